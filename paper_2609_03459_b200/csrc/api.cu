@@ -634,7 +634,7 @@ static int backward_any(tt_emb* h, const float* grad_out, float* const* core_gra
         int mask = 1 << (K - 1);                     // last core: the fixed-order sum of the stripes
         for (int k = 2; k <= K - 1; ++k)
             if (td.midfast[k] >= 0) mask |= 1 << (k - 1);   // middle cores: the slice's owner CTA
-        if (K >= 3 && td.midfast[2] >= 0) mask |= 1;        // first core: the sum over the children of a first digit
+        if (K >= 3) mask |= 1;                              // first core: the sum over the children of a first digit
         td.sgd_mask = mask;
         if (mask != (1 << K) - 1) rest = true;
     }

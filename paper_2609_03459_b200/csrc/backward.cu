@@ -1447,111 +1447,6 @@ __global__ void k_tfill(WsView w, int k)
     }
 }
 
-// dP_{k-1}[parent] (or the first core's gradient slice when k = 2) = sum over children v of
-//   out[m][a] = sum_{j,b} dP_k[v][(m*d_k + j)*r_k + b] * G_k[i_k(v)][a][j][b]
-// one CTA per parent, children in sorted order; the slice is staged in shared memory (padded rows)
-__global__ void __launch_bounds__(256) k_mid_down(WsView w, int k)
-{
-    tt_pdl_enter();
-    extern __shared__ float sm[];
-    const uint32_t count = w.counters[CTR_LEVEL0 + k - 1];
-    for (uint32_t pn = blockIdx.x; pn < count; pn += gridDim.x) {
-        const int t = tt_find_table(w.tb[k - 1], w.T, pn);
-        const TableDesc& td = w.tdesc[t];
-        if (td.midfast[k] >= 0) continue;  // handled by k_mid_mma + k_mid_sum
-        const int kc = k - 1;
-        const int M = td.P[kc], ra = td.r[kc], cols = td.d[kc] * td.r[kc + 1];
-        const int ld = cols + 1;
-        float* Bs = sm;                  // ra * ld
-        float* dPs = sm + ra * ld;       // M * cols
-        const int nout = M * ra;
-        // each thread owns outputs o = tid, tid + 256, ... (at most 16 per thread: M*ra <= 4096)
-        float acc[16];
-#pragma unroll
-        for (int i = 0; i < 16; ++i) acc[i] = 0.f;
-        const uint32_t c0 = w.cstart[k - 1][pn], c1 = w.cstart[k - 1][pn + 1];
-        for (uint32_t v = c0; v < c1; ++v) {
-            const uint32_t ik = w.val[k][v] % (uint32_t)td.n[kc];
-            const float* Bsl = td.core[kc] + (size_t)ik * td.slice_floats[kc];
-            for (int i = threadIdx.x; i < ra * cols; i += blockDim.x) Bs[(i / cols) * ld + (i % cols)] = __ldg(Bsl + i);
-            const float* dp = w.dP[k] + (size_t)v * w.stride[k];
-            for (int i = threadIdx.x; i < M * cols; i += blockDim.x) dPs[i] = dp[i];
-            __syncthreads();
-#pragma unroll
-            for (int i = 0; i < 16; ++i) {
-                const int o = threadIdx.x + i * 256;
-                if (o < nout) {
-                    const int m = o / ra, a = o - m * ra;
-                    const float* x = dPs + m * cols;
-                    const float* y = Bs + a * ld;
-                    float s = 0.f;
-                    for (int c = 0; c < cols; ++c) s = fmaf(x[c], y[c], s);
-                    acc[i] += s;
-                }
-            }
-            __syncthreads();
-        }
-        float* dst;
-        if (k == 2) dst = td.grad[0] + (size_t)w.val[1][pn] * td.slice_floats[0];
-        else dst = w.dP[k - 1] + (size_t)pn * w.stride[k - 1];
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            const int o = threadIdx.x + i * 256;
-            if (o < nout) dst[o] = acc[i];
-        }
-    }
-}
-
-// gradient of slice i_k of core k (1-based, 2 <= k <= K-1) of table t:
-//   dG_k[i_k][a][c] = sum over level-k nodes v with digit i_k of sum_m P_{k-1}[parent(v)][m][a] * dP_k[v][m*cols + c]
-// one CTA per (table, slice); nodes come from the digit-major list, i.e. in ascending parent order
-__global__ void __launch_bounds__(256) k_mid_slice(WsView w, int k)
-{
-    tt_pdl_enter();
-    extern __shared__ float sm[];
-    const int t = blockIdx.y;
-    const TableDesc& td = w.tdesc[t];
-    const int kc = k - 1;
-    if ((int)blockIdx.x >= td.n[kc] || td.midfast[k] >= 0) return;
-    const uint32_t ik = blockIdx.x;
-    const int M = td.P[kc], ra = td.r[kc], cols = td.d[kc] * td.r[kc + 1];
-    const int nout = ra * cols;
-    float* Pls = sm;             // M * ra
-    float* dPs = sm + M * ra;    // M * cols
-    const uint32_t space = td.prefix_space[k - 1];
-    const uint32_t j0 = tt_trank(w, td, k, ik * space), j1 = tt_trank(w, td, k, (ik + 1) * space);
-    float* dst = td.grad[kc] + (size_t)ik * td.slice_floats[kc];
-    for (int o0 = 0; o0 < nout; o0 += 256 * 16) {
-        float acc[16];
-#pragma unroll
-        for (int i = 0; i < 16; ++i) acc[i] = 0.f;
-        for (uint32_t jn = j0; jn < j1; ++jn) {
-            const uint32_t v = w.tnode[k][jn];
-            const float* pl = tt_left_operand(w, td, k, v);
-            for (int i = threadIdx.x; i < M * ra; i += blockDim.x) Pls[i] = pl[i];
-            const float* dp = w.dP[k] + (size_t)v * w.stride[k];
-            for (int i = threadIdx.x; i < M * cols; i += blockDim.x) dPs[i] = dp[i];
-            __syncthreads();
-#pragma unroll
-            for (int i = 0; i < 16; ++i) {
-                const int o = o0 + threadIdx.x + i * 256;
-                if (o < nout) {
-                    const int a = o / cols, c = o - a * cols;
-                    float s = 0.f;
-                    for (int m = 0; m < M; ++m) s = fmaf(Pls[m * ra + a], dPs[m * cols + c], s);
-                    acc[i] += s;
-                }
-            }
-            __syncthreads();
-        }
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            const int o = o0 + threadIdx.x + i * 256;
-            if (o < nout) dst[o] = acc[i];
-        }
-    }
-}
-
 // ---- tensor-core middle-core backward (P_{k-1} = 4 or 2 rows, r_{k-1} in {16,32}, d_k * r_k in {32,64,128}) ----
 //
 // One CTA of 4 warps per (table, slice i_k).  The nodes with digit i_k arrive in ascending parent order from the
@@ -1802,6 +1697,264 @@ __global__ void __launch_bounds__(128, 5) k_mid_mma(WsView w, int k, int variant
     fold(true);   // also writes the zeros of a slice without nodes
 }
 
+// ---- tensor-core middle-core backward for every other shape (any M = P_{k-1}, r_{k-1}, d_k * r_k) ----
+//
+// The same two products as k_mid_mma, cut into 64 x 64 output tiles so that wide slices spread over the SMs (rank 64:
+// 64 slices of 64 x 256, i.e. 256 tiles of dG) and narrow ones fit one tile:
+//   z < dgz   one tile of dG_k[i_k]: 64 values of a by 64 columns; k runs over the slice's stacked rows (node, m), 32 per
+//             pass, staged with cp.async in two buffers, row addresses looked up two passes ahead
+//   z >= dgz  Y: tiles of 64 stacked rows by 64 values of a, dealt out to the slice's `yctas` CTAs; k runs over the
+//             columns, 32 per pass
+// A warp owns a 32 x 32 quarter of the tile (8 fragment loads per k step for 8 tile products of 3xTF32); row tiles and
+// column blocks outside the shape are skipped.  Pitches of 72 (fragments run down the rows) and 36 floats (along the
+// rows) keep the fragment loads free of bank conflicts.  Every k step is added in rounded fp32
+// (tt_mma_3xtf32_rounded).  No fused update of the slice: the Y CTAs of other tiles still read it.
+// Bound by the operand path (16 fragment loads for 24 tensor instructions) and, for short node lists, by a CTA's look-ups.
+// Middle stage, 2x4x4x4 with rank 64 (65 536 lookups): 5.05 ms with one FP32 thread per output element over the whole
+// node list, 0.16 ms as tiles; 3x3x5 with ranks 6 and 4 (4 tables, 1 M lookups): 0.41 and 0.06 ms.
+#define MT_EDGE 64
+#define MT_KROWS 32
+#define MT_PA (MT_EDGE + 8)
+#define MT_PC (MT_KROWS + 4)
+
+// 4-byte asynchronous copy global -> shared
+__device__ __forceinline__ void tt_cp_async4(void* smem_dst, const void* gsrc)
+{
+    const unsigned d = (unsigned)__cvta_generic_to_shared(smem_dst);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d), "l"(gsrc) : "memory");
+}
+
+// dst[row][0 .. 4 * W4) = src[row][off .. off + avail), the rest of the row (and rows without a source) zero; 128 threads
+template <int ROWS, int W4>
+__device__ __forceinline__ void tt_stage_rows(float* dst, int pitch, const float* const* src, int off, int avail, bool vec)
+{
+    if (vec) {
+        for (int i = threadIdx.x; i < ROWS * W4; i += 128) {
+            const int row = i / W4, c4 = i % W4;
+            const float* p = src[row];
+            float* d = dst + row * pitch + 4 * c4;
+            if (p && 4 * c4 < avail) tt_cp_async16(d, p + off + 4 * c4);
+            else *reinterpret_cast<float4*>(d) = make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+    } else {
+        for (int i = threadIdx.x; i < ROWS * W4 * 4; i += 128) {
+            const int row = i / (W4 * 4), c = i % (W4 * 4);
+            const float* p = src[row];
+            float* d = dst + row * pitch + c;
+            if (p && c < avail) tt_cp_async4(d, p + off + c);
+            else *d = 0.f;
+        }
+    }
+}
+
+// sum += A . B over 8 k values: mtl row tiles of 16, ntl column blocks of 8.  The A fragment of row tile mt is
+// {a0, a1, a2, a3}[16 mt * astep], the B fragment of block nt {b0, b1}[8 nt * bstep]
+__device__ __forceinline__ void tt_quarter_step(float (&sum)[2][4][4], const float* a0, const float* a1, const float* a2, const float* a3,
+                                                int astep, const float* b0, const float* b1, int bstep, int mtl, int ntl)
+{
+    Tf32Pair a[2][4];
+#pragma unroll
+    for (int mt = 0; mt < 2; ++mt)
+        if (mt < mtl) {
+            a[mt][0] = tt_split_tf32(a0[16 * mt * astep]);
+            a[mt][1] = tt_split_tf32(a1[16 * mt * astep]);
+            a[mt][2] = tt_split_tf32(a2[16 * mt * astep]);
+            a[mt][3] = tt_split_tf32(a3[16 * mt * astep]);
+        }
+#pragma unroll
+    for (int nt = 0; nt < 4; ++nt)
+        if (nt < ntl) {
+            Tf32Pair b[2];
+            b[0] = tt_split_tf32(b0[8 * nt * bstep]);
+            b[1] = tt_split_tf32(b1[8 * nt * bstep]);
+#pragma unroll
+            for (int mt = 0; mt < 2; ++mt)
+                if (mt < mtl) tt_mma_3xtf32_rounded(sum[mt][nt], a[mt], b);
+        }
+}
+
+__global__ void __launch_bounds__(128, 4) k_mid_tile(WsView w, int k, int lbase, int dgz, int yctas)
+{
+    tt_pdl_enter();
+    __shared__ __align__(16) float sm[2 * 2 * MT_EDGE * MT_PC];   // = 2 * 2 * MT_KROWS * MT_PA
+    static_assert(MT_EDGE * MT_PC == MT_KROWS * MT_PA, "both roles stage the same number of floats");
+    constexpr int STAGE = MT_EDGE * MT_PC;
+    const TableDesc& td = w.tdesc[w.vlist[lbase + blockIdx.y]];
+    const int kc = k - 1;
+    if ((int)blockIdx.x >= td.n[kc]) return;
+    const uint32_t ik = blockIdx.x;
+    const int M = td.P[kc], ra = td.r[kc], cols = td.d[kc] * td.r[kc + 1];
+    const bool vec = (ra & 3) == 0 && (cols & 3) == 0;   // then every row, node and slice starts on a 16-byte boundary
+    const uint32_t space = td.prefix_space[k - 1];
+    const uint32_t j0 = tt_trank(w, td, k, ik * space), j1 = tt_trank(w, td, k, (ik + 1) * space);
+    const uint32_t R = (j1 - j0) * (uint32_t)M;          // stacked rows
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, g = lane >> 2, t = lane & 3;
+    const int wr = wid >> 1, wc = wid & 1;               // this warp's quarter
+    const int ach = (ra + MT_EDGE - 1) / MT_EDGE;
+    float sum[2][4][4];
+#pragma unroll
+    for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+        for (int nt = 0; nt < 4; ++nt)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) sum[mt][nt][i] = 0.f;
+
+    if ((int)blockIdx.z < dgz) {
+        // ------------------------------------------------------------------------------ a tile of the slice gradient
+        const int cch = (cols + MT_EDGE - 1) / MT_EDGE;
+        if ((int)blockIdx.z >= ach * cch) return;
+        const int a0 = (int)blockIdx.z / cch * MT_EDGE, c0 = (int)blockIdx.z % cch * MT_EDGE;
+        const int mtl = min(2, max(0, (ra - a0 - 32 * wr + 15) / 16)), ntl = min(4, max(0, (cols - c0 - 32 * wc + 7) / 8));
+        __shared__ const float* s_a[3][MT_KROWS];
+        __shared__ const float* s_d[3][MT_KROWS];
+        const uint32_t passes = (R + MT_KROWS - 1) / MT_KROWS;
+        auto lookup = [&](uint32_t r, const float*& pa, const float*& pd) {   // threads 0..31: row r * 32 + tid
+            pa = nullptr; pd = nullptr;
+            const uint32_t row = r * MT_KROWS + lane;
+            if (row < R) {
+                const uint32_t jn = row / (uint32_t)M, m = row - jn * (uint32_t)M;
+                const uint32_t v = w.tnode[k][j0 + jn];
+                pa = tt_left_operand(w, td, k, v) + (size_t)m * ra + a0;
+                pd = w.dP[k] + (size_t)v * w.stride[k] + (size_t)m * cols + c0;
+            }
+        };
+        auto issue = [&](uint32_t r) {
+            float* st = sm + (r & 1u) * (2 * STAGE);
+            tt_stage_rows<MT_KROWS, MT_EDGE / 4>(st, MT_PA, s_a[r % 3u], 0, ra - a0, vec);
+            tt_stage_rows<MT_KROWS, MT_EDGE / 4>(st + STAGE, MT_PA, s_d[r % 3u], 0, cols - c0, vec);
+            asm volatile("cp.async.commit_group;" ::: "memory");
+        };
+        if (wid < 2) {   // passes 0 and 1 side by side
+            const float *pa, *pd;
+            lookup((uint32_t)wid, pa, pd);
+            s_a[wid][lane] = pa;
+            s_d[wid][lane] = pd;
+        }
+        __syncthreads();
+        if (passes > 0) issue(0);
+        for (uint32_t r = 0; r < passes; ++r) {
+            const float *pa = nullptr, *pd = nullptr;
+            if (wid == 0) lookup(r + 2, pa, pd);
+            if (r + 1 < passes) {
+                issue(r + 1);
+                asm volatile("cp.async.wait_group 1;" ::: "memory");
+            } else {
+                asm volatile("cp.async.wait_group 0;" ::: "memory");
+            }
+            __syncthreads();
+            if (mtl > 0 && ntl > 0) {
+                const float* A = sm + (r & 1u) * (2 * STAGE) + 32 * wr + g;
+                const float* D = sm + (r & 1u) * (2 * STAGE) + STAGE + 32 * wc + g;
+#pragma unroll
+                for (int p = 0; p < MT_KROWS / 8; ++p) {
+                    if (r * MT_KROWS + 8 * p >= R) break;
+                    const float* Aa = A + (8 * p + t) * MT_PA;
+                    const float* Da = D + (8 * p + t) * MT_PA;
+                    tt_quarter_step(sum, Aa, Aa + 8, Aa + 4 * MT_PA, Aa + 4 * MT_PA + 8, 1, Da, Da + 4 * MT_PA, 1, mtl, ntl);
+                }
+            }
+            if (wid == 0) { s_a[(r + 2) % 3u][lane] = pa; s_d[(r + 2) % 3u][lane] = pd; }   // the ring slot of pass r - 1
+            __syncthreads();
+        }
+        float* const dst = td.grad[kc] + (size_t)ik * td.slice_floats[kc];
+#pragma unroll
+        for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+            for (int nt = 0; nt < 4; ++nt)
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int a = a0 + 32 * wr + 16 * mt + 8 * h + g, c = c0 + 32 * wc + 8 * nt + 2 * t;
+                    if (a >= ra || c >= cols) continue;
+                    float* d = dst + (size_t)a * cols + c;
+                    if (vec) *reinterpret_cast<float2*>(d) = make_float2(sum[mt][nt][2 * h], sum[mt][nt][2 * h + 1]);
+                    else {
+                        d[0] = sum[mt][nt][2 * h];
+                        if (c + 1 < cols) d[1] = sum[mt][nt][2 * h + 1];
+                    }
+                }
+        return;
+    }
+
+    // ---------------------------------------------------------------------------------- tiles of Y
+    __shared__ const float* s_row[MT_EDGE];    // dP row of each stacked row
+    __shared__ const float* s_core[MT_EDGE];   // row of the slice for each a
+    __shared__ float* s_out[MT_EDGE];
+    const uint32_t items = (R + MT_EDGE - 1) / MT_EDGE * (uint32_t)ach;
+    const int cpasses = (cols + MT_KROWS - 1) / MT_KROWS;
+    for (uint32_t it = blockIdx.z - (uint32_t)dgz; it < items; it += (uint32_t)yctas) {
+        const int a0 = (int)(it % (uint32_t)ach) * MT_EDGE;
+        const uint32_t row0 = it / (uint32_t)ach * MT_EDGE;
+        if (tid < MT_EDGE) {
+            const uint32_t row = row0 + tid;
+            const float* pd = nullptr;
+            float* py = nullptr;
+            if (row < R) {
+                const uint32_t jn = row / (uint32_t)M, m = row - jn * (uint32_t)M;
+                const uint32_t v = w.tnode[k][j0 + jn];
+                pd = w.dP[k] + (size_t)v * w.stride[k] + (size_t)m * cols;
+                py = w.Y[k] + (size_t)v * w.stride[k - 1] + (size_t)m * ra;
+            }
+            s_row[tid] = pd;
+            s_out[tid] = py;
+        } else {
+            const int a = a0 + tid - MT_EDGE;
+            s_core[tid - MT_EDGE] = a < ra ? td.core[kc] + (size_t)ik * td.slice_floats[kc] + (size_t)a * cols : nullptr;
+        }
+        __syncthreads();
+        const int mtl = min(2, max(0, (int)(min(R - row0, (uint32_t)MT_EDGE) - 32 * wr + 15) / 16));
+        const int ntl = min(4, max(0, (ra - a0 - 32 * wc + 7) / 8));
+        auto issue = [&](int c) {
+            float* st = sm + (c & 1) * (2 * STAGE);
+            const int off = c * MT_KROWS, avail = cols - off;
+            tt_stage_rows<MT_EDGE, MT_KROWS / 4>(st, MT_PC, s_row, off, avail, vec);
+            tt_stage_rows<MT_EDGE, MT_KROWS / 4>(st + STAGE, MT_PC, s_core, off, avail, vec);
+            asm volatile("cp.async.commit_group;" ::: "memory");
+        };
+        issue(0);
+        for (int c = 0; c < cpasses; ++c) {
+            if (c + 1 < cpasses) {
+                issue(c + 1);
+                asm volatile("cp.async.wait_group 1;" ::: "memory");
+            } else {
+                asm volatile("cp.async.wait_group 0;" ::: "memory");
+            }
+            __syncthreads();
+            if (mtl > 0 && ntl > 0) {
+                const float* D = sm + (c & 1) * (2 * STAGE) + (32 * wr + g) * MT_PC + t;
+                const float* B = sm + (c & 1) * (2 * STAGE) + STAGE + (32 * wc + g) * MT_PC + t;
+#pragma unroll
+                for (int p = 0; p < MT_KROWS / 8; ++p) {
+                    if (c * MT_KROWS + 8 * p >= cols) break;
+                    const float* Da = D + 8 * p;
+                    const float* Ba = B + 8 * p;
+                    tt_quarter_step(sum, Da, Da + 8 * MT_PC, Da + 4, Da + 8 * MT_PC + 4, MT_PC, Ba, Ba + 4, MT_PC, mtl, ntl);
+                }
+            }
+            __syncthreads();
+        }
+#pragma unroll
+        for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                float* out = s_out[32 * wr + 16 * mt + 8 * h + g];
+#pragma unroll
+                for (int nt = 0; nt < 4; ++nt) {
+                    const int a = a0 + 32 * wc + 8 * nt + 2 * t;
+                    if (out && a < ra) {
+                        if (vec) *reinterpret_cast<float2*>(out + a) = make_float2(sum[mt][nt][2 * h], sum[mt][nt][2 * h + 1]);
+                        else {
+                            out[a] = sum[mt][nt][2 * h];
+                            if (a + 1 < ra) out[a + 1] = sum[mt][nt][2 * h + 1];
+                        }
+                    }
+                    sum[mt][nt][2 * h] = 0.f;
+                    sum[mt][nt][2 * h + 1] = 0.f;
+                }
+            }
+        __syncthreads();   // the addresses are rewritten for the next tile
+    }
+}
+
 // dP_{k-1}[parent] (k = 2: the first core's gradient slice) = sum of the Y rows of the parent's children,
 // which are contiguous in sorted order; one warp per parent
 __global__ void __launch_bounds__(256) k_mid_sum(WsView w, int k)
@@ -1814,10 +1967,21 @@ __global__ void __launch_bounds__(256) k_mid_sum(WsView w, int k)
     for (uint32_t pn = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; pn < count; pn += nwarps) {
         const int t = tt_find_table(w.tb[k - 1], w.T, pn);
         const TableDesc& td = w.tdesc[t];
-        if (td.midfast[k] < 0) continue;
-        const int nout4 = td.P[k - 1] * td.r[k - 1] / 4;
+        const int nout = td.P[k - 1] * td.r[k - 1], nout4 = nout / 4;
         const uint32_t c0 = w.cstart[k - 1][pn], c1 = w.cstart[k - 1][pn + 1];
         float* dst = k == 2 ? td.grad[0] + (size_t)w.val[1][pn] * td.slice_floats[0] : w.dP[k - 1] + (size_t)pn * w.stride[k - 1];
+        if (nout & 3) {   // slices of the first core are not 16-byte aligned
+            for (int f = lane; f < nout; f += 32) {
+                float s = 0.f;
+                for (uint32_t v = c0; v < c1; ++v) s += __ldg(w.Y[k] + (size_t)v * strideY + f);
+                dst[f] = s;
+                if (k == 2 && w.fused_lr != 0.f) {
+                    float* c = td.core[0] + (size_t)w.val[1][pn] * td.slice_floats[0] + f;
+                    *c = *c - w.fused_lr * s;
+                }
+            }
+            continue;
+        }
         for (int f = lane; f < nout4; f += 32) {
             float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
             for (uint32_t v = c0; v < c1; ++v) {
@@ -1866,25 +2030,26 @@ cudaError_t tt_launch_bwd_middle(tt_emb* h, cudaStream_t s)
     WsView& w = h->v;
     cudaError_t e;
     for (int k = h->K - 1; k >= 2; --k) {
-        int max_n = 1, max_down = 1, max_slice = 1;
-        bool any_generic = false, any_fast[11] = {false, false, false, false, false, false, false, false, false, false, false};
+        bool any_fast[TT_NUM_MIDFAST] = {};
+        int dgz = 1, tile_rows = 1;   // generic shapes: tiles of the slice gradient, most stacked rows of a slice
         for (int t = 0; t < h->T; ++t) {
             const TableDesc& td = h->tab[t];
             const int kc = k - 1;
-            const int M = td.P[kc], ra = td.r[kc], cols = td.d[kc] * td.r[kc + 1];
-            if (td.n[kc] > max_n) max_n = td.n[kc];
-            if (ra * (cols + 1) + M * cols > max_down) max_down = ra * (cols + 1) + M * cols;
-            if (M * ra + M * cols > max_slice) max_slice = M * ra + M * cols;
-            if (td.midfast[k] < 0) any_generic = true; else any_fast[td.midfast[k]] = true;
+            if (td.midfast[k] >= 0) { any_fast[td.midfast[k]] = true; continue; }
+            const int tiles = ((td.r[kc] + MT_EDGE - 1) / MT_EDGE) * ((td.d[kc] * td.r[kc + 1] + MT_EDGE - 1) / MT_EDGE);
+            if (tiles > dgz) dgz = tiles;
+            const int64_t rows = (int64_t)(td.prefix_space[k - 1] < w.cap[k] ? td.prefix_space[k - 1] : w.cap[k]) * td.P[kc];
+            const int64_t yt = (rows + MT_EDGE - 1) / MT_EDGE * ((td.r[kc] + MT_EDGE - 1) / MT_EDGE);
+            if (yt > tile_rows) tile_rows = (int)(yt < 65535 ? yt : 65535);
         }
+        const int ngen = h->mcount[k][0];
         // level K-1's digit-major list already exists: the forward built it to order its sweep
         if (k != h->K - 1 && (e = tt_launch_tlist(h, k, s)) != cudaSuccess) return e;
-        const dim3 sg(max_n, h->T);
         // the shape variants are independent (different tables): run them side by side so that the tail of one
         // (a few long node lists) overlaps the others
         int nfast = 0;
-        for (int v = 0; v < 11; ++v) nfast += any_fast[v] ? 1 : 0;
-        const bool fork = nfast > 1 && !h->serial;
+        for (int v = 0; v < TT_NUM_MIDFAST; ++v) nfast += any_fast[v] ? 1 : 0;
+        const bool fork = nfast + (ngen > 0 ? 1 : 0) > 1 && !h->serial;
         if (fork && (e = tt_fork(h, s, 4)) != cudaSuccess) return e;
         int slot = 0;
         auto st = [&]() { return fork ? h->side[(slot++) & 3] : s; };
@@ -1902,19 +2067,17 @@ cudaError_t tt_launch_bwd_middle(tt_emb* h, cudaStream_t s)
         if (any_fast[8]) { if ((e = tt_launch_mid<4, 8, 32>(mgrid(8), st(), w, k, 8, mlist(8))) != cudaSuccess) return e; tt_note_launch(); }
         if (any_fast[9]) { if ((e = tt_launch_mid<2, 8, 32>(mgrid(9), st(), w, k, 9, mlist(9))) != cudaSuccess) return e; tt_note_launch(); }
         if (any_fast[10]) { if ((e = tt_launch_mid<2, 8, 16>(mgrid(10), st(), w, k, 10, mlist(10))) != cudaSuccess) return e; tt_note_launch(); }
+        if (ngen > 0) {
+            // Y tiles: as many CTAs per slice as fill the SMs about four times over, no more than there can be tiles
+            const int slices = h->mmaxn[k][0] * ngen;
+            int yctas = (h->sm_count * 16 + slices - 1) / slices;
+            if (yctas > tile_rows) yctas = tile_rows;
+            if ((e = tt_launch_pdl(k_mid_tile, dim3(h->mmaxn[k][0], ngen, dgz + yctas), dim3(128), 0, st(), w, k, mlist(-1), dgz, yctas)) != cudaSuccess) return e;
+            tt_note_launch();
+        }
         if (fork && (e = tt_join(h, s, 4)) != cudaSuccess) return e;
-        if (nfast > 0) {
-            if ((e = tt_launch_pdl(k_mid_sum, dim3(h->sm_count * 8), dim3(256), 0, s, w, k)) != cudaSuccess) return e;
-            tt_note_launch();
-        }
-        if (any_generic) {
-            if ((e = cudaFuncSetAttribute(k_mid_slice, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(max_slice * sizeof(float)))) != cudaSuccess) return e;
-            k_mid_slice<<<sg, 256, (size_t)max_slice * sizeof(float), s>>>(w, k);
-            tt_note_launch();
-            if ((e = cudaFuncSetAttribute(k_mid_down, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(max_down * sizeof(float)))) != cudaSuccess) return e;
-            k_mid_down<<<h->sm_count * 8, 256, (size_t)max_down * sizeof(float), s>>>(w, k);
-            tt_note_launch();
-        }
+        if ((e = tt_launch_pdl(k_mid_sum, dim3(h->sm_count * 8), dim3(256), 0, s, w, k)) != cudaSuccess) return e;
+        tt_note_launch();
     }
     return cudaGetLastError();
 }

@@ -42,3 +42,19 @@ __device__ __forceinline__ void tt_mma_3xtf32(float (&d)[4], const Tf32Pair (&a)
     tt_mma_tf32(d, a[0].hi, a[1].hi, a[2].hi, a[3].hi, b[0].lo, b[1].lo);
     tt_mma_tf32(d, a[0].hi, a[1].hi, a[2].hi, a[3].hi, b[0].hi, b[1].hi);
 }
+
+// sum += A.B with the product formed from zero and added in fp32.  The tensor core truncates when it adds into its
+// accumulator, so a chain of products drifts towards zero; here only the three products of one k step share an
+// accumulator (the two small ones first) and the sums over k are rounded, as in a chain of fmaf.
+__device__ __forceinline__ void tt_mma_3xtf32_rounded(float (&sum)[4], const Tf32Pair (&a)[4], const Tf32Pair (&b)[2])
+{
+    float d[4];
+    asm volatile(
+        "mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%10,%10,%10};"
+        : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+        : "r"(a[0].lo), "r"(a[1].lo), "r"(a[2].lo), "r"(a[3].lo), "r"(b[0].hi), "r"(b[1].hi), "f"(0.f));
+    tt_mma_tf32(d, a[0].hi, a[1].hi, a[2].hi, a[3].hi, b[0].lo, b[1].lo);
+    tt_mma_tf32(d, a[0].hi, a[1].hi, a[2].hi, a[3].hi, b[0].hi, b[1].hi);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) sum[i] += d[i];
+}
