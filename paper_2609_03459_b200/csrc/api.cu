@@ -449,7 +449,7 @@ extern "C" int tt_emb_bind(tt_emb_t h, float* const* core_ptrs, void* workspace,
             v.dP[k] = (float*)(base + h->off_dP[k]);
             v.Y[k] = (float*)(base + h->off_Y[k]);
         }
-        v.carry = (float*)(base + h->off_carry);
+        h->carry = (float*)(base + h->off_carry);
         v.gpart = (float*)(base + h->off_gpart);
         v.gpart_stride = h->gpart_floats > 0 ? h->gpart_floats : 4;
     }

@@ -20,6 +20,7 @@
 #include "scan.cuh"
 #include "mma.cuh"
 #include "quad_mid.cuh"
+#include <type_traits>
 
 #define HT_SIZE 4096
 #define HT_TILE 2048
@@ -230,6 +231,13 @@ struct RowAcc {
             }
         }
     }
+    // v += the first piece (CPL = 1) of a row in shared memory
+    __device__ void add_shared(const void* x)
+    {
+        const float* f = reinterpret_cast<const float*>(x);
+#pragma unroll
+        for (int i = 0; i < (VEC ? 4 : 1); ++i) v[i] += f[i];
+    }
     __device__ void store(float* __restrict__ row, int D, int lane) const
     {
         if (VEC) {
@@ -253,14 +261,15 @@ template <bool VEC, int CPL>
 __global__ void __launch_bounds__(256) k_dE(WsView w, const float* __restrict__ grad_out)
 {
     tt_pdl_enter();
+    constexpr int NF = !VEC && CPL <= 4 ? 16 / CPL : 4;   // narrow rows: more of them in flight
     const int lane = threadIdx.x & 31;
     const int64_t chunk = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const uint32_t U = w.counters[CTR_LEVEL0 + w.K];
     const uint32_t Ltot = w.cnt[U];
-    const int64_t a64 = chunk * TT_DE_CHUNK;
+    const int64_t a64 = chunk * w.de_chunk;
     if (a64 >= Ltot) return;
     const uint32_t a = (uint32_t)a64;
-    const uint32_t b = min(a + (uint32_t)TT_DE_CHUNK, Ltot);
+    const uint32_t b = min(a + w.de_chunk, Ltot);
     const int D = w.D;
     const size_t gstride = (size_t)w.T * D;
     const uint32_t prev = a > 0 ? w.pairs[a - 1].x : HT_EMPTY;
@@ -276,13 +285,13 @@ __global__ void __launch_bounds__(256) k_dE(WsView w, const float* __restrict__ 
         const bool weighted = w.wsorted && (w.psw || w.pool_mean);
         const float wmine = (weighted && p0 + lane < b) ? __ldg(&w.wsorted[p0 + lane]) : 1.f;
         const int n = (int)min(32u, b - p0);
-        // four rows of grad_out in flight at a time (their addresses need the table of each pair's slot; positions are
+        // NF rows of grad_out in flight at a time (their addresses need the table of each pair's slot; positions are
         // sorted, so the table changes rarely), then the rows are folded in position order
         const int tmine = lane < n ? tt_find_table_from(w.tb[w.K], w.T, mine.x, tcur) : tcur;
-        for (int j0 = 0; j0 < n; j0 += 4) {
-            RowAcc<VEC, CPL> rowv[4];
+        for (int j0 = 0; j0 < n; j0 += NF) {
+            RowAcc<VEC, CPL> rowv[NF];
 #pragma unroll
-            for (int jj = 0; jj < 4; ++jj) {
+            for (int jj = 0; jj < NF; ++jj) {
                 const int j = min(j0 + jj, n - 1);
                 const uint32_t bag = __shfl_sync(0xffffffffu, mine.y, j);
                 const int tj = __shfl_sync(0xffffffffu, tmine, j);
@@ -290,7 +299,7 @@ __global__ void __launch_bounds__(256) k_dE(WsView w, const float* __restrict__ 
                 if (j0 + jj < n) rowv[jj].add_row(grad_out + (size_t)bag * gstride + (size_t)tj * D, D, lane, 1.f);
             }
 #pragma unroll
-            for (int jj = 0; jj < 4; ++jj) {
+            for (int jj = 0; jj < NF; ++jj) {
                 const int j = j0 + jj;
                 if (j >= n) break;
                 const uint32_t sl = __shfl_sync(0xffffffffu, mine.x, j);
@@ -316,53 +325,84 @@ __global__ void __launch_bounds__(256) k_dE(WsView w, const float* __restrict__ 
     else acc.store(w.E + (size_t)cur * D, D, lane);
 }
 
-// the chunk in which a border-crossing segment starts adds up the pieces in position order
+// The chunk in which a border-crossing segment starts adds up its pieces: its own tail, the tails of the chunks that the
+// segment fills, the head in the chunk where it ends (the sort has left the segment's end in cnt).  A warp adds a few
+// pieces by itself; a popular row spans hundreds of chunks, and one warp would walk them one memory round trip after the
+// other, so those are left to the whole CTA: 256 threads as 256 / (D / VEC) piece slots side by side, each with every
+// slots-th piece, then the slots in order.  (One warp per row: 4 M lookups,
+// D = 16, dE 187 us in chunks of 512 and 302 us in chunks of 128; now 142 and 121 us.)
+#define DE_FIX_OWN 8    // pieces that a warp adds by itself
 template <bool VEC, int CPL>
 __global__ void __launch_bounds__(256) k_dE_fix(WsView w)
 {
     tt_pdl_enter();
+    using piece_t = typename std::conditional<VEC, float4, float>::type;
+    __shared__ piece_t s_part[256];
+    __shared__ uint32_t s_chunk[8], s_slot[8], s_pieces[8];
+    __shared__ uint32_t s_n;
+    if (threadIdx.x == 0) s_n = 0;
+    __syncthreads();
     const int lane = threadIdx.x & 31;
     const int64_t chunk = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const uint32_t U = w.counters[CTR_LEVEL0 + w.K];
     const uint32_t Ltot = w.cnt[U];
-    const int64_t a64 = chunk * TT_DE_CHUNK;
-    if (a64 >= Ltot) return;
-    const uint32_t a = (uint32_t)a64;
-    const uint32_t b = min(a + (uint32_t)TT_DE_CHUNK, Ltot);
-    if (b >= Ltot) return;
-    const uint32_t first = w.pairs[a].x, last = w.pairs[b - 1].x;
-    const uint32_t prev = a > 0 ? w.pairs[a - 1].x : HT_EMPTY;
-    const uint32_t next = w.pairs[b].x;
-    if (next != last) return;                         // nothing continues past this chunk
-    if (first == last && prev == first) return;       // the segment started earlier: not the owner
+    const int64_t a64 = chunk * w.de_chunk;
     const int D = w.D;
-    RowAcc<VEC, CPL> acc;
-    acc.clear();
-    acc.add_row(w.carry + ((size_t)chunk * 2 + 1) * D, D, lane);
-    const int64_t nchunks = ((int64_t)Ltot + TT_DE_CHUNK - 1) / TT_DE_CHUNK;
-    // A popular row spans thousands of chunks.  Look at 32 following chunks at once: every lane classifies one
-    // ("whole chunk is this row and it goes on" = a tail piece to add; otherwise its head piece ends the row),
-    // a ballot finds where the row ends, and the pieces are added in position order.
-    for (int64_t c0 = chunk + 1; c0 < nchunks; c0 += 32) {
-        const int64_t c2 = c0 + lane;
-        bool through = false;
-        if (c2 < nchunks) {
-            const uint32_t a2 = (uint32_t)(c2 * TT_DE_CHUNK);
-            const uint32_t b2 = min(a2 + (uint32_t)TT_DE_CHUNK, Ltot);
-            const uint32_t last2 = w.pairs[b2 - 1].x;
-            const uint32_t next2 = b2 < Ltot ? w.pairs[b2].x : HT_EMPTY;
-            through = last2 == last && next2 == last;
-        }
-        const unsigned stops = __ballot_sync(0xffffffffu, !through);   // chunks beyond the end count as stops
-        const int nthrough = stops ? __ffs(stops) - 1 : 32;
-#pragma unroll 8
-        for (int i = 0; i < nthrough; ++i) acc.add_row(w.carry + ((size_t)(c0 + i) * 2 + 1) * D, D, lane);
-        if (nthrough < 32) {
-            if (c0 + nthrough < nchunks) acc.add_row(w.carry + (size_t)(c0 + nthrough) * 2 * D, D, lane);
-            break;
+    if (a64 < Ltot) {
+        const uint32_t a = (uint32_t)a64;
+        const uint32_t b = min(a + w.de_chunk, Ltot);
+        const uint32_t first = w.pairs[a].x, last = w.pairs[b - 1].x;
+        const uint32_t prev = a > 0 ? w.pairs[a - 1].x : HT_EMPTY;
+        const uint32_t next = b < Ltot ? w.pairs[b].x : HT_EMPTY;
+        // something continues past this chunk, and it started here
+        if (b < Ltot && next == last && !(first == last && prev == first)) {
+            const uint32_t pieces = (w.cnt[last] - 1u) / w.de_chunk - (uint32_t)chunk + 1u;
+            if (pieces > DE_FIX_OWN) {
+                if (lane == 0) {
+                    const uint32_t i = atomicAdd(&s_n, 1u);
+                    s_chunk[i] = (uint32_t)chunk;
+                    s_slot[i] = last;
+                    s_pieces[i] = pieces;
+                }
+            } else {
+                RowAcc<VEC, CPL> acc;
+                acc.clear();
+#pragma unroll 4
+                for (uint32_t i = 0; i + 1 < pieces; ++i) acc.add_row(w.carry + ((size_t)(chunk + i) * 2 + 1) * D, D, lane);
+                acc.add_row(w.carry + (size_t)(chunk + pieces - 1) * 2 * D, D, lane);
+                acc.store(w.E + (size_t)last * D, D, lane);
+            }
         }
     }
-    acc.store(w.E + (size_t)last * D, D, lane);
+    __syncthreads();
+    const int cols = VEC ? D / 4 : D;                   // pieces of a row that the threads own
+    const int width = cols < 256 ? cols : 256;
+    const uint32_t slots = 256u / (uint32_t)width, slot = threadIdx.x / width;
+    for (uint32_t q = 0; q < s_n; ++q) {
+        const uint32_t pieces = s_pieces[q];
+        const piece_t* src = reinterpret_cast<const piece_t*>(w.carry) + (size_t)s_chunk[q] * 2 * cols;
+        for (int c0 = 0; c0 < cols; c0 += width) {
+            const int c = c0 + threadIdx.x % width;
+            RowAcc<VEC, 1> acc;                         // one piece of the row
+            acc.clear();
+            if (slot < slots && c < cols) {
+#pragma unroll 8
+                for (uint32_t i = slot; i < pieces; i += slots) {
+                    const piece_t* x = src + ((size_t)i * 2 + (i + 1 < pieces ? 1 : 0)) * cols + c;
+                    acc.add_row(reinterpret_cast<const float*>(x), VEC ? 4 : 1, 0);
+                }
+                acc.store(reinterpret_cast<float*>(&s_part[threadIdx.x]), VEC ? 4 : 1, 0);
+            }
+            __syncthreads();
+            if (slot == 0 && c < cols) {
+                acc.clear();
+                for (uint32_t i = 0; i < slots; ++i)
+                    acc.add_shared(&s_part[i * width + threadIdx.x]);
+                acc.store(w.E + (size_t)s_slot[q] * D + (VEC ? 4 * c : c), VEC ? 4 : 1, 0);
+            }
+            __syncthreads();
+        }
+    }
 }
 
 // Fast variant for D/4 <= 32 float4 chunks per row: LPR lanes cover a row, 32/LPR rows per load instruction,
@@ -378,10 +418,10 @@ __global__ void __launch_bounds__(256, 5) k_dE_fast(WsView w, const float* __res
     const int64_t chunk = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const uint32_t U = w.counters[CTR_LEVEL0 + w.K];
     const uint32_t Ltot = w.cnt[U];
-    const int64_t a64 = chunk * TT_DE_CHUNK;
+    const int64_t a64 = chunk * w.de_chunk;
     if (a64 >= Ltot) return;
     const uint32_t a = (uint32_t)a64;
-    const uint32_t b = min(a + (uint32_t)TT_DE_CHUNK, Ltot);
+    const uint32_t b = min(a + w.de_chunk, Ltot);
     const int D = w.D, D4 = D >> 2;
     const bool lane_on = lr < D4;
     const uint32_t prev = a > 0 ? w.pairs[a - 1].x : HT_EMPTY;
@@ -479,10 +519,10 @@ __global__ void __launch_bounds__(32 * DE_WARPS, 4) k_dE_stage(WsView w, const f
     const int64_t chunk = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const uint32_t U = w.counters[CTR_LEVEL0 + w.K];
     const uint32_t Ltot = w.cnt[U];
-    const int64_t a64 = chunk * TT_DE_CHUNK;
+    const int64_t a64 = chunk * w.de_chunk;
     if (a64 >= Ltot) return;
     const uint32_t a = (uint32_t)a64;
-    const uint32_t b = min(a + (uint32_t)TT_DE_CHUNK, Ltot);
+    const uint32_t b = min(a + w.de_chunk, Ltot);
     const uint32_t prev = a > 0 ? w.pairs[a - 1].x : HT_EMPTY;
     const uint32_t next = b < Ltot ? w.pairs[b].x : HT_EMPTY;
     const float4* __restrict__ G4 = reinterpret_cast<const float4*>(grad_out);
@@ -607,10 +647,30 @@ __global__ void __launch_bounds__(32 * DE_WARPS, 4) k_dE_stage(WsView w, const f
     }
 }
 
+// Positions per warp, and where the warps leave the pieces of segments that cross a chunk border.  A chunk is walked
+// serially, so short batches want short chunks (1024 positions: 65 thousand lookups kept 64 warps busy) and long ones
+// chunks that amortise the borders.  dE with 32 / 128 / 256 / 512 / 1024 positions per warp, us: 65 k lookups (D = 128,
+// at least 160 there) 39 / 39 / 60 / 101 / 185; 0.5 M (D = 32) 33 / 31 / 42 / 62 / 103; 1.6 M (D = 64) 72 / 70 / 70 / 85 /
+// 113; 4 M (D = 16) 173 / 122 / 121 / 142 / 173.
+static void tt_de_partition(tt_emb* h)
+{
+    WsView& w = h->v;
+    int64_t c = w.L / 2048 < 128 ? w.L / 2048 : 128;
+    if (c < w.L / 32768) c = w.L / 32768;
+    c = c < 32 ? 32 : (c > TT_DE_CHUNK ? TT_DE_CHUNK : c / 32 * 32);
+    // the pieces of more than L / TT_DE_CHUNK chunks go where the unsorted pairs were (the sort has consumed them): 8 bytes
+    // per lookup, so a chunk holds at least about D positions
+    const uintptr_t u0 = (reinterpret_cast<uintptr_t>(w.upairs) + 15) & ~(uintptr_t)15;
+    const size_t room = reinterpret_cast<uintptr_t>(w.upairs + h->max_lookups + 1) - u0;
+    while (c < TT_DE_CHUNK && (size_t)((w.L + c - 1) / c) * 2 * h->D * sizeof(float) > room) c += 32;
+    w.de_chunk = (uint32_t)c;
+    w.carry = c < TT_DE_CHUNK ? reinterpret_cast<float*>(u0) : h->carry;
+}
+
 template <bool VEC, int CPL>
 static cudaError_t launch_dE_t(tt_emb* h, const float* grad_out, cudaStream_t s)
 {
-    const int64_t chunks = (h->v.L + TT_DE_CHUNK - 1) / TT_DE_CHUNK;
+    const int64_t chunks = (h->v.L + h->v.de_chunk - 1) / h->v.de_chunk;
     const int grid = (int)((chunks + 7) / 8);
     if (grid > 0) {
         const int D4 = h->D / 4;
@@ -640,12 +700,15 @@ cudaError_t tt_launch_bwd_dE(tt_emb* h, const float* grad_out, cudaStream_t s)
 {
     const int D = h->D;
     const bool vec = (D % 4 == 0) && ((reinterpret_cast<uintptr_t>(grad_out) & 15) == 0);
+    tt_de_partition(h);
     if (vec) {
         if (D <= 128) return launch_dE_t<true, 1>(h, grad_out, s);
         if (D <= 256) return launch_dE_t<true, 2>(h, grad_out, s);
         if (D <= 512) return launch_dE_t<true, 4>(h, grad_out, s);
         return launch_dE_t<true, 8>(h, grad_out, s);
     }
+    if (D <= 32) return launch_dE_t<false, 1>(h, grad_out, s);
+    if (D <= 64) return launch_dE_t<false, 2>(h, grad_out, s);
     if (D <= 128) return launch_dE_t<false, 4>(h, grad_out, s);
     if (D <= 256) return launch_dE_t<false, 8>(h, grad_out, s);
     if (D <= 512) return launch_dE_t<false, 16>(h, grad_out, s);

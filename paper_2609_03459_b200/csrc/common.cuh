@@ -14,7 +14,7 @@
 #define TT_HEAD_TILES 4                                 // leading scan tiles of a table that are emitted first (see PopScan)
 #define TT_LSCAN_ITEMS 2                                // the short scans of the prefix-level bitmaps
 #define TT_LSCAN_TILE (TT_SCAN_THREADS * TT_LSCAN_ITEMS)
-#define TT_DE_CHUNK 1024                                  // sorted lookups per warp in the dE segment reduction
+#define TT_DE_CHUNK 1024                                  // most sorted lookups per warp in the dE segment reduction
 #define TT_NUM_STAGES 33                                // 0..8 pipeline stages, 9..20 forward sweep variants -1..10, 21..32 backward sweep variants
 #define TT_STRIPES 8                                     // L2-resident partial copies of the last core's gradient
 #define TT_NUM_MIDFAST 11                                // tensor-core instances of the middle-core backward (backward.cu)
@@ -87,7 +87,8 @@ struct WsView {
     uint2* upairs;                      // [L] (slot, bag) in lookup order, written by the pooling kernel (null: forward only)
     float* dP[TT_MAXK + 1];             // dP_k per level-k node, 2 <= k <= K-1
     float* Y[TT_MAXK + 1];              // per level-k node: its contribution to dP_{k-1} of its parent
-    float* carry;                       // [chunks][2][D]
+    float* carry;                       // [chunks][2][D] pieces of the segments that cross a chunk border
+    uint32_t de_chunk;                  // sorted lookups per warp in the dE segment reduction (at most TT_DE_CHUNK)
     float* gpart;                       // [TT_STRIPES][gpart_stride] partial copies of all tables' last-core gradients
     int64_t gpart_stride;               // floats per stripe
     uint2* tbm[TT_MAXK + 1];            // digit-major node bitmaps, levels 2..K-1
@@ -146,6 +147,7 @@ struct tt_emb {
     const char* region_name[96];
     size_t off_guard_list;      // device copy of the (offset, length) pairs + the check's result word
     void* ws_base;
+    float* carry;         // workspace region of v.carry for chunks of TT_DE_CHUNK lookups
     size_t scan_tmp_elems;
     int64_t gpart_floats;
     WsView v;             // filled at bind
