@@ -178,9 +178,9 @@ extern "C" int tt_emb_create(const tt_emb_config_t* cfg, tt_emb_t* out_handle)
     // work units: every table is cut into `units` equal-cost slices, one CTA each
     // about 8 waves of 8 resident CTAs per SM: fine enough that the last wave and table-size differences do not matter
     int Q = (64 * h->sm_count + T - 1) / T;   // (32 * and 128 * measured: 16.8 / 16.5 ms per training step against 16.4)
-    {   // ... but not so fine that a unit holds only a handful of groups (each unit pays two binary searches)
+    {   // ... but not so fine that a unit holds fewer than sixteen groups, one batch of its four warps
         uint64_t groups = level_space[K - 1] < (uint64_t)h->capU ? level_space[K - 1] : (uint64_t)h->capU;
-        const int64_t by_groups = (int64_t)(groups / (uint64_t)T / 64);
+        const int64_t by_groups = (int64_t)(groups / (uint64_t)T / TT_UNIT_GROUPS);
         if (Q > by_groups) Q = (int)by_groups;
     }
     if (Q < 8) Q = 8;
@@ -211,6 +211,7 @@ extern "C" int tt_emb_create(const tt_emb_config_t* cfg, tt_emb_t* out_handle)
             else if (PMv == 4 && Mv == 2 && RBv == 16 && quad_ok) td.fast = 9;
             else if (PMv == 4 && Mv == 2 && RBv == 8) td.fast = 10;   // D = 16 with rank 8: FP32 pipe (slices of 16 columns)
         }
+        td.unit_groups = td.fast == 3 ? 4 * TT_UNIT_GROUPS : TT_UNIT_GROUPS;
         for (int k = 0; k < TT_MAXK; ++k) td.midfast[k] = -1;
         for (int k = 2; k <= K - 1; ++k) {
             const int Mv = td.P[k - 1], rav = td.r[k - 1], colsv = td.d[k - 1] * td.r[k];
@@ -291,7 +292,7 @@ extern "C" int tt_emb_create(const tt_emb_config_t* cfg, tt_emb_t* out_handle)
         tot += v.cap[K - 1];
         if (tot < ((unsigned __int128)1 << 31)) break;
     }
-    h->cost_shift = shift;
+    v.cost_shift = shift;
 
     // ---- workspace plan
     // every region is followed by at least 64 guard bytes (written at bind, checked on demand by tt_emb_check_guards)

@@ -1499,14 +1499,16 @@ __device__ __forceinline__ uint32_t tt_trank(const WsView& w, const TableDesc& t
     return e.y + __popc(e.x & ((1u << (key & 31)) - 1u));
 }
 
-__global__ void k_tfill(WsView w, int k)
+__global__ void k_tfill(WsView w, int k, int costs)
 {
     tt_pdl_enter();
     const uint32_t count = w.counters[CTR_LEVEL0 + k];
     for (uint32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < count; v += gridDim.x * blockDim.x) {
         const int t = tt_find_table(w.tb[k], w.T, v);
         const TableDesc& td = w.tdesc[t];
-        w.tnode[k][tt_trank(w, td, k, tt_tkey(td, k, w.val[k][v]))] = v;
+        const uint32_t rank = tt_trank(w, td, k, tt_tkey(td, k, w.val[k][v]));
+        w.tnode[k][rank] = v;
+        if (costs) w.cost[rank] = tt_group_cost(w, td, v);
     }
 }
 
@@ -2064,7 +2066,7 @@ __global__ void __launch_bounds__(256) k_mid_sum(WsView w, int k)
 
 // Digit-major ("transposed") list of the level-k nodes: a second presence-bitmap sort, keyed by
 // (i_k, parent prefix) instead of (parent prefix, i_k); tnode[k][rank] = node.
-cudaError_t tt_launch_tlist(tt_emb* h, int k, cudaStream_t s)
+cudaError_t tt_launch_tlist(tt_emb* h, int k, bool costs, cudaStream_t s)
 {
     WsView& w = h->v;
     cudaError_t e;
@@ -2074,7 +2076,7 @@ cudaError_t tt_launch_tlist(tt_emb* h, int k, cudaStream_t s)
     tt_note_launch();
     TPopScan tp{w, k};
     if ((e = tt_scan(tp, w.ttotal_words[k], w.scan_tmp, s)) != cudaSuccess) return e;
-    if ((e = tt_launch_pdl(k_tfill, dim3(g), dim3(256), 0, s, w, k)) != cudaSuccess) return e;
+    if ((e = tt_launch_pdl(k_tfill, dim3(g), dim3(256), 0, s, w, k, costs ? 1 : 0)) != cudaSuccess) return e;
     tt_note_launch();
     return cudaGetLastError();
 }
@@ -2107,7 +2109,7 @@ cudaError_t tt_launch_bwd_middle(tt_emb* h, cudaStream_t s)
         }
         const int ngen = h->mcount[k][0];
         // level K-1's digit-major list already exists: the forward built it to order its sweep
-        if (k != h->K - 1 && (e = tt_launch_tlist(h, k, s)) != cudaSuccess) return e;
+        if (k != h->K - 1 && (e = tt_launch_tlist(h, k, false, s)) != cudaSuccess) return e;
         // the shape variants are independent (different tables): run them side by side so that the tail of one
         // (a few long node lists) overlaps the others
         int nfast = 0;

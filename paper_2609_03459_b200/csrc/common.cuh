@@ -10,10 +10,18 @@
 #define TT_SCAN_THREADS 256
 #define TT_SCAN_ITEMS 16
 #define TT_SCAN_TILE (TT_SCAN_THREADS * TT_SCAN_ITEMS)  // elements per scan tile
-#define TT_POOL_MAX_SHARES 262144                       // shares of the lookups that the pooling warps take in order
+#define TT_POOL_MAX_SHARES 131072                       // shares of the lookups that the pooling warps take in order
 #define TT_HEAD_TILES 4                                 // leading scan tiles of a table that are emitted first (see PopScan)
 #define TT_LSCAN_ITEMS 2                                // the short scans of the prefix-level bitmaps
 #define TT_LSCAN_TILE (TT_SCAN_THREADS * TT_LSCAN_ITEMS)
+#define TT_CSCAN_ITEMS 4                                // the scan of the group costs
+#define TT_PSCAN_ITEMS 4                                // the scan of row bitmaps of up to TT_PSCAN_WORDS words
+#define TT_PSCAN_WORDS (1u << 21)
+// fewest groups of a work unit; 4x as many for D = 128, rank 32, whose warps each reuse a 32 KB slice over their groups.
+// Sweeps with at least 4 / 8 / 16 / 32 / 64 groups per unit, forward + backward, us: 8 tables x 8 k groups (rank 16) 385 / 352 /
+// 325 / 319 / 343; 4 tables x 9 k (D = 32, rank 8) 119 / 117 / 107 / 122 / 188; four cores, 4.7 k groups 304 / 310 / 319 / 422 /
+// 576; D = 128, rank 32, 27 k groups (forward) 236 / 164 / 145 / 137 / 129
+#define TT_UNIT_GROUPS 16
 #define TT_DE_CHUNK 1024                                  // most sorted lookups per warp in the dE segment reduction
 #define TT_NUM_STAGES 33                                // 0..8 pipeline stages, 9..20 forward sweep variants -1..10, 21..32 backward sweep variants
 #define TT_STRIPES 8                                     // L2-resident partial copies of the last core's gradient
@@ -43,6 +51,7 @@ struct TableDesc {
     int32_t units;                      // work units (CTAs) this table is cut into
     int32_t unit_base;                  // first global unit id
     int32_t sgd_mask;                   // bit k: the fused backward + SGD call updates core k inside the kernel that finalises its gradient
+    int32_t unit_groups;                // a work unit holds at least this many groups
     int32_t fast;                       // register-tiled kernel variant for this table's shapes, -1 = generic path
     int32_t midfast[TT_MAXK];           // same for the middle-core backward of level k (index k), -1 = generic
 };
@@ -52,6 +61,7 @@ struct WsView {
     int32_t T, K, D;
     int32_t ablation;                   // study switches: bit 0 no prefix reuse, bit 1 static (equal-count) schedule,
                                         // bit 2 no de-duplication (every lookup is its own row and its own group; implies bit 0)
+    int32_t cost_shift;                 // cost unit of the schedule = 2^cost_shift FMAs
     float fused_lr;                     // != 0: the kernels that finalise a gradient also apply G -= fused_lr * dG (cores in sgd_mask)
     int32_t stride[TT_MAXK + 1];        // floats per node of the level-k partial-product buffers (max over tables)
     int64_t B, L;                       // current batch / lookups
@@ -132,7 +142,6 @@ struct tt_emb {
     int mbase[TT_MAXK + 1][TT_NUM_MIDFAST + 1], mcount[TT_MAXK + 1][TT_NUM_MIDFAST + 1], mmaxn[TT_MAXK + 1][TT_NUM_MIDFAST + 1];
     int32_t* vlist_host;
     size_t off_vlist;
-    int cost_shift;       // cost unit of the schedule = 2^cost_shift FMAs
     TableDesc* tab;       // host copy [T]
     size_t ws_bytes;
     size_t off_status, off_counters, off_tdesc, off_tlstart, off_bm, off_scan, off_cost, off_E;
@@ -181,7 +190,7 @@ cudaError_t tt_stage_end(tt_emb* h, int stage, cudaStream_t s);
 // ---- launchers implemented in the .cu files (all enqueue on `s`, return cudaGetLastError()) ----
 cudaError_t tt_launch_grouping(tt_emb* h, cudaStream_t s);
 cudaError_t tt_launch_schedule(tt_emb* h, cudaStream_t s);
-cudaError_t tt_launch_tlist(tt_emb* h, int k, cudaStream_t s);   // digit-major list of the level-k nodes
+cudaError_t tt_launch_tlist(tt_emb* h, int k, bool costs, cudaStream_t s);   // digit-major list of the level-k nodes (with their costs: level K-1)
 cudaError_t tt_launch_contraction(tt_emb* h, cudaStream_t s);
 cudaError_t tt_launch_pooling(tt_emb* h, float* out, cudaStream_t s);
 cudaError_t tt_launch_bwd_sort(tt_emb* h, cudaStream_t s);
@@ -289,6 +298,16 @@ __device__ __forceinline__ const float* tt_left_operand(const WsView& w, const T
     return w.pbuf[k - 1] + (size_t)w.parent[k][v] * w.stride[k - 1];
 }
 
+// cost of group g (a level-(K-1) node): FMAs of its intermediate product and of its rows, c_k = P_{k-1} r_{k-1} d_k r_k
+__device__ __forceinline__ uint32_t tt_group_cost(const WsView& w, const TableDesc& td, uint32_t g)
+{
+    const int K = w.K;
+    const uint32_t nchild = w.cstart[K - 1][g + 1] - w.cstart[K - 1][g];
+    const uint64_t c_last = (uint64_t)td.P[K - 1] * td.r[K - 1] * td.d[K - 1];
+    const uint64_t c_mid = K >= 3 ? (uint64_t)td.P[K - 2] * td.r[K - 2] * td.d[K - 2] * td.r[K - 1] : 0;
+    return (uint32_t)(((c_mid + (uint64_t)nchild * c_last) >> w.cost_shift) + 1);
+}
+
 // group range [g0, g1) of work unit q of table t: an equal-cost slice of the table's level-(K-1) groups in sweep order
 // (called by one thread per unit, once per forward: k_unit_ranges)
 __device__ __forceinline__ void tt_unit_range(const WsView& w, int t, int q, uint32_t& g0, uint32_t& g1)
@@ -297,10 +316,10 @@ __device__ __forceinline__ void tt_unit_range(const WsView& w, int t, int q, uin
     const int lvl = w.K - 1;
     const uint32_t a = w.tb[lvl][t], b = w.tb[lvl][t + 1];
     // the host sizes the grid for the largest possible number of groups; with fewer groups in this batch the table is
-    // cut into fewer units (at least 16 groups each) and the surplus CTAs leave at once
+    // cut into fewer units (at least td.unit_groups groups each) and the surplus CTAs leave at once
     int Q = td.units;
     {
-        const int by_groups = (int)((b - a) >> 4);
+        const int by_groups = (int)((b - a) / (uint32_t)td.unit_groups);
         if (Q > by_groups) Q = by_groups < 1 ? 1 : by_groups;
     }
     if (q >= Q) { g0 = a; g1 = a; return; }

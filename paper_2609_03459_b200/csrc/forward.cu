@@ -16,26 +16,14 @@
 
 // ---------------------------------------------------------------------------------------------- schedule
 
+// cost of every group in sweep order -> exclusive prefix sums, in place.  The costs are written by the kernel that fills the
+// sweep order (k_tfill; k_costs where the order is the natural one): formed inside the two scan kernels, each cost was
+// three dependent look-ups that a thread made sixteen times in a row (20 us per kernel for five thousand groups).
 struct CostScan {
     WsView w;
-    int shift;
     __device__ uint32_t size() const { return w.counters[CTR_LEVEL0 + w.K - 1]; }
-    __device__ int locate(uint32_t j0) const { return tt_find_table(w.tb[w.K - 1], w.T, j0); }
-    __device__ uint32_t value(uint32_t j, int hint) const
-    {
-        // position j of the sweep order: digit-major for K >= 3 (groups that share the big slice of core K-1 are
-        // neighbours, so that slice is fetched from L2 once per run instead of once per group), natural for K = 2
-        const int K = w.K;
-        const int t = tt_find_table_from(w.tb[K - 1], w.T, j, hint);
-        const uint32_t g = (K >= 3 && !(w.ablation & 1)) ? w.tnode[K - 1][j] : j;
-        const TableDesc& td = w.tdesc[t];
-        const uint32_t nchild = w.cstart[K - 1][g + 1] - w.cstart[K - 1][g];
-        // c_k = P_{k-1} r_{k-1} d_k r_k
-        uint64_t c_last = (uint64_t)td.P[K - 1] * td.r[K - 1] * td.d[K - 1];
-        uint64_t c_mid = K >= 3 ? (uint64_t)td.P[K - 2] * td.r[K - 2] * td.d[K - 2] * td.r[K - 1] : 0;
-        uint64_t c = ((c_mid + (uint64_t)nchild * c_last) >> shift) + 1;
-        return (uint32_t)c;
-    }
+    __device__ int locate(uint32_t) const { return 0; }
+    __device__ uint32_t value(uint32_t j, int) const { return w.cost[j]; }
     __device__ void emit(uint32_t g, uint32_t excl, uint32_t, int) const { w.cost[g] = excl; }
     __device__ void total(uint32_t tot) const
     {
@@ -43,6 +31,15 @@ struct CostScan {
         w.counters[CTR_COST_TOTAL] = tot;
     }
 };
+
+// natural sweep order (K = 2; study switch "no prefix reuse")
+__global__ void __launch_bounds__(256) k_costs(WsView w)
+{
+    tt_pdl_enter();
+    const uint32_t count = w.counters[CTR_LEVEL0 + w.K - 1];
+    for (uint32_t g = blockIdx.x * blockDim.x + threadIdx.x; g < count; g += gridDim.x * blockDim.x)
+        w.cost[g] = tt_group_cost(w, w.tdesc[tt_find_table(w.tb[w.K - 1], w.T, g)], g);
+}
 
 // group range of every work unit (table, q), once per forward: the sweeps of the forward and of the backward read
 // two words instead of bisecting the cost array at the start of every CTA (two chains of ~20 dependent loads each:
@@ -60,14 +57,15 @@ __global__ void __launch_bounds__(128) k_unit_ranges(WsView w)
 
 cudaError_t tt_launch_schedule(tt_emb* h, cudaStream_t s)
 {
+    cudaError_t e;
     if (h->K >= 3 && !(h->ablation & 1)) {
-        cudaError_t e = tt_launch_tlist(h, h->K - 1, s);
-        if (e != cudaSuccess) return e;
+        if ((e = tt_launch_tlist(h, h->K - 1, true, s)) != cudaSuccess) return e;
+    } else {
+        if ((e = tt_launch_pdl(k_costs, dim3(h->sm_count * 8), dim3(256), 0, s, h->v)) != cudaSuccess) return e;
+        tt_note_launch();
     }
-    // cost unit: 2^shift FMAs, chosen at create time so that the worst-case total fits 32 bits
-    CostScan cs{h->v, h->cost_shift};
-    cudaError_t e = tt_scan(cs, h->v.cap[h->v.K - 1], h->v.scan_tmp, s);
-    if (e != cudaSuccess) return e;
+    CostScan cs{h->v};
+    if ((e = tt_scan<CostScan, TT_CSCAN_ITEMS>(cs, h->v.cap[h->v.K - 1], h->v.scan_tmp, s)) != cudaSuccess) return e;
     const int total = h->T * h->units_per_table;
     if ((e = tt_launch_pdl(k_unit_ranges, dim3((total + 127) / 128), dim3(128), 0, s, h->v)) != cudaSuccess) return e;
     tt_note_launch();

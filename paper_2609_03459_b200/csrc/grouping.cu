@@ -113,6 +113,7 @@ __device__ __forceinline__ void tt_emit_set_bits(uint32_t* __restrict__ val, uin
 
 // ---------------------------------------------------------------------------------------------- level K: rows
 
+template <int TILE>
 struct PopScan {
     WsView w;
     __device__ uint32_t size() const { return w.total_words; }
@@ -133,6 +134,12 @@ struct PopScan {
     // those tiles are densely set and emit a hundred times the rows of a tile further down (70 us against 6), and in
     // ascending order the dense tiles of the last tables ran alone at the end of the kernel.
     __device__ uint32_t tile_of(uint32_t cta) const
+    {
+        constexpr uint32_t PER = TT_SCAN_TILE / TILE;   // the order is that of the long scan's tiles, cut finer
+        const uint32_t big = big_tile_of(cta / PER);
+        return big == 0xffffffffu ? big : big * PER + cta % PER;
+    }
+    __device__ uint32_t big_tile_of(uint32_t cta) const
     {
         const uint32_t head = (uint32_t)TT_HEAD_TILES * (uint32_t)w.T;
         if (cta < head) {
@@ -366,8 +373,16 @@ cudaError_t tt_launch_grouping(tt_emb* h, cudaStream_t s)
         if ((e = tt_launch_pdl(k_mark, dim3(g1), dim3(256), 0, s, w)) != cudaSuccess) return e;
         tt_note_launch();
     }
-    PopScan ps{w};
-    if ((e = tt_scan(ps, w.total_words, w.scan_tmp, s, (unsigned)(TT_HEAD_TILES * w.T) + w.rest_tiles)) != cudaSuccess) return e;
+    // short bitmaps in finer tiles, so that they spread over the SMs
+    const unsigned ptiles = (unsigned)(TT_HEAD_TILES * w.T) + w.rest_tiles;
+    if (w.total_words <= TT_PSCAN_WORDS) {
+        PopScan<TT_SCAN_THREADS * TT_PSCAN_ITEMS> ps{w};
+        e = tt_scan<decltype(ps), TT_PSCAN_ITEMS>(ps, w.total_words, w.scan_tmp, s, ptiles * (TT_SCAN_ITEMS / TT_PSCAN_ITEMS));
+    } else {
+        PopScan<TT_SCAN_TILE> ps{w};
+        e = tt_scan(ps, w.total_words, w.scan_tmp, s, ptiles);
+    }
+    if (e != cudaSuccess) return e;
     for (int k = w.K - 1; k >= 1; --k) {
         {
             const uint32_t want = (w.total_words_l[k] + 7u) / 8u;   // a warp per word
