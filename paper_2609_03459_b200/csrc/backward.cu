@@ -2020,47 +2020,79 @@ __global__ void __launch_bounds__(128, 4) k_mid_tile(WsView w, int k, int lbase,
     }
 }
 
-// dP_{k-1}[parent] (k = 2: the first core's gradient slice) = sum of the Y rows of the parent's children,
-// which are contiguous in sorted order; one warp per parent
-__global__ void __launch_bounds__(256) k_mid_sum(WsView w, int k)
+// dP_{k-1}[parent] (k = 2: the first core's gradient slice) = sum of the Y rows of the parent's children, which are
+// contiguous in sorted order.  One warp per parent and block of 32 float4 (or 32 floats where a row is no multiple of four
+// floats); where there are no more of these than CTAs, as with the few parents of many children at k = 2, the eight warps of
+// a CTA share one.  Rows narrower than 32 pieces
+// put several children side by side, and eight children per lane are in flight at a time, the last ones included (a loop
+// over the remainder would make a round trip for each).  Bound by the latency of those round trips where there are few
+// parents: 331 parents of 112 children (16 floats) took 31 us with one warp per parent and one
+// child at a time, 7 us now; bound by HBM on large batches (0.7 GB of Y in 90 us).
+template <bool VEC>
+__device__ __forceinline__ void tt_mid_sum_item(const WsView& w, const TableDesc& td, int k, uint32_t pn, uint32_t f0, float4 (*s_sum)[32], int share, int shares)
+{
+    constexpr int NF = 8;
+    using piece_t = typename std::conditional<VEC, float4, float>::type;
+    constexpr uint32_t PF = VEC ? 4 : 1;
+    const uint32_t lane = threadIdx.x & 31;
+    const uint32_t pitch = (uint32_t)w.stride[k - 1] / PF, np = (uint32_t)(td.P[k - 1] * td.r[k - 1]) / PF;
+    const uint32_t c0 = w.cstart[k - 1][pn], n = w.cstart[k - 1][pn + 1] - c0;
+    uint32_t lpr = 32;
+    while (lpr > 1 && lpr / 2 >= np) lpr >>= 1;
+    const uint32_t slots = 32u / lpr, slot = lane / lpr, f = f0 + lane % lpr;
+    const piece_t* y = reinterpret_cast<const piece_t*>(w.Y[k]) + (size_t)c0 * pitch + f;
+    RowAcc<VEC, 1> s;
+    s.clear();
+    if (f < np)
+        for (uint32_t v0 = slot + slots * (uint32_t)share; v0 < n; v0 += NF * slots * (uint32_t)shares) {
+            piece_t x[NF];
+#pragma unroll
+            for (int i = 0; i < NF; ++i) {
+                const uint32_t v = v0 + (uint32_t)i * slots * (uint32_t)shares;
+                x[i] = v < n ? __ldg(y + (size_t)v * pitch) : piece_t{};
+            }
+#pragma unroll
+            for (int i = 0; i < NF; ++i) s.add_shared(&x[i]);
+        }
+    for (uint32_t o = lpr; o < 32; o <<= 1)
+#pragma unroll
+        for (uint32_t i = 0; i < PF; ++i) s.v[i] += __shfl_xor_sync(0xffffffffu, s.v[i], o);
+    if (shares > 1) {   // the warps of the CTA, in order
+        s.store(reinterpret_cast<float*>(&s_sum[share][lane]), (int)PF, 0);
+        __syncthreads();
+        if (share == 0)
+            for (int i = 1; i < shares; ++i) s.add_shared(&s_sum[i][lane]);
+        __syncthreads();
+        if (share != 0) return;
+    }
+    if (f >= np || slot != 0) return;
+    float* dst = (k == 2 ? td.grad[0] + (size_t)w.val[1][pn] * td.slice_floats[0] : w.dP[k - 1] + (size_t)pn * w.stride[k - 1]) + PF * f;
+    s.store(dst, (int)PF, 0);
+    if (k == 2 && w.fused_lr != 0.f) {   // the slices of present first digits are final here: the fused update goes with them
+        float* c = td.core[0] + (size_t)w.val[1][pn] * td.slice_floats[0] + PF * f;
+        RowAcc<VEC, 1> u;
+#pragma unroll
+        for (uint32_t i = 0; i < PF; ++i) u.v[i] = c[i] - w.fused_lr * s.v[i];
+        u.store(c, (int)PF, 0);
+    }
+}
+
+// blocks: of 32 pieces, in the widest row of level k - 1
+__global__ void __launch_bounds__(256) k_mid_sum(WsView w, int k, uint32_t blocks)
 {
     tt_pdl_enter();
-    const int lane = threadIdx.x & 31;
-    const uint32_t count = w.counters[CTR_LEVEL0 + k - 1];
-    const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
-    const int strideY = w.stride[k - 1];
-    for (uint32_t pn = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; pn < count; pn += nwarps) {
-        const int t = tt_find_table(w.tb[k - 1], w.T, pn);
-        const TableDesc& td = w.tdesc[t];
-        const int nout = td.P[k - 1] * td.r[k - 1], nout4 = nout / 4;
-        const uint32_t c0 = w.cstart[k - 1][pn], c1 = w.cstart[k - 1][pn + 1];
-        float* dst = k == 2 ? td.grad[0] + (size_t)w.val[1][pn] * td.slice_floats[0] : w.dP[k - 1] + (size_t)pn * w.stride[k - 1];
-        if (nout & 3) {   // slices of the first core are not 16-byte aligned
-            for (int f = lane; f < nout; f += 32) {
-                float s = 0.f;
-                for (uint32_t v = c0; v < c1; ++v) s += __ldg(w.Y[k] + (size_t)v * strideY + f);
-                dst[f] = s;
-                if (k == 2 && w.fused_lr != 0.f) {
-                    float* c = td.core[0] + (size_t)w.val[1][pn] * td.slice_floats[0] + f;
-                    *c = *c - w.fused_lr * s;
-                }
-            }
-            continue;
-        }
-        for (int f = lane; f < nout4; f += 32) {
-            float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-            for (uint32_t v = c0; v < c1; ++v) {
-                const float4 x = __ldg(reinterpret_cast<const float4*>(w.Y[k] + (size_t)v * strideY) + f);
-                s.x += x.x; s.y += x.y; s.z += x.z; s.w += x.w;
-            }
-            reinterpret_cast<float4*>(dst)[f] = s;
-            if (k == 2 && w.fused_lr != 0.f) {   // first core: the slices of present first digits are final here
-                float4* c4 = reinterpret_cast<float4*>(td.core[0] + (size_t)w.val[1][pn] * td.slice_floats[0]) + f;
-                float4 u = *c4;
-                u.x = u.x - w.fused_lr * s.x; u.y = u.y - w.fused_lr * s.y; u.z = u.z - w.fused_lr * s.z; u.w = u.w - w.fused_lr * s.w;
-                *c4 = u;
-            }
-        }
+    __shared__ float4 s_sum[8][32];
+    const int wid = threadIdx.x >> 5;
+    const uint64_t items = (uint64_t)w.counters[CTR_LEVEL0 + k - 1] * blocks;
+    const int shares = items <= gridDim.x ? 8 : 1;
+    const uint64_t first = shares > 1 ? blockIdx.x : (uint64_t)blockIdx.x * 8 + wid, step = (uint64_t)gridDim.x * (8 / shares);
+    for (uint64_t it = first; it < items; it += step) {
+        const uint32_t pn = (uint32_t)(it / blocks), f0 = (uint32_t)(it % blocks) * 32u;
+        const TableDesc& td = w.tdesc[tt_find_table(w.tb[k - 1], w.T, pn)];
+        const uint32_t nout = (uint32_t)(td.P[k - 1] * td.r[k - 1]);
+        if (nout & 3) {   // the first core's slices are not 16-byte aligned
+            if (f0 < nout) tt_mid_sum_item<false>(w, td, k, pn, f0, s_sum, shares > 1 ? wid : 0, shares);
+        } else if (4 * f0 < nout) tt_mid_sum_item<true>(w, td, k, pn, f0, s_sum, shares > 1 ? wid : 0, shares);
     }
 }
 
@@ -2096,10 +2128,13 @@ cudaError_t tt_launch_bwd_middle(tt_emb* h, cudaStream_t s)
     cudaError_t e;
     for (int k = h->K - 1; k >= 2; --k) {
         bool any_fast[TT_NUM_MIDFAST] = {};
+        uint32_t sum_blocks = 1;
         int dgz = 1, tile_rows = 1;   // generic shapes: tiles of the slice gradient, most stacked rows of a slice
         for (int t = 0; t < h->T; ++t) {
             const TableDesc& td = h->tab[t];
             const int kc = k - 1;
+            const uint32_t nout = (uint32_t)(td.P[kc] * td.r[kc]), pieces = (nout & 3) ? nout : nout / 4;
+            if ((pieces + 31) / 32 > sum_blocks) sum_blocks = (pieces + 31) / 32;
             if (td.midfast[k] >= 0) { any_fast[td.midfast[k]] = true; continue; }
             const int tiles = ((td.r[kc] + MT_EDGE - 1) / MT_EDGE) * ((td.d[kc] * td.r[kc + 1] + MT_EDGE - 1) / MT_EDGE);
             if (tiles > dgz) dgz = tiles;
@@ -2141,7 +2176,7 @@ cudaError_t tt_launch_bwd_middle(tt_emb* h, cudaStream_t s)
             tt_note_launch();
         }
         if (fork && (e = tt_join(h, s, 4)) != cudaSuccess) return e;
-        if ((e = tt_launch_pdl(k_mid_sum, dim3(h->sm_count * 8), dim3(256), 0, s, w, k)) != cudaSuccess) return e;
+        if ((e = tt_launch_pdl(k_mid_sum, dim3(h->sm_count * 8), dim3(256), 0, s, w, k, sum_blocks)) != cudaSuccess) return e;
         tt_note_launch();
     }
     return cudaGetLastError();
