@@ -578,6 +578,7 @@ static int forward_any(tt_emb* h, const void* indices, bool idx32, const int64_t
     h->have_forward = false;
     for (int i = 0; i < 4; ++i) h->ev_valid[i] = false;
     for (int i = 9; i < 9 + TT_NUM_VARIANTS + 1; ++i) h->ev_valid[i] = false;
+    TT_CUDA(tt_plan_pooling(h, out));
     TT_STAGE(h, 0, s, tt_launch_grouping(h, s));
     TT_STAGE(h, 1, s, tt_launch_schedule(h, s));
     TT_STAGE(h, 2, s, tt_launch_contraction(h, s));

@@ -20,6 +20,7 @@
 #include "scan.cuh"
 #include "mma.cuh"
 #include "quad_mid.cuh"
+#include "group.cuh"
 #include <type_traits>
 
 #define HT_SIZE 4096
@@ -1464,54 +1465,6 @@ cudaError_t tt_launch_bwd_contraction(tt_emb* h, cudaStream_t s)
 
 // ---------------------------------------------------------------------------------------------- 4. middle cores
 
-__device__ __forceinline__ uint32_t tt_tkey(const TableDesc& td, int k, uint32_t val)
-{
-    // digit-major key of a level-k node: i_k * (number of possible parents) + parent prefix value
-    const uint32_t nk = (uint32_t)td.n[k - 1];
-    return (val % nk) * td.prefix_space[k - 1] + val / nk;
-}
-
-__global__ void k_tmark(WsView w, int k)
-{
-    tt_pdl_enter();
-    const uint32_t count = w.counters[CTR_LEVEL0 + k];
-    for (uint32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < count; v += gridDim.x * blockDim.x) {
-        const int t = tt_find_table(w.tb[k], w.T, v);
-        const TableDesc& td = w.tdesc[t];
-        const uint32_t key = tt_tkey(td, k, w.val[k][v]);
-        atomicOr(&w.tbm[k][td.tword_base[k] + (key >> 5)].x, 1u << (key & 31));
-    }
-}
-
-struct TPopScan {
-    WsView w;
-    int k;
-    __device__ uint32_t size() const { return w.ttotal_words[k]; }
-    __device__ int locate(uint32_t) const { return 0; }
-    __device__ uint32_t value(uint32_t i, int) const { return __popc(w.tbm[k][i].x); }
-    __device__ void emit(uint32_t i, uint32_t excl, uint32_t, int) const { w.tbm[k][i].y = excl; }
-    __device__ void total(uint32_t) const {}
-};
-
-__device__ __forceinline__ uint32_t tt_trank(const WsView& w, const TableDesc& td, int k, uint32_t key)
-{
-    const uint2 e = w.tbm[k][td.tword_base[k] + (key >> 5)];
-    return e.y + __popc(e.x & ((1u << (key & 31)) - 1u));
-}
-
-__global__ void k_tfill(WsView w, int k, int costs)
-{
-    tt_pdl_enter();
-    const uint32_t count = w.counters[CTR_LEVEL0 + k];
-    for (uint32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < count; v += gridDim.x * blockDim.x) {
-        const int t = tt_find_table(w.tb[k], w.T, v);
-        const TableDesc& td = w.tdesc[t];
-        const uint32_t rank = tt_trank(w, td, k, tt_tkey(td, k, w.val[k][v]));
-        w.tnode[k][rank] = v;
-        if (costs) w.cost[rank] = tt_group_cost(w, td, v);
-    }
-}
-
 // ---- tensor-core middle-core backward (P_{k-1} = 4 or 2 rows, r_{k-1} in {16,32}, d_k * r_k in {32,64,128}) ----
 //
 // One CTA of 4 warps per (table, slice i_k).  The nodes with digit i_k arrive in ascending parent order from the
@@ -2096,23 +2049,6 @@ __global__ void __launch_bounds__(256) k_mid_sum(WsView w, int k, uint32_t block
     }
 }
 
-// Digit-major ("transposed") list of the level-k nodes: a second presence-bitmap sort, keyed by
-// (i_k, parent prefix) instead of (parent prefix, i_k); tnode[k][rank] = node.
-cudaError_t tt_launch_tlist(tt_emb* h, int k, bool costs, cudaStream_t s)
-{
-    WsView& w = h->v;
-    cudaError_t e;
-    if ((e = cudaMemsetAsync(w.tbm[k], 0, (size_t)w.ttotal_words[k] * sizeof(uint2), s)) != cudaSuccess) return e;
-    const int g = h->sm_count * 8;
-    if ((e = tt_launch_pdl(k_tmark, dim3(g), dim3(256), 0, s, w, k)) != cudaSuccess) return e;
-    tt_note_launch();
-    TPopScan tp{w, k};
-    if ((e = tt_scan(tp, w.ttotal_words[k], w.scan_tmp, s)) != cudaSuccess) return e;
-    if ((e = tt_launch_pdl(k_tfill, dim3(g), dim3(256), 0, s, w, k, costs ? 1 : 0)) != cudaSuccess) return e;
-    tt_note_launch();
-    return cudaGetLastError();
-}
-
 template <int M, int RA, int COLS>
 static cudaError_t tt_launch_mid(dim3 grid, cudaStream_t st, const WsView& w, int k, int variant, int lbase)
 {
@@ -2144,7 +2080,7 @@ cudaError_t tt_launch_bwd_middle(tt_emb* h, cudaStream_t s)
         }
         const int ngen = h->mcount[k][0];
         // level K-1's digit-major list already exists: the forward built it to order its sweep
-        if (k != h->K - 1 && (e = tt_launch_tlist(h, k, false, s)) != cudaSuccess) return e;
+        if (k != h->K - 1 && (e = tt_launch_tlist(h, k, s)) != cudaSuccess) return e;
         // the shape variants are independent (different tables): run them side by side so that the tail of one
         // (a few long node lists) overlaps the others
         int nfast = 0;

@@ -17,6 +17,9 @@
 #define TT_CSCAN_ITEMS 4                                // the scan of the group costs
 #define TT_PSCAN_ITEMS 4                                // the scan of row bitmaps of up to TT_PSCAN_WORDS words
 #define TT_PSCAN_WORDS (1u << 21)
+// most lookups whose marking pass also checks the offsets: one launch less, but the tables' ranges come from all over the
+// offsets (99 M lookups, 60 tables: grouping 0.76 ms with two kernels, 0.81 ms with one; 0.5 M, 8 tables: 3 us shorter)
+#define TT_FUSED_INGEST (1 << 22)
 // fewest groups of a work unit; 4x as many for D = 128, rank 32, whose warps each reuse a 32 KB slice over their groups.
 // Sweeps with at least 4 / 8 / 16 / 32 / 64 groups per unit, forward + backward, us: 8 tables x 8 k groups (rank 16) 385 / 352 /
 // 325 / 319 / 343; 4 tables x 9 k (D = 32, rank 8) 119 / 117 / 107 / 122 / 188; four cores, 4.7 k groups 304 / 310 / 319 / 422 /
@@ -85,6 +88,7 @@ struct WsView {
     uint32_t* parent[TT_MAXK + 1];      // levels 3..K-1: parent node at level k-1 (null elsewhere: nothing reads it)
     uint32_t* tb[TT_MAXK + 1];          // [T+1] node range of each table at level k
     uint32_t* cost;                     // [cap_{K-1}+1] exclusive scan of per-group cost (+ total)
+    int64_t pool_shares;                // shares of the lookups in the pooling pass (0: it takes no shares)
     int64_t* pool_bounds;               // [shares + 1] first bag of every share of the pooling pass (k_pool_bounds)
     uint2* unit_rng;                    // [T * units per table] group range of every work unit (k_unit_ranges)
     int32_t units_per_table;
@@ -156,6 +160,7 @@ struct tt_emb {
     const char* region_name[96];
     size_t off_guard_list;      // device copy of the (offset, length) pairs + the check's result word
     void* ws_base;
+    int pool_grid;        // CTAs of the pooling kernel (tt_plan_pooling)
     float* carry;         // workspace region of v.carry for chunks of TT_DE_CHUNK lookups
     size_t scan_tmp_elems;
     int64_t gpart_floats;
@@ -190,7 +195,8 @@ cudaError_t tt_stage_end(tt_emb* h, int stage, cudaStream_t s);
 // ---- launchers implemented in the .cu files (all enqueue on `s`, return cudaGetLastError()) ----
 cudaError_t tt_launch_grouping(tt_emb* h, cudaStream_t s);
 cudaError_t tt_launch_schedule(tt_emb* h, cudaStream_t s);
-cudaError_t tt_launch_tlist(tt_emb* h, int k, bool costs, cudaStream_t s);   // digit-major list of the level-k nodes (with their costs: level K-1)
+cudaError_t tt_launch_tlist(tt_emb* h, int k, cudaStream_t s);   // digit-major list of the level-k nodes (backward, k < K-1)
+cudaError_t tt_plan_pooling(tt_emb* h, const float* out);          // grid and shares of the pooling pass, before the schedule
 cudaError_t tt_launch_contraction(tt_emb* h, cudaStream_t s);
 cudaError_t tt_launch_pooling(tt_emb* h, float* out, cudaStream_t s);
 cudaError_t tt_launch_bwd_sort(tt_emb* h, cudaStream_t s);
@@ -297,6 +303,10 @@ __device__ __forceinline__ const float* tt_left_operand(const WsView& w, const T
     }
     return w.pbuf[k - 1] + (size_t)w.parent[k][v] * w.stride[k - 1];
 }
+
+// groups swept in digit-major order (neighbours share the big slice of core K-1, which is then fetched from L2 once per
+// run instead of once per group); otherwise in natural order
+__host__ __device__ __forceinline__ bool tt_digit_major(const WsView& w) { return w.K >= 3 && !(w.ablation & 1); }
 
 // cost of group g (a level-(K-1) node): FMAs of its intermediate product and of its rows, c_k = P_{k-1} r_{k-1} d_k r_k
 __device__ __forceinline__ uint32_t tt_group_cost(const WsView& w, const TableDesc& td, uint32_t g)

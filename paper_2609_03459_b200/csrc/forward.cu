@@ -14,64 +14,6 @@
 #include "mma.cuh"
 #include "quad_mid.cuh"
 
-// ---------------------------------------------------------------------------------------------- schedule
-
-// cost of every group in sweep order -> exclusive prefix sums, in place.  The costs are written by the kernel that fills the
-// sweep order (k_tfill; k_costs where the order is the natural one): formed inside the two scan kernels, each cost was
-// three dependent look-ups that a thread made sixteen times in a row (20 us per kernel for five thousand groups).
-struct CostScan {
-    WsView w;
-    __device__ uint32_t size() const { return w.counters[CTR_LEVEL0 + w.K - 1]; }
-    __device__ int locate(uint32_t) const { return 0; }
-    __device__ uint32_t value(uint32_t j, int) const { return w.cost[j]; }
-    __device__ void emit(uint32_t g, uint32_t excl, uint32_t, int) const { w.cost[g] = excl; }
-    __device__ void total(uint32_t tot) const
-    {
-        w.cost[size()] = tot;
-        w.counters[CTR_COST_TOTAL] = tot;
-    }
-};
-
-// natural sweep order (K = 2; study switch "no prefix reuse")
-__global__ void __launch_bounds__(256) k_costs(WsView w)
-{
-    tt_pdl_enter();
-    const uint32_t count = w.counters[CTR_LEVEL0 + w.K - 1];
-    for (uint32_t g = blockIdx.x * blockDim.x + threadIdx.x; g < count; g += gridDim.x * blockDim.x)
-        w.cost[g] = tt_group_cost(w, w.tdesc[tt_find_table(w.tb[w.K - 1], w.T, g)], g);
-}
-
-// group range of every work unit (table, q), once per forward: the sweeps of the forward and of the backward read
-// two words instead of bisecting the cost array at the start of every CTA (two chains of ~20 dependent loads each:
-// contraction 2.27 -> 2.16 ms, backward sweeps 4.49 -> 4.43 ms on the 60-table training step)
-__global__ void __launch_bounds__(128) k_unit_ranges(WsView w)
-{
-    tt_pdl_enter();
-    const int total = w.T * w.units_per_table;
-    const int u = blockIdx.x * blockDim.x + threadIdx.x;
-    if (u >= total) return;
-    uint32_t g0, g1;
-    tt_unit_range(w, u / w.units_per_table, u % w.units_per_table, g0, g1);
-    w.unit_rng[u] = make_uint2(g0, g1);
-}
-
-cudaError_t tt_launch_schedule(tt_emb* h, cudaStream_t s)
-{
-    cudaError_t e;
-    if (h->K >= 3 && !(h->ablation & 1)) {
-        if ((e = tt_launch_tlist(h, h->K - 1, true, s)) != cudaSuccess) return e;
-    } else {
-        if ((e = tt_launch_pdl(k_costs, dim3(h->sm_count * 8), dim3(256), 0, s, h->v)) != cudaSuccess) return e;
-        tt_note_launch();
-    }
-    CostScan cs{h->v};
-    if ((e = tt_scan<CostScan, TT_CSCAN_ITEMS>(cs, h->v.cap[h->v.K - 1], h->v.scan_tmp, s)) != cudaSuccess) return e;
-    const int total = h->T * h->units_per_table;
-    if ((e = tt_launch_pdl(k_unit_ranges, dim3((total + 127) / 128), dim3(128), 0, s, h->v)) != cudaSuccess) return e;
-    tt_note_launch();
-    return cudaGetLastError();
-}
-
 // ---------------------------------------------------------------------------------------------- products
 
 // P_k for every level-k node, 2 <= k <= K-2 (only K = 4 has such a level); one CTA per node, grid-stride
@@ -738,40 +680,15 @@ __device__ __forceinline__ uint32_t tt_lookup_slot(const WsView& w, const TableD
 // first warp finished at 84 % of the kernel, the median one at 90 %.  Eight shares per warp: more of them cost more
 // in pipeline fill and drain per share than they give in balance (4 / 8 / 16 / 32: 2.62 / 2.39 / 2.50 / 2.76 ms).
 #define TT_POOL_MAX_CHUNKS 8
-__host__ __device__ __forceinline__ int64_t tt_pool_chunks(int64_t L, int64_t W)
+// grid and shares of a pooling kernel with W warps
+static void tt_pool_set(tt_emb* h, int64_t grid, int warps)
 {
-    int64_t c = L / (W * 512);                          // at least 512 lookups per share
+    const int64_t W = grid * warps;
+    int64_t c = h->v.L / (W * 512);                     // at least 512 lookups per share
     c = c < 1 ? 1 : (c > TT_POOL_MAX_CHUNKS ? TT_POOL_MAX_CHUNKS : c);
     while (W * c > TT_POOL_MAX_SHARES && c > 1) --c;
-    return c;
-}
-
-// first bag of every share: share ci starts at the first bag whose offset is >= L ci / C (the same search for both
-// neighbours of a boundary, whatever the offsets hold).  One thread per boundary: the bisections (21 dependent loads for
-// two million bags) run side by side here instead of at the start of every share in the pooling warps.
-__global__ void __launch_bounds__(256) k_pool_bounds(WsView w, int64_t C)
-{
-    tt_pdl_enter();
-    const int64_t nb = (int64_t)w.T * w.B;
-    for (int64_t ci = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; ci <= C; ci += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t target = (w.L * ci) / C;
-        int64_t lo = 0, hi = nb;
-        while (lo < hi) {
-            const int64_t mid = (lo + hi) >> 1;
-            if (__ldg(w.offsets + mid) < target) lo = mid + 1; else hi = mid;
-        }
-        w.pool_bounds[ci] = ci == 0 ? 0 : (ci == C ? nb : lo);
-    }
-}
-
-static cudaError_t launch_pool_bounds(tt_emb* h, int64_t W, cudaStream_t s)
-{
-    const int64_t C = W * tt_pool_chunks(h->v.L, W);
-    const int64_t want = (C + 1 + 255) / 256;
-    const int grid = (int)(want < (int64_t)h->sm_count * 8 ? want : (int64_t)h->sm_count * 8);
-    cudaError_t e = tt_launch_pdl(k_pool_bounds, dim3(grid), dim3(256), 0, s, h->v, C);
-    if (e == cudaSuccess) tt_note_launch();
-    return e;
+    h->pool_grid = (int)grid;
+    h->v.pool_shares = W * c;
 }
 
 template <int LPR, int CPL, bool WT>  // lanes per row, float4 chunks per lane, weighted / mean pooling
@@ -788,8 +705,7 @@ __global__ void __launch_bounds__(256, (CPL == 1 ? 6 : (CPL == 2 ? 2 : 1))) k_po
     const uint32_t capK = w.cap[w.K];
     // Skew-aware split: the grid is exactly resident (persistent warps); a share holds the bags whose first
     // lookup falls into it (offsets is the cost prefix sum).
-    const int64_t W = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    const int64_t C = W * tt_pool_chunks(w.L, W);
+    const int64_t C = w.pool_shares;
     auto clampL = [&](int64_t x) { return x < 0 ? (int64_t)0 : (x > w.L ? w.L : x); };
     for (;;) {
     // shares are handed out in order through a counter: a warp whose shares hold popular (L2-resident) rows takes more of them
@@ -915,8 +831,7 @@ __global__ void __launch_bounds__(32 * POOL_WARPS, 4) k_pool_async(WsView w, flo
     const bool lane_on = lr < D4;
     const float4* __restrict__ E4 = reinterpret_cast<const float4*>(w.E);
     const uint32_t capK = w.cap[w.K];
-    const int64_t W = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    const int64_t C = W * tt_pool_chunks(w.L, W);
+    const int64_t C = w.pool_shares;
     // lookup positions and bag indices fit in 32 bits (L and T * B are below 2^31, checked when the handle is made)
     typedef int32_t pos_t;
     auto clampL = [&](int64_t x) { return x < 0 ? (pos_t)0 : (x > w.L ? (pos_t)w.L : (pos_t)x); };
@@ -1064,8 +979,7 @@ __global__ void __launch_bounds__(32 * POOL_WARPS, 4) k_pool_stream(WsView w, fl
     const bool lane_on = lr < D4;
     const float4* __restrict__ E4 = reinterpret_cast<const float4*>(w.E);
     const uint32_t capK = w.cap[w.K];
-    const int64_t W = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    const int64_t C = W * tt_pool_chunks(w.L, W);
+    const int64_t C = w.pool_shares;
     const bool stream_ok = !(*w.status & TT_EMB_STATUS_OFFSETS);
     // lookup positions and bag indices fit in 32 bits (L and T * B are below 2^31, checked when the handle is made)
     typedef int32_t pos_t;
@@ -1368,45 +1282,52 @@ __global__ void __launch_bounds__(32 * POOL_WARPS, 4) k_pool_stream(WsView w, fl
 
 
 template <int R4, bool WT>
-static cudaError_t launch_pool_async(tt_emb* h, float* out, cudaStream_t s)
+static cudaError_t launch_pool_async(tt_emb* h, float* out, bool plan, cudaStream_t s)
 {
     const size_t smem = (size_t)POOL_WARPS * 32 * R4 * sizeof(float4);
     cudaError_t e = cudaFuncSetAttribute(k_pool_async<R4, WT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    int per_sm = 0;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_pool_async<R4, WT>, 32 * POOL_WARPS, smem)) != cudaSuccess) return e;
-    if (per_sm < 1) per_sm = 1;
     const int64_t nb = (int64_t)h->v.T * h->v.B;
-    int64_t grid = (int64_t)per_sm * h->sm_count;
-    const int64_t need = (nb + POOL_WARPS - 1) / POOL_WARPS;
-    if (grid > need) grid = need;
-    if (grid < 1) grid = 1;
-    if ((e = launch_pool_bounds(h, grid * POOL_WARPS, s)) != cudaSuccess) return e;
+    if (plan) {
+        int per_sm = 0;
+        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_pool_async<R4, WT>, 32 * POOL_WARPS, smem)) != cudaSuccess) return e;
+        if (per_sm < 1) per_sm = 1;
+        int64_t grid = (int64_t)per_sm * h->sm_count;
+        const int64_t need = (nb + POOL_WARPS - 1) / POOL_WARPS;
+        if (grid > need) grid = need;
+        if (grid < 1) grid = 1;
+        tt_pool_set(h, grid, POOL_WARPS);
+        return cudaSuccess;
+    }
+    const int grid = h->pool_grid;
     if (h->v.L < (int64_t)(R4 == 16 ? TT_POOL_STREAM_BELOW_WIDE : TT_POOL_STREAM_BELOW) * nb) {   // few lookups per bag: windows across bags
         if ((e = cudaFuncSetAttribute(k_pool_stream<R4, WT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
-        if ((e = tt_launch_pdl(k_pool_stream<R4, WT>, dim3((int)grid), dim3(32 * POOL_WARPS), smem, s, h->v, out)) != cudaSuccess) return e;
+        if ((e = tt_launch_pdl(k_pool_stream<R4, WT>, dim3(grid), dim3(32 * POOL_WARPS), smem, s, h->v, out)) != cudaSuccess) return e;
         tt_note_launch();
         return cudaGetLastError();
     }
-    if ((e = tt_launch_pdl(k_pool_async<R4, WT>, dim3((int)grid), dim3(32 * POOL_WARPS), smem, s, h->v, out)) != cudaSuccess) return e;
+    if ((e = tt_launch_pdl(k_pool_async<R4, WT>, dim3(grid), dim3(32 * POOL_WARPS), smem, s, h->v, out)) != cudaSuccess) return e;
     tt_note_launch();
     return cudaGetLastError();
 }
 
 template <int LPR, int CPL, bool WT>
-static cudaError_t launch_pool_vec(tt_emb* h, float* out, cudaStream_t s)
+static cudaError_t launch_pool_vec(tt_emb* h, float* out, bool plan, cudaStream_t s)
 {
-    int per_sm = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_pool_vec<LPR, CPL, WT>, 256, 0);
-    if (e != cudaSuccess) return e;
-    if (per_sm < 1) per_sm = 1;
-    const int64_t nb = (int64_t)h->v.T * h->v.B;
-    int64_t grid = (int64_t)per_sm * h->sm_count;
-    const int64_t need = (nb + 7) / 8;
-    if (grid > need) grid = need;
-    if (grid < 1) grid = 1;
-    if ((e = launch_pool_bounds(h, grid * 8, s)) != cudaSuccess) return e;
-    if ((e = tt_launch_pdl(k_pool_vec<LPR, CPL, WT>, dim3((int)grid), dim3(256), 0, s, h->v, out)) != cudaSuccess) return e;
+    cudaError_t e;
+    if (plan) {
+        int per_sm = 0;
+        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_pool_vec<LPR, CPL, WT>, 256, 0)) != cudaSuccess) return e;
+        if (per_sm < 1) per_sm = 1;
+        const int64_t nb = (int64_t)h->v.T * h->v.B;
+        int64_t grid = (int64_t)per_sm * h->sm_count;
+        const int64_t need = (nb + 7) / 8;
+        if (grid > need) grid = need;
+        if (grid < 1) grid = 1;
+        tt_pool_set(h, grid, 8);
+        return cudaSuccess;
+    }
+    if ((e = tt_launch_pdl(k_pool_vec<LPR, CPL, WT>, dim3(h->pool_grid), dim3(256), 0, s, h->v, out)) != cudaSuccess) return e;
     tt_note_launch();
     return cudaGetLastError();
 }
@@ -1472,29 +1393,38 @@ __global__ void __launch_bounds__(256) k_pool_scalar(WsView w, float* __restrict
 }
 
 template <bool WT>
-static cudaError_t launch_pool_sized(tt_emb* h, int D4, float* out, cudaStream_t s)
+static cudaError_t launch_pool_sized(tt_emb* h, int D4, float* out, bool plan, cudaStream_t s)
 {
-    if (D4 > 8 && D4 <= 16) return launch_pool_async<16, WT>(h, out, s);
-    if (D4 > 4 && D4 <= 8) return launch_pool_async<8, WT>(h, out, s);
-    if (D4 <= 4) return launch_pool_vec<4, 1, WT>(h, out, s);
-    if (D4 <= 8) return launch_pool_vec<8, 1, WT>(h, out, s);
-    if (D4 <= 16) return launch_pool_vec<16, 1, WT>(h, out, s);
-    if (D4 <= 32) return launch_pool_vec<32, 1, WT>(h, out, s);
-    if (D4 <= 64) return launch_pool_vec<32, 2, WT>(h, out, s);
-    if (D4 <= 128) return launch_pool_vec<32, 4, WT>(h, out, s);
-    return launch_pool_vec<32, 8, WT>(h, out, s);
+    if (D4 > 8 && D4 <= 16) return launch_pool_async<16, WT>(h, out, plan, s);
+    if (D4 > 4 && D4 <= 8) return launch_pool_async<8, WT>(h, out, plan, s);
+    if (D4 <= 4) return launch_pool_vec<4, 1, WT>(h, out, plan, s);
+    if (D4 <= 8) return launch_pool_vec<8, 1, WT>(h, out, plan, s);
+    if (D4 <= 16) return launch_pool_vec<16, 1, WT>(h, out, plan, s);
+    if (D4 <= 32) return launch_pool_vec<32, 1, WT>(h, out, plan, s);
+    if (D4 <= 64) return launch_pool_vec<32, 2, WT>(h, out, plan, s);
+    if (D4 <= 128) return launch_pool_vec<32, 4, WT>(h, out, plan, s);
+    return launch_pool_vec<32, 8, WT>(h, out, plan, s);
+}
+
+static bool tt_pool_vectors(const tt_emb* h, const float* out)
+{
+    return h->D % 4 == 0 && (reinterpret_cast<uintptr_t>(out) & 15) == 0;
+}
+
+cudaError_t tt_plan_pooling(tt_emb* h, const float* out)
+{
+    h->v.pool_shares = 0;
+    if (!tt_pool_vectors(h, out)) return cudaSuccess;   // a warp takes bags, not shares
+    return (h->v.psw || h->v.pool_mean) ? launch_pool_sized<true>(h, h->D / 4, nullptr, true, nullptr)
+                                        : launch_pool_sized<false>(h, h->D / 4, nullptr, true, nullptr);
 }
 
 cudaError_t tt_launch_pooling(tt_emb* h, float* out, cudaStream_t s)
 {
     WsView& w = h->v;
-    const int64_t nb = (int64_t)w.T * w.B;
-    const int64_t want = (nb + 7) / 8;  // 8 warps per CTA, one warp per bag
-    int grid = (int)want;
-    if (grid < 1) grid = 1;
     const int D = w.D;
-    const bool vec_ok = (D % 4 == 0) && ((reinterpret_cast<uintptr_t>(out) & 15) == 0);
-    if (!vec_ok) {
+    if (!tt_pool_vectors(h, out)) {
+        const int64_t want = ((int64_t)w.T * w.B + 7) / 8;  // 8 warps per CTA, one warp per bag
         int pgrid = (int)(want < (int64_t)h->sm_count * 8 ? want : (int64_t)h->sm_count * 8);
         const dim3 pg(pgrid < 1 ? 1 : pgrid);
         cudaError_t e0 = D <= 32 ? tt_launch_pdl(k_pool_scalar<1>, pg, dim3(256), 0, s, w, out)
@@ -1505,7 +1435,5 @@ cudaError_t tt_launch_pooling(tt_emb* h, float* out, cudaStream_t s)
         tt_note_launch();
         return cudaGetLastError();
     }
-    const int D4 = D / 4;
-    (void)grid;
-    return (w.psw || w.pool_mean) ? launch_pool_sized<true>(h, D4, out, s) : launch_pool_sized<false>(h, D4, out, s);
+    return (w.psw || w.pool_mean) ? launch_pool_sized<true>(h, D / 4, out, false, s) : launch_pool_sized<false>(h, D / 4, out, false, s);
 }
