@@ -232,6 +232,9 @@ extern "C" int tt_emb_create(const tt_emb_config_t* cfg, tt_emb_t* out_handle)
         td.gpart_off = gpart;
         gpart += (td.core_floats[K - 1] + 3) / 4 * 4;
     }
+    h->warp_groups = true;
+    for (int t = 0; t < T; ++t)
+        if (h->tab[t].fast < 0 || h->tab[t].fast == 4) h->warp_groups = false;
     h->units_total = unit_base;
     h->units_per_table = Q;
     // vlist[0..T): table ids grouped by kernel variant; vlist[T..2T): all tables.  Inside each list the tables come
@@ -405,6 +408,7 @@ extern "C" int tt_emb_bind(tt_emb_t h, float* const* core_ptrs, void* workspace,
     int sms = 0;
     if (!tt_device_ok(&sms)) return TT_EMB_ERR_ARCH;
     cudaStream_t s = (cudaStream_t)stream;
+    h->cluster_ok = tt_group_cluster_ok();
     const int T = h->T, K = h->K;
     for (int t = 0; t < T; ++t)
         for (int k = 0; k < K; ++k) {

@@ -64,6 +64,8 @@ struct WsView {
     int32_t T, K, D;
     int32_t ablation;                   // study switches: bit 0 no prefix reuse, bit 1 static (equal-count) schedule,
                                         // bit 2 no de-duplication (every lookup is its own row and its own group; implies bit 0)
+    int32_t equal_units;                // 1: work units of equal group counts instead of equal costs (study switch; small batches,
+                                        // whose schedule is made in one cluster without the scan of the costs)
     int32_t cost_shift;                 // cost unit of the schedule = 2^cost_shift FMAs
     float fused_lr;                     // != 0: the kernels that finalise a gradient also apply G -= fused_lr * dG (cores in sgd_mask)
     int32_t stride[TT_MAXK + 1];        // floats per node of the level-k partial-product buffers (max over tables)
@@ -160,6 +162,8 @@ struct tt_emb {
     const char* region_name[96];
     size_t off_guard_list;      // device copy of the (offset, length) pairs + the check's result word
     void* ws_base;
+    bool warp_groups;     // every table is swept by warps that take groups one batch at a time (not by whole CTAs)
+    int cluster_ok;       // the device takes the cluster of group_cluster.cu
     int pool_grid;        // CTAs of the pooling kernel (tt_plan_pooling)
     float* carry;         // workspace region of v.carry for chunks of TT_DE_CHUNK lookups
     size_t scan_tmp_elems;
@@ -194,6 +198,8 @@ cudaError_t tt_stage_end(tt_emb* h, int stage, cudaStream_t s);
 
 // ---- launchers implemented in the .cu files (all enqueue on `s`, return cudaGetLastError()) ----
 cudaError_t tt_launch_grouping(tt_emb* h, cudaStream_t s);
+cudaError_t tt_launch_group_cluster(tt_emb* h, bool rows, cudaStream_t s);
+int tt_group_cluster_ok();
 cudaError_t tt_launch_schedule(tt_emb* h, cudaStream_t s);
 cudaError_t tt_launch_tlist(tt_emb* h, int k, cudaStream_t s);   // digit-major list of the level-k nodes (backward, k < K-1)
 cudaError_t tt_plan_pooling(tt_emb* h, const float* out);          // grid and shares of the pooling pass, before the schedule
@@ -333,12 +339,12 @@ __device__ __forceinline__ void tt_unit_range(const WsView& w, int t, int q, uin
         if (Q > by_groups) Q = by_groups < 1 ? 1 : by_groups;
     }
     if (q >= Q) { g0 = a; g1 = a; return; }
-    const uint64_t ca = w.cost[a], cb = w.cost[b];
-    if (w.ablation & 2) {   // study switch: static schedule, equal group counts
+    if (w.equal_units) {   // equal group counts
         g0 = a + (uint32_t)((uint64_t)(b - a) * (uint64_t)q / Q);
         g1 = a + (uint32_t)((uint64_t)(b - a) * (uint64_t)(q + 1) / Q);
         return;
     }
+    const uint64_t ca = w.cost[a], cb = w.cost[b];
     const uint64_t lo_c = ca + (cb - ca) * (uint64_t)q / Q, hi_c = ca + (cb - ca) * (uint64_t)(q + 1) / Q;
     // first group whose exclusive cost >= target
     auto lower = [&](uint64_t target) {

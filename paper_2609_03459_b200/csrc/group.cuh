@@ -1,6 +1,8 @@
 // Device functions of the grouping and of the schedule, one element (lookup, bitmap word, node, share) at a time, shared by
 // the kernels that run each step over the whole chip (grouping.cu) and by the one that runs all steps in one cluster
 // (group_cluster.cu).
+// The scan functors hold the workspace view by value where a kernel gets the functor as its parameter, by reference inside
+// a kernel that has the view.
 #pragma once
 #include "common.cuh"
 #include "scan.cuh"
@@ -111,9 +113,9 @@ __device__ __forceinline__ void tt_emit_set_bits(uint32_t* __restrict__ val, uin
 
 // ---- level K: rows
 
-template <int TILE>
+template <int TILE, class View = WsView>
 struct PopScan {
-    WsView w;
+    View w;
     __device__ uint32_t size() const { return w.total_words; }
     // every table starts on a scan-tile boundary: the table of a tile's first word is the table of all its words
     __device__ int locate(uint32_t i0) const
@@ -201,38 +203,25 @@ __device__ __forceinline__ uint32_t tt_rank_incl(const WsView& w, const TableDes
     return e.y + __popc(e.x & (0xffffffffu >> (31 - (x & 31))));
 }
 
-// Presence bits of word i of level k < K (one bit per possible length-k prefix of every table) from the scanned bitmap of
-// level k + 1: prefix p is present when some node of level k + 1 lies in [p n_{k+1}, (p + 1) n_{k+1}).  Called by a whole
-// warp, one lane per prefix (the two rank look-ups of a prefix are dependent loads: 32 of them one after the other per
-// thread took 25 us even for the few words of level 1); the word is written whole (no memset, no atomics).
-__device__ __forceinline__ unsigned tt_prefix_word(const WsView& w, int k, uint32_t i, int lane)
+// Whether prefix p of level k < K is present, from the scanned bitmap of level k + 1: some node of that level lies in
+// [p n_{k+1}, (p + 1) n_{k+1}).
+__device__ __forceinline__ bool tt_prefix_present(const WsView& w, const TableDesc& td, int k, uint32_t p)
 {
     const int c = k + 1;
-    int lo_t = 0, hi_t = w.T;
-    while (hi_t - lo_t > 1) {
-        const int mid = (lo_t + hi_t) >> 1;
-        if (w.tdesc[mid].lword_base[k] <= i) lo_t = mid; else hi_t = mid;
-    }
-    const TableDesc& td = w.tdesc[lo_t];
-    const uint32_t p = ((i - td.lword_base[k]) << 5) + lane;
     const uint32_t radix = (uint32_t)td.n[k];                       // radix of digit k + 1
     const uint32_t space_c = c == w.K ? (uint32_t)td.N : td.prefix_space[c];
     const uint64_t lo = (uint64_t)p * radix;
-    bool present = false;
-    if (p < td.prefix_space[k] && lo < space_c) {                    // rows past N do not exist
-        uint64_t hi = lo + radix;
-        if (hi > space_c) hi = space_c;
-        present = tt_rank_incl(w, td, c, (uint32_t)hi - 1u) != tt_rank_excl(w, td, c, (uint32_t)lo);
-    }
-    const unsigned bits = __ballot_sync(0xffffffffu, present);
-    if (lane == 0) w.bml[k][i] = make_uint2(bits, 0u);
-    return bits;
+    if (p >= td.prefix_space[k] || lo >= space_c) return false;      // rows past N do not exist
+    uint64_t hi = lo + radix;
+    if (hi > space_c) hi = space_c;
+    return tt_rank_incl(w, td, c, (uint32_t)hi - 1u) != tt_rank_excl(w, td, c, (uint32_t)lo);
 }
 
 // Level k < K from its own presence bitmap: the ascending distinct prefixes of every table.  Runs after the scan of
 // level k + 1 and k_prefix_bits, which sets this level's bits.
+template <class View = WsView>
 struct LevelScan {
-    WsView w;
+    View w;
     int k;
     __device__ uint32_t size() const { return w.total_words_l[k]; }
     __device__ int locate(uint32_t i0) const
@@ -310,8 +299,9 @@ __device__ __forceinline__ void tt_tmark_node(const WsView& w, const TableDesc& 
     atomicOr(&w.tbm[k][td.tword_base[k] + (key >> 5)].x, 1u << (key & 31));
 }
 
+template <class View = WsView>
 struct TPopScan {
-    WsView w;
+    View w;
     int k;
     __device__ uint32_t size() const { return w.ttotal_words[k]; }
     __device__ int locate(uint32_t) const { return 0; }
@@ -340,8 +330,9 @@ __device__ __forceinline__ void tt_tfill_node(const WsView& w, const TableDesc& 
 // cost of every group in sweep order -> exclusive prefix sums, in place.  The costs are written by the kernel that fills the
 // sweep order (k_tfill; k_costs where the order is the natural one): formed inside the two scan kernels, each cost was
 // three dependent look-ups that a thread made sixteen times in a row (20 us per kernel for five thousand groups).
+template <class View = WsView>
 struct CostScan {
-    WsView w;
+    View w;
     __device__ uint32_t size() const { return w.counters[CTR_LEVEL0 + w.K - 1]; }
     __device__ int locate(uint32_t) const { return 0; }
     __device__ int locate_from(uint32_t, int hint) const { return hint; }

@@ -1,0 +1,250 @@
+// Grouping and schedule of small batches in one kernel: one cluster of sixteen CTAs runs every step, with the cluster's
+// hardware barrier between the steps.
+//
+// The steps of grouping.cu are a chain of fifteen dependent kernels (marks, a scan per level, links, the digit-major list,
+// costs, boundaries), 3 to 5 us each however little they do.  Sixteen SMs do the same work on a few thousand lookups in
+// less than the launches cost: 1 k lookups, one table, grouping and schedule 74 -> 34 us, now bound by the latency of the
+// dependent loads in each step (one to three L2 round trips between two barriers).  The step functions are those of
+// group.cuh; only the distribution over threads differs.  Where every table is swept by warps that take one batch of groups
+// at a time, units of equal group counts do as well as units of equal cost, so the costs and their scan are left out.
+#include "common.cuh"
+#include "scan.cuh"
+#include "group.cuh"
+
+#define GC_THREADS 1024
+#define GC_CTAS 16
+
+// all writes of the cluster's threads before the barrier are visible to all of them after it
+__device__ __forceinline__ void gc_sync()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// elements that each CTA takes
+__device__ __forceinline__ uint32_t gc_run(uint32_t n) { return (n + GC_CTAS - 1) / GC_CTAS; }
+
+// Exclusive scan of f over n elements: every CTA takes a run of them.  The CTAs' sums go straight into the shared memory of
+// all sixteen (`sums`, a slot of its own for every scan of the kernel); a run of up to GC_TILE elements stays in registers
+// between the sum and the second pass.  One barrier inside, none at the end.
+#define GC_IT 4
+#define GC_TILE (GC_THREADS * GC_IT)
+template <class F>
+__device__ __forceinline__ void gc_scan(const F& f, uint32_t n, uint32_t* sums, uint32_t* sm)
+{
+    const uint32_t rank = blockIdx.x, tid = threadIdx.x;
+    const uint32_t per = gc_run(n);
+    const uint32_t lo = min(n, rank * per), hi = min(n, lo + per);
+    const int lane = tid & 31, wid = tid >> 5;
+    int hint = lo < hi ? f.locate(lo) : 0;
+    uint32_t v[GC_IT], ex[GC_IT];
+    int at[GC_IT];
+    uint32_t carry = 0, tot = 0;
+    // values of one tile; exclusive prefixes of its elements inside their warps, the warps' in sm
+    auto load = [&](uint32_t base) {
+#pragma unroll
+        for (int j = 0; j < GC_IT; ++j) {
+            const uint32_t i = base + (uint32_t)j * GC_THREADS + tid;
+            v[j] = 0;
+            if (i < hi) {
+                hint = f.locate_from(i, hint);
+                v[j] = f.value(i, hint);
+            }
+            at[j] = hint;
+        }
+#pragma unroll
+        for (int j = 0; j < GC_IT; ++j) {
+            const uint32_t a = base + (uint32_t)j * GC_THREADS + tid < hi ? tt_scan_amount(f, v[j], 0) : 0u;
+            uint32_t incl = a;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += y;
+            }
+            ex[j] = incl - a;
+            if (lane == 31) sm[j * (GC_THREADS / 32) + wid] = incl;   // element order: stripe j, then warp
+        }
+        __syncthreads();
+        if (wid == 0) {   // exclusive scan of the warps' sums, GC_IT per lane
+            uint32_t x[GC_IT], s = 0;
+#pragma unroll
+            for (int j = 0; j < GC_IT; ++j) { x[j] = sm[lane * GC_IT + j]; s += x[j]; }
+            uint32_t incl = s;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += y;
+            }
+            uint32_t run = incl - s;
+#pragma unroll
+            for (int j = 0; j < GC_IT; ++j) { sm[lane * GC_IT + j] = run; run += x[j]; }
+            if (lane == 31) sm[GC_THREADS / 32 * GC_IT] = run;
+        }
+        __syncthreads();
+        tot = sm[GC_THREADS / 32 * GC_IT];
+    };
+    auto emit = [&](uint32_t base) {
+#pragma unroll
+        for (int j = 0; j < GC_IT; ++j) {
+            const uint32_t i = base + (uint32_t)j * GC_THREADS + tid;
+            if (i < hi) f.emit(i, carry + sm[j * (GC_THREADS / 32) + wid] + ex[j], v[j], at[j]);
+        }
+        carry += tot;
+    };
+    const bool one = per <= GC_TILE;
+    if (one) load(lo);
+    else {
+        uint32_t amount = 0;
+        for (uint32_t i = lo + tid; i < hi; i += GC_THREADS) amount += tt_scan_amount(f, f.value(i, hint), 0);
+        tt_block_excl_scan(amount, sm, tot);
+    }
+    if (tid < GC_CTAS) {   // this CTA's sum to every CTA
+        uint32_t remote;
+        const uint32_t local = (uint32_t)__cvta_generic_to_shared(sums + rank);
+        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(local), "r"(tid));
+        asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(remote), "r"(tot) : "memory");
+    }
+    gc_sync();
+    uint32_t all = 0;
+#pragma unroll
+    for (uint32_t i = 0; i < GC_CTAS; ++i) {
+        const uint32_t x = sums[i];
+        carry += i < rank ? x : 0u;
+        all += x;
+    }
+    if (rank == 0 && tid == 0) f.total(all);
+    if (one) emit(lo);
+    else
+        for (uint32_t base = lo; base < hi; base += GC_TILE) {
+            hint = base == lo ? f.locate(lo) : hint;
+            load(base);
+            emit(base);
+            __syncthreads();
+        }
+}
+
+// rows: from the row ids on (workspace regions cleared here); otherwise the row bitmap is scanned already
+__global__ void __launch_bounds__(GC_THREADS) k_group_cluster(const __grid_constant__ WsView w, int rows)
+{
+    tt_pdl_enter();
+    __shared__ uint32_t sm[GC_THREADS / 32 * GC_IT + 1];
+    __shared__ uint32_t sums[TT_MAXK + 1][GC_CTAS];   // [k]: the scan of level k, [K] later that of the costs; [0]: of the digit-major bitmap
+    const int K = w.K;
+    const uint32_t tid = threadIdx.x, first = blockIdx.x * GC_THREADS + tid, step = GC_CTAS * GC_THREADS;
+    const int lane = tid & 31, wid = tid >> 5;
+    const bool digit_major = tt_digit_major(w);
+    if (rows) {
+        if (first < 16 + 64) reinterpret_cast<uint32_t*>(w.status)[first] = 0u;   // status and counters are adjacent
+        uint4* bm4 = reinterpret_cast<uint4*>(w.bm);                             // a whole number of scan tiles
+        for (uint32_t i = first; i < w.total_words / 2; i += step) bm4[i] = make_uint4(0u, 0u, 0u, 0u);
+    }
+    if (digit_major)
+        for (uint32_t i = first; i < w.ttotal_words[K - 1]; i += step) w.tbm[K - 1][i] = make_uint2(0u, 0u);
+    gc_sync();   // also: every CTA runs before another writes into its shared memory
+    if (rows) {
+        tt_check_offsets(w, first, step);
+        tt_mark_rows<false>(w, first, step, (int64_t)step * 4);
+        gc_sync();
+        gc_scan(PopScan<TT_SCAN_TILE, const WsView&>{w}, w.total_words, sums[K], sm);
+        gc_sync();
+    }
+    for (int k = K - 1; k >= 1; --k) {
+        // presence bits of the words that this CTA scans, a warp per word, four words at a time
+        const uint32_t n = w.total_words_l[k], per = gc_run(n), lo = min(n, blockIdx.x * per), hi = min(n, lo + per);
+        const LevelScan<const WsView&> ls{w, k};
+        int t = lo < hi ? ls.locate(lo) : 0;
+        for (uint32_t i0 = lo + wid; i0 < hi; i0 += GC_THREADS / 32 * 4) {
+            bool present[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const uint32_t i = i0 + (uint32_t)j * (GC_THREADS / 32);
+                present[j] = false;
+                if (i < hi) {
+                    t = ls.locate_from(i, t);
+                    const TableDesc& td = w.tdesc[t];
+                    present[j] = tt_prefix_present(w, td, k, ((i - td.lword_base[k]) << 5) + lane);
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const uint32_t i = i0 + (uint32_t)j * (GC_THREADS / 32);
+                const unsigned bits = __ballot_sync(0xffffffffu, present[j]);
+                if (lane == 0 && i < hi) w.bml[k][i] = make_uint2(bits, 0u);
+            }
+        }
+        __syncthreads();
+        gc_scan(ls, n, sums[k], sm);
+        gc_sync();
+    }
+    // links of all levels in one pass over their nodes, share boundaries by the threads that come last
+    uint32_t nodes = 0;
+    for (int k = K - 1; k >= 1; --k) nodes += w.counters[CTR_LEVEL0 + k];
+    if (first < (uint32_t)(K - 1)) tt_link_end(w, (int)first + 1);
+    for (uint32_t x = first; x < nodes; x += step) {
+        uint32_t v = x;
+        int k = K - 1;
+        while (v >= w.counters[CTR_LEVEL0 + k]) v -= w.counters[CTR_LEVEL0 + k--];
+        const TableDesc& td = w.tdesc[tt_find_table(w.tb[k], w.T, v)];
+        if (digit_major && k == K - 1) tt_tmark_node(w, td, k, v);
+        tt_link_node(w, td, k, v);
+    }
+    if (w.pool_shares > 0)
+        for (int64_t ci = step - 1 - first; ci <= w.pool_shares; ci += step) tt_pool_bound(w, ci);
+    const int64_t units = (int64_t)w.T * w.units_per_table;
+    if (w.equal_units)
+        for (int64_t u = step - 1 - first; u < units; u += step) tt_unit_bounds(w, (int)u);
+    gc_sync();
+    const uint32_t groups = w.counters[CTR_LEVEL0 + K - 1];
+    if (digit_major) {
+        gc_scan(TPopScan<const WsView&>{w, K - 1}, w.ttotal_words[K - 1], sums[0], sm);
+        gc_sync();
+        for (uint32_t v = first; v < groups; v += step)
+            tt_tfill_node(w, w.tdesc[tt_find_table(w.tb[K - 1], w.T, v)], K - 1, v, !w.equal_units);
+    } else if (!w.equal_units) {
+        for (uint32_t g = first; g < groups; g += step)
+            w.cost[g] = tt_group_cost(w, w.tdesc[tt_find_table(w.tb[K - 1], w.T, g)], g);
+    }
+    if (w.equal_units) return;
+    gc_sync();
+    gc_scan(CostScan<const WsView&>{w}, groups, sums[K], sm);
+    gc_sync();
+    for (int64_t u = first; u < units; u += step) tt_unit_bounds(w, (int)u);
+}
+
+cudaError_t tt_launch_group_cluster(tt_emb* h, bool rows, cudaStream_t s)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(GC_CTAS);
+    cfg.blockDim = dim3(GC_THREADS);
+    cfg.stream = s;
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = GC_CTAS;
+    at[1].val.clusterDim.y = 1;
+    at[1].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 2;
+    cudaError_t e = cudaLaunchKernelEx(&cfg, k_group_cluster, h->v, rows ? 1 : 0);
+    if (e == cudaSuccess) tt_note_launch();
+    return e;
+}
+
+// whether the device takes the cluster (sixteen CTAs are past the portable eight): asked once per handle
+int tt_group_cluster_ok()
+{
+    if (cudaFuncSetAttribute(k_group_cluster, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) { cudaGetLastError(); return 0; }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(GC_CTAS);
+    cfg.blockDim = dim3(GC_THREADS);
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = GC_CTAS;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, k_group_cluster, &cfg) != cudaSuccess) { cudaGetLastError(); return 0; }
+    return n > 0;
+}

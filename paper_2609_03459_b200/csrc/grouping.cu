@@ -35,12 +35,25 @@ __global__ void __launch_bounds__(256, 8) k_mark(WsView w)
 
 // ---------------------------------------------------------------------------------------------- prefix levels
 
+// Presence bitmap of level k < K (one bit per possible length-k prefix of every table) from level k + 1.  One warp per word,
+// one lane per prefix (the two rank look-ups of a prefix are dependent loads: 32 of them one after the other per thread
+// took 25 us even for the few words of level 1); the words are written whole (no memset, no atomics).
 __global__ void __launch_bounds__(256) k_prefix_bits(WsView w, int k)
 {
     tt_pdl_enter();
+    const int lane = threadIdx.x & 31;
     const uint32_t nwords = w.total_words_l[k];
     const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
-    for (uint32_t i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < nwords; i += nwarps) tt_prefix_word(w, k, i, threadIdx.x & 31);
+    for (uint32_t i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < nwords; i += nwarps) {
+        int lo_t = 0, hi_t = w.T;
+        while (hi_t - lo_t > 1) {
+            const int mid = (lo_t + hi_t) >> 1;
+            if (w.tdesc[mid].lword_base[k] <= i) lo_t = mid; else hi_t = mid;
+        }
+        const TableDesc& td = w.tdesc[lo_t];
+        const unsigned bits = __ballot_sync(0xffffffffu, tt_prefix_present(w, td, k, ((i - td.lword_base[k]) << 5) + lane));
+        if (lane == 0) w.bml[k][i] = make_uint2(bits, 0u);
+    }
 }
 
 // Links of all levels (blockIdx.y = K - 1 - k), and the marks of the digit-major order of the level-(K-1) nodes (`mark`)
@@ -114,10 +127,31 @@ __global__ void __launch_bounds__(256) k_nodedup_levels(WsView w)
     }
 }
 
+// 0: a kernel per step; 1: one cluster of sixteen SMs (group_cluster.cu) from the prefix levels on; 2: one cluster for
+// everything.  The cluster saves a dozen launches and loses where a step has work for more SMs: scans and links of large
+// prefix spaces, marks and scan of long row bitmaps.  Whole call with 0 / 1 / 2, us: 1 table of 1 M rows (33 k words), 1 k
+// lookups 73 / 53 / 43; 2 tables, 98 k words, 18 k lookups (training) 254 / 229 / 228; 8 tables, 573 k words, 8 k lookups
+// 95 / 78 / 95; 16 tables, prefix bitmaps of 10 k words 127 / 115; of 30 k words 221 / 253.
+#define TT_CLUSTER_LEVEL_WORDS (1u << 14)
+#define TT_CLUSTER_ROW_WORDS (1u << 17)
+#define TT_CLUSTER_LOOKUPS (1 << 15)
+static int tt_use_cluster(const tt_emb* h)
+{
+    const WsView& w = h->v;
+    if (!h->cluster_ok || w.ablation) return 0;
+    for (int k = 1; k < w.K; ++k)
+        if (w.total_words_l[k] > TT_CLUSTER_LEVEL_WORDS) return 0;
+    if (w.K >= 3 && w.ttotal_words[w.K - 1] > TT_CLUSTER_LEVEL_WORDS) return 0;
+    return w.total_words <= TT_CLUSTER_ROW_WORDS && w.L <= TT_CLUSTER_LOOKUPS ? 2 : 1;
+}
+
 cudaError_t tt_launch_grouping(tt_emb* h, cudaStream_t s)
 {
     WsView& w = h->v;
     cudaError_t e;
+    const int cluster = tt_use_cluster(h);
+    w.equal_units = (cluster != 0 && h->warp_groups) || (w.ablation & 2) ? 1 : 0;
+    if (cluster == 2) return tt_launch_group_cluster(h, true, s);
     // status word + counters are adjacent; bitmap follows its own region
     if ((e = cudaMemsetAsync(w.status, 0, (16 + 64) * sizeof(uint32_t), s)) != cudaSuccess) return e;
     const int64_t nb = (int64_t)w.T * w.B + 1;
@@ -131,7 +165,7 @@ cudaError_t tt_launch_grouping(tt_emb* h, cudaStream_t s)
         return cudaGetLastError();
     }
     if ((e = cudaMemsetAsync(w.bm, 0, (size_t)w.total_words * sizeof(uint2), s)) != cudaSuccess) return e;
-    if (tt_digit_major(w) && (e = cudaMemsetAsync(w.tbm[w.K - 1], 0, (size_t)w.ttotal_words[w.K - 1] * sizeof(uint2), s)) != cudaSuccess) return e;
+    if (cluster == 0 && tt_digit_major(w) && (e = cudaMemsetAsync(w.tbm[w.K - 1], 0, (size_t)w.ttotal_words[w.K - 1] * sizeof(uint2), s)) != cudaSuccess) return e;
     {
         int64_t want = (w.L + 1023) / 1024;
         const bool fused = w.L <= TT_FUSED_INGEST;
@@ -154,6 +188,7 @@ cudaError_t tt_launch_grouping(tt_emb* h, cudaStream_t s)
         e = tt_scan(ps, w.total_words, w.scan_tmp, s, ptiles);
     }
     if (e != cudaSuccess) return e;
+    if (cluster == 1) return tt_launch_group_cluster(h, false, s);
     for (int k = w.K - 1; k >= 1; --k) {
         {
             const uint32_t want = (w.total_words_l[k] + 7u) / 8u;   // a warp per word
@@ -161,8 +196,8 @@ cudaError_t tt_launch_grouping(tt_emb* h, cudaStream_t s)
             if ((e = tt_launch_pdl(k_prefix_bits, dim3(g), dim3(256), 0, s, w, k)) != cudaSuccess) return e;
             tt_note_launch();
         }
-        LevelScan ls{w, k};
-        if ((e = tt_scan<LevelScan, TT_LSCAN_ITEMS>(ls, w.total_words_l[k], w.scan_tmp, s)) != cudaSuccess) return e;
+        LevelScan<> ls{w, k};
+        if ((e = tt_scan<LevelScan<>, TT_LSCAN_ITEMS>(ls, w.total_words_l[k], w.scan_tmp, s)) != cudaSuccess) return e;
         if ((w.ablation & 1) && k == w.K - 1) {   // the scan still sets the bits of level K-2; its nodes are replaced
             if ((e = tt_launch_pdl(k_unique_groups, dim3(h->sm_count * 8), dim3(256), 0, s, w)) != cudaSuccess) return e;
             tt_note_launch();
@@ -196,7 +231,7 @@ static cudaError_t launch_tfill(tt_emb* h, int k, bool costs, cudaStream_t s)
 {
     WsView& w = h->v;
     cudaError_t e;
-    TPopScan tp{w, k};
+    TPopScan<> tp{w, k};
     if ((e = tt_scan(tp, w.ttotal_words[k], w.scan_tmp, s)) != cudaSuccess) return e;
     if ((e = tt_launch_pdl(k_tfill, dim3(h->sm_count * 8), dim3(256), 0, s, w, k, costs ? 1 : 0)) != cudaSuccess) return e;
     tt_note_launch();
@@ -240,14 +275,15 @@ cudaError_t tt_launch_schedule(tt_emb* h, cudaStream_t s)
 {
     WsView& w = h->v;
     cudaError_t e;
+    if (tt_use_cluster(h) != 0) return cudaSuccess;   // done with the grouping
     if (tt_digit_major(w)) {
         if ((e = launch_tfill(h, w.K - 1, true, s)) != cudaSuccess) return e;
     } else {
         if ((e = tt_launch_pdl(k_costs, dim3(h->sm_count * 8), dim3(256), 0, s, w)) != cudaSuccess) return e;
         tt_note_launch();
     }
-    CostScan cs{w};
-    if ((e = tt_scan<CostScan, TT_CSCAN_ITEMS>(cs, w.cap[w.K - 1], w.scan_tmp, s)) != cudaSuccess) return e;
+    CostScan<> cs{w};
+    if ((e = tt_scan<CostScan<>, TT_CSCAN_ITEMS>(cs, w.cap[w.K - 1], w.scan_tmp, s)) != cudaSuccess) return e;
     int64_t want = (int64_t)w.T * w.units_per_table;
     if (want < w.pool_shares + 1) want = w.pool_shares + 1;
     want = (want + 127) / 128;
