@@ -175,21 +175,9 @@ extern "C" int tt_emb_create(const tt_emb_config_t* cfg, tt_emb_t* out_handle)
     h->capU = (cfg->max_unique_rows > 0 && cfg->max_unique_rows < bound) ? cfg->max_unique_rows : bound;
     if (h->ablation & 4) h->capU = cfg->max_lookups > 0 ? cfg->max_lookups : 1;   // one row slot per lookup
 
-    // work units: every table is cut into `units` equal-cost slices, one CTA each
-    // about 8 waves of 8 resident CTAs per SM: fine enough that the last wave and table-size differences do not matter
-    int Q = (64 * h->sm_count + T - 1) / T;   // (32 * and 128 * measured: 16.8 / 16.5 ms per training step against 16.4)
-    {   // ... but not so fine that a unit holds fewer than sixteen groups, one batch of its four warps
-        uint64_t groups = level_space[K - 1] < (uint64_t)h->capU ? level_space[K - 1] : (uint64_t)h->capU;
-        const int64_t by_groups = (int64_t)(groups / (uint64_t)T / TT_UNIT_GROUPS);
-        if (Q > by_groups) Q = (int)by_groups;
-    }
-    if (Q < 8) Q = 8;
-    if (Q > 16384) Q = 16384;
-    int unit_base = 0;
     int64_t gpart = 0;
     for (int t = 0; t < T; ++t) {
         TableDesc& td = h->tab[t];
-        td.units = Q;
         td.fast = -1;
         if (K >= 3 && td.d[K - 1] == 4) {
             // (P_{K-1}, r_{K-1}, P_{K-2}) combinations with a register-tiled variant (see forward.cu)
@@ -211,7 +199,7 @@ extern "C" int tt_emb_create(const tt_emb_config_t* cfg, tt_emb_t* out_handle)
             else if (PMv == 4 && Mv == 2 && RBv == 16 && quad_ok) td.fast = 9;
             else if (PMv == 4 && Mv == 2 && RBv == 8) td.fast = 10;   // D = 16 with rank 8: FP32 pipe (slices of 16 columns)
         }
-        td.unit_groups = td.fast == 3 ? 4 * TT_UNIT_GROUPS : TT_UNIT_GROUPS;
+        td.unit_groups = td.fast == 3 ? 4 * TT_UNIT_GROUPS : td.fast >= 0 ? TT_UNIT_GROUPS : TT_UNIT_GROUPS_ANY;
         for (int k = 0; k < TT_MAXK; ++k) td.midfast[k] = -1;
         for (int k = 2; k <= K - 1; ++k) {
             const int Mv = td.P[k - 1], rav = td.r[k - 1], colsv = td.d[k - 1] * td.r[k];
@@ -227,10 +215,28 @@ extern "C" int tt_emb_create(const tt_emb_config_t* cfg, tt_emb_t* out_handle)
             else if (Mv == 2 && rav == 8 && colsv == 32) td.midfast[k] = 9;
             else if (Mv == 2 && rav == 8 && colsv == 16) td.midfast[k] = 10;
         }
-        td.unit_base = unit_base;
-        unit_base += Q;
         td.gpart_off = gpart;
         gpart += (td.core_floats[K - 1] + 3) / 4 * 4;
+    }
+
+    // work units: every table is cut into `units` equal-cost slices, one CTA each
+    // about 8 waves of 8 resident CTAs per SM: fine enough that the last wave and table-size differences do not matter
+    int Q = (64 * h->sm_count + T - 1) / T;   // (32 * and 128 * measured: 16.8 / 16.5 ms per training step against 16.4)
+    {   // ... but not so fine that a unit holds only a few groups
+        int unit_groups = h->tab[0].unit_groups;
+        for (int t = 1; t < T; ++t)
+            if (h->tab[t].unit_groups < unit_groups) unit_groups = h->tab[t].unit_groups;
+        uint64_t groups = level_space[K - 1] < (uint64_t)h->capU ? level_space[K - 1] : (uint64_t)h->capU;
+        const int64_t by_groups = K == 2 ? h->capU / T / TT_UNIT_ROWS : (int64_t)(groups / (uint64_t)T / (uint64_t)unit_groups);
+        if (Q > by_groups) Q = (int)by_groups;
+    }
+    if (Q < 8) Q = 8;
+    if (Q > 16384) Q = 16384;
+    int unit_base = 0;
+    for (int t = 0; t < T; ++t) {
+        h->tab[t].units = Q;
+        h->tab[t].unit_base = unit_base;
+        unit_base += Q;
     }
     h->warp_groups = true;
     for (int t = 0; t < T; ++t)

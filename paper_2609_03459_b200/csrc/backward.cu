@@ -21,12 +21,12 @@
 #include "mma.cuh"
 #include "quad_mid.cuh"
 #include "group.cuh"
+#include "generic.cuh"
 #include <type_traits>
 
 #define HT_SIZE 4096
 #define HT_TILE 2048
 #define HT_EMPTY 0xffffffffu
-#define RB 8  // rows per batch in the last-level kernel
 
 // ---------------------------------------------------------------------------------------------- small utilities
 
@@ -718,63 +718,49 @@ cudaError_t tt_launch_bwd_dE(tt_emb* h, const float* grad_out, cudaStream_t s)
 
 // ---------------------------------------------------------------------------------------------- 3. last level
 
-// generic fallback (any shape): the whole CTA works on one group at a time
-__device__ __forceinline__ void tt_sweep_bwd_generic(const WsView& w, const TableDesc& td, uint32_t g0, uint32_t g1,
-                                                     float* gk, float* Pl, float* Cs, float* dCs, float* dEs)
+// any shape: batches of groups spread flat over the CTA (generic.cuh)
+__global__ void __launch_bounds__(GEN_THREADS, 3) k_sweep_bwd_any(WsView w, int vbase)
 {
-    const int K = w.K, kl = K - 1, km = K - 2;
-    const int Pm = td.P[K - 1], rb = td.r[K - 1], dK = td.d[kl], D = w.D;
-    const int sliceK = td.slice_floats[kl];
-    const uint32_t nK = (uint32_t)td.n[kl];
-    for (int i = threadIdx.x; i < Pm * rb; i += blockDim.x) dCs[i] = 0.f;
-    __syncthreads();
-    for (uint32_t jpos = g0; jpos < g1; ++jpos) {
-        const uint32_t g = K >= 3 ? w.tnode[K - 1][jpos] : jpos;
-        const uint32_t val = w.val[K - 1][g];
-        if (K >= 3) {
-            const int M = td.P[km], ra = td.r[km], cols = td.d[km] * rb;
-            const float* src = tt_left_operand(w, td, K - 1, g);
-            for (int i = threadIdx.x; i < M * ra; i += blockDim.x) Pl[i] = src[i];
-            __syncthreads();
-            const uint32_t im = val % (uint32_t)td.n[km];
-            tt_mid_product(Pl, td.core[km] + (size_t)im * td.slice_floats[km], Cs, M, ra, cols);
-        } else {
-            const float* src = td.core[0] + (size_t)val * td.slice_floats[0];
-            for (int i = threadIdx.x; i < Pm * rb; i += blockDim.x) Cs[i] = src[i];
-        }
-        __syncthreads();
-        const uint32_t u0 = w.cstart[K - 1][g], u1 = w.cstart[K - 1][g + 1];
-        for (uint32_t ub = u0; ub < u1; ub += RB) {
-            const int nr = (int)min((uint32_t)RB, u1 - ub);
-            for (int i = threadIdx.x; i < nr * D; i += blockDim.x) dEs[i] = w.E[(size_t)ub * D + i];
-            __syncthreads();
-            // dG_K[i_K][b][j] += sum_p C[p][b] * dE[p][j]     ("dD = C^T . dE")
-            for (int it = threadIdx.x; it < nr * sliceK; it += blockDim.x) {
-                const int rr = it / sliceK, e = it - rr * sliceK;
-                const int bb = e / dK, j = e - bb * dK;
-                const float* de = dEs + rr * D + j;
-                float acc = 0.f;
-                for (int p = 0; p < Pm; ++p) acc = fmaf(Cs[p * rb + bb], de[p * dK], acc);
-                const uint32_t iK = w.val[K][ub + rr] % nK;
-                atomicAdd(gk + (size_t)iK * sliceK + e, acc);
-            }
-            // dC[p][b] += sum_j dE[p][j] * D[b][j]             ("dC = dE . D^T", summed over the group: Eq. 2)
-            for (int it = threadIdx.x; it < Pm * rb; it += blockDim.x) {
-                const int p = it / rb, bb = it - p * rb;
-                float acc = 0.f;
-                for (int rr = 0; rr < nr; ++rr) {
-                    const uint32_t iK = w.val[K][ub + rr] % nK;
-                    const float* Dsl = td.core[kl] + (size_t)iK * sliceK + bb * dK;
-                    const float* de = dEs + rr * D + p * dK;
-                    for (int j = 0; j < dK; ++j) acc = fmaf(de[j], __ldg(Dsl + j), acc);
-                }
-                dCs[it] += acc;
+    tt_pdl_enter();
+    extern __shared__ __align__(16) float sm[];
+    __shared__ GenBatch b;
+    const int t = w.vlist[vbase + blockIdx.y], K = w.K;
+    const uint2 rng = w.unit_rng[t * w.units_per_table + blockIdx.x];
+    const TableDesc& td = w.tdesc[t];
+    const int stripe = (blockIdx.x + blockIdx.y) % TT_STRIPES;
+    float* gk = w.gpart + (size_t)stripe * w.gpart_stride + td.gpart_off;
+    float *Cs = sm, *dCs = sm + GEN_C_FLOATS;
+    const bool vec = (td.d[K - 1] & 3) == 0;
+    const int Pm = td.P[K - 1], rb = td.r[K - 1], pitch = gen_pitch(rb);
+    const uint32_t ng = (uint32_t)gen_groups(td, K);
+    uint2 groups, range;
+    gen_unit(w, t, rng, groups, range);
+    for (uint32_t base = groups.x; base < groups.y; base += ng) {
+        const int cnt = (int)min(ng, groups.y - base);
+        for (int i = threadIdx.x; i < cnt * Pm * pitch; i += GEN_THREADS) dCs[i] = 0.f;
+        gen_batch_begin(w, td, base, cnt, range, b);
+        gen_batch_c(w, td, cnt, b, Cs);
+        const uint32_t rows = b.row0[cnt];
+        for (uint32_t r0 = 0; r0 < rows; r0 += GEN_ROWS) {
+            const int n = (int)min((uint32_t)GEN_ROWS, rows - r0);
+            gen_rows(w, td, cnt, r0, n, b);
+            if (vec) {
+                gen_backward_slice<true>(w, td, n, b, Cs, gk);
+                gen_backward_dc<true>(w, td, r0, n, b, dCs);
+            } else {
+                gen_backward_slice<false>(w, td, n, b, Cs, gk);
+                gen_backward_dc<false>(w, td, r0, n, b, dCs);
             }
             __syncthreads();
         }
         // hand dC to the level above (K = 2: it is the gradient of the first core's slice itself)
-        float* dst = K >= 3 ? w.dP[K - 1] + (size_t)g * w.stride[K - 1] : td.grad[0] + (size_t)val * td.slice_floats[0];
-        for (int i = threadIdx.x; i < Pm * rb; i += blockDim.x) { dst[i] = dCs[i]; dCs[i] = 0.f; }
+        for (int it = threadIdx.x; it < cnt * Pm * rb; it += GEN_THREADS) {
+            const int q = it / (Pm * rb), e = it - q * (Pm * rb), p = e / rb;
+            float* dst = K >= 3 ? w.dP[K - 1] + (size_t)b.g[q] * w.stride[K - 1] : td.grad[0] + (size_t)b.val[q] * td.slice_floats[0];
+            const float x = dCs[q * (Pm * pitch) + p * pitch + (e - p * rb)];
+            if (b.part[q]) atomicAdd(dst + e, x);   // K = 2: the first core's gradient starts at zero
+            else dst[e] = x;
+        }
         __syncthreads();
     }
 }
@@ -1346,14 +1332,6 @@ __global__ void __launch_bounds__(128, (V == 5 || V == 6 || V == 8 || V == 9 || 
     const TableDesc& td = w.tdesc[t];
     const int stripe = (blockIdx.x + blockIdx.y) % TT_STRIPES;
     float* gk = w.gpart + (size_t)stripe * w.gpart_stride + td.gpart_off;
-    if (V < 0) {
-        float* Pl = sm;
-        float* Cs = Pl + pl_floats;
-        float* dCs = Cs + c_floats;
-        float* dEs = dCs + c_floats;
-        tt_sweep_bwd_generic(w, td, g0, g1, gk, Pl, Cs, dCs, dEs);
-        return;
-    }
     __shared__ uint32_t next;
     if (threadIdx.x == 0) next = g0;
     __syncthreads();
@@ -1405,17 +1383,22 @@ static cudaError_t launch_sweep_bwd(tt_emb* h, int max_pl, int max_c, cudaStream
     if (V == 6) max_c = 8 * (16 + 8);
     if (V == 8) max_c = 4 * (32 + 8);
     if (V == 9) max_c = 4 * (16 + 8);
-    size_t smem = V < 0 ? (size_t)(max_pl + 2 * max_c + RB * h->D) * sizeof(float)
-                        : (size_t)4 * (max_pl + max_c) * sizeof(float);
+    size_t smem = (size_t)4 * (max_pl + max_c) * sizeof(float);
     if (V == 5) smem = (size_t)4 * 8 * 8 * 36 * sizeof(float);    // eight C tiles per warp, rows padded by four floats
     if (V == 6) smem = (size_t)4 * 8 * 8 * 20 * sizeof(float);
     if (V == 8) smem = (size_t)4 * 8 * 4 * 36 * sizeof(float);
     if (V == 9) smem = (size_t)4 * 8 * 4 * 20 * sizeof(float);
     if (V == 1) smem = (size_t)4 * 4 * 16 * 20 * sizeof(float);   // four C tiles per warp
-    cudaError_t e = cudaFuncSetAttribute(k_sweep_bwd<V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
+    cudaError_t e;
     if ((e = tt_stage_begin(h, 9 + TT_NUM_VARIANTS + 1 + V + 1, s)) != cudaSuccess) return e;
-    if ((e = tt_launch_pdl(k_sweep_bwd<V>, dim3(h->units_per_table, n), dim3(128), smem, s, h->v, max_pl, max_c, h->vbase[V + 1])) != cudaSuccess) return e;
+    if constexpr (V < 0) {
+        smem = 2 * GEN_C_FLOATS * sizeof(float);
+        if ((e = cudaFuncSetAttribute(k_sweep_bwd_any, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
+        if ((e = tt_launch_pdl(k_sweep_bwd_any, dim3(h->units_per_table, n), dim3(GEN_THREADS), smem, s, h->v, h->vbase[0])) != cudaSuccess) return e;
+    } else {
+        if ((e = cudaFuncSetAttribute(k_sweep_bwd<V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
+        if ((e = tt_launch_pdl(k_sweep_bwd<V>, dim3(h->units_per_table, n), dim3(128), smem, s, h->v, max_pl, max_c, h->vbase[V + 1])) != cudaSuccess) return e;
+    }
     tt_note_launch();
     if ((e = tt_stage_end(h, 9 + TT_NUM_VARIANTS + 1 + V + 1, s)) != cudaSuccess) return e;
     return cudaGetLastError();

@@ -25,6 +25,10 @@
 // 325 / 319 / 343; 4 tables x 9 k (D = 32, rank 8) 119 / 117 / 107 / 122 / 188; four cores, 4.7 k groups 304 / 310 / 319 / 422 /
 // 576; D = 128, rank 32, 27 k groups (forward) 236 / 164 / 145 / 137 / 129
 #define TT_UNIT_GROUPS 16
+// ... and of the any-shape sweeps, whose CTAs take a batch of groups at a time (3x3x5, 29 k groups, forward + backward sweep
+// with at least 1 / 4 / 8 / 16 groups: 332 / 285 / 252 / 253 us; 8x8 with K = 2, 420 k lookups, whole call 1.16 ms with 8, 1.68 with 16)
+#define TT_UNIT_GROUPS_ANY 8
+#define TT_UNIT_ROWS 64   // fewest rows of a unit of a K = 2 table
 #define TT_DE_CHUNK 1024                                  // most sorted lookups per warp in the dE segment reduction
 #define TT_NUM_STAGES 33                                // 0..8 pipeline stages, 9..20 forward sweep variants -1..10, 21..32 backward sweep variants
 #define TT_STRIPES 8                                     // L2-resident partial copies of the last core's gradient
@@ -324,12 +328,20 @@ __device__ __forceinline__ uint32_t tt_group_cost(const WsView& w, const TableDe
     return (uint32_t)(((c_mid + (uint64_t)nchild * c_last) >> w.cost_shift) + 1);
 }
 
-// group range [g0, g1) of work unit q of table t: an equal-cost slice of the table's level-(K-1) groups in sweep order
+// group range (K = 2: row range) [g0, g1) of work unit q of table t: an equal-cost slice of the table's level-(K-1) groups in sweep order
 // (called by one thread per unit, once per forward: k_unit_ranges)
 __device__ __forceinline__ void tt_unit_range(const WsView& w, int t, int q, uint32_t& g0, uint32_t& g1)
 {
     const TableDesc& td = w.tdesc[t];
     const int lvl = w.K - 1;
+    if (w.K == 2) {   // ranges of rows, see generic.cuh
+        const uint32_t u0 = w.tb[2][t], n = w.tb[2][t + 1] - u0;
+        const uint32_t Q = min((uint32_t)td.units, max(1u, n / TT_UNIT_ROWS));
+        if ((uint32_t)q >= Q) { g0 = u0; g1 = u0; return; }
+        g0 = u0 + (uint32_t)((uint64_t)n * (uint32_t)q / Q);
+        g1 = u0 + (uint32_t)((uint64_t)n * (uint32_t)(q + 1) / Q);
+        return;
+    }
     const uint32_t a = w.tb[lvl][t], b = w.tb[lvl][t + 1];
     // the host sizes the grid for the largest possible number of groups; with fewer groups in this batch the table is
     // cut into fewer units (at least td.unit_groups groups each) and the surplus CTAs leave at once

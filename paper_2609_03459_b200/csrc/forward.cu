@@ -13,6 +13,7 @@
 #include "scan.cuh"
 #include "mma.cuh"
 #include "quad_mid.cuh"
+#include "generic.cuh"
 
 // ---------------------------------------------------------------------------------------------- products
 
@@ -503,39 +504,30 @@ __device__ __forceinline__ void tt_sweep_pair_cta(const WsView& w, const TableDe
     }
 }
 
-// generic fallback: the whole CTA works on one group at a time (any shape)
-__device__ __forceinline__ void tt_sweep_generic(const WsView& w, const TableDesc& td, uint32_t g0, uint32_t g1, float* Pl, float* Cs)
+// any shape: batches of groups spread flat over the CTA (generic.cuh)
+__global__ void __launch_bounds__(GEN_THREADS) k_sweep_fwd_any(WsView w, int vbase)
 {
-    const int K = w.K, kl = K - 1, km = K - 2;
-    const int Pm = td.P[K - 1], rb = td.r[K - 1], dK = td.d[kl], D = w.D;
-    const uint32_t nK = (uint32_t)td.n[kl];
-    for (uint32_t jpos = g0; jpos < g1; ++jpos) {
-        const uint32_t g = (K >= 3 && !(w.ablation & 1)) ? w.tnode[K - 1][jpos] : jpos;
-        const uint32_t val = w.val[K - 1][g];
-        if (K >= 3) {
-            const int M = td.P[km], ra = td.r[km], cols = td.d[km] * rb;
-            const float* src = tt_left_operand(w, td, K - 1, g);
-            for (int i = threadIdx.x; i < M * ra; i += blockDim.x) Pl[i] = src[i];
+    tt_pdl_enter();
+    extern __shared__ __align__(16) float sm[];
+    __shared__ GenBatch b;
+    const int t = w.vlist[vbase + blockIdx.y];
+    const uint2 rng = w.unit_rng[t * w.units_per_table + blockIdx.x];
+    const TableDesc& td = w.tdesc[t];
+    const bool vec = (td.d[w.K - 1] & 3) == 0;   // then slices, their rows and the row buffer's rows are whole float4s
+    const uint32_t ng = (uint32_t)gen_groups(td, w.K);
+    uint2 groups, range;
+    gen_unit(w, t, rng, groups, range);
+    for (uint32_t base = groups.x; base < groups.y; base += ng) {
+        const int cnt = (int)min(ng, groups.y - base);
+        gen_batch_begin(w, td, base, cnt, range, b);
+        gen_batch_c(w, td, cnt, b, sm);
+        const uint32_t rows = b.row0[cnt];
+        for (uint32_t r0 = 0; r0 < rows; r0 += GEN_ROWS) {
+            const int n = (int)min((uint32_t)GEN_ROWS, rows - r0);
+            gen_rows(w, td, cnt, r0, n, b);
+            if (vec) gen_forward_rows<true>(w, td, n, b, sm);
+            else gen_forward_rows<false>(w, td, n, b, sm);
             __syncthreads();
-            const uint32_t im = val % (uint32_t)td.n[km];
-            tt_mid_product(Pl, td.core[km] + (size_t)im * td.slice_floats[km], Cs, M, ra, cols);
-        } else {
-            const float* src = td.core[0] + (size_t)val * td.slice_floats[0];
-            for (int i = threadIdx.x; i < Pm * rb; i += blockDim.x) Cs[i] = src[i];
-        }
-        __syncthreads();
-        const uint32_t u0 = w.cstart[K - 1][g], u1 = w.cstart[K - 1][g + 1];
-        const int items = (int)(u1 - u0) * D;
-        for (int it = threadIdx.x; it < items; it += blockDim.x) {
-            const int rr = it / D, e = it - rr * D;
-            const int p = e / dK, j = e - p * dK;
-            const uint32_t u = u0 + rr;
-            const uint32_t iK = w.val[K][u] % nK;
-            const float* Dsl = td.core[kl] + (size_t)iK * td.slice_floats[kl];
-            const float* c = Cs + p * rb;
-            float acc = 0.f;
-            for (int b = 0; b < rb; ++b) acc = fmaf(c[b], __ldg(Dsl + b * dK + j), acc);
-            w.E[(size_t)u * D + e] = acc;
         }
         __syncthreads();
     }
@@ -545,7 +537,7 @@ __device__ __forceinline__ void tt_sweep_generic(const WsView& w, const TableDes
 // one instantiation per shape variant V so that each gets its own register budget.  blockIdx.y walks the
 // tables of variant V (w.vlist), blockIdx.x the table's equal-cost slices.
 template <int V>
-__global__ void __launch_bounds__(128, (V >= 0 && V != 3 && V != 4) ? 6 : 1) k_sweep_fwd(WsView w, int pl_floats, int c_floats, int vbase)
+__global__ void __launch_bounds__(128, (V != 3 && V != 4) ? 6 : 1) k_sweep_fwd(WsView w, int pl_floats, int c_floats, int vbase)
 {
     tt_pdl_enter();
     extern __shared__ __align__(16) float sm[];
@@ -554,10 +546,6 @@ __global__ void __launch_bounds__(128, (V >= 0 && V != 3 && V != 4) ? 6 : 1) k_s
     const uint2 rng = w.unit_rng[t * w.units_per_table + blockIdx.x];
     const uint32_t g0 = rng.x, g1 = rng.y;
     const TableDesc& td = w.tdesc[t];
-    if (V < 0) {
-        tt_sweep_generic(w, td, g0, g1, sm, sm + pl_floats);
-        return;
-    }
     if (threadIdx.x == 0) next = g0;
     __syncthreads();
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -597,11 +585,17 @@ static cudaError_t launch_sweep_fwd(tt_emb* h, int max_pl, int max_c, cudaStream
 {
     const int n = h->vcount[V + 1];
     if (n == 0) return cudaSuccess;
-    const size_t smem = tt_sweep_smem(V, max_pl, max_c);
-    cudaError_t e = cudaFuncSetAttribute(k_sweep_fwd<V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
+    cudaError_t e;
     if ((e = tt_stage_begin(h, 9 + V + 1, s)) != cudaSuccess) return e;
-    if ((e = tt_launch_pdl(k_sweep_fwd<V>, dim3(h->units_per_table, n), dim3(128), smem, s, h->v, max_pl, max_c, h->vbase[V + 1])) != cudaSuccess) return e;
+    if constexpr (V < 0) {
+        const size_t smem = GEN_C_FLOATS * sizeof(float);
+        if ((e = cudaFuncSetAttribute(k_sweep_fwd_any, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
+        if ((e = tt_launch_pdl(k_sweep_fwd_any, dim3(h->units_per_table, n), dim3(GEN_THREADS), smem, s, h->v, h->vbase[0])) != cudaSuccess) return e;
+    } else {
+        const size_t smem = tt_sweep_smem(V, max_pl, max_c);
+        if ((e = cudaFuncSetAttribute(k_sweep_fwd<V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
+        if ((e = tt_launch_pdl(k_sweep_fwd<V>, dim3(h->units_per_table, n), dim3(128), smem, s, h->v, max_pl, max_c, h->vbase[V + 1])) != cudaSuccess) return e;
+    }
     tt_note_launch();
     if ((e = tt_stage_end(h, 9 + V + 1, s)) != cudaSuccess) return e;
     return cudaGetLastError();

@@ -150,7 +150,7 @@ cudaError_t tt_launch_grouping(tt_emb* h, cudaStream_t s)
     WsView& w = h->v;
     cudaError_t e;
     const int cluster = tt_use_cluster(h);
-    w.equal_units = (cluster != 0 && h->warp_groups) || (w.ablation & 2) ? 1 : 0;
+    w.equal_units = (cluster != 0 && (h->warp_groups || w.K == 2)) || (w.ablation & 2) ? 1 : 0;   // (units of K = 2 are ranges of rows)
     if (cluster == 2) return tt_launch_group_cluster(h, true, s);
     // status word + counters are adjacent; bitmap follows its own region
     if ((e = cudaMemsetAsync(w.status, 0, (16 + 64) * sizeof(uint32_t), s)) != cudaSuccess) return e;
@@ -248,7 +248,7 @@ cudaError_t tt_launch_tlist(tt_emb* h, int k, cudaStream_t s)
     return launch_tfill(h, k, false, s);
 }
 
-// natural sweep order (K = 2; study switch "no prefix reuse")
+// natural sweep order (study switch "no prefix reuse")
 __global__ void __launch_bounds__(256) k_costs(WsView w)
 {
     tt_pdl_enter();
@@ -278,12 +278,14 @@ cudaError_t tt_launch_schedule(tt_emb* h, cudaStream_t s)
     if (tt_use_cluster(h) != 0) return cudaSuccess;   // done with the grouping
     if (tt_digit_major(w)) {
         if ((e = launch_tfill(h, w.K - 1, true, s)) != cudaSuccess) return e;
-    } else {
+    } else if (w.K >= 3) {
         if ((e = tt_launch_pdl(k_costs, dim3(h->sm_count * 8), dim3(256), 0, s, w)) != cudaSuccess) return e;
         tt_note_launch();
     }
-    CostScan<> cs{w};
-    if ((e = tt_scan<CostScan<>, TT_CSCAN_ITEMS>(cs, w.cap[w.K - 1], w.scan_tmp, s)) != cudaSuccess) return e;
+    if (w.K >= 3) {
+        CostScan<> cs{w};
+        if ((e = tt_scan<CostScan<>, TT_CSCAN_ITEMS>(cs, w.cap[w.K - 1], w.scan_tmp, s)) != cudaSuccess) return e;
+    }
     int64_t want = (int64_t)w.T * w.units_per_table;
     if (want < w.pool_shares + 1) want = w.pool_shares + 1;
     want = (want + 127) / 128;
