@@ -22,6 +22,8 @@
 #include "quad_mid.cuh"
 #include "group.cuh"
 #include "generic.cuh"
+#include "wide.cuh"
+#include "tiles.cuh"
 #include <type_traits>
 
 #define HT_SIZE 4096
@@ -1319,6 +1321,97 @@ __device__ __forceinline__ void tt_sweep_bwd_quad(const WsView& w, const TableDe
     }
 }
 
+// rank-64 four-core shape (wide.cuh).  dG_K: a warp takes one row, a lane two values of b over the 32 rows of C and dE.  dC (32 x
+// 64) = sum over the group's rows of dE . D^T: two warps per group, half the columns each, as 3xTF32 tiles whose k is two rows
+// by four columns, every pair of rows added in rounded fp32 (a group has up to n_K rows).
+__global__ void __launch_bounds__(WIDE_THREADS, 2) k_sweep_bwd_wide(WsView w, int vbase)
+{
+    tt_pdl_enter();
+    extern __shared__ __align__(16) float sm[];
+    __shared__ WideBatch batches[2];
+    float *Bs = sm, *As = Bs + 64 * WIDE_BP, *Cs = As + 8 * WIDE_GROUPS * WIDE_AP;
+    const int t = w.vlist[vbase + blockIdx.y], K = w.K, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const uint2 rng = w.unit_rng[t * w.units_per_table + blockIdx.x];
+    const TableDesc& td = w.tdesc[t];
+    const int stripe = (blockIdx.x + blockIdx.y) % TT_STRIPES;
+    float* gk = w.gpart + (size_t)stripe * w.gpart_stride + td.gpart_off;
+    const uint32_t nK = (uint32_t)td.n[K - 1];
+    WideLoop loop(w, td, rng, batches, Bs, As, Cs);
+    while (loop.next()) {
+        const WideBatch& b = loop.batch();
+        const uint32_t rows = wide_rows(b);
+        float4* stage = reinterpret_cast<float4*>(As) + wid * 64;   // this warp's rows of dE, one at a time
+        for (uint32_t r = wid; r < rows; r += WIDE_THREADS / 32) {
+            uint32_t u;
+            const int q = wide_row(b, r, u);
+            __syncwarp();
+            tt_cp_async16(stage + lane, reinterpret_cast<const float4*>(w.E + (size_t)u * w.D) + lane);
+            const uint32_t iK = w.val[K][u] - b.val[q] * nK;
+            asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
+            __syncwarp();
+            const float* c = Cs + q * (32 * WIDE_CP) + lane;
+            float4 x0 = make_float4(0.f, 0.f, 0.f, 0.f), x1 = x0;
+#pragma unroll 8
+            for (int p = 0; p < 32; ++p) {
+                const float4 d = stage[p];
+                const float y0 = c[p * WIDE_CP], y1 = c[p * WIDE_CP + 32];
+                x0.x = fmaf(y0, d.x, x0.x); x0.y = fmaf(y0, d.y, x0.y); x0.z = fmaf(y0, d.z, x0.z); x0.w = fmaf(y0, d.w, x0.w);
+                x1.x = fmaf(y1, d.x, x1.x); x1.y = fmaf(y1, d.y, x1.y); x1.z = fmaf(y1, d.z, x1.z); x1.w = fmaf(y1, d.w, x1.w);
+            }
+            float* dst = gk + (size_t)iK * 256 + lane * 4;
+            tt_red_v4(dst, x0.x, x0.y, x0.z, x0.w);
+            tt_red_v4(dst + 128, x1.x, x1.y, x1.z, x1.w);
+        }
+        const int q = wid >> 1, n0 = 32 * (wid & 1), g = lane >> 2, j = lane & 3;
+        if (b.im[q] != 0xffffffffu) {
+            float sum[2][4][4];
+#pragma unroll
+            for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+                for (int nt = 0; nt < 4; ++nt)
+#pragma unroll
+                    for (int x = 0; x < 4; ++x) sum[mt][nt][x] = 0.f;
+            const uint32_t u1 = b.u1[q], row_base = b.val[q] * nK;
+#pragma unroll 1
+            for (uint32_t u = b.u0[q]; u < u1; u += 2) {
+                const bool two = u + 1 < u1;
+                const float* dE = w.E + (size_t)u * w.D + 4 * g + j;
+                const float* D0 = td.core[K - 1] + (size_t)(w.val[K][u] - row_base) * 256 + 4 * (n0 + g) + j;
+                const float* D1 = td.core[K - 1] + (size_t)(w.val[K][two ? u + 1 : u] - row_base) * 256 + 4 * (n0 + g) + j;
+                float e[2][4], d[4][2];
+#pragma unroll
+                for (int mt = 0; mt < 2; ++mt) {
+                    e[mt][0] = __ldg(dE + 64 * mt);
+                    e[mt][1] = __ldg(dE + 64 * mt + 32);
+                    e[mt][2] = two ? __ldg(dE + w.D + 64 * mt) : 0.f;
+                    e[mt][3] = two ? __ldg(dE + w.D + 64 * mt + 32) : 0.f;
+                }
+#pragma unroll
+                for (int nt = 0; nt < 4; ++nt) { d[nt][0] = __ldg(D0 + 32 * nt); d[nt][1] = __ldg(D1 + 32 * nt); }
+                Tf32Pair a[2][4];
+#pragma unroll
+                for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+                    for (int x = 0; x < 4; ++x) a[mt][x] = tt_split_tf32(e[mt][x]);
+#pragma unroll
+                for (int nt = 0; nt < 4; ++nt) {
+                    Tf32Pair f[2] = {tt_split_tf32(d[nt][0]), tt_split_tf32(d[nt][1])};
+#pragma unroll
+                    for (int mt = 0; mt < 2; ++mt) tt_mma_3xtf32_rounded(sum[mt][nt], a[mt], f);
+                }
+            }
+            float* dst = w.dP[K - 1] + (size_t)b.g[q] * w.stride[K - 1] + n0 + 2 * j;
+#pragma unroll
+            for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+                for (int nt = 0; nt < 4; ++nt) {
+                    *reinterpret_cast<float2*>(dst + (16 * mt + g) * 64 + 8 * nt) = make_float2(sum[mt][nt][0], sum[mt][nt][1]);
+                    *reinterpret_cast<float2*>(dst + (16 * mt + g + 8) * 64 + 8 * nt) = make_float2(sum[mt][nt][2], sum[mt][nt][3]);
+                }
+        }
+    }
+}
+
 // One CTA (4 warps) per work unit (table, q); last-core gradients go to one of TT_STRIPES L2-resident partial
 // copies with vector reductions, added up in fixed stripe order by k_reduce_gpart.
 template <int V>
@@ -1342,7 +1435,6 @@ __global__ void __launch_bounds__(128, (V == 5 || V == 6 || V == 8 || V == 9 || 
     if (V == 1) tt_sweep_bwd_quad<16, 16, 4, 4>(w, td, g1, gk, sm + (size_t)wid * (4 * 16 * 20), &next, lane);
     if (V == 2) tt_sweep_bwd_fast<16, 8, 4, 4, 1, true>(w, td, g1, gk, As, Cs, &next, lane);
     if (V == 3) tt_sweep_bwd_fast<32, 32, 4, 4, 2, true>(w, td, g1, gk, As, Cs, &next, lane);
-    if (V == 4) tt_sweep_bwd_fast<32, 64, 2, 8, 2, false>(w, td, g1, gk, As, Cs, &next, lane);
     if (V == 5) tt_sweep_bwd_quad<8, 32, 2, 4>(w, td, g1, gk, sm + (size_t)wid * (8 * 8 * 36), &next, lane);
     if (V == 6) tt_sweep_bwd_quad<8, 16, 2, 4>(w, td, g1, gk, sm + (size_t)wid * (8 * 8 * 20), &next, lane);
     if (V == 7) tt_sweep_bwd_fast<8, 8, 2, 2, 1, false>(w, td, g1, gk, As, Cs, &next, lane);   // 8 x 8: the FP32 pipe wins (0.39 against 0.41 ms)
@@ -1395,6 +1487,9 @@ static cudaError_t launch_sweep_bwd(tt_emb* h, int max_pl, int max_c, cudaStream
         smem = 2 * GEN_C_FLOATS * sizeof(float);
         if ((e = cudaFuncSetAttribute(k_sweep_bwd_any, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
         if ((e = tt_launch_pdl(k_sweep_bwd_any, dim3(h->units_per_table, n), dim3(GEN_THREADS), smem, s, h->v, h->vbase[0])) != cudaSuccess) return e;
+    } else if constexpr (V == 4) {
+        if ((e = cudaFuncSetAttribute(k_sweep_bwd_wide, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)WIDE_SMEM)) != cudaSuccess) return e;
+        if ((e = tt_launch_pdl(k_sweep_bwd_wide, dim3(h->units_per_table, n), dim3(WIDE_THREADS), WIDE_SMEM, s, h->v, h->vbase[V + 1])) != cudaSuccess) return e;
     } else {
         if ((e = cudaFuncSetAttribute(k_sweep_bwd<V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
         if ((e = tt_launch_pdl(k_sweep_bwd<V>, dim3(h->units_per_table, n), dim3(128), smem, s, h->v, max_pl, max_c, h->vbase[V + 1])) != cudaSuccess) return e;
@@ -1706,74 +1801,11 @@ __global__ void __launch_bounds__(128, 5) k_mid_mma(WsView w, int k, int variant
 //             pass, staged with cp.async in two buffers, row addresses looked up two passes ahead
 //   z >= dgz  Y: tiles of 64 stacked rows by 64 values of a, dealt out to the slice's `yctas` CTAs; k runs over the
 //             columns, 32 per pass
-// A warp owns a 32 x 32 quarter of the tile (8 fragment loads per k step for 8 tile products of 3xTF32); row tiles and
-// column blocks outside the shape are skipped.  Pitches of 72 (fragments run down the rows) and 36 floats (along the
-// rows) keep the fragment loads free of bank conflicts.  Every k step is added in rounded fp32
-// (tt_mma_3xtf32_rounded).  No fused update of the slice: the Y CTAs of other tiles still read it.
+// A warp owns a 32 x 32 quarter of the tile (tiles.cuh; 16 fragment loads per k step for 8 tile products of 3xTF32); row
+// tiles and column blocks outside the shape are skipped.  No fused update of the slice: the Y CTAs of other tiles still read it.
 // Bound by the operand path (16 fragment loads for 24 tensor instructions) and, for short node lists, by a CTA's look-ups.
 // Middle stage, 2x4x4x4 with rank 64 (65 536 lookups): 5.05 ms with one FP32 thread per output element over the whole
 // node list, 0.16 ms as tiles; 3x3x5 with ranks 6 and 4 (4 tables, 1 M lookups): 0.41 and 0.06 ms.
-#define MT_EDGE 64
-#define MT_KROWS 32
-#define MT_PA (MT_EDGE + 8)
-#define MT_PC (MT_KROWS + 4)
-
-// 4-byte asynchronous copy global -> shared
-__device__ __forceinline__ void tt_cp_async4(void* smem_dst, const void* gsrc)
-{
-    const unsigned d = (unsigned)__cvta_generic_to_shared(smem_dst);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d), "l"(gsrc) : "memory");
-}
-
-// dst[row][0 .. 4 * W4) = src[row][off .. off + avail), the rest of the row (and rows without a source) zero; 128 threads
-template <int ROWS, int W4>
-__device__ __forceinline__ void tt_stage_rows(float* dst, int pitch, const float* const* src, int off, int avail, bool vec)
-{
-    if (vec) {
-        for (int i = threadIdx.x; i < ROWS * W4; i += 128) {
-            const int row = i / W4, c4 = i % W4;
-            const float* p = src[row];
-            float* d = dst + row * pitch + 4 * c4;
-            if (p && 4 * c4 < avail) tt_cp_async16(d, p + off + 4 * c4);
-            else *reinterpret_cast<float4*>(d) = make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-    } else {
-        for (int i = threadIdx.x; i < ROWS * W4 * 4; i += 128) {
-            const int row = i / (W4 * 4), c = i % (W4 * 4);
-            const float* p = src[row];
-            float* d = dst + row * pitch + c;
-            if (p && c < avail) tt_cp_async4(d, p + off + c);
-            else *d = 0.f;
-        }
-    }
-}
-
-// sum += A . B over 8 k values: mtl row tiles of 16, ntl column blocks of 8.  The A fragment of row tile mt is
-// {a0, a1, a2, a3}[16 mt * astep], the B fragment of block nt {b0, b1}[8 nt * bstep]
-__device__ __forceinline__ void tt_quarter_step(float (&sum)[2][4][4], const float* a0, const float* a1, const float* a2, const float* a3,
-                                                int astep, const float* b0, const float* b1, int bstep, int mtl, int ntl)
-{
-    Tf32Pair a[2][4];
-#pragma unroll
-    for (int mt = 0; mt < 2; ++mt)
-        if (mt < mtl) {
-            a[mt][0] = tt_split_tf32(a0[16 * mt * astep]);
-            a[mt][1] = tt_split_tf32(a1[16 * mt * astep]);
-            a[mt][2] = tt_split_tf32(a2[16 * mt * astep]);
-            a[mt][3] = tt_split_tf32(a3[16 * mt * astep]);
-        }
-#pragma unroll
-    for (int nt = 0; nt < 4; ++nt)
-        if (nt < ntl) {
-            Tf32Pair b[2];
-            b[0] = tt_split_tf32(b0[8 * nt * bstep]);
-            b[1] = tt_split_tf32(b1[8 * nt * bstep]);
-#pragma unroll
-            for (int mt = 0; mt < 2; ++mt)
-                if (mt < mtl) tt_mma_3xtf32_rounded(sum[mt][nt], a[mt], b);
-        }
-}
-
 __global__ void __launch_bounds__(128, 4) k_mid_tile(WsView w, int k, int lbase, int dgz, int yctas)
 {
     tt_pdl_enter();

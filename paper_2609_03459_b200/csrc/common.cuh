@@ -22,8 +22,8 @@
 #define TT_FUSED_INGEST (1 << 22)
 // fewest groups of a work unit; 4x as many for D = 128, rank 32, whose warps each reuse a 32 KB slice over their groups.
 // Sweeps with at least 4 / 8 / 16 / 32 / 64 groups per unit, forward + backward, us: 8 tables x 8 k groups (rank 16) 385 / 352 /
-// 325 / 319 / 343; 4 tables x 9 k (D = 32, rank 8) 119 / 117 / 107 / 122 / 188; four cores, 4.7 k groups 304 / 310 / 319 / 422 /
-// 576; D = 128, rank 32, 27 k groups (forward) 236 / 164 / 145 / 137 / 129
+// 325 / 319 / 343; 4 tables x 9 k (D = 32, rank 8) 119 / 117 / 107 / 122 / 188; four cores, 4.7 k groups 178 / 173 / 170 / 235;
+// D = 128, rank 32, 27 k groups (forward) 236 / 164 / 145 / 137 / 129
 #define TT_UNIT_GROUPS 16
 // ... and of the any-shape sweeps, whose CTAs take a batch of groups at a time (3x3x5, 29 k groups, forward + backward sweep
 // with at least 1 / 4 / 8 / 16 groups: 332 / 285 / 252 / 253 us; 8x8 with K = 2, 420 k lookups, whole call 1.16 ms with 8, 1.68 with 16)

@@ -14,25 +14,124 @@
 #include "mma.cuh"
 #include "quad_mid.cuh"
 #include "generic.cuh"
+#include "wide.cuh"
+#include "tiles.cuh"
 
 // ---------------------------------------------------------------------------------------------- products
 
-// P_k for every level-k node, 2 <= k <= K-2 (only K = 4 has such a level); one CTA per node, grid-stride
-__global__ void __launch_bounds__(128) k_mid_level(WsView w, int k)
+// P_2 for every level-2 node of a four-core table: P_2 = G_1[i_1] . G_2[i_2].  A CTA keeps to one i_2 and 64 columns of its
+// slice and multiplies the slices of all present i_1, 64 stacked rows at a time (tiles.cuh); a prefix's node is a rank
+// look-up in the level's bitmap, so the nodes of one i_2 need no list.  (One CTA per node read its slice for itself: 3403
+// nodes of 2 x 64 by 64 x 256 took 70 us, bound by 0.2 GB of slices from L2; 16 us this way.)
+__global__ void __launch_bounds__(128, 4) k_level2(WsView w)
+{
+    tt_pdl_enter();
+    __shared__ __align__(16) float sm[2 * (MT_EDGE * MT_PC + MT_KROWS * MT_PA)];
+    __shared__ const float* s_row[MT_EDGE];     // rows of G_1
+    __shared__ float* s_out[MT_EDGE];
+    __shared__ const float* s_slice[128];       // rows of the slice of G_2
+    __shared__ int s_any;
+    const TableDesc& td = w.tdesc[blockIdx.y];
+    const int M = td.d[0], ra = td.r[1], cols = td.d[1] * td.r[2], c0 = (int)blockIdx.z * MT_EDGE;
+    if ((int)blockIdx.x >= td.n[1] || c0 >= cols) return;
+    const bool vec = (ra & 3) == 0 && (cols & 3) == 0;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, g = lane >> 2, t = lane & 3, wr = wid >> 1, wc = wid & 1;
+    s_slice[tid] = tid < ra ? td.core[1] + (size_t)blockIdx.x * td.slice_floats[1] + (size_t)tid * cols + c0 : nullptr;   // r <= 128
+    const int rows = td.n[0] * M, kpasses = (ra + MT_KROWS - 1) / MT_KROWS;
+    const int ntl = min(4, max(0, (cols - c0 - 32 * wc + 7) / 8));
+    constexpr int STAGE = MT_EDGE * MT_PC + MT_KROWS * MT_PA;
+    for (int row0 = 0; row0 < rows; row0 += MT_EDGE) {
+        if (tid == 0) s_any = 0;
+        __syncthreads();
+        if (tid < MT_EDGE) {
+            const int row = row0 + tid;
+            const float* src = nullptr;
+            float* out = nullptr;
+            if (row < rows) {
+                const uint32_t p = (uint32_t)(row / M), m = (uint32_t)row - p * (uint32_t)M;
+                const uint32_t x = p * (uint32_t)td.n[1] + blockIdx.x;
+                const uint2 e = w.bml[2][td.lword_base[2] + (x >> 5)];
+                const uint32_t v = e.y + __popc(e.x & ((1u << (x & 31)) - 1u));
+                if (((e.x >> (x & 31)) & 1u) && v < w.counters[CTR_LEVEL0 + 2]) {
+                    src = td.core[0] + (size_t)row * ra;
+                    out = w.pbuf[2] + (size_t)v * w.stride[2] + (size_t)m * cols + c0;
+                    s_any = 1;
+                }
+            }
+            s_row[tid] = src;
+            s_out[tid] = out;
+        }
+        __syncthreads();
+        if (!s_any) continue;
+        float sum[2][4][4];
+#pragma unroll
+        for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+            for (int nt = 0; nt < 4; ++nt)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) sum[mt][nt][i] = 0.f;
+        const int mtl = min(2, max(0, (min(rows - row0, MT_EDGE) - 32 * wr + 15) / 16));
+        auto issue = [&](int kp) {
+            float* st = sm + (kp & 1) * STAGE;
+            tt_stage_rows<MT_EDGE, MT_KROWS / 4>(st, MT_PC, s_row, kp * MT_KROWS, ra - kp * MT_KROWS, vec);
+            tt_stage_rows<MT_KROWS, MT_EDGE / 4>(st + MT_EDGE * MT_PC, MT_PA, s_slice + kp * MT_KROWS, 0, cols - c0, vec);
+            asm volatile("cp.async.commit_group;" ::: "memory");
+        };
+        issue(0);
+        for (int kp = 0; kp < kpasses; ++kp) {
+            if (kp + 1 < kpasses) {
+                issue(kp + 1);
+                asm volatile("cp.async.wait_group 1;" ::: "memory");
+            } else {
+                asm volatile("cp.async.wait_group 0;" ::: "memory");
+            }
+            __syncthreads();
+            if (mtl > 0 && ntl > 0) {
+                const float* A = sm + (kp & 1) * STAGE + (32 * wr + g) * MT_PC + t;
+                const float* D = sm + (kp & 1) * STAGE + MT_EDGE * MT_PC + t * MT_PA + 32 * wc + g;
+#pragma unroll
+                for (int p = 0; p < MT_KROWS / 8; ++p) {
+                    if (kp * MT_KROWS + 8 * p >= ra) break;
+                    const float* Aa = A + 8 * p;
+                    const float* Da = D + 8 * p * MT_PA;
+                    tt_quarter_step(sum, Aa, Aa + 8 * MT_PC, Aa + 4, Aa + 8 * MT_PC + 4, MT_PC, Da, Da + 4 * MT_PA, 1, mtl, ntl);
+                }
+            }
+            __syncthreads();
+        }
+#pragma unroll
+        for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                float* out = s_out[32 * wr + 16 * mt + 8 * h + g];
+#pragma unroll
+                for (int nt = 0; nt < 4; ++nt) {
+                    const int c = 32 * wc + 8 * nt + 2 * t;
+                    if (!out || c0 + c >= cols) continue;
+                    if (vec) *reinterpret_cast<float2*>(out + c) = make_float2(sum[mt][nt][2 * h], sum[mt][nt][2 * h + 1]);
+                    else {
+                        out[c] = sum[mt][nt][2 * h];
+                        if (c0 + c + 1 < cols) out[c + 1] = sum[mt][nt][2 * h + 1];
+                    }
+                }
+            }
+    }
+}
+
+// study switches: nodes that no bitmap finds (every lookup or row its own); one CTA per node
+__global__ void __launch_bounds__(128) k_level2_nodes(WsView w)
 {
     tt_pdl_enter();
     extern __shared__ float sm[];
-    const uint32_t count = w.counters[CTR_LEVEL0 + k];
+    const uint32_t count = w.counters[CTR_LEVEL0 + 2];
     for (uint32_t v = blockIdx.x; v < count; v += gridDim.x) {
-        const int t = tt_find_table(w.tb[k], w.T, v);
-        const TableDesc& td = w.tdesc[t];
-        const int kc = k - 1;
-        const int M = td.P[kc], ra = td.r[kc], cols = td.d[kc] * td.r[kc + 1];
-        const float* src = tt_left_operand(w, td, k, v);
+        const TableDesc& td = w.tdesc[tt_find_table(w.tb[2], w.T, v)];
+        const int M = td.P[1], ra = td.r[1], cols = td.d[1] * td.r[2];
+        const float* src = tt_left_operand(w, td, 2, v);
         for (int i = threadIdx.x; i < M * ra; i += blockDim.x) sm[i] = src[i];
         __syncthreads();
-        const uint32_t ik = w.val[k][v] % (uint32_t)td.n[kc];
-        tt_mid_product(sm, td.core[kc] + (size_t)ik * td.slice_floats[kc], w.pbuf[k] + (size_t)v * w.stride[k], M, ra, cols);
+        const uint32_t ik = w.val[2][v] % (uint32_t)td.n[1];
+        tt_mid_product(sm, td.core[1] + (size_t)ik * td.slice_floats[1], w.pbuf[2] + (size_t)v * w.stride[2], M, ra, cols);
         __syncthreads();
     }
 }
@@ -108,7 +207,7 @@ __device__ __forceinline__ void tt_warp_mid(const float* As, const float* __rest
 // E rows u0..u1 of the group whose C (PM x RB, row-major) is in Cs.  d_K = 4.
 template <int PM, int RB, int TP>
 __device__ __forceinline__ void tt_warp_rows(const float* Cs, const WsView& w, const TableDesc& td, uint32_t u0, uint32_t u1,
-                                             uint32_t row_base, int lane, int part = 0, int nparts = 1)   // this warp takes every nparts-th batch
+                                             uint32_t row_base, int lane)
 {
     constexpr int LR = PM / TP;   // lanes per row
     constexpr int RW = 32 / LR;   // rows per batch
@@ -124,7 +223,7 @@ __device__ __forceinline__ void tt_warp_rows(const float* Cs, const WsView& w, c
     const int K = w.K;
     const float* __restrict__ GK = td.core[K - 1];
     const uint32_t* __restrict__ rows = w.val[K];
-    for (uint32_t ub = u0 + (uint32_t)(part * RW); ub < u1; ub += (uint32_t)(RW * nparts)) {
+    for (uint32_t ub = u0; ub < u1; ub += RW) {
         const uint32_t u = ub + slot;
         const bool act = u < u1;
         const uint32_t iK = act ? rows[u] - row_base : 0u;
@@ -338,9 +437,8 @@ __device__ __forceinline__ void tt_sweep_fast(const WsView& w, const TableDesc& 
 
 // Tensor-core variants: a warp takes NG = 16 / MROWS consecutive groups of the digit-major order at a time; their
 // intermediate products are formed together (quad_mid.cuh), then each group's rows are produced from its C in shared
-// memory: on the tensor cores too (TP = 0), or on the FP32 pipe with TP rows of C per lane where C is too large for
-// register-resident fragments.
-template <int PM, int RB, int MROWS, int KTMAX, int TP>
+// memory, on the tensor cores too.
+template <int PM, int RB, int MROWS, int KTMAX>
 __device__ __forceinline__ void tt_sweep_quad(const WsView& w, const TableDesc& td, uint32_t g1, float* Cs4, uint32_t* next, int lane)
 {
     constexpr int COLS = PM / MROWS * RB;   // d_{K-1} * r_{K-1}
@@ -365,142 +463,56 @@ __device__ __forceinline__ void tt_sweep_quad(const WsView& w, const TableDesc& 
             u0q = w.cstart[K - 1][gq];
             u1q = w.cstart[K - 1][gq + 1];
         }
-        tt_quad_mid<COLS, MROWS, KTMAX, (TP == 0 ? RB : 0)>(td.core[km], td.slice_floats[km], ra, cnt, imq, srcq, Cs4, lane);
+        tt_quad_mid<COLS, MROWS, KTMAX, RB>(td.core[km], td.slice_floats[km], ra, cnt, imq, srcq, Cs4, lane);
         __syncwarp();
         for (int q = 0; q < cnt; ++q) {
             const uint32_t val = __shfl_sync(0xffffffffu, valq, q);
             const uint32_t u0 = __shfl_sync(0xffffffffu, u0q, q), u1 = __shfl_sync(0xffffffffu, u1q, q);
-            if constexpr (TP == 0 && PM < 16) tt_warp_rows_mma_t<PM, RB, RB + 4>(Cs4 + (size_t)q * (PM * (RB + 4)), w, td, u0, u1, val * nK, lane);
-            else if constexpr (TP == 0) tt_warp_rows_mma<PM, RB, RB + 4>(Cs4 + (size_t)q * (PM * (RB + 4)), w, td, u0, u1, val * nK, lane);
-            else tt_warp_rows<PM, RB, TP>(Cs4 + (size_t)q * (PM * RB), w, td, u0, u1, val * nK, lane);
+            if constexpr (PM < 16) tt_warp_rows_mma_t<PM, RB, RB + 4>(Cs4 + (size_t)q * (PM * (RB + 4)), w, td, u0, u1, val * nK, lane);
+            else tt_warp_rows_mma<PM, RB, RB + 4>(Cs4 + (size_t)q * (PM * (RB + 4)), w, td, u0, u1, val * nK, lane);
         }
         __syncwarp();
     }
 }
 
-// Stacked product of two 8-row groups against this warp's 64 columns of the slice B (ra <= 64 rows, COLS columns): the
-// 64 x 64 block is fetched into shared memory in one go (32 cp.async per lane, one L2 round trip instead of one per 16
-// rows and 32 columns), then the 3xTF32 tiles run from shared memory.  Row stride 68 floats: fragment loads 2-way at worst.
-template <int COLS>
-__device__ __forceinline__ void tt_pair_mid_staged(const float* __restrict__ B, int ra, const float* __restrict__ srcA,
-                                                   const float* __restrict__ srcB, bool selA, bool selB, float* Cs2, float* stg,
-                                                   int lane, int wid, bool stage)
+// rank-64 four-core shape (wide.cuh): a warp makes one row, a lane one of its 32 rows of C by the four columns of the slice
+__global__ void __launch_bounds__(WIDE_THREADS, 2) k_sweep_fwd_wide(WsView w, int vbase)
 {
-    constexpr int RS = 68;
-    const int g = lane >> 2, t = lane & 3;
-    const int c0 = 64 * wid;   // first column of this warp's block
-    if (stage)                 // (the block of the previous pair is still there when the pair shares its slice)
-        for (int i = lane; i < 64 * 16; i += 32) {
-            const int k = i >> 4, f = i & 15;
-            if (k < ra) tt_cp_async16(stg + k * RS + 4 * f, B + (size_t)k * COLS + c0 + 4 * f);
-        }
-    asm volatile("cp.async.commit_group;" ::: "memory");
-    float araw[8][4];   // rows g (first group) and g + 8 (second group) of the stacked operand, unsplit
-#pragma unroll
-    for (int kt = 0; kt < 8; ++kt) {
-        const int k0 = 8 * kt + t, k1 = k0 + 4;
-        araw[kt][0] = (selA && k0 < ra) ? __ldg(srcA + g * ra + k0) : 0.f;
-        araw[kt][1] = (selB && k0 < ra) ? __ldg(srcB + g * ra + k0) : 0.f;
-        araw[kt][2] = (selA && k1 < ra) ? __ldg(srcA + g * ra + k1) : 0.f;
-        araw[kt][3] = (selB && k1 < ra) ? __ldg(srcB + g * ra + k1) : 0.f;
-    }
-    asm volatile("cp.async.wait_group 0;" ::: "memory");
-    __syncwarp();
-    const int kta = (ra + 7) >> 3;
-    float* dstA = Cs2 + g * COLS + c0 + 8 * t;                  // group 0, row g of P
-    float* dstB = Cs2 + (size_t)8 * COLS + g * COLS + c0 + 8 * t;   // group 1
-#pragma unroll 1
-    for (int nb = 0; nb < 2; ++nb) {
-        float acc[4][4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) { acc[j][0] = 0.f; acc[j][1] = 0.f; acc[j][2] = 0.f; acc[j][3] = 0.f; }
-#pragma unroll
-        for (int kt = 0; kt < 8; ++kt) {
-            if (kt < kta) {
-                const int k0 = 8 * kt + t, k1 = k0 + 4;
-                const float4 f0 = k0 < ra ? *reinterpret_cast<const float4*>(stg + k0 * RS + 32 * nb + 4 * g) : make_float4(0.f, 0.f, 0.f, 0.f);
-                const float4 f1 = k1 < ra ? *reinterpret_cast<const float4*>(stg + k1 * RS + 32 * nb + 4 * g) : make_float4(0.f, 0.f, 0.f, 0.f);
-                Tf32Pair a[4];
-#pragma unroll
-                for (int x = 0; x < 4; ++x) a[x] = tt_split_tf32(araw[kt][x]);
-                const float v0[4] = {f0.x, f0.y, f0.z, f0.w};
-                const float v1[4] = {f1.x, f1.y, f1.z, f1.w};
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    Tf32Pair b[2];
-                    b[0] = tt_split_tf32(v0[j]);
-                    b[1] = tt_split_tf32(v1[j]);
-                    tt_mma_3xtf32(acc[j], a, b);
-                }
-            }
-        }
-        if (selA) {
-            *reinterpret_cast<float4*>(dstA + 32 * nb) = make_float4(acc[0][0], acc[1][0], acc[2][0], acc[3][0]);
-            *reinterpret_cast<float4*>(dstA + 32 * nb + 4) = make_float4(acc[0][1], acc[1][1], acc[2][1], acc[3][1]);
-        }
-        if (selB) {
-            *reinterpret_cast<float4*>(dstB + 32 * nb) = make_float4(acc[0][2], acc[1][2], acc[2][2], acc[3][2]);
-            *reinterpret_cast<float4*>(dstB + 32 * nb + 4) = make_float4(acc[0][3], acc[1][3], acc[2][3], acc[3][3]);
-        }
-    }
-    __syncwarp();   // the block is overwritten by the next call
-}
-
-// Rank-64 four-core shape: the stage K-1 product of one group is 8 x 64 by 64 x 256 and there are few groups (tens of
-// thousands), so the whole CTA works on one pair of groups at a time: the four warps each compute two of the eight
-// column blocks of the stacked 16-row tensor-core product into one shared C buffer (16 KB per CTA instead of per
-// warp), then two warps per group produce its rows.  Four times the parallelism per pair of the warp-per-pair form.
-template <int PM, int RB>
-__device__ __forceinline__ void tt_sweep_pair_cta(const WsView& w, const TableDesc& td, uint32_t g0, uint32_t g1, float* Cs2,
-                                                  int lane, int wid)
-{
-    constexpr int MROWS = 8, COLS = PM / MROWS * RB;
-    static_assert(COLS == 256, "four warps x 64 columns");
-    __shared__ uint32_t m_val[2], m_im[2], m_u0[2], m_u1[2];
-    __shared__ const float* m_src[2];
-    const int K = w.K, km = K - 2;
-    const int ra = td.r[km];
+    tt_pdl_enter();
+    extern __shared__ __align__(16) float sm[];
+    __shared__ WideBatch batches[2];
+    float *Bs = sm, *As = Bs + 64 * WIDE_BP, *Cs = As + 8 * WIDE_GROUPS * WIDE_AP;
+    const int t = w.vlist[vbase + blockIdx.y], K = w.K, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const uint2 rng = w.unit_rng[t * w.units_per_table + blockIdx.x];
+    const TableDesc& td = w.tdesc[t];
     const uint32_t nK = (uint32_t)td.n[K - 1];
-    uint32_t staged = 0xffffffffu;   // slice whose blocks the warps hold in shared memory (the same for all four warps)
-    for (uint32_t base = g0; base < g1; base += 2) {
-        const int cnt = (int)min(2u, g1 - base);
-        if (threadIdx.x < 2) {
-            const int q = threadIdx.x;
-            if (q < cnt) {
-                const uint32_t pos = base + q;
-                const uint32_t gq = (w.ablation & 1) ? pos : w.tnode[K - 1][pos];
-                const uint32_t v = w.val[K - 1][gq];
-                m_val[q] = v;
-                m_im[q] = v % (uint32_t)td.n[km];
-                m_src[q] = tt_left_operand(w, td, K - 1, gq);
-                m_u0[q] = w.cstart[K - 1][gq];
-                m_u1[q] = w.cstart[K - 1][gq + 1];
-            } else {
-                m_val[q] = 0; m_im[q] = 0xffffffffu; m_src[q] = nullptr; m_u0[q] = 0; m_u1[q] = 0;
+    WideLoop loop(w, td, rng, batches, Bs, As, Cs);
+    while (loop.next()) {
+        const WideBatch& b = loop.batch();
+        const uint32_t rows = wide_rows(b);
+        float4* stage = reinterpret_cast<float4*>(As) + wid * 64;   // this warp's slices of the last core, one at a time
+        for (uint32_t r = wid; r < rows; r += WIDE_THREADS / 32) {
+            uint32_t u;
+            const int q = wide_row(b, r, u);
+            const float4* D = reinterpret_cast<const float4*>(td.core[K - 1]) + (size_t)(w.val[K][u] - b.val[q] * nK) * 64;
+            __syncwarp();
+            tt_cp_async16(stage + lane, D + lane);
+            tt_cp_async16(stage + lane + 32, D + lane + 32);
+            asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
+            __syncwarp();
+            const float4* c4 = reinterpret_cast<const float4*>(Cs + q * (32 * WIDE_CP) + lane * WIDE_CP);
+            float4 e = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 4
+            for (int i = 0; i < 16; ++i) {
+                const float4 c = c4[i];
+                const float4 d0 = stage[4 * i], d1 = stage[4 * i + 1], d2 = stage[4 * i + 2], d3 = stage[4 * i + 3];
+                e.x = fmaf(c.x, d0.x, e.x); e.y = fmaf(c.x, d0.y, e.y); e.z = fmaf(c.x, d0.z, e.z); e.w = fmaf(c.x, d0.w, e.w);
+                e.x = fmaf(c.y, d1.x, e.x); e.y = fmaf(c.y, d1.y, e.y); e.z = fmaf(c.y, d1.z, e.z); e.w = fmaf(c.y, d1.w, e.w);
+                e.x = fmaf(c.z, d2.x, e.x); e.y = fmaf(c.z, d2.y, e.y); e.z = fmaf(c.z, d2.z, e.z); e.w = fmaf(c.z, d2.w, e.w);
+                e.x = fmaf(c.w, d3.x, e.x); e.y = fmaf(c.w, d3.y, e.y); e.z = fmaf(c.w, d3.z, e.z); e.w = fmaf(c.w, d3.w, e.w);
             }
+            reinterpret_cast<float4*>(w.E + (size_t)u * w.D)[lane] = e;
         }
-        __syncthreads();
-        const float* B0 = td.core[km] + (size_t)m_im[0] * td.slice_floats[km];
-        float* stg = Cs2 + 2 * PM * RB + (size_t)wid * (64 * 68);   // this warp's staged 64 x 64 block of the slice
-        // neighbouring pairs of the digit-major order share the slice: its 64 KB are fetched again only when it changes
-        if (cnt == 2 && m_im[1] == m_im[0]) {
-            tt_pair_mid_staged<COLS>(B0, ra, m_src[0], m_src[1], true, true, Cs2, stg, lane, wid, staged != m_im[0]);
-            staged = m_im[0];
-        } else {
-            tt_pair_mid_staged<COLS>(B0, ra, m_src[0], m_src[1], true, false, Cs2, stg, lane, wid, staged != m_im[0]);
-            staged = m_im[0];
-            if (cnt == 2) {
-                tt_pair_mid_staged<COLS>(td.core[km] + (size_t)m_im[1] * td.slice_floats[km], ra, m_src[0], m_src[1], false, true, Cs2,
-                                         stg, lane, wid, true);
-                staged = m_im[1];
-            }
-        }
-        __syncthreads();
-        {
-            const int q = wid >> 1;   // warps 0,1: first group; warps 2,3: second group
-            if (q < cnt) tt_warp_rows<PM, RB, 2>(Cs2 + (size_t)q * (PM * RB), w, td, m_u0[q], m_u1[q], m_val[q] * nK, lane, wid & 1, 2);
-        }
-        __syncthreads();
     }
 }
 
@@ -537,7 +549,7 @@ __global__ void __launch_bounds__(GEN_THREADS) k_sweep_fwd_any(WsView w, int vba
 // one instantiation per shape variant V so that each gets its own register budget.  blockIdx.y walks the
 // tables of variant V (w.vlist), blockIdx.x the table's equal-cost slices.
 template <int V>
-__global__ void __launch_bounds__(128, (V != 3 && V != 4) ? 6 : 1) k_sweep_fwd(WsView w, int pl_floats, int c_floats, int vbase)
+__global__ void __launch_bounds__(128, V != 3 ? 6 : 1) k_sweep_fwd(WsView w, int pl_floats, int c_floats, int vbase)
 {
     tt_pdl_enter();
     extern __shared__ __align__(16) float sm[];
@@ -549,18 +561,17 @@ __global__ void __launch_bounds__(128, (V != 3 && V != 4) ? 6 : 1) k_sweep_fwd(W
     if (threadIdx.x == 0) next = g0;
     __syncthreads();
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    if (V == 0) tt_sweep_quad<16, 32, 4, 4, 0>(w, td, g1, sm + (size_t)wid * (4 * 16 * 36), &next, lane);
-    if (V == 1) tt_sweep_quad<16, 16, 4, 4, 0>(w, td, g1, sm + (size_t)wid * (4 * 16 * 20), &next, lane);
-    if (V == 3) tt_sweep_quad<32, 32, 4, 4, 0>(w, td, g1, sm + (size_t)wid * (4 * 32 * 36), &next, lane);
-    if (V == 4) tt_sweep_pair_cta<32, 64>(w, td, g0, g1, sm, lane, wid);
+    if (V == 0) tt_sweep_quad<16, 32, 4, 4>(w, td, g1, sm + (size_t)wid * (4 * 16 * 36), &next, lane);
+    if (V == 1) tt_sweep_quad<16, 16, 4, 4>(w, td, g1, sm + (size_t)wid * (4 * 16 * 20), &next, lane);
+    if (V == 3) tt_sweep_quad<32, 32, 4, 4>(w, td, g1, sm + (size_t)wid * (4 * 32 * 36), &next, lane);
     float* As = sm + (size_t)wid * (pl_floats + c_floats);
     float* Cs = As + pl_floats;
-    if (V == 2) tt_sweep_quad<16, 8, 4, 4, 0>(w, td, g1, sm + (size_t)wid * (4 * 16 * 12), &next, lane);
-    if (V == 5) tt_sweep_quad<8, 32, 2, 4, 0>(w, td, g1, sm + (size_t)wid * (8 * 8 * 36), &next, lane);
-    if (V == 6) tt_sweep_quad<8, 16, 2, 4, 0>(w, td, g1, sm + (size_t)wid * (8 * 8 * 20), &next, lane);
-    if (V == 7) tt_sweep_quad<8, 8, 2, 4, 0>(w, td, g1, sm + (size_t)wid * (8 * 8 * 12), &next, lane);
-    if (V == 8) tt_sweep_quad<4, 32, 2, 4, 0>(w, td, g1, sm + (size_t)wid * (8 * 4 * 36), &next, lane);
-    if (V == 9) tt_sweep_quad<4, 16, 2, 4, 0>(w, td, g1, sm + (size_t)wid * (8 * 4 * 20), &next, lane);
+    if (V == 2) tt_sweep_quad<16, 8, 4, 4>(w, td, g1, sm + (size_t)wid * (4 * 16 * 12), &next, lane);
+    if (V == 5) tt_sweep_quad<8, 32, 2, 4>(w, td, g1, sm + (size_t)wid * (8 * 8 * 36), &next, lane);
+    if (V == 6) tt_sweep_quad<8, 16, 2, 4>(w, td, g1, sm + (size_t)wid * (8 * 8 * 20), &next, lane);
+    if (V == 7) tt_sweep_quad<8, 8, 2, 4>(w, td, g1, sm + (size_t)wid * (8 * 8 * 12), &next, lane);
+    if (V == 8) tt_sweep_quad<4, 32, 2, 4>(w, td, g1, sm + (size_t)wid * (8 * 4 * 36), &next, lane);
+    if (V == 9) tt_sweep_quad<4, 16, 2, 4>(w, td, g1, sm + (size_t)wid * (8 * 4 * 20), &next, lane);
     if (V == 10) tt_sweep_fast<4, 8, 2, 2, 1, false>(w, td, g1, As, Cs, &next, lane);
 }
 
@@ -576,7 +587,6 @@ static size_t tt_sweep_smem(int V, int max_pl, int max_c)
     if (V == 7) return (size_t)4 * 8 * 8 * 12 * sizeof(float);
     if (V == 8) return (size_t)4 * 8 * 4 * 36 * sizeof(float);
     if (V == 9) return (size_t)4 * 8 * 4 * 20 * sizeof(float);
-    if (V == 4) return (size_t)(2 * 32 * 64 + 4 * 64 * 68) * sizeof(float);   // one pair of C tiles per CTA + a staged slice block per warp
     return (size_t)4 * (max_pl + max_c) * sizeof(float);
 }
 
@@ -591,6 +601,9 @@ static cudaError_t launch_sweep_fwd(tt_emb* h, int max_pl, int max_c, cudaStream
         const size_t smem = GEN_C_FLOATS * sizeof(float);
         if ((e = cudaFuncSetAttribute(k_sweep_fwd_any, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
         if ((e = tt_launch_pdl(k_sweep_fwd_any, dim3(h->units_per_table, n), dim3(GEN_THREADS), smem, s, h->v, h->vbase[0])) != cudaSuccess) return e;
+    } else if constexpr (V == 4) {
+        if ((e = cudaFuncSetAttribute(k_sweep_fwd_wide, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)WIDE_SMEM)) != cudaSuccess) return e;
+        if ((e = tt_launch_pdl(k_sweep_fwd_wide, dim3(h->units_per_table, n), dim3(WIDE_THREADS), WIDE_SMEM, s, h->v, h->vbase[V + 1])) != cudaSuccess) return e;
     } else {
         const size_t smem = tt_sweep_smem(V, max_pl, max_c);
         if ((e = cudaFuncSetAttribute(k_sweep_fwd<V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
@@ -613,13 +626,20 @@ cudaError_t tt_launch_contraction(tt_emb* h, cudaStream_t s)
             if (k == h->K - 1 && f > max_c) max_c = f;
         }
     }
-    for (int k = 2; k <= h->K - 2; ++k) {
-        int grid = h->sm_count * 16;
-        cudaError_t e0 = tt_launch_pdl(k_mid_level, dim3(grid), dim3(128), (size_t)max_pl * sizeof(float), s, w, k);
-        if (e0 != cudaSuccess) return e0;
+    cudaError_t e;
+    if (h->K == 4 && (h->ablation & 1) == 0) {
+        int max_n = 1, max_z = 1;
+        for (int t = 0; t < h->T; ++t) {
+            const int z = (h->tab[t].d[1] * h->tab[t].r[2] + MT_EDGE - 1) / MT_EDGE;
+            if (h->tab[t].n[1] > max_n) max_n = h->tab[t].n[1];
+            if (z > max_z) max_z = z;
+        }
+        if ((e = tt_launch_pdl(k_level2, dim3(max_n, h->T, max_z), dim3(128), 0, s, w)) != cudaSuccess) return e;
+        tt_note_launch();
+    } else if (h->K == 4) {
+        if ((e = tt_launch_pdl(k_level2_nodes, dim3(h->sm_count * 16), dim3(128), (size_t)max_pl * sizeof(float), s, w)) != cudaSuccess) return e;
         tt_note_launch();
     }
-    cudaError_t e;
     // tables of different shape variants are independent: their kernels run side by side on forked streams
     int nvar = 0;
     for (int vi = 0; vi <= TT_NUM_VARIANTS; ++vi) nvar += h->vcount[vi] > 0 ? 1 : 0;
