@@ -147,7 +147,8 @@ int tt_emb_set_pooling(tt_emb_t h, int32_t mode, const float* per_sample_weights
  * core_grads HOST array of T*K DEVICE pointers, each shaped like the matching core (slice-major);
  *            fully OVERWRITTEN (untouched slices become zero), not accumulated.
  * Lookups are sorted by row and reduced by segments (dE); first- and middle-core slices each have a single
- * owner that sums its sorted contributions; last-core slices are accumulated with vector reductions into a
+ * owner that sums its sorted contributions (K = 2: a first-core slice may have several, which add their sums);
+ * last-core slices are accumulated with vector reductions into a
  * few L2-resident partial copies that are then added in a fixed order.  Needs enable_backward = 1.
  * Asynchronous.
  */
@@ -182,8 +183,8 @@ int tt_emb_sgd_step(tt_emb_t h, float* const* core_grads, float lr, tt_emb_strea
  * every core's gradient has a kernel that writes its final value (the fixed-order sum of the last core's partial
  * copies, the owner CTA of a middle-core slice, the sum over the children of a first digit); with lr != 0 that
  * kernel also applies G <- G - lr * dG to the elements it has just finished, so the gradient is not read again.
- * Cores whose gradient is finalised by a kernel that other blocks still read the core in (generic shape path,
- * K = 2 first core) are updated by the plain kernel at the end of the call.  core_grads is still fully written
+ * Cores whose gradient is finalised by a kernel that other blocks still read the core in (middle cores of shapes
+ * without a kernel of their own, K = 2 first core) are updated by the plain kernel at the end of the call.  core_grads is still fully written
  * (gradients at the pre-update cores), the result equals the two separate calls up to the rounding of identical
  * expressions.  Arguments and errors as tt_emb_backward; lr = 0 is tt_emb_backward.  Asynchronous.
  */
