@@ -967,7 +967,10 @@ __global__ void __launch_bounds__(32 * POOL_WARPS, 4) k_pool_async(WsView w, flo
 // window with one boundary is summed into two partial sums in one unrolled pass; a window with several bags in it is
 // summed by the whole warp at once, each sub-warp taking consecutive rows and the pieces of a bag that crosses
 // sub-warps being joined afterwards (from two boundaries on for rows of up to 128 bytes, from five on for wider rows,
-// where a sub-warp has sixteen rows to walk); a window with empty bags, weights or mean pooling is summed bag by bag.
+// where a sub-warp has sixteen rows to walk); a window with empty bags in it is summed bag by bag.  Weights and
+// mean pooling take the same ways (the factor with the row, 1 / length where a bag is written): 131 k bags of 1 to 30 weighted
+// rows of 128 bytes 73 -> 63 us, of 1 to 8 rows of 256 bytes with mean 51 -> 41 us, of one weighted row 33 -> 17 us against
+// bag by bag.
 // 2 million bags of 128-byte rows, stream against one bag per window: 2 / 4 / 8 lookups each 0.20 / 0.28 / 0.51 ms
 // against 0.82; 1 to 15 lookups 0.54 against 0.83, 1 to 31 0.83 against 0.91, 1 to 63 1.22 against 1.27, 1 to 100 1.69
 // against 1.72, 1 to 200 3.09 against 3.00 ms.  256-byte rows: 2 / 4 / 8 lookups 0.29 / 0.44 / 0.74 ms against 0.88-0.92;
@@ -978,6 +981,14 @@ __global__ void __launch_bounds__(32 * POOL_WARPS, 4) k_pool_async(WsView w, flo
 // clamped (offsets[bag], offsets[bag + 1]) pair as the header promises, and windows stop at the end of their bag.
 #define TT_POOL_STREAM_BELOW 33        // rows of up to 128 bytes
 #define TT_POOL_STREAM_BELOW_WIDE 12   // rows of up to 256 bytes
+// a += v, or a += f * v with weights
+template <bool WT>
+__device__ __forceinline__ void pool_add(float4& a, const float4& v, float f)
+{
+    if (WT) a = make_float4(fmaf(f, v.x, a.x), fmaf(f, v.y, a.y), fmaf(f, v.z, a.z), fmaf(f, v.w, a.w));
+    else tt_add4(a, v);
+}
+
 template <int R4, bool WT>   // R4: float4 pieces per staged row, 16 (D <= 64) or 8 (D <= 32)
 __global__ void __launch_bounds__(32 * POOL_WARPS, 4) k_pool_stream(WsView w, float* __restrict__ out)
 {
@@ -1119,7 +1130,7 @@ __global__ void __launch_bounds__(32 * POOL_WARPS, 4) k_pool_stream(WsView w, fl
         __syncwarp();
         // Windows with bag boundaries in them are summed by the whole warp at once.  Lane i looks at bag + i, which ends at
         // e_mine; a bag starts at row e - pos of the window for every end e inside it.
-        if (!WT && stream_ok && o_hi < pos + n) {
+        if (stream_ok && o_hi < pos + n) {
             const pos_t wend = pos + n;
             const int ei = (int)(bag - ebase) + lane;
             const pos_t e0 = __shfl_sync(0xffffffffu, ends_reg, ei & 31), e1 = __shfl_sync(0xffffffffu, ends_nx, ei & 31);
@@ -1133,8 +1144,12 @@ __global__ void __launch_bounds__(32 * POOL_WARPS, 4) k_pool_stream(WsView w, fl
 #pragma unroll
                 for (int jj = 0; jj < 32 / RPI; ++jj) {
                     const int j = RPI * jj + sub;
-                    if (j < n && lane_on)
-                        __stcs(o4 + (size_t)j * ostride, ((valid >> j) & 1u) ? buf[j * R4 + lr] : make_float4(0.f, 0.f, 0.f, 0.f));
+                    const float wj = WT ? __shfl_sync(0xffffffffu, wt, j) : 1.f;   // (the mean of one lookup is the lookup)
+                    if (j < n && lane_on) {
+                        float4 v = ((valid >> j) & 1u) ? buf[j * R4 + lr] : make_float4(0.f, 0.f, 0.f, 0.f);
+                        if (WT) v = make_float4(wj * v.x, wj * v.y, wj * v.z, wj * v.w);
+                        __stcs(o4 + (size_t)j * ostride, v);
+                    }
                 }
                 __syncwarp();
                 pos += n;
@@ -1154,7 +1169,8 @@ __global__ void __launch_bounds__(32 * POOL_WARPS, 4) k_pool_stream(WsView w, fl
                 for (int jj = 0; jj < 32 / RPI; ++jj) {
                     const int j = RPI * jj + sub;
                     const float4 v = buf[j * R4 + lr];
-                    if (j < c) tt_add4(pa, v); else tt_add4(pb, v);
+                    const float wj = WT ? __shfl_sync(0xffffffffu, wt, j) : 1.f;
+                    if (j < c) pool_add<WT>(pa, v, wj); else pool_add<WT>(pb, v, wj);
                 }
                 acc.x += pa.x; acc.y += pa.y; acc.z += pa.z; acc.w += pa.w;
                 close_bag();
@@ -1193,20 +1209,32 @@ __global__ void __launch_bounds__(32 * POOL_WARPS, 4) k_pool_stream(WsView w, fl
                 // they waited for instructions: 2.39 -> 1.90 ms on the 240-table workload, ncu `no_instruction` stalls)
                 // (the row of out of the bag being summed moves on by one bag per segment end; masks shifted to the sub-warp)
                 {
-                    const int j0 = sub * R4, ns = min(R4, n - j0);
+                    // (weights come by shuffle: then all sub-warps take the same number of steps, and those past the window's
+                    // last row do nothing)
+                    const int j0 = sub * R4, ns = min(R4, WT ? n : n - j0);
+                    int len = 0;                                  // rows of the running bag, for the mean
                     unsigned vs = valid >> j0, cs = closes >> j0;
                     float4* orow = row_of(j0);
                     const size_t ostride = (size_t)w.T * D4;
                     const float4* src = buf + j0 * R4 + lr;
 #pragma unroll 1
                     for (int jj = 0; jj < ns; ++jj, vs >>= 1, cs >>= 1, src += R4) {
+                        const float wj = WT ? __shfl_sync(0xffffffffu, wt, j0 + jj) : 1.f;
                         if (vs & 1u) {
                             const float4 v = *src;
-                            tt_add4(run, v);
+                            pool_add<WT>(run, v, wj);
                         }
+                        if (WT) ++len;
                         if (cs & 1u) {
                             if (head_open) { head = run; head_closed = true; head_open = false; }
-                            else if (lane_on) __stcs(orow, run);
+                            else if (lane_on) {
+                                if (WT && w.pool_mean) {
+                                    const float inv = 1.f / (float)len;
+                                    run = make_float4(run.x * inv, run.y * inv, run.z * inv, run.w * inv);
+                                }
+                                __stcs(orow, run);
+                            }
+                            if (WT) len = 0;
                             run = make_float4(0.f, 0.f, 0.f, 0.f);
                             orow += ostride;
                         }
@@ -1217,9 +1245,16 @@ __global__ void __launch_bounds__(32 * POOL_WARPS, 4) k_pool_stream(WsView w, fl
                 const unsigned hc = __ballot_sync(0xffffffffu, head_closed), ho = __ballot_sync(0xffffffffu, head_open);
 #pragma unroll
                 for (int s2 = 0; s2 < RPI; ++s2) {
+                    float inv = 1.f;
+                    if (WT && w.pool_mean) {   // the bag that is open at the sub-warp's first row: bag + kb
+                        const int kb = __popc(starts & ((2u << (s2 * R4)) - 2u));
+                        const pos_t e_end = __shfl_sync(0xffffffffu, e_mine, kb), e_beg = __shfl_sync(0xffffffffu, e_mine, kb > 0 ? kb - 1 : 0);
+                        inv = 1.f / (float)(e_end - (kb > 0 ? e_beg : o_lo));
+                    }
                     if (((hc >> (s2 * R4)) & 1u) && sub == s2 && lane_on) {
                         float4 sum = carry;
                         tt_add4(sum, head);
+                        if (WT && w.pool_mean) sum = make_float4(sum.x * inv, sum.y * inv, sum.z * inv, sum.w * inv);
                         __stcs(row_of(s2 * R4), sum);
                     }
                     float4 tail;
@@ -1268,11 +1303,11 @@ __global__ void __launch_bounds__(32 * POOL_WARPS, 4) k_pool_stream(WsView w, fl
                 continue;
             }
             float4 part = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (!WT && plain && seg == 32) {
+            if (plain && seg == 32) {
 #pragma unroll
                 for (int jj = 0; jj < 32 / RPI; ++jj) {
                     const float4 v = buf[(RPI * jj + sub) * R4 + lr];
-                    tt_add4(part, v);
+                    pool_add<WT>(part, v, WT ? __shfl_sync(0xffffffffu, wt, RPI * jj + sub) : 1.f);
                 }
             } else {
                 for (int jj = r / RPI; RPI * jj < r + seg; ++jj) {
