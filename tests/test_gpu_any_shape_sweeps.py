@@ -31,6 +31,11 @@ def test_rows_and_gradients(binding, n, d, r):  # noqa: F811
     N = int(np.prod(n))
     spec = TableSpec(N=N, n=n, d=d, r=r, alpha=0.7, core_dist="normal", core_scale=0.3)
     wl = workloads.custom([spec, spec], 211, (0, 60), seed=N + r[1], with_grad=True)
+    if wl.D == 1:
+        # the first core's gradient is one number, a sum of 6 k terms: with random signs it can cancel to 1/2000 of the sum of
+        # their magnitudes (about 1400), where fp32 is only bound to 2^-24 * 1400 = 8e-5; of one sign it is well conditioned
+        wl.grad_out = np.abs(wl.grad_out)
+        wl.cores = [[np.abs(c) for c in t] for t in wl.cores]
     emb = binding.from_workload(wl, enable_backward=True)
     assert emb.table_variant(0) == -1
     out = emb.forward(dev(wl.indices), dev(wl.offsets), wl.B)
