@@ -20,9 +20,17 @@
 // ---------------------------------------------------------------------------------------------- products
 
 // P_2 for every level-2 node of a four-core table: P_2 = G_1[i_1] . G_2[i_2].  A CTA keeps to one i_2 and 64 columns of its
-// slice and multiplies the slices of all present i_1, 64 stacked rows at a time (tiles.cuh); a prefix's node is a rank
-// look-up in the level's bitmap, so the nodes of one i_2 need no list.  (One CTA per node read its slice for itself: 3403
-// nodes of 2 x 64 by 64 x 256 took 70 us, bound by 0.2 GB of slices from L2; 16 us this way.)
+// slice, looks for the present i_1 in the level's bitmap, LEVEL2_SCAN of them at a time (a prefix's node is a rank look-up
+// there, so the nodes of one i_2 need no list), and multiplies the slices that it found, 64 stacked rows at a time
+// (tiles.cuh).  One CTA per node reads its slice for itself: 3403 nodes of 2 x 64 by 64 x 256 took 70 us, bound by 0.2 GB of
+// slices from L2, and take 16 us this way.
+#define LEVEL2_SCAN 256
+// CTAs that share the first digits of one i_2, a block of LEVEL2_SCAN each in turn (popular prefixes are often the first ones)
+__host__ __device__ __forceinline__ uint32_t tt_level2_parts(const TableDesc& td)
+{
+    const uint32_t most = ((uint32_t)td.n[0] + LEVEL2_SCAN - 1) / LEVEL2_SCAN, want = 2048u / (uint32_t)td.n[1];
+    return want < 1u ? 1u : (want < most ? want : most);
+}
 __global__ void __launch_bounds__(128, 4) k_level2(WsView w)
 {
     tt_pdl_enter();
@@ -30,95 +38,111 @@ __global__ void __launch_bounds__(128, 4) k_level2(WsView w)
     __shared__ const float* s_row[MT_EDGE];     // rows of G_1
     __shared__ float* s_out[MT_EDGE];
     __shared__ const float* s_slice[128];       // rows of the slice of G_2
-    __shared__ int s_any;
+    __shared__ uint2 s_list[LEVEL2_SCAN];       // present first digits and their nodes
+    __shared__ int s_count;
     const TableDesc& td = w.tdesc[blockIdx.y];
     const int M = td.d[0], ra = td.r[1], cols = td.d[1] * td.r[2], c0 = (int)blockIdx.z * MT_EDGE;
-    if ((int)blockIdx.x >= td.n[1] || c0 >= cols) return;
+    const uint32_t n2 = (uint32_t)td.n[1], i2 = blockIdx.x % n2, part = blockIdx.x / n2, parts = tt_level2_parts(td);
+    if (part >= parts || c0 >= cols) return;
+    const uint32_t n1 = (uint32_t)td.n[0];
     const bool vec = (ra & 3) == 0 && (cols & 3) == 0;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, g = lane >> 2, t = lane & 3, wr = wid >> 1, wc = wid & 1;
-    s_slice[tid] = tid < ra ? td.core[1] + (size_t)blockIdx.x * td.slice_floats[1] + (size_t)tid * cols + c0 : nullptr;   // r <= 128
-    const int rows = td.n[0] * M, kpasses = (ra + MT_KROWS - 1) / MT_KROWS;
+    s_slice[tid] = tid < ra ? td.core[1] + (size_t)i2 * td.slice_floats[1] + (size_t)tid * cols + c0 : nullptr;   // r <= 128
+    const int kpasses = (ra + MT_KROWS - 1) / MT_KROWS;
     const int ntl = min(4, max(0, (cols - c0 - 32 * wc + 7) / 8));
+    const uint32_t count = w.counters[CTR_LEVEL0 + 2];
     constexpr int STAGE = MT_EDGE * MT_PC + MT_KROWS * MT_PA;
-    for (int row0 = 0; row0 < rows; row0 += MT_EDGE) {
-        if (tid == 0) s_any = 0;
+    for (uint32_t base = part * LEVEL2_SCAN; base < n1; base += parts * LEVEL2_SCAN) {
+        if (tid == 0) s_count = 0;
         __syncthreads();
-        if (tid < MT_EDGE) {
-            const int row = row0 + tid;
-            const float* src = nullptr;
-            float* out = nullptr;
-            if (row < rows) {
-                const uint32_t p = (uint32_t)(row / M), m = (uint32_t)row - p * (uint32_t)M;
-                const uint32_t x = p * (uint32_t)td.n[1] + blockIdx.x;
-                const uint2 e = w.bml[2][td.lword_base[2] + (x >> 5)];
-                const uint32_t v = e.y + __popc(e.x & ((1u << (x & 31)) - 1u));
-                if (((e.x >> (x & 31)) & 1u) && v < w.counters[CTR_LEVEL0 + 2]) {
-                    src = td.core[0] + (size_t)row * ra;
-                    out = w.pbuf[2] + (size_t)v * w.stride[2] + (size_t)m * cols + c0;
-                    s_any = 1;
-                }
-            }
-            s_row[tid] = src;
-            s_out[tid] = out;
-        }
-        __syncthreads();
-        if (!s_any) continue;
-        float sum[2][4][4];
+        uint2 e[LEVEL2_SCAN / 128];
 #pragma unroll
-        for (int mt = 0; mt < 2; ++mt)
-#pragma unroll
-            for (int nt = 0; nt < 4; ++nt)
-#pragma unroll
-                for (int i = 0; i < 4; ++i) sum[mt][nt][i] = 0.f;
-        const int mtl = min(2, max(0, (min(rows - row0, MT_EDGE) - 32 * wr + 15) / 16));
-        auto issue = [&](int kp) {
-            float* st = sm + (kp & 1) * STAGE;
-            tt_stage_rows<MT_EDGE, MT_KROWS / 4>(st, MT_PC, s_row, kp * MT_KROWS, ra - kp * MT_KROWS, vec);
-            tt_stage_rows<MT_KROWS, MT_EDGE / 4>(st + MT_EDGE * MT_PC, MT_PA, s_slice + kp * MT_KROWS, 0, cols - c0, vec);
-            asm volatile("cp.async.commit_group;" ::: "memory");
-        };
-        issue(0);
-        for (int kp = 0; kp < kpasses; ++kp) {
-            if (kp + 1 < kpasses) {
-                issue(kp + 1);
-                asm volatile("cp.async.wait_group 1;" ::: "memory");
-            } else {
-                asm volatile("cp.async.wait_group 0;" ::: "memory");
-            }
-            __syncthreads();
-            if (mtl > 0 && ntl > 0) {
-                const float* A = sm + (kp & 1) * STAGE + (32 * wr + g) * MT_PC + t;
-                const float* D = sm + (kp & 1) * STAGE + MT_EDGE * MT_PC + t * MT_PA + 32 * wc + g;
-#pragma unroll
-                for (int p = 0; p < MT_KROWS / 8; ++p) {
-                    if (kp * MT_KROWS + 8 * p >= ra) break;
-                    const float* Aa = A + 8 * p;
-                    const float* Da = D + 8 * p * MT_PA;
-                    tt_quarter_step(sum, Aa, Aa + 8 * MT_PC, Aa + 4, Aa + 8 * MT_PC + 4, MT_PC, Da, Da + 4 * MT_PA, 1, mtl, ntl);
-                }
-            }
-            __syncthreads();
+        for (int j = 0; j < LEVEL2_SCAN / 128; ++j) {
+            const uint32_t p = base + 128 * j + tid;
+            e[j] = p < n1 ? w.bml[2][td.lword_base[2] + ((p * n2 + i2) >> 5)] : make_uint2(0u, 0u);
         }
 #pragma unroll
-        for (int mt = 0; mt < 2; ++mt)
+        for (int j = 0; j < LEVEL2_SCAN / 128; ++j) {
+            const uint32_t p = base + 128 * j + tid, bit = (p * n2 + i2) & 31;
+            const uint32_t v = e[j].y + __popc(e[j].x & ((1u << bit) - 1u));
+            const bool present = ((e[j].x >> bit) & 1u) && v < count;
+            const unsigned found = __ballot_sync(0xffffffffu, present);
+            int at = 0;
+            if (lane == 0 && found) at = atomicAdd(&s_count, __popc(found));
+            at = __shfl_sync(0xffffffffu, at, 0);
+            if (present) s_list[at + __popc(found & ((1u << lane) - 1u))] = make_uint2(p, v);
+        }
+        __syncthreads();
+        const int rows = s_count * M;               // at most 256 x 1024
+        for (int row0 = 0; row0 < rows; row0 += MT_EDGE) {
+            if (tid < MT_EDGE) {
+                const int q = (row0 + tid) / M, m = row0 + tid - q * M;
+                const bool some = row0 + tid < rows;
+                const uint2 x = some ? s_list[q] : make_uint2(0u, 0u);
+                s_row[tid] = some ? td.core[0] + ((size_t)x.x * M + m) * ra : nullptr;
+                s_out[tid] = some ? w.pbuf[2] + (size_t)x.y * w.stride[2] + (size_t)m * cols + c0 : nullptr;
+            }
+            __syncthreads();
+            float sum[2][4][4];
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                float* out = s_out[32 * wr + 16 * mt + 8 * h + g];
+            for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
-                for (int nt = 0; nt < 4; ++nt) {
-                    const int c = 32 * wc + 8 * nt + 2 * t;
-                    if (!out || c0 + c >= cols) continue;
-                    if (vec) *reinterpret_cast<float2*>(out + c) = make_float2(sum[mt][nt][2 * h], sum[mt][nt][2 * h + 1]);
-                    else {
-                        out[c] = sum[mt][nt][2 * h];
-                        if (c0 + c + 1 < cols) out[c + 1] = sum[mt][nt][2 * h + 1];
+                for (int nt = 0; nt < 4; ++nt)
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) sum[mt][nt][i] = 0.f;
+            const int mtl = min(2, max(0, (min(rows - row0, MT_EDGE) - 32 * wr + 15) / 16));
+            auto issue = [&](int kp) {
+                float* st = sm + (kp & 1) * STAGE;
+                tt_stage_rows<MT_EDGE, MT_KROWS / 4>(st, MT_PC, s_row, kp * MT_KROWS, ra - kp * MT_KROWS, vec);
+                tt_stage_rows<MT_KROWS, MT_EDGE / 4>(st + MT_EDGE * MT_PC, MT_PA, s_slice + kp * MT_KROWS, 0, cols - c0, vec);
+                asm volatile("cp.async.commit_group;" ::: "memory");
+            };
+            issue(0);
+            for (int kp = 0; kp < kpasses; ++kp) {
+                if (kp + 1 < kpasses) {
+                    issue(kp + 1);
+                    asm volatile("cp.async.wait_group 1;" ::: "memory");
+                } else {
+                    asm volatile("cp.async.wait_group 0;" ::: "memory");
+                }
+                __syncthreads();
+                if (mtl > 0 && ntl > 0) {
+                    const float* A = sm + (kp & 1) * STAGE + (32 * wr + g) * MT_PC + t;
+                    const float* D = sm + (kp & 1) * STAGE + MT_EDGE * MT_PC + t * MT_PA + 32 * wc + g;
+#pragma unroll
+                    for (int p = 0; p < MT_KROWS / 8; ++p) {
+                        if (kp * MT_KROWS + 8 * p >= ra) break;
+                        const float* Aa = A + 8 * p;
+                        const float* Da = D + 8 * p * MT_PA;
+                        tt_quarter_step(sum, Aa, Aa + 8 * MT_PC, Aa + 4, Aa + 8 * MT_PC + 4, MT_PC, Da, Da + 4 * MT_PA, 1, mtl, ntl);
                     }
                 }
+                __syncthreads();
             }
+#pragma unroll
+            for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    float* out = s_out[32 * wr + 16 * mt + 8 * h + g];
+#pragma unroll
+                    for (int nt = 0; nt < 4; ++nt) {
+                        const int c = 32 * wc + 8 * nt + 2 * t;
+                        if (!out || c0 + c >= cols) continue;
+                        if (vec) *reinterpret_cast<float2*>(out + c) = make_float2(sum[mt][nt][2 * h], sum[mt][nt][2 * h + 1]);
+                        else {
+                            out[c] = sum[mt][nt][2 * h];
+                            if (c0 + c + 1 < cols) out[c + 1] = sum[mt][nt][2 * h + 1];
+                        }
+                    }
+                }
+            __syncthreads();   // the addresses are rewritten for the next tile
+        }
+        __syncthreads();   // all have read the count
     }
 }
 
-// study switches: nodes that no bitmap finds (every lookup or row its own); one CTA per node
+// Few nodes per slice, or few of the possible prefixes present; also the study switches, whose nodes no bitmap finds (every
+// lookup or row its own).  One CTA per node
 __global__ void __launch_bounds__(128) k_level2_nodes(WsView w)
 {
     tt_pdl_enter();
@@ -614,6 +638,26 @@ static cudaError_t launch_sweep_fwd(tt_emb* h, int max_pl, int max_c, cudaStream
     return cudaGetLastError();
 }
 
+// Whether level 2 is multiplied digit by digit.  k_level2 starts CTAs for every i_2 and looks at every possible prefix; a node
+// by itself costs a read of its slice.  Forward call by node / by digit, us: n = 64^4, rank 64, 131 k lookups 238 / 201; n =
+// (1 M, 8, 8, 8), rank 64, 1 k lookups (8 k possible prefixes per lookup) 529 / 595, 131 k (61) 3760 / 2547; n = (4096, 4096,
+// 8, 8), rank 64, 131 k (128) 1456 / 1559 and 6553 / 4155 (popular and spread rows), rank 9 952 / 1063 and 1360 / 1598; n = (8,
+// 1 M, 8, 8), 131 k lookups (an eighth of a node per slice) 596 / 2320.
+#define LEVEL2_PER_SLICE 4
+#define LEVEL2_SPARSE 64
+static bool tt_level2_by_digit(const tt_emb* h)
+{
+    const WsView& w = h->v;
+    if (w.ablation & 1) return false;
+    const uint64_t nodes = w.L < (int64_t)w.cap[2] ? (uint64_t)w.L : w.cap[2];   // at most
+    uint64_t slices = 0, space = 0;
+    for (int t = 0; t < h->T; ++t) {
+        slices += (uint64_t)h->tab[t].n[1];
+        space += h->tab[t].prefix_space[2];
+    }
+    return nodes >= LEVEL2_PER_SLICE * slices && space <= LEVEL2_SPARSE * nodes;
+}
+
 cudaError_t tt_launch_contraction(tt_emb* h, cudaStream_t s)
 {
     WsView& w = h->v;
@@ -627,14 +671,15 @@ cudaError_t tt_launch_contraction(tt_emb* h, cudaStream_t s)
         }
     }
     cudaError_t e;
-    if (h->K == 4 && (h->ablation & 1) == 0) {
-        int max_n = 1, max_z = 1;
+    if (h->K == 4 && tt_level2_by_digit(h)) {
+        uint32_t max_x = 1, max_z = 1;
         for (int t = 0; t < h->T; ++t) {
-            const int z = (h->tab[t].d[1] * h->tab[t].r[2] + MT_EDGE - 1) / MT_EDGE;
-            if (h->tab[t].n[1] > max_n) max_n = h->tab[t].n[1];
+            const TableDesc& td = h->tab[t];
+            const uint32_t x = (uint32_t)td.n[1] * tt_level2_parts(td), z = (uint32_t)((td.d[1] * td.r[2] + MT_EDGE - 1) / MT_EDGE);
+            if (x > max_x) max_x = x;
             if (z > max_z) max_z = z;
         }
-        if ((e = tt_launch_pdl(k_level2, dim3(max_n, h->T, max_z), dim3(128), 0, s, w)) != cudaSuccess) return e;
+        if ((e = tt_launch_pdl(k_level2, dim3(max_x, h->T, max_z), dim3(128), 0, s, w)) != cudaSuccess) return e;
         tt_note_launch();
     } else if (h->K == 4) {
         if ((e = tt_launch_pdl(k_level2_nodes, dim3(h->sm_count * 16), dim3(128), (size_t)max_pl * sizeof(float), s, w)) != cudaSuccess) return e;
