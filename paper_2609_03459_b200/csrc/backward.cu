@@ -24,6 +24,7 @@
 #include "generic.cuh"
 #include "wide.cuh"
 #include "tiles.cuh"
+#include "rows.cuh"
 #include <type_traits>
 
 #define HT_SIZE 4096
@@ -1820,7 +1821,7 @@ __global__ void __launch_bounds__(128, 4) k_mid_tile(WsView w, int k, int lbase,
     const bool vec = (ra & 3) == 0 && (cols & 3) == 0;   // then every row, node and slice starts on a 16-byte boundary
     const uint32_t space = td.prefix_space[k - 1];
     const uint32_t j0 = tt_trank(w, td, k, ik * space), j1 = tt_trank(w, td, k, (ik + 1) * space);
-    const uint32_t R = (j1 - j0) * (uint32_t)M;          // stacked rows
+    const uint64_t R = tt_stacked_rows(j1 - j0, M);
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, g = lane >> 2, t = lane & 3;
     const int wr = wid >> 1, wc = wid & 1;               // this warp's quarter
     const int ach = (ra + MT_EDGE - 1) / MT_EDGE;
@@ -1840,54 +1841,63 @@ __global__ void __launch_bounds__(128, 4) k_mid_tile(WsView w, int k, int lbase,
         const int mtl = min(2, max(0, (ra - a0 - 32 * wr + 15) / 16)), ntl = min(4, max(0, (cols - c0 - 32 * wc + 7) / 8));
         __shared__ const float* s_a[3][MT_KROWS];
         __shared__ const float* s_d[3][MT_KROWS];
-        const uint32_t passes = (R + MT_KROWS - 1) / MT_KROWS;
-        auto lookup = [&](uint32_t r, const float*& pa, const float*& pd) {   // threads 0..31: row r * 32 + tid
+        const uint64_t passes = (R + MT_KROWS - 1) / MT_KROWS;
+        // this lane's row of a pass of 32 rows (a warp looks up one pass); the first of the passes that the warp looks up
+        StackedRow at = tt_stacked_row((uint64_t)(wid < 2 ? wid : 0) * MT_KROWS + lane, M);
+        auto lookup = [&](const float*& pa, const float*& pd) {
             pa = nullptr; pd = nullptr;
-            const uint32_t row = r * MT_KROWS + lane;
-            if (row < R) {
-                const uint32_t jn = row / (uint32_t)M, m = row - jn * (uint32_t)M;
-                const uint32_t v = w.tnode[k][j0 + jn];
-                pa = tt_left_operand(w, td, k, v) + (size_t)m * ra + a0;
-                pd = w.dP[k] + (size_t)v * w.stride[k] + (size_t)m * cols + c0;
+            if (at.node < j1 - j0) {
+                const uint32_t v = w.tnode[k][j0 + at.node];
+                pa = tt_left_operand(w, td, k, v) + (size_t)at.m * ra + a0;
+                pd = w.dP[k] + (size_t)v * w.stride[k] + (size_t)at.m * cols + c0;
             }
         };
-        auto issue = [&](uint32_t r) {
-            float* st = sm + (r & 1u) * (2 * STAGE);
-            tt_stage_rows<MT_KROWS, MT_EDGE / 4>(st, MT_PA, s_a[r % 3u], 0, ra - a0, vec);
-            tt_stage_rows<MT_KROWS, MT_EDGE / 4>(st + STAGE, MT_PA, s_d[r % 3u], 0, cols - c0, vec);
+        // the pass's buffer, and its addresses in the ring of three
+        auto issue = [&](int buf, int ring) {
+            float* st = sm + buf * (2 * STAGE);
+            tt_stage_rows<MT_KROWS, MT_EDGE / 4>(st, MT_PA, s_a[ring], 0, ra - a0, vec);
+            tt_stage_rows<MT_KROWS, MT_EDGE / 4>(st + STAGE, MT_PA, s_d[ring], 0, cols - c0, vec);
             asm volatile("cp.async.commit_group;" ::: "memory");
         };
         if (wid < 2) {   // passes 0 and 1 side by side
             const float *pa, *pd;
-            lookup((uint32_t)wid, pa, pd);
+            lookup(pa, pd);
             s_a[wid][lane] = pa;
             s_d[wid][lane] = pd;
         }
         __syncthreads();
-        if (passes > 0) issue(0);
-        for (uint32_t r = 0; r < passes; ++r) {
+        if (passes > 0) issue(0, 0);
+        at = tt_stacked_next(at, MT_KROWS, M);   // (warp 0: to pass 1)
+        int buf = 0, ring = 0;                   // of the current pass
+        for (uint64_t left = R; left > 0; left -= min(left, (uint64_t)MT_KROWS)) {
+            const int ring1 = ring == 2 ? 0 : ring + 1, ring2 = ring == 0 ? 2 : ring - 1;
             const float *pa = nullptr, *pd = nullptr;
-            if (wid == 0) lookup(r + 2, pa, pd);
-            if (r + 1 < passes) {
-                issue(r + 1);
+            if (wid == 0) {
+                at = tt_stacked_next(at, MT_KROWS, M);
+                lookup(pa, pd);
+            }
+            if (left > MT_KROWS) {
+                issue(buf ^ 1, ring1);
                 asm volatile("cp.async.wait_group 1;" ::: "memory");
             } else {
                 asm volatile("cp.async.wait_group 0;" ::: "memory");
             }
             __syncthreads();
             if (mtl > 0 && ntl > 0) {
-                const float* A = sm + (r & 1u) * (2 * STAGE) + 32 * wr + g;
-                const float* D = sm + (r & 1u) * (2 * STAGE) + STAGE + 32 * wc + g;
+                const float* A = sm + buf * (2 * STAGE) + 32 * wr + g;
+                const float* D = sm + buf * (2 * STAGE) + STAGE + 32 * wc + g;
 #pragma unroll
                 for (int p = 0; p < MT_KROWS / 8; ++p) {
-                    if (r * MT_KROWS + 8 * p >= R) break;
+                    if (8 * p >= left) break;
                     const float* Aa = A + (8 * p + t) * MT_PA;
                     const float* Da = D + (8 * p + t) * MT_PA;
                     tt_quarter_step(sum, Aa, Aa + 8, Aa + 4 * MT_PA, Aa + 4 * MT_PA + 8, 1, Da, Da + 4 * MT_PA, 1, mtl, ntl);
                 }
             }
-            if (wid == 0) { s_a[(r + 2) % 3u][lane] = pa; s_d[(r + 2) % 3u][lane] = pd; }   // the ring slot of pass r - 1
+            if (wid == 0) { s_a[ring2][lane] = pa; s_d[ring2][lane] = pd; }   // the ring slot of the pass before
             __syncthreads();
+            buf ^= 1;
+            ring = ring1;
         }
         float* const dst = td.grad[kc] + (size_t)ik * td.slice_floats[kc];
 #pragma unroll
@@ -1912,20 +1922,19 @@ __global__ void __launch_bounds__(128, 4) k_mid_tile(WsView w, int k, int lbase,
     __shared__ const float* s_row[MT_EDGE];    // dP row of each stacked row
     __shared__ const float* s_core[MT_EDGE];   // row of the slice for each a
     __shared__ float* s_out[MT_EDGE];
-    const uint32_t items = (R + MT_EDGE - 1) / MT_EDGE * (uint32_t)ach;
+    const uint64_t items = (R + MT_EDGE - 1) / MT_EDGE * (uint32_t)ach;   // (one or two of a: r <= 128)
     const int cpasses = (cols + MT_KROWS - 1) / MT_KROWS;
-    for (uint32_t it = blockIdx.z - (uint32_t)dgz; it < items; it += (uint32_t)yctas) {
-        const int a0 = (int)(it % (uint32_t)ach) * MT_EDGE;
-        const uint32_t row0 = it / (uint32_t)ach * MT_EDGE;
+    for (uint64_t it = blockIdx.z - (uint32_t)dgz; it < items; it += (uint32_t)yctas) {
+        const int a0 = (int)(it & (uint32_t)(ach - 1)) * MT_EDGE;
+        const uint64_t row0 = (it >> (ach - 1)) * MT_EDGE;
         if (tid < MT_EDGE) {
-            const uint32_t row = row0 + tid;
+            const StackedRow r = tt_stacked_next(tt_stacked_row(row0, M), tid, M);
             const float* pd = nullptr;
             float* py = nullptr;
-            if (row < R) {
-                const uint32_t jn = row / (uint32_t)M, m = row - jn * (uint32_t)M;
-                const uint32_t v = w.tnode[k][j0 + jn];
-                pd = w.dP[k] + (size_t)v * w.stride[k] + (size_t)m * cols;
-                py = w.Y[k] + (size_t)v * w.stride[k - 1] + (size_t)m * ra;
+            if (r.node < j1 - j0) {
+                const uint32_t v = w.tnode[k][j0 + r.node];
+                pd = w.dP[k] + (size_t)v * w.stride[k] + (size_t)r.m * cols;
+                py = w.Y[k] + (size_t)v * w.stride[k - 1] + (size_t)r.m * ra;
             }
             s_row[tid] = pd;
             s_out[tid] = py;
@@ -1934,7 +1943,7 @@ __global__ void __launch_bounds__(128, 4) k_mid_tile(WsView w, int k, int lbase,
             s_core[tid - MT_EDGE] = a < ra ? td.core[kc] + (size_t)ik * td.slice_floats[kc] + (size_t)a * cols : nullptr;
         }
         __syncthreads();
-        const int mtl = min(2, max(0, (int)(min(R - row0, (uint32_t)MT_EDGE) - 32 * wr + 15) / 16));
+        const int mtl = min(2, max(0, ((int)min(R - row0, (uint64_t)MT_EDGE) - 32 * wr + 15) / 16));
         const int ntl = min(4, max(0, (ra - a0 - 32 * wc + 7) / 8));
         auto issue = [&](int c) {
             float* st = sm + (c & 1) * (2 * STAGE);
