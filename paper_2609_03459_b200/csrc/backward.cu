@@ -2089,7 +2089,8 @@ cudaError_t tt_launch_bwd_middle(tt_emb* h, cudaStream_t s)
     for (int k = h->K - 1; k >= 2; --k) {
         bool any_fast[TT_NUM_MIDFAST] = {};
         uint32_t sum_blocks = 1;
-        int dgz = 1, tile_rows = 1;   // generic shapes: tiles of the slice gradient, most stacked rows of a slice
+        int dgz = 1;                  // generic shapes: tiles of the slice gradient,
+        int64_t ytiles = 1;           // most tiles of Y of a slice
         for (int t = 0; t < h->T; ++t) {
             const TableDesc& td = h->tab[t];
             const int kc = k - 1;
@@ -2100,7 +2101,7 @@ cudaError_t tt_launch_bwd_middle(tt_emb* h, cudaStream_t s)
             if (tiles > dgz) dgz = tiles;
             const int64_t rows = (int64_t)(td.prefix_space[k - 1] < w.cap[k] ? td.prefix_space[k - 1] : w.cap[k]) * td.P[kc];
             const int64_t yt = (rows + MT_EDGE - 1) / MT_EDGE * ((td.r[kc] + MT_EDGE - 1) / MT_EDGE);
-            if (yt > tile_rows) tile_rows = (int)(yt < 65535 ? yt : 65535);
+            if (yt > ytiles) ytiles = yt;
         }
         const int ngen = h->mcount[k][0];
         // level K-1's digit-major list already exists: the forward built it to order its sweep
@@ -2128,10 +2129,7 @@ cudaError_t tt_launch_bwd_middle(tt_emb* h, cudaStream_t s)
         if (any_fast[9]) { if ((e = tt_launch_mid<2, 8, 32>(mgrid(9), st(), w, k, 9, mlist(9))) != cudaSuccess) return e; tt_note_launch(); }
         if (any_fast[10]) { if ((e = tt_launch_mid<2, 8, 16>(mgrid(10), st(), w, k, 10, mlist(10))) != cudaSuccess) return e; tt_note_launch(); }
         if (ngen > 0) {
-            // Y tiles: as many CTAs per slice as fill the SMs about four times over, no more than there can be tiles
-            const int slices = h->mmaxn[k][0] * ngen;
-            int yctas = (h->sm_count * 16 + slices - 1) / slices;
-            if (yctas > tile_rows) yctas = tile_rows;
+            const int yctas = tt_ctas_per_slice(h->sm_count, (int64_t)h->mmaxn[k][0] * ngen, ytiles);
             if ((e = tt_launch_pdl(k_mid_tile, dim3(h->mmaxn[k][0], ngen, dgz + yctas), dim3(128), 0, st(), w, k, mlist(-1), dgz, yctas)) != cudaSuccess) return e;
             tt_note_launch();
         }

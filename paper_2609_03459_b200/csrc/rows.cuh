@@ -32,3 +32,11 @@ TT_HD StackedRow tt_stacked_next(StackedRow r, uint32_t n, int M)
     r.m = m - q * (uint32_t)M;
     return r;
 }
+
+// CTAs per slice for work of `tiles` tiles a slice at most: they fill the SMs four times over with four CTAs each.  The
+// slices of all tables of a handle may be 2^31 and more.
+TT_HD int tt_ctas_per_slice(int sm_count, int64_t slices, int64_t tiles)
+{
+    const int64_t want = ((int64_t)sm_count * 16 + slices - 1) / slices, most = tiles < 65535 ? tiles : 65535;
+    return (int)(want < most ? want : most);
+}

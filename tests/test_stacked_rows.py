@@ -1,5 +1,5 @@
 """Arithmetic of stacked rows (csrc/rows.cuh), compiled for the host: positions and counts around 2^31 and 2^32 rows, up to
-2^31 - 1 nodes of 1024 rows."""
+2^31 - 1 nodes of 1024 rows; CTAs per slice for 2^31 slices and more."""
 import ctypes
 import os
 import subprocess
@@ -13,6 +13,7 @@ extern "C" {
 uint64_t rows(uint32_t nodes, int M) { return tt_stacked_rows(nodes, M); }
 uint64_t at(uint64_t row, int M) { StackedRow r = tt_stacked_row(row, M); return ((uint64_t)r.node << 32) | r.m; }
 uint64_t after(uint32_t node, uint32_t m, uint32_t n, int M) { StackedRow r = {node, m}; r = tt_stacked_next(r, n, M); return ((uint64_t)r.node << 32) | r.m; }
+int ctas(int sm_count, int64_t slices, int64_t tiles) { return tt_ctas_per_slice(sm_count, slices, tiles); }
 }
 """
 
@@ -27,6 +28,7 @@ def lib(tmp_path_factory):
     so.rows.argtypes = [ctypes.c_uint32, ctypes.c_int]
     so.at.argtypes = [ctypes.c_uint64, ctypes.c_int]
     so.after.argtypes = [ctypes.c_uint32] * 3 + [ctypes.c_int]
+    so.ctas.argtypes = [ctypes.c_int, ctypes.c_int64, ctypes.c_int64]
     return so
 
 
@@ -41,3 +43,9 @@ def test_positions(lib, nodes, M):
         for n in (0, 1, 31, 32, 63, 64):
             if row + n < total:
                 assert lib.after(row // M, row % M, n, M) == ((row + n) // M) << 32 | (row + n) % M
+
+
+@pytest.mark.parametrize("slices,tiles,want", [
+    (1, 1, 1), (1, 10**12, 2368), (60, 1, 1), (60, 100, 40), (2368, 9, 1), (3 * 800_000_000, 1, 1), (2**31 - 1, 2**40, 1), (2**40, 5, 1)])
+def test_ctas_per_slice(lib, slices, tiles, want):
+    assert lib.ctas(148, slices, tiles) == want
