@@ -22,8 +22,10 @@
 // P_2 for every level-2 node of a four-core table: P_2 = G_1[i_1] . G_2[i_2].  A CTA keeps to one i_2 and 64 columns of its
 // slice, looks for the present i_1 in the level's bitmap, LEVEL2_SCAN of them at a time (a prefix's node is a rank look-up
 // there, so the nodes of one i_2 need no list), and multiplies the slices that it found, 64 stacked rows at a time
-// (tiles.cuh).  One CTA per node reads its slice for itself: 3403 nodes of 2 x 64 by 64 x 256 took 70 us, bound by 0.2 GB of
-// slices from L2, and take 16 us this way.
+// with fp32 FMAs: a thread makes eight rows by four columns, in the order of tt_mid_product (3xTF32 tiles took the same time, the
+// staging bounds both, and put the error of `out` against 64 bits at 1.29e-7 instead of 1.09e-7 for 3x3x3x5, rank 9).  One CTA
+// per node reads its slice for itself: 3403 nodes of 2 x 64 by 64 x 256 took 70 us, bound by 0.2 GB of slices from L2, and
+// take 16 us this way.
 #define LEVEL2_SCAN 256
 // CTAs that share the first digits of one i_2, a block of LEVEL2_SCAN each in turn (popular prefixes are often the first ones)
 __host__ __device__ __forceinline__ uint32_t tt_level2_parts(const TableDesc& td)
@@ -46,10 +48,9 @@ __global__ void __launch_bounds__(128, 4) k_level2(WsView w)
     if (part >= parts || c0 >= cols) return;
     const uint32_t n1 = (uint32_t)td.n[0];
     const bool vec = (ra & 3) == 0 && (cols & 3) == 0;
-    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, g = lane >> 2, t = lane & 3, wr = wid >> 1, wc = wid & 1;
+    const int tid = threadIdx.x, lane = tid & 31, ty = tid >> 4, tx = tid & 15;
     s_slice[tid] = tid < ra ? td.core[1] + (size_t)i2 * td.slice_floats[1] + (size_t)tid * cols + c0 : nullptr;   // r <= 128
     const int kpasses = (ra + MT_KROWS - 1) / MT_KROWS;
-    const int ntl = min(4, max(0, (cols - c0 - 32 * wc + 7) / 8));
     const uint32_t count = w.counters[CTR_LEVEL0 + 2];
     constexpr int STAGE = MT_EDGE * MT_PC + MT_KROWS * MT_PA;
     for (uint32_t base = part * LEVEL2_SCAN; base < n1; base += parts * LEVEL2_SCAN) {
@@ -83,14 +84,11 @@ __global__ void __launch_bounds__(128, 4) k_level2(WsView w)
                 s_out[tid] = some ? w.pbuf[2] + (size_t)x.y * w.stride[2] + (size_t)m * cols + c0 : nullptr;
             }
             __syncthreads();
-            float sum[2][4][4];
+            float sum[8][4];                        // rows ty + 8 i, columns 4 tx ..
 #pragma unroll
-            for (int mt = 0; mt < 2; ++mt)
+            for (int i = 0; i < 8; ++i)
 #pragma unroll
-                for (int nt = 0; nt < 4; ++nt)
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) sum[mt][nt][i] = 0.f;
-            const int mtl = min(2, max(0, (min(rows - row0, MT_EDGE) - 32 * wr + 15) / 16));
+                for (int j = 0; j < 4; ++j) sum[i][j] = 0.f;
             auto issue = [&](int kp) {
                 float* st = sm + (kp & 1) * STAGE;
                 tt_stage_rows<MT_EDGE, MT_KROWS / 4>(st, MT_PC, s_row, kp * MT_KROWS, ra - kp * MT_KROWS, vec);
@@ -106,35 +104,39 @@ __global__ void __launch_bounds__(128, 4) k_level2(WsView w)
                     asm volatile("cp.async.wait_group 0;" ::: "memory");
                 }
                 __syncthreads();
-                if (mtl > 0 && ntl > 0) {
-                    const float* A = sm + (kp & 1) * STAGE + (32 * wr + g) * MT_PC + t;
-                    const float* D = sm + (kp & 1) * STAGE + MT_EDGE * MT_PC + t * MT_PA + 32 * wc + g;
+                const float* A = sm + (kp & 1) * STAGE + ty * MT_PC;
+                const float* B = sm + (kp & 1) * STAGE + MT_EDGE * MT_PC + 4 * tx;
+                const int kn = min(MT_KROWS, ra - kp * MT_KROWS);   // zeros up to the next multiple of four
+                if (c0 + 4 * tx < cols)
+#pragma unroll 2
+                    for (int k = 0; k < kn; k += 4) {
+                        float4 x[8];
 #pragma unroll
-                    for (int p = 0; p < MT_KROWS / 8; ++p) {
-                        if (kp * MT_KROWS + 8 * p >= ra) break;
-                        const float* Aa = A + 8 * p;
-                        const float* Da = D + 8 * p * MT_PA;
-                        tt_quarter_step(sum, Aa, Aa + 8 * MT_PC, Aa + 4, Aa + 8 * MT_PC + 4, MT_PC, Da, Da + 4 * MT_PA, 1, mtl, ntl);
+                        for (int i = 0; i < 8; ++i) x[i] = *reinterpret_cast<const float4*>(A + 8 * i * MT_PC + k);
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) {
+                            const float4 y = *reinterpret_cast<const float4*>(B + (k + q) * MT_PA);
+#pragma unroll
+                            for (int i = 0; i < 8; ++i) {
+                                const float f = q == 0 ? x[i].x : q == 1 ? x[i].y : q == 2 ? x[i].z : x[i].w;
+                                sum[i][0] = fmaf(f, y.x, sum[i][0]); sum[i][1] = fmaf(f, y.y, sum[i][1]);
+                                sum[i][2] = fmaf(f, y.z, sum[i][2]); sum[i][3] = fmaf(f, y.w, sum[i][3]);
+                            }
+                        }
                     }
-                }
                 __syncthreads();
             }
 #pragma unroll
-            for (int mt = 0; mt < 2; ++mt)
+            for (int i = 0; i < 8; ++i) {
+                float* out = s_out[ty + 8 * i];
+                if (!out || c0 + 4 * tx >= cols) continue;
+                out += 4 * tx;
+                if ((cols & 3) == 0) *reinterpret_cast<float4*>(out) = make_float4(sum[i][0], sum[i][1], sum[i][2], sum[i][3]);
+                else
 #pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    float* out = s_out[32 * wr + 16 * mt + 8 * h + g];
-#pragma unroll
-                    for (int nt = 0; nt < 4; ++nt) {
-                        const int c = 32 * wc + 8 * nt + 2 * t;
-                        if (!out || c0 + c >= cols) continue;
-                        if (vec) *reinterpret_cast<float2*>(out + c) = make_float2(sum[mt][nt][2 * h], sum[mt][nt][2 * h + 1]);
-                        else {
-                            out[c] = sum[mt][nt][2 * h];
-                            if (c0 + c + 1 < cols) out[c + 1] = sum[mt][nt][2 * h + 1];
-                        }
-                    }
-                }
+                    for (int j = 0; j < 4; ++j)
+                        if (c0 + 4 * tx + j < cols) out[j] = sum[i][j];
+            }
             __syncthreads();   // the addresses are rewritten for the next tile
         }
         __syncthreads();   // all have read the count

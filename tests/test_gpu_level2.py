@@ -70,3 +70,16 @@ def test_rows(binding, n, d, r):  # noqa: F811
     for L in (1, 60, 50_000):
         check(emb, cores, n, torch.randint(0, int(np.prod(n)), (L,), device="cuda"))
     assert emb.check_guards() is None
+
+
+def test_products_keep_32_bits(binding):  # noqa: F811
+    # ranks of one and last cores of ones: a row is the product of two numbers, rounded once
+    import torch
+    n, d = (300, 7, 2, 2), (3, 5, 1, 1)
+    emb, cores = handle(binding, n, d, (1, 1, 1, 1, 1), 8400)
+    cores[2].fill_(1.0), cores[3].fill_(1.0)
+    for L in (20, 8400):         # by node, by digit
+        ids = torch.randperm(8400, device="cuda")[:L]
+        out = emb.forward(ids, torch.arange(L + 1, device="cuda"), L)
+        a, b = cores[0][ids // 28].reshape(L, 3, 1), cores[1][ids // 4 % 7].reshape(L, 1, 5)
+        assert torch.equal(out, (a * b).reshape(L, 15)), L
