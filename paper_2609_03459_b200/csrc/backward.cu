@@ -1337,7 +1337,7 @@ __global__ void __launch_bounds__(WIDE_THREADS, 2) k_sweep_bwd_wide(WsView w, in
     const int stripe = (blockIdx.x + blockIdx.y) % TT_STRIPES;
     float* gk = w.gpart + (size_t)stripe * w.gpart_stride + td.gpart_off;
     const uint32_t nK = (uint32_t)td.n[K - 1];
-    WideLoop loop(w, td, rng, batches, Bs, As, Cs);
+    WideLoop<true> loop(w, td, rng, batches, Bs, As, Cs);
     while (loop.next()) {
         const WideBatch& b = loop.batch();
         const uint32_t rows = wide_rows(b);

@@ -512,7 +512,7 @@ __global__ void __launch_bounds__(WIDE_THREADS, 2) k_sweep_fwd_wide(WsView w, in
     const uint2 rng = w.unit_rng[t * w.units_per_table + blockIdx.x];
     const TableDesc& td = w.tdesc[t];
     const uint32_t nK = (uint32_t)td.n[K - 1];
-    WideLoop loop(w, td, rng, batches, Bs, As, Cs);
+    WideLoop<false> loop(w, td, rng, batches, Bs, As, Cs);
     while (loop.next()) {
         const WideBatch& b = loop.batch();
         const uint32_t rows = wide_rows(b);
