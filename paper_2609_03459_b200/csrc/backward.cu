@@ -727,6 +727,7 @@ __global__ void __launch_bounds__(GEN_THREADS, 3) k_sweep_bwd_any(WsView w, int 
     tt_pdl_enter();
     extern __shared__ __align__(16) float sm[];
     __shared__ GenBatch b;
+    __shared__ float4 s_part[GEN_THREADS];
     const int t = w.vlist[vbase + blockIdx.y], K = w.K;
     const uint2 rng = w.unit_rng[t * w.units_per_table + blockIdx.x];
     const TableDesc& td = w.tdesc[t];
@@ -749,10 +750,10 @@ __global__ void __launch_bounds__(GEN_THREADS, 3) k_sweep_bwd_any(WsView w, int 
             gen_rows(w, td, cnt, r0, n, b);
             if (vec) {
                 gen_backward_slice<true>(w, td, n, b, Cs, gk);
-                gen_backward_dc<true>(w, td, r0, n, b, dCs);
+                gen_backward_dc<true>(w, td, r0, n, b, dCs, s_part);
             } else {
                 gen_backward_slice<false>(w, td, n, b, Cs, gk);
-                gen_backward_dc<false>(w, td, r0, n, b, dCs);
+                gen_backward_dc<false>(w, td, r0, n, b, dCs, s_part);
             }
             __syncthreads();
         }

@@ -242,13 +242,21 @@ __device__ __forceinline__ void gen_backward_slice(const WsView& w, const TableD
 
 // dC += dE . G_K[i_K]^T over the n looked-up rows, r0 the first of them: an item is two by two elements of one group's dC
 // over the group's rows among them, eight rows to a partial sum.  Where the rows belong to few groups, a group's rows are
-// cut into `parts` so that all threads have an item; the parts meet in shared memory.
+// cut into `parts` so that all threads have an item; the parts meet in s_part [GEN_THREADS] and are added in order.
 template <bool VEC>
-__device__ __forceinline__ void gen_backward_dc(const WsView& w, const TableDesc& td, uint32_t r0, int n, const GenBatch& b, float* dCs)
+__device__ __forceinline__ void gen_backward_dc(const WsView& w, const TableDesc& td, uint32_t r0, int n, const GenBatch& b, float* dCs, float4* s_part)
 {
     const int K = w.K, Pm = td.P[K - 1], rb = td.r[K - 1], dK = td.d[K - 1], pitch = gen_pitch(rb), slice = td.slice_floats[K - 1];
     const int q0 = (int)b.q[0], nq = (int)b.q[n - 1] - q0 + 1, ab = (rb + 1) / 2, per = (Pm + 1) / 2 * ab, items = nq * per;
     const int parts = items < GEN_THREADS ? min(16, GEN_THREADS / items) : 1;
+    auto add = [&](int ie, const float4& x) {
+        const int qq = ie / per, e = ie - qq * per, p = e / ab * 2, a = (e - e / ab * ab) * 2;
+        float* dst = dCs + (q0 + qq) * (Pm * pitch) + p * pitch + a;
+        dst[0] += x.x;
+        if (a + 1 < rb) dst[1] += x.y;
+        if (p + 1 < Pm) dst[pitch] += x.z;
+        if (p + 1 < Pm && a + 1 < rb) dst[pitch + 1] += x.w;
+    };
     for (int it = threadIdx.x; it < items * parts; it += GEN_THREADS) {
         const int part = it / items, ie = it - part * items, qq = ie / per, e = ie - qq * per, p = e / ab * 2, a = (e - e / ab * ab) * 2;
         const int q = q0 + qq;
@@ -283,14 +291,19 @@ __device__ __forceinline__ void gen_backward_dc(const WsView& w, const TableDesc
 #pragma unroll
             for (int s = 0; s < 2; ++s) { sum[s][0] += acc[s][0]; sum[s][1] += acc[s][1]; }
         }
-        float* dst = dCs + q * (Pm * pitch) + p * pitch + a;
-#pragma unroll
-        for (int s = 0; s < 2; ++s)
-#pragma unroll
-            for (int t = 0; t < 2; ++t) {
-                if ((s && !pn) || (t && !an)) continue;
-                if (parts > 1) atomicAdd(dst + s * pitch + t, sum[s][t]);
-                else dst[s * pitch + t] += sum[s][t];
+        const float4 x = make_float4(sum[0][0], sum[0][1], sum[1][0], sum[1][1]);
+        if (parts > 1) s_part[it] = x;               // then a thread has one item
+        else add(ie, x);
+    }
+    if (parts > 1) {
+        __syncthreads();
+        if ((int)threadIdx.x < items) {
+            float4 x = s_part[threadIdx.x];
+            for (int part = 1; part < parts; ++part) {
+                const float4 y = s_part[part * items + threadIdx.x];
+                x.x += y.x; x.y += y.y; x.z += y.z; x.w += y.w;
             }
+            add((int)threadIdx.x, x);
+        }
     }
 }

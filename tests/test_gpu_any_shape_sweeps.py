@@ -49,3 +49,23 @@ def test_rows_and_gradients(binding, n, d, r):  # noqa: F811
     for ablation in (1, 2, 4):
         study = binding.from_workload(wl, ablation=ablation)
         assert_close(study.forward(dev(wl.indices), dev(wl.offsets), wl.B).cpu().numpy(), oracle.forward_workload(wl), f"out, switch {ablation}")
+
+
+@pytest.mark.parametrize("n,d,r", [((2, 3, 400), (3, 3, 5), (1, 6, 4, 1)), ((1, 2, 900), (4, 2, 8), (1, 3, 7, 1))])
+def test_gradients_above_the_last_core_repeat_bit_for_bit(binding, n, d, r):  # noqa: F811
+    # few groups of many rows: a group's rows are cut into parts, which are added in order.  Every row is looked up once, so that
+    # the gradients of the rows do not depend on the order of the sorted look-ups
+    rng = np.random.default_rng(7)
+    N = int(np.prod(n))
+    spec = TableSpec(N=N, n=n, d=d, r=r, alpha=1.0, core_dist="normal", core_scale=1.0)
+    wl = workloads.custom([spec], N, 1, seed=11, with_grad=True)
+    wl.indices, wl.offsets = rng.permutation(N).astype(np.int64), np.arange(N + 1, dtype=np.int64)
+    emb = binding.from_workload(wl, enable_backward=True)
+    first = None
+    for _ in range(8):
+        emb.forward(dev(wl.indices), dev(wl.offsets), wl.B)
+        emb.backward(dev(wl.grad_out))
+        grads = emb.get_grads()[0][:2]
+        first = first or grads
+        for k in range(2):
+            assert np.array_equal(grads[k], first[k]), k
