@@ -22,6 +22,8 @@ pytestmark = pytest.mark.gpu
     ((9, 4, 3), (3, 2, 2), (1, 128, 20, 1)),         # two tiles of a
     ((4, 5, 4, 6), (2, 4, 4, 4), (1, 64, 64, 64, 1)),
     ((3, 4, 5, 3), (3, 2, 3, 2), (1, 5, 7, 9, 1)),
+    ((3, 9500, 3), (2, 5, 2), (1, 65, 3, 1)),        # so many slices that the CTAs of dG make Y too; two tiles of a
+    ((90, 4800, 2), (3, 3, 5), (1, 6, 4, 1)),
 ])
 def test_gradients_and_fused_update(binding, n, d, r):  # noqa: F811
     spec = TableSpec(N=int(np.prod(n)) - 1, n=n, d=d, r=r, alpha=0.9, core_dist="normal", core_scale=0.3)
