@@ -1,12 +1,19 @@
-// Grouping and schedule of small batches in one kernel: one cluster of sixteen CTAs runs every step, with the cluster's
-// hardware barrier between the steps.
+// Grouping and schedule in one kernel, where the bitmaps are short (tt_use_cluster): one cluster of sixteen CTAs runs every
+// step, with the cluster's hardware barrier between the steps.
 //
 // The steps of grouping.cu are a chain of fifteen dependent kernels (marks, a scan per level, links, the digit-major list,
 // costs, boundaries), 3 to 5 us each however little they do.  Sixteen SMs do the same work on a few thousand lookups in
 // less than the launches cost: 1 k lookups, one table, grouping and schedule 74 -> 34 us, now bound by the latency of the
 // dependent loads in each step (one to three L2 round trips between two barriers).  The step functions are those of
-// group.cuh; only the distribution over threads differs.  Where every table is swept by warps that take one batch of groups
-// at a time, units of equal group counts do as well as units of equal cost, so the costs and their scan are left out.
+// group.cuh; only the distribution over threads differs.
+// Where every table is swept by warps that take one batch of groups at a time, the units hold equal group counts instead of
+// equal costs, whatever the batch, and the costs and their scan are left out.  Whole forward calls with equal counts / equal costs
+// (4x4x4, rank 16), us: 1 table, 11 k lookups 55 / 67, 0.5 M 136 / 147, 10 M 743 / 773; 8 tables of 10 M rows, 4 M lookups 811 / 860;
+// the other way only for few lookups of large tables whose popular prefixes hold hundreds of rows (1 table of 40 M rows, 11 k
+// lookups, popular rows first 107 / 97; 2 tables 127 / 118).
+// The cluster needs sixteen SMs of one GPC at one moment.  Calls of 1 k lookups beside another stream's kernels, cluster / a
+// kernel per step, us: idle GPU 47 / 77; copies of 1 GB, median of the calls that meet them 0.66 / 2.2 ms (each kernel of the
+// chain waits for its turn); matrix products 0.72 / 0.70 ms; forwards of 16 tables 0.11 / 0.84 ms.
 #include "common.cuh"
 #include "scan.cuh"
 #include "group.cuh"

@@ -129,20 +129,28 @@ __global__ void __launch_bounds__(256) k_nodedup_levels(WsView w)
 
 // 0: a kernel per step; 1: one cluster of sixteen SMs (group_cluster.cu) from the prefix levels on; 2: one cluster for
 // everything.  The cluster saves a dozen launches and loses where a step has work for more SMs: scans and links of large
-// prefix spaces, marks and scan of long row bitmaps.  Whole call with 0 / 1 / 2, us: 1 table of 1 M rows (33 k words), 1 k
-// lookups 73 / 53 / 43; 2 tables, 98 k words, 18 k lookups (training) 254 / 229 / 228; 8 tables, 573 k words, 8 k lookups
-// 95 / 78 / 95; 16 tables, prefix bitmaps of 10 k words 127 / 115; of 30 k words 221 / 253.
+// prefix spaces, marks and scan of long row bitmaps, checks of many offsets.  Whole call with 0 / 1 / 2, us: 1 table of 1 M
+// rows (33 k words), 1 k lookups 73 / 53 / 43; 2 tables, 98 k words, 18 k lookups (training) 254 / 229 / 228; 8 tables, 573 k
+// words, 8 k lookups 95 / 78 / 95; 16 tables, prefix bitmaps of 10 k words 127 / 115; of 30 k words 221 / 253.
+// Up to 8 k words whatever the batch (0 / 1: 1 table of 10 M rows, 2 M lookups 333 / 308, 10 M lookups 773 / 743; 2 of 40 M rows,
+// 8 k words, 4 M lookups 489 / 475, 20 M 2046 / 2046); between 8 k and 16 k words only with few lookups, which leave most
+// of the prefixes out (8 tables of 10 M rows, 12 k words, spread rows: 85 k lookups 167 / 164, 4 M 725 / 747, 16 M 1434 / 1464).
+// Offsets (20 k lookups, 1 / 2): 0.26 M 92 / 87 and 108 / 110, 1 M 189 / 203.
+#define TT_CLUSTER_ANY_WORDS (1u << 13)
 #define TT_CLUSTER_LEVEL_WORDS (1u << 14)
+#define TT_CLUSTER_LEVEL_LOOKUPS (1 << 21)
 #define TT_CLUSTER_ROW_WORDS (1u << 17)
 #define TT_CLUSTER_LOOKUPS (1 << 15)
+#define TT_CLUSTER_OFFSETS (1 << 18)
 static int tt_use_cluster(const tt_emb* h)
 {
     const WsView& w = h->v;
     if (!h->cluster_ok || w.ablation) return 0;
+    uint32_t words = w.K >= 3 ? w.ttotal_words[w.K - 1] : 0u;
     for (int k = 1; k < w.K; ++k)
-        if (w.total_words_l[k] > TT_CLUSTER_LEVEL_WORDS) return 0;
-    if (w.K >= 3 && w.ttotal_words[w.K - 1] > TT_CLUSTER_LEVEL_WORDS) return 0;
-    return w.total_words <= TT_CLUSTER_ROW_WORDS && w.L <= TT_CLUSTER_LOOKUPS ? 2 : 1;
+        if (w.total_words_l[k] > words) words = w.total_words_l[k];
+    if (words > (w.L <= TT_CLUSTER_LEVEL_LOOKUPS ? TT_CLUSTER_LEVEL_WORDS : TT_CLUSTER_ANY_WORDS)) return 0;
+    return w.total_words <= TT_CLUSTER_ROW_WORDS && w.L <= TT_CLUSTER_LOOKUPS && (int64_t)w.T * w.B <= TT_CLUSTER_OFFSETS ? 2 : 1;
 }
 
 cudaError_t tt_launch_grouping(tt_emb* h, cudaStream_t s)
