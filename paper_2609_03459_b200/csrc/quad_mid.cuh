@@ -2,7 +2,7 @@
 // tensor cores.
 //
 // Groups are walked in digit-major order, so neighbours share the slice B = G_{K-1}[i_{K-1}] (r_a x cols).  With
-// P_{K-2} of MROWS = 4 (or 2, 8) rows per group, NG = 16 / MROWS = 4 (or 8, 2) groups stack into one 16 x r_a operand, and
+// P_{K-2} of MROWS = 4 (or 2) rows per group, NG = 16 / MROWS = 4 (or 8) groups stack into one 16 x r_a operand, and
 //     [C_0; ..; C_{NG-1}] = [P_0; ..; P_{NG-1}] . B
 // is a 16 x cols product of m16n8k8 tiles in 3xTF32 (see mma.cuh).  The slice then enters the SM once per NG
 // groups instead of once per group (the FP32-pipe form of this product was bound by the L1 operand path), and the
@@ -14,20 +14,17 @@
 // One pass.  Lane (g = lane / 4, t = lane % 4) feeds rows g and g + 8 of the stacked operand: row g belongs to group
 // g / MROWS (source srcA, taken when selA), row g + 8 to group (8 + g) / MROWS (srcB, selB); m = g % MROWS is the row
 // of P inside the group.  src points at P (MROWS x ra, row-major).  ra <= 8 * KTMAX, any value (the k range is padded
-// with zeros).  Results go to Cs4 + q * MROWS * COLS + m * COLS + column for group q (C_q as [MROWS][COLS] =
-// [PM][RB] row-major).
+// with zeros).  Results go to the group's C tile in Cs4, stored as [PM][RB + 4]: rows of r_{K-1} = RB values padded by four
+// floats, which makes the row stage's fragment loads from shared memory conflict-free.
 //
 // Column mapping: a block of 32 columns is one float4 load per lane and k row (8 lanes x 16 bytes = 128 bytes per
 // row); tile j of the block takes component j, i.e. tile column n' stands for slice column 32 * block + 4 n' + j, so
 // that a lane ends up with 8 consecutive columns of each of its two rows (two float4 stores per row).
-// RBP > 0: C tiles are stored as [PM][RBP + 4] (rows of r_{K-1} = RBP values padded by four floats), which makes the
-// row stage's fragment loads from shared memory conflict-free; RBP = 0: plain [MROWS][COLS] tiles.
-template <int COLS, int MROWS, int KTMAX, int RBP = 0>
+template <int COLS, int MROWS, int KTMAX, int RB>
 __device__ __forceinline__ void tt_quad_mid_mma(const float* __restrict__ B, int ra, const float* __restrict__ srcA,
-                                                const float* __restrict__ srcB, bool selA, bool selB, float* Cs4, int lane,
-                                                int nb0 = 0, int nb1 = COLS / 32)   // column blocks of 32 this warp computes
+                                                const float* __restrict__ srcB, bool selA, bool selB, float* Cs4, int lane)
 {
-    static_assert((MROWS == 2 || MROWS == 4 || MROWS == 8) && KTMAX % 2 == 0, "stacking of 8, 4 or 2 groups");
+    static_assert((MROWS == 2 || MROWS == 4) && KTMAX % 2 == 0, "stacking of 8 or 4 groups");
     const int g = lane >> 2, t = lane & 3, m = g & (MROWS - 1);
     const int kta = (ra + 7) >> 3;
     // the stacked operand stays unsplit in registers (KTMAX * 4) and is split where it is used: half the registers of
@@ -43,20 +40,17 @@ __device__ __forceinline__ void tt_quad_mid_mma(const float* __restrict__ B, int
     }
     const float4* __restrict__ B4 = reinterpret_cast<const float4*>(B);
     constexpr int C4N = COLS / 4;
-    constexpr int DSUB = RBP > 0 ? COLS / RBP : 1;              // d_{K-1}: rows of C per row of P
-    constexpr int TILE = RBP > 0 ? MROWS * DSUB * (RBP + 4) : MROWS * COLS;
-    float* dstA = Cs4 + (size_t)(g / MROWS) * TILE + (RBP > 0 ? 0 : m * COLS + 8 * t);
-    float* dstB = Cs4 + (size_t)((8 + g) / MROWS) * TILE + (RBP > 0 ? 0 : m * COLS + 8 * t);
+    constexpr int DSUB = COLS / RB;                             // d_{K-1}: rows of C per row of P
+    constexpr int TILE = MROWS * DSUB * (RB + 4);
+    float* dstA = Cs4 + (size_t)(g / MROWS) * TILE;
+    float* dstB = Cs4 + (size_t)((8 + g) / MROWS) * TILE;
     // offset of columns [32 nb + 8 t, + 8) of row m inside a tile
     auto coff = [&](int nb) {
-        if (RBP > 0) {
-            const int col = 32 * nb + 8 * t;
-            return (m * DSUB + col / RBP) * (RBP + 4) + col % RBP;
-        }
-        return 32 * nb;
+        const int col = 32 * nb + 8 * t;
+        return (m * DSUB + col / RB) * (RB + 4) + col % RB;
     };
 #pragma unroll 1
-    for (int nb = nb0; nb < nb1; ++nb) {
+    for (int nb = 0; nb < COLS / 32; ++nb) {
         float acc[4][4];
 #pragma unroll
         for (int j = 0; j < 4; ++j) { acc[j][0] = 0.f; acc[j][1] = 0.f; acc[j][2] = 0.f; acc[j][3] = 0.f; }
@@ -100,7 +94,7 @@ __device__ __forceinline__ void tt_quad_mid_mma(const float* __restrict__ B, int
 
 // All passes of one batch of cnt <= 16 / MROWS groups.  Lane q < cnt holds group q's slice index (imq) and operand
 // pointer (srcq).
-template <int COLS, int MROWS, int KTMAX, int RBP = 0>
+template <int COLS, int MROWS, int KTMAX, int RB>
 __device__ __forceinline__ void tt_quad_mid(const float* __restrict__ core_mid, size_t slice_floats, int ra, int cnt, uint32_t imq,
                                             const float* srcq, float* Cs4, int lane)
 {
@@ -115,7 +109,7 @@ __device__ __forceinline__ void tt_quad_mid(const float* __restrict__ core_mid, 
         const uint32_t im = __shfl_sync(0xffffffffu, imq, first);
         const unsigned sel = __ballot_sync(0xffffffffu, lane < 16 / MROWS && ((remaining >> lane) & 1u) && imq == im) & ((1u << (16 / MROWS)) - 1u);
         const bool selA = (sel >> qA) & 1u, selB = (sel >> qB) & 1u;
-        tt_quad_mid_mma<COLS, MROWS, KTMAX, RBP>(core_mid + (size_t)im * slice_floats, ra, srcA, srcB, selA, selB, Cs4, lane);
+        tt_quad_mid_mma<COLS, MROWS, KTMAX, RB>(core_mid + (size_t)im * slice_floats, ra, srcA, srcB, selA, selB, Cs4, lane);
         remaining &= ~sel;
     }
 }
