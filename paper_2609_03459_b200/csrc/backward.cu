@@ -1802,12 +1802,13 @@ __global__ void __launch_bounds__(128, 5) k_mid_mma(WsView w, int k, int variant
 //   z < dgz   one tile of dG_k[i_k]: 64 values of a by 64 columns; k runs over the slice's stacked rows (node, m), 32 per
 //             pass, staged with cp.async in two buffers, row addresses looked up two passes ahead
 //   z >= dgz  Y: tiles of 64 stacked rows by 64 values of a, dealt out to the slice's `yctas` CTAs; k runs over the
-//             columns, 32 per pass.  yctas = 0: to the CTAs of dG, after their tile
+//             columns, 32 per pass.  FOLD: to the CTAs of dG, after their tile
 // A warp owns a 32 x 32 quarter of the tile (tiles.cuh; 16 fragment loads per k step for 8 tile products of 3xTF32); row
 // tiles and column blocks outside the shape are skipped.  No fused update of the slice: the Y CTAs of other tiles still read it.
 // Bound by the operand path (16 fragment loads for 24 tensor instructions) and, for short node lists, by a CTA's look-ups.
 // Middle stage, 2x4x4x4 with rank 64 (65 536 lookups): 5.05 ms with one FP32 thread per output element over the whole
 // node list, 0.16 ms as tiles; 3x3x5 with ranks 6 and 4 (4 tables, 1 M lookups): 0.41 and 0.06 ms.
+template <bool FOLD>
 __global__ void __launch_bounds__(128, 4) k_mid_tile(WsView w, int k, int lbase, int dgz, int yctas)
 {
     tt_pdl_enter();
@@ -1835,8 +1836,9 @@ __global__ void __launch_bounds__(128, 4) k_mid_tile(WsView w, int k, int lbase,
             for (int i = 0; i < 4; ++i) sum[mt][nt][i] = 0.f;
 
     const int cch = (cols + MT_EDGE - 1) / MT_EDGE;
-    if ((int)blockIdx.z < min(dgz, ach * cch)) {
+    if ((int)blockIdx.z < (FOLD ? min(dgz, ach * cch) : dgz)) {
         // ------------------------------------------------------------------------------ a tile of the slice gradient
+        if (!FOLD && (int)blockIdx.z >= ach * cch) return;
         const int a0 = (int)blockIdx.z / cch * MT_EDGE, c0 = (int)blockIdx.z % cch * MT_EDGE;
         const int mtl = min(2, max(0, (ra - a0 - 32 * wr + 15) / 16)), ntl = min(4, max(0, (cols - c0 - 32 * wc + 7) / 8));
         __shared__ const float* s_a[3][MT_KROWS];
@@ -1907,19 +1909,25 @@ __global__ void __launch_bounds__(128, 4) k_mid_tile(WsView w, int k, int lbase,
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                     const int a = a0 + 32 * wr + 16 * mt + 8 * h + g, c = c0 + 32 * wc + 8 * nt + 2 * t;
+                    if (a >= ra || c >= cols) continue;
                     float* d = dst + (size_t)a * cols + c;
-                    if (a < ra && c < cols) {
-                        if (vec) *reinterpret_cast<float2*>(d) = make_float2(sum[mt][nt][2 * h], sum[mt][nt][2 * h + 1]);
-                        else {
-                            d[0] = sum[mt][nt][2 * h];
-                            if (c + 1 < cols) d[1] = sum[mt][nt][2 * h + 1];
-                        }
+                    if (vec) *reinterpret_cast<float2*>(d) = make_float2(sum[mt][nt][2 * h], sum[mt][nt][2 * h + 1]);
+                    else {
+                        d[0] = sum[mt][nt][2 * h];
+                        if (c + 1 < cols) d[1] = sum[mt][nt][2 * h + 1];
                     }
-                    sum[mt][nt][2 * h] = 0.f;
-                    sum[mt][nt][2 * h + 1] = 0.f;
                 }
+        if constexpr (FOLD) {
+#pragma unroll
+            for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+                for (int nt = 0; nt < 4; ++nt)
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) sum[mt][nt][i] = 0.f;
+        } else {
+            return;
+        }
     }
-    if (yctas > 0 && (int)blockIdx.z < dgz) return;
 
     // ---------------------------------------------------------------------------------- tiles of Y
     __shared__ const float* s_row[MT_EDGE];    // dP row of each stacked row
@@ -1927,7 +1935,7 @@ __global__ void __launch_bounds__(128, 4) k_mid_tile(WsView w, int k, int lbase,
     __shared__ float* s_out[MT_EDGE];
     const uint64_t items = (R + MT_EDGE - 1) / MT_EDGE * (uint32_t)ach;   // (one or two of a: r <= 128)
     const int cpasses = (cols + MT_KROWS - 1) / MT_KROWS;
-    const uint32_t first = yctas > 0 ? blockIdx.z - (uint32_t)dgz : blockIdx.z, step = (uint32_t)(yctas > 0 ? yctas : dgz);
+    const uint32_t first = FOLD ? blockIdx.z : blockIdx.z - (uint32_t)dgz, step = (uint32_t)(FOLD ? dgz : yctas);
     for (uint64_t it = first; it < items; it += step) {
         const int a0 = (int)(it & (uint32_t)(ach - 1)) * MT_EDGE;
         const uint64_t row0 = (it >> (ach - 1)) * MT_EDGE;
@@ -2135,8 +2143,9 @@ cudaError_t tt_launch_bwd_middle(tt_emb* h, cudaStream_t s)
         if (ngen > 0) {
             // very many slices fill the chip with their dG tiles, and most of them have no or few nodes: no CTAs of their own for Y
             const int64_t slices = (int64_t)h->mmaxn[k][0] * ngen;
-            const int yctas = slices >= 64 * h->sm_count ? 0 : tt_ctas_per_slice(h->sm_count, slices, ytiles);
-            if ((e = tt_launch_pdl(k_mid_tile, dim3(h->mmaxn[k][0], ngen, dgz + yctas), dim3(128), 0, st(), w, k, mlist(-1), dgz, yctas)) != cudaSuccess) return e;
+            const bool fold = slices >= 64 * h->sm_count;
+            const int yctas = fold ? 0 : tt_ctas_per_slice(h->sm_count, slices, ytiles);
+            if ((e = tt_launch_pdl(fold ? k_mid_tile<true> : k_mid_tile<false>, dim3(h->mmaxn[k][0], ngen, dgz + yctas), dim3(128), 0, st(), w, k, mlist(-1), dgz, yctas)) != cudaSuccess) return e;
             tt_note_launch();
         }
         if (fork && (e = tt_join(h, s, 4)) != cudaSuccess) return e;
