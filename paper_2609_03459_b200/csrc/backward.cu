@@ -15,7 +15,8 @@
 //             at 2.6 per clock per SM on this part, too slow for a CTA-private copy).
 //   4. middle cores: dP_{k-1} of a parent = sum over its (contiguous) children; the gradient of slice i_k
 //             = sum over the level-k nodes with that digit, enumerated by a second, digit-major bitmap sort.
-//             Each output has exactly one owner, which sums in sorted order: no atomics.
+//             Each output has exactly one owner, which sums in sorted order: no atomics.  (K = 2 has no middle
+//             cores; a first-core slice whose group is cut across work units gets its pieces by atomic additions.)
 #include "common.cuh"
 #include "scan.cuh"
 #include "mma.cuh"

@@ -72,8 +72,8 @@ struct WsView {
     int32_t T, K, D;
     int32_t ablation;                   // study switches: bit 0 no prefix reuse, bit 1 static (equal-count) schedule,
                                         // bit 2 no de-duplication (every lookup is its own row and its own group; implies bit 0)
-    int32_t equal_units;                // 1: work units of equal group counts instead of equal costs (study switch; small batches,
-                                        // whose schedule is made in one cluster without the scan of the costs)
+    int32_t equal_units;                // 1: work units of equal group counts instead of equal costs (study switch; schedules made in
+                                        // one cluster for tables swept by warps, without the scan of the costs: group_cluster.cu)
     int32_t cost_shift;                 // cost unit of the schedule = 2^cost_shift FMAs
     uint32_t many_groups;               // from this many groups on, the units of 4x4x4 and of D = 32, rank 8 hold at least 2 * TT_UNIT_GROUPS
     float fused_lr;                     // != 0: the kernels that finalise a gradient also apply G -= fused_lr * dG (cores in sgd_mask)
@@ -100,8 +100,8 @@ struct WsView {
     uint32_t* tb[TT_MAXK + 1];          // [T+1] node range of each table at level k
     uint32_t* cost;                     // [cap_{K-1}+1] exclusive scan of per-group cost (+ total)
     int64_t pool_shares;                // shares of the lookups in the pooling pass (0: it takes no shares)
-    int64_t* pool_bounds;               // [shares + 1] first bag of every share of the pooling pass (k_pool_bounds)
-    uint2* unit_rng;                    // [T * units per table] group range of every work unit (k_unit_ranges)
+    int64_t* pool_bounds;               // [shares + 1] first bag of every share of the pooling pass (tt_pool_bound)
+    uint2* unit_rng;                    // [T * units per table] group range of every work unit (tt_unit_bounds)
     int32_t units_per_table;
     float* pbuf[TT_MAXK + 1];           // partial products P_k of level-k nodes, 2 <= k <= K-2
     float* E;                           // [capU][D] rows (forward) / dE (backward)
@@ -334,7 +334,7 @@ __device__ __forceinline__ uint32_t tt_group_cost(const WsView& w, const TableDe
 }
 
 // group range (K = 2: row range) [g0, g1) of work unit q of table t: an equal-cost slice of the table's level-(K-1) groups in sweep order
-// (called by one thread per unit, once per forward: k_unit_ranges)
+// (called by one thread per unit, once per forward: k_partition, k_group_cluster)
 __device__ __forceinline__ void tt_unit_range(const WsView& w, int t, int q, uint32_t& g0, uint32_t& g1)
 {
     const TableDesc& td = w.tdesc[t];

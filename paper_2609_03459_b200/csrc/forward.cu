@@ -1,9 +1,10 @@
-// Forward path: cost-balanced schedule, prefix products, fused last-two-level contraction, bag pooling.
+// Forward path: prefix products, fused last-two-level contraction, bag pooling.
 //
 // Work is organised around the sorted prefix tree built by the grouping pass.  A "group" is a node of
 // level K-1 (a distinct (i_1..i_{K-1}) prefix); its children are the distinct rows that share it.
-//   * schedule: cost(group) = c_mid + children * c_last (FMA counts), exclusive scan, and every table is
-//     cut into `units` slices of equal cost; one CTA per unit, dispatched dynamically by the hardware.
+//   * schedule (grouping.cu, group_cluster.cu): cost(group) = c_mid + children * c_last (FMA counts), exclusive scan, and
+//     every table is cut into `units` slices of equal cost (or equal counts); one CTA per unit, dispatched dynamically by
+//     the hardware.
 //   * contraction: per group the partial product C = P_{K-2} . G_{K-1}[i_{K-1}] is formed once in shared
 //     memory (paper Sec. 3.2 "Intermediate Computation") and every child row E = C . G_K[i_K] is produced
 //     from it ("Embedding Computation"); C never goes to global memory.
@@ -733,7 +734,7 @@ __device__ __forceinline__ uint32_t tt_lookup_slot(const WsView& w, const TableD
     return slot;
 }
 
-// Pooling partition: the lookups are cut into C = W * chunks equal shares of whole bags (k_pool_bounds), and the
+// Pooling partition: the lookups are cut into C = W * chunks equal shares of whole bags (tt_pool_bound), and the
 // warps take the shares in order from a counter.  All resident warps therefore work inside one moving window of
 // about W shares at a time - a few tables - so the rows that several bags share are still in L2 when the next
 // bag asks for them; one contiguous share per warp would spread the warps over all tables at once.  Equal lookups are

@@ -178,8 +178,12 @@ cudaError_t tt_launch_grouping(tt_emb* h, cudaStream_t s)
         int64_t want = (w.L + 1023) / 1024;
         const bool fused = w.L <= TT_FUSED_INGEST;
         if (fused && want < g0) want = g0;
-        // marks of one small table meet on its popular words: fewer lookups in flight, so that more of them find the bit set
-        // (655 k lookups of one table, grouping 119 / 95 us with eight / two CTAs per SM; eight tables 108 / 112)
+        // the marks of one table meet on its few popular words: with fewer lookups in flight, more of them find the bit set.  More
+        // tables spread the same lookups over more popular words, longer batches pay for the idle SMs.  Whole call with eight / two
+        // CTAs per SM (popular rows first, exponent 1.2, unless stated): one table, 0.5 M lookups 173 / 167, 191 / 179 and 209 / 187
+        // us (1 M, 10 M, 40 M rows; spread rows 125 / 120, exponent 0.8 141 / 136 and, spread, 106 / 106), 2 M lookups 341 / 320 (exponent
+        // 0.8 211 / 215, spread 187 / 196), 10 M 1026 / 1056; two tables, 1 M lookups 206 / 187 (spread 155 / 153); three, 1.5 M 241 /
+        // 226; four, 0.8 M 162 / 160 (spread 143 / 146); eight, 1 M 171 / 172 (spread 195 / 201); sixty 232 / 236
         const int per_sm = w.T == 1 && w.L <= (1 << 20) ? 2 : 8;
         if (want > h->sm_count * per_sm) want = h->sm_count * per_sm;
         if (!fused) {
