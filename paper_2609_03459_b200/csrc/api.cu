@@ -199,7 +199,7 @@ extern "C" int tt_emb_create(const tt_emb_config_t* cfg, tt_emb_t* out_handle)
             else if (PMv == 4 && Mv == 2 && RBv == 16 && quad_ok) td.fast = 9;
             else if (PMv == 4 && Mv == 2 && RBv == 8) td.fast = 10;   // D = 16 with rank 8: FP32 pipe (slices of 16 columns)
         }
-        td.unit_groups = td.fast == 3 ? 4 * TT_UNIT_GROUPS : td.fast >= 5 && td.fast <= 9 && td.fast != 7 ? 2 * TT_UNIT_GROUPS : td.fast >= 0 ? TT_UNIT_GROUPS : TT_UNIT_GROUPS_ANY;
+        td.unit_groups = td.fast == 3 ? 4 * TT_UNIT_GROUPS : td.fast >= 0 ? TT_UNIT_GROUPS : TT_UNIT_GROUPS_ANY;
         for (int k = 0; k < TT_MAXK; ++k) td.midfast[k] = -1;
         for (int k = 2; k <= K - 1; ++k) {
             const int Mv = td.P[k - 1], rav = td.r[k - 1], colsv = td.d[k - 1] * td.r[k];
@@ -302,7 +302,7 @@ extern "C" int tt_emb_create(const tt_emb_config_t* cfg, tt_emb_t* out_handle)
         if (tot < ((unsigned __int128)1 << 31)) break;
     }
     v.cost_shift = shift;
-    v.many_groups = 2u * TT_UNIT_GROUPS * 16u * (uint32_t)h->sm_count;
+    v.paired_groups = (uint32_t)(TT_PAIRED_GROUPS * h->sm_count);
 
     // ---- workspace plan
     // every region is followed by at least 64 guard bytes (written at bind, checked on demand by tt_emb_check_guards)

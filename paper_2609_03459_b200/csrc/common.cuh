@@ -20,15 +20,18 @@
 // most lookups whose marking pass also checks the offsets: one launch less, but the tables' ranges come from all over the
 // offsets (99 M lookups, 60 tables: grouping 0.76 ms with two kernels, 0.81 ms with one; 0.5 M, 8 tables: 3 us shorter)
 #define TT_FUSED_INGEST (1 << 22)
-// fewest groups of a work unit: one batch of its four warps, i.e. 16, or 32 where the warps of both sweeps take eight groups at
-// a time (D = 32 and 16 with ranks 16 and 32; 8 tables, D = 32, rank 32, 8 M lookups with 16 / 32 / 64: forward 420 / 350 / 331 us,
-// backward 1023 / 867 / 790; one table, 0.1 M lookups of spread rows 53 / 42 / 53 and 72 / 59 / 73).  The other stacked shapes
-// have units enough at 32 where a batch has more groups than sixteen such units per SM (4x4x4, 8 tables, 8 M lookups of spread
-// rows, 16 / 32: rank 16 249 + 545 / 210 + 468, rank 32 471 + 738 / 399 + 743, rank 8 159 + 399 / 139 + 401; one table, 0.1 M
-// lookups, popular rows first, rank 32 60 + 100 / 67 + 112).  64 for D = 128, rank 32, whose warps each reuse a 32 KB slice over
-// their groups (27 k groups, forward with at least 4 / 8 / 16 / 32 / 64: 236 / 164 / 145 / 137 / 129 us); 16 for four cores, rank 64
-// (4.7 k groups, 178 / 173 / 170 / 235 with 4 / 8 / 16 / 32), and for D = 16, rank 8, whose warps take single groups
+// fewest groups of a work unit; 4x as many for D = 128, rank 32, whose warps each reuse a 32 KB slice over their groups.
+// Sweeps with at least 4 / 8 / 16 / 32 / 64 groups per unit, forward + backward, us: 8 tables x 8 k groups (rank 16) 385 / 352 /
+// 325 / 319 / 343; 4 tables x 9 k (D = 32, rank 8) 119 / 117 / 107 / 122 / 188; four cores, 4.7 k groups 178 / 173 / 170 / 235;
+// D = 128, rank 32, 27 k groups (forward) 236 / 164 / 145 / 137 / 129.
+// D = 32 and 16 with ranks 16 and 32 take eight groups per warp in both sweeps, 32 per round of a CTA's four warps.  Where the
+// groups fill the chip twice over with units of 16 (TT_PAIRED_GROUPS per SM: six such CTAs fit an SM), they get units of at
+// most 32, so that every warp has its eight (training call of 8 tables, 8 M lookups of spread rows, 180 k groups, rank 32, units
+// of 16 / 32: 1973 / 1700 us; 15 % to 18 % on 0.1 M to 8 M lookups); below, finer units balance better than full warps (33
+// tables, 12 k groups 247 / 275; 18 tables, 69 bags each 1.12 times longer with 32).  At least 32 instead of at most 32 leaves
+// units of 33 groups, whose fifth batch costs a second round (53 tables, 19 k groups, forward 282 / 334).
 #define TT_UNIT_GROUPS 16
+#define TT_PAIRED_GROUPS (2 * 6 * TT_UNIT_GROUPS)
 // ... and of the any-shape sweeps, whose CTAs take a batch of groups at a time (3x3x5, 29 k groups, forward + backward sweep
 // with at least 1 / 4 / 8 / 16 groups: 332 / 285 / 252 / 253 us; 8x8 with K = 2, 420 k lookups, whole call 1.16 ms with 8, 1.68 with 16)
 #define TT_UNIT_GROUPS_ANY 8
@@ -75,7 +78,7 @@ struct WsView {
     int32_t equal_units;                // 1: work units of equal group counts instead of equal costs (study switch; schedules made in
                                         // one cluster for tables swept by warps, without the scan of the costs: group_cluster.cu)
     int32_t cost_shift;                 // cost unit of the schedule = 2^cost_shift FMAs
-    uint32_t many_groups;               // from this many groups on, the units of 4x4x4 and of D = 32, rank 8 hold at least 2 * TT_UNIT_GROUPS
+    uint32_t paired_groups;             // from this many groups on, units of shapes with eight groups per warp hold 2 * TT_UNIT_GROUPS
     float fused_lr;                     // != 0: the kernels that finalise a gradient also apply G -= fused_lr * dG (cores in sgd_mask)
     int32_t stride[TT_MAXK + 1];        // floats per node of the level-k partial-product buffers (max over tables)
     int64_t B, L;                       // current batch / lookups
@@ -352,8 +355,8 @@ __device__ __forceinline__ void tt_unit_range(const WsView& w, int t, int q, uin
     // cut into fewer units (at least td.unit_groups groups each) and the surplus CTAs leave at once
     int Q = td.units;
     {
-        const bool many = (td.fast <= 2 || td.fast == 7) && td.fast >= 0 && w.tb[lvl][w.T] >= w.many_groups;
-        const int by_groups = (int)((b - a) / (uint32_t)(many ? 2 * TT_UNIT_GROUPS : td.unit_groups));
+        const bool pair = (td.fast == 5 || td.fast == 6 || td.fast == 8 || td.fast == 9) && w.tb[lvl][w.T] >= w.paired_groups;
+        const int by_groups = (int)(pair ? (b - a + 2 * TT_UNIT_GROUPS - 1) / (2 * TT_UNIT_GROUPS) : (b - a) / (uint32_t)td.unit_groups);
         if (Q > by_groups) Q = by_groups < 1 ? 1 : by_groups;
     }
     if (q >= Q) { g0 = a; g1 = a; return; }
