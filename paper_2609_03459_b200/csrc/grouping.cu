@@ -25,10 +25,22 @@ __global__ void __launch_bounds__(256) k_check_offsets(WsView w)
 
 // FUSED: offsets and row ids in one pass (the marks take the tables' ranges from the offsets themselves); otherwise
 // k_check_offsets has run.  The registers of eight CTAs per SM: every lookup is one or two requests and little else.
+// Bound by the requests of the lookups that find their bit not set: the lookups of a popular row that are in flight before
+// its first mark lands queue up on one word.  So a CTA marks 32 lookups, waits for them and then takes all of its share.  Grouping
+// without / with, us: one table, 0.5 M lookups (exponent 1.2, 1 M, 10 M, 40 M rows) 91 / 61, 95 / 63, 102 / 72, spread rows 67 / 47,
+// 72 / 52, 87 / 69; 8 tables, 1.6 M lookups 126 / 112; 60 tables, 99 M lookups 865 / 770.  8 / 16 / 64 / 128 lookups instead of
+// 32: 102 / 103 / 107 / 115 for 103 us (one table of 16 M rows, 0.5 M lookups).  A second test of the word past L1 before the
+// atomic (the copy in L1 is often an old one) costs more than the requests it saves: 8 tables 124 us, 60 tables 950.
+#define TT_MARK_SEEDS_FROM (1 << 16)   // 8 k lookups: call 78.5 us with them, 78.0 without
 template <bool FUSED>
 __global__ void __launch_bounds__(256, 8) k_mark(WsView w)
 {
     tt_pdl_enter();
+    // one warp's lookups first: the popular rows are marked by then, and the other warps find their bits set
+    if (w.L >= TT_MARK_SEEDS_FROM) {
+        if (threadIdx.x < 32) tt_mark_rows<!FUSED>(w, (int64_t)blockIdx.x * blockDim.x * 4 + threadIdx.x, w.L, w.L);
+        __syncthreads();
+    }
     if (FUSED) tt_check_offsets(w, (int64_t)blockIdx.x * blockDim.x + threadIdx.x, (int64_t)gridDim.x * blockDim.x);
     tt_mark_rows<!FUSED>(w, (int64_t)blockIdx.x * blockDim.x * 4 + threadIdx.x, blockDim.x, (int64_t)gridDim.x * blockDim.x * 4);
 }
@@ -178,14 +190,7 @@ cudaError_t tt_launch_grouping(tt_emb* h, cudaStream_t s)
         int64_t want = (w.L + 1023) / 1024;
         const bool fused = w.L <= TT_FUSED_INGEST;
         if (fused && want < g0) want = g0;
-        // the marks of one table meet on its few popular words: with fewer lookups in flight, more of them find the bit set.  More
-        // tables spread the same lookups over more popular words, longer batches pay for the idle SMs.  Whole call with eight / two
-        // CTAs per SM (popular rows first, exponent 1.2, unless stated): one table, 0.5 M lookups 173 / 167, 191 / 179 and 209 / 187
-        // us (1 M, 10 M, 40 M rows; spread rows 125 / 120, exponent 0.8 141 / 136 and, spread, 106 / 106), 2 M lookups 341 / 320 (exponent
-        // 0.8 211 / 215, spread 187 / 196), 10 M 1026 / 1056; two tables, 1 M lookups 206 / 187 (spread 155 / 153); three, 1.5 M 241 /
-        // 226; four, 0.8 M 162 / 160 (spread 143 / 146); eight, 1 M 171 / 172 (spread 195 / 201); sixty 232 / 236
-        const int per_sm = w.T == 1 && w.L <= (1 << 20) ? 2 : 8;
-        if (want > h->sm_count * per_sm) want = h->sm_count * per_sm;
+        if (want > h->sm_count * 8) want = h->sm_count * 8;
         if (!fused) {
             if ((e = tt_launch_pdl(k_check_offsets, dim3(g0), dim3(256), 0, s, w)) != cudaSuccess) return e;
             tt_note_launch();
