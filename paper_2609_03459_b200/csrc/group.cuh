@@ -7,6 +7,58 @@
 #include "common.cuh"
 #include "scan.cuh"
 
+// ---- shares of the pooling pass
+
+// Share ci starts with the first bag whose offset is >= L ci / C.  The pass that checks the offsets writes the boundaries as
+// it goes: bag i + 1 is the first bag of every share whose target lies in (offsets[i], offsets[i + 1]].  (A bisection of
+// the offsets per share, 15 dependent loads each, took 6 us of its step in the cluster: 8 tables, 33 k bags, 33 k shares, call 652 -> 646 us.  With
+// many bags per share the search is cheaper than two quotients per bag: 60 k shares of 2 M bags grouping and schedule 811 / 806
+// us, of 7.9 M bags 1024 / 1052.)
+
+#define TT_POOL_BAGS_PER_SHARE 64
+__device__ __forceinline__ bool tt_pool_bounds_by_bag(const WsView& w)
+{
+    return w.pool_shares > 0 && w.L > 0 && (int64_t)w.T * w.B <= TT_POOL_BAGS_PER_SHARE * w.pool_shares;
+}
+
+// first share whose target is past lookup x: the smallest ci with L ci >= C (x + 1).  C (x + 1) < 2^48 is exact in fp64, the
+// quotient is off by one at most
+__device__ __forceinline__ int64_t tt_first_share(const WsView& w, int64_t x, double invL)
+{
+    const int64_t num = w.pool_shares * (x + 1);
+    int64_t ci = (int64_t)((double)num * invL);
+    if (ci * w.L < num) ++ci;
+    else if (ci > 0 && (ci - 1) * w.L >= num) --ci;
+    return ci;
+}
+// the shares that start after bag i, 0 <= o = offsets[i] <= o_next = offsets[i + 1] <= L
+__device__ __forceinline__ void tt_pool_bounds_after(const WsView& w, int64_t i, int64_t o, int64_t o_next, double invL)
+{
+    const int64_t C = w.pool_shares, nb = (int64_t)w.T * w.B;
+    const int64_t c0 = tt_first_share(w, o, invL), c1 = i + 1 < nb ? tt_first_share(w, o_next, invL) : C;
+    for (int64_t ci = c0; ci < c1 && ci < C; ++ci) w.pool_bounds[ci] = i + 1;
+    if (i == 0)
+        for (int64_t ci = 0; ci < c0 && ci < C; ++ci) w.pool_bounds[ci] = 0;
+    if (i + 1 == nb) w.pool_bounds[C] = nb;
+}
+// otherwise, and with offsets that the check has flagged, the boundaries come from a search: the same one for both neighbours
+// of a boundary, so that the shares have no gaps whatever the offsets hold
+__device__ __forceinline__ bool tt_pool_bounds_missing(const WsView& w)
+{
+    return w.pool_shares > 0 && (!tt_pool_bounds_by_bag(w) || (__ldcg(w.status) & TT_EMB_STATUS_OFFSETS));
+}
+__device__ __forceinline__ void tt_pool_bound(const WsView& w, int64_t ci)
+{
+    const int64_t C = w.pool_shares, nb = (int64_t)w.T * w.B;
+    const int64_t target = (w.L * ci) / C;
+    int64_t lo = 0, hi = nb;
+    while (lo < hi) {
+        const int64_t mid = (lo + hi) >> 1;
+        if (__ldg(w.offsets + mid) < target) lo = mid + 1; else hi = mid;
+    }
+    w.pool_bounds[ci] = ci == 0 ? 0 : (ci == C ? nb : lo);
+}
+
 // ---- ingest
 
 // first lookup of table t, from the offsets (clamped: malformed ones set a status bit and are used as they are otherwise)
@@ -16,17 +68,31 @@ __device__ __forceinline__ int64_t tt_table_start(const WsView& w, int t)
     return o < 0 ? 0 : (o > w.L ? w.L : o);
 }
 
-// the offsets: non-decreasing, from 0 to L; first lookup of every table into tl_start.  Threads first, first + step, ..
+// the offsets: non-decreasing, from 0 to L; first lookup of every table into tl_start, boundaries of the pooling shares.  Threads
+// first, first + step, ..
 __device__ __forceinline__ void tt_check_offsets(const WsView& w, int64_t first, int64_t step)
 {
     const int64_t nb = (int64_t)w.T * w.B;
     bool bad = false;
-    for (int64_t i = first; i <= nb; i += step) {
-        const int64_t o = __ldg(w.offsets + i);
+    auto check = [&](int64_t i, int64_t o) {
         if (o < 0 || o > w.L) bad = true;
         if (i == 0 && o != 0) bad = true;
         if (i == nb && o != w.L) bad = true;
-        if (i < nb && __ldg(w.offsets + i + 1) < o) bad = true;
+    };
+    if (tt_pool_bounds_by_bag(w)) {
+        const double invL = 1.0 / (double)w.L;
+        for (int64_t i = first; i <= nb; i += step) {
+            const int64_t o = __ldg(w.offsets + i), o_next = i < nb ? __ldg(w.offsets + i + 1) : o;
+            check(i, o);
+            if (o_next < o) bad = true;
+            else if (i < nb && o >= 0 && o_next <= w.L) tt_pool_bounds_after(w, i, o, o_next, invL);
+        }
+    } else {
+        for (int64_t i = first; i <= nb; i += step) {
+            const int64_t o = __ldg(w.offsets + i);
+            check(i, o);
+            if (i < nb && __ldg(w.offsets + i + 1) < o) bad = true;
+        }
     }
     for (int64_t t = first; t <= w.T; t += step) w.tl_start[t] = tt_table_start(w, (int)t);
     if (bad) atomicOr(w.status, TT_EMB_STATUS_OFFSETS);
@@ -355,20 +421,6 @@ struct CostScan {
         w.counters[CTR_COST_TOTAL] = tot;
     }
 };
-
-// first bag of share ci: the first bag whose offset is >= L ci / C (the same search for both neighbours of a boundary,
-// whatever the offsets hold)
-__device__ __forceinline__ void tt_pool_bound(const WsView& w, int64_t ci)
-{
-    const int64_t C = w.pool_shares, nb = (int64_t)w.T * w.B;
-    const int64_t target = (w.L * ci) / C;
-    int64_t lo = 0, hi = nb;
-    while (lo < hi) {
-        const int64_t mid = (lo + hi) >> 1;
-        if (__ldg(w.offsets + mid) < target) lo = mid + 1; else hi = mid;
-    }
-    w.pool_bounds[ci] = ci == 0 ? 0 : (ci == C ? nb : lo);
-}
 
 // group range of work unit u = (table, q)
 __device__ __forceinline__ void tt_unit_bounds(const WsView& w, int u)

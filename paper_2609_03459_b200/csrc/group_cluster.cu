@@ -182,7 +182,7 @@ __global__ void __launch_bounds__(GC_THREADS) k_group_cluster(const __grid_const
         gc_scan(ls, n, sums[k], sm);
         gc_sync();
     }
-    // links of all levels in one pass over their nodes, share boundaries by the threads that come last
+    // links of all levels in one pass over their nodes, unit boundaries by the threads that come last
     uint32_t nodes = 0;
     for (int k = K - 1; k >= 1; --k) nodes += w.counters[CTR_LEVEL0 + k];
     if (first < (uint32_t)(K - 1)) tt_link_end(w, (int)first + 1);
@@ -194,7 +194,7 @@ __global__ void __launch_bounds__(GC_THREADS) k_group_cluster(const __grid_const
         if (digit_major && k == K - 1) tt_tmark_node(w, td, k, v);
         tt_link_node(w, td, k, v);
     }
-    if (w.pool_shares > 0)
+    if (tt_pool_bounds_missing(w))
         for (int64_t ci = step - 1 - first; ci <= w.pool_shares; ci += step) tt_pool_bound(w, ci);
     const int64_t units = (int64_t)w.T * w.units_per_table;
     if (w.equal_units)

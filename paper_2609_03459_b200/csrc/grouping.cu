@@ -287,7 +287,7 @@ __global__ void __launch_bounds__(128) k_partition(WsView w)
     const int64_t units = (int64_t)w.T * w.units_per_table;
     const int64_t first = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
     for (int64_t u = first; u < units; u += step) tt_unit_bounds(w, (int)u);
-    if (w.pool_shares > 0)
+    if (tt_pool_bounds_missing(w))
         for (int64_t ci = first; ci <= w.pool_shares; ci += step) tt_pool_bound(w, ci);
 }
 
