@@ -26,6 +26,7 @@
 #include "wide.cuh"
 #include "tiles.cuh"
 #include "rows.cuh"
+#include "stream.cuh"
 #include <type_traits>
 
 #define HT_SIZE 4096
@@ -1131,10 +1132,13 @@ __device__ __forceinline__ void tt_warp_rows_bwd_mma(const float* Cs, const WsVi
     const int rc = t >> 1, jc = 2 * (t & 1);  // dG C fragment: row rc of the pair, columns jc, jc+1
     for (uint32_t ub0 = u0; ub0 < u1; ub0 += 32) {
     const uint32_t ub1 = min(ub0 + 32u, u1);
+    // last digits of the 32 rows, one per lane (a load per pair put two dependent loads before every product: 240-table workload,
+    // sweep 4.47 -> 4.16 ms)
+    const uint32_t ids = ub0 + lane < u1 ? rows[ub0 + lane] - row_base : 0u;
     for (uint32_t ub = ub0; ub < ub1; ub += 2) {
         const bool two = ub + 1 < u1;
         const uint32_t ua = ub, uc = two ? ub + 1 : ub;
-        const uint32_t iKa = rows[ua] - row_base, iKc = rows[uc] - row_base;
+        const uint32_t iKa = __shfl_sync(0xffffffffu, ids, ua - ub0), iKc = __shfl_sync(0xffffffffu, ids, uc - ub0);
         const float* __restrict__ Ea = w.E + (size_t)ua * (PM * 4);
         const float* __restrict__ Ec = w.E + (size_t)uc * (PM * 4);
         // ---- loads: dE as A fragments (dC), slices as B fragments (dC), dE as B fragments (dG)
@@ -1324,6 +1328,192 @@ __device__ __forceinline__ void tt_sweep_bwd_quad(const WsView& w, const TableDe
     }
 }
 
+// The same with the rows of the batch as one stream (stream.cuh).  Per step of four rows:
+//   dC += sum_{row, j} dE[p][j] D[b][j]: k = (row, j), two k steps.  Lane t of a quad takes row t: k = t and t + 4 are j = 0, 1 in
+//         the first step and 2, 3 in the second, so that a fragment is one 16-byte load.  C of 8 or 4 rows: transposed.
+//   dG_K[i_K] += C^T . dE: n = (row, j), two tiles: n / 2 is the row (tt_stream_row), j = 2 (n % 2) + tile, so that an operand of both
+//         tiles is one 8-byte load and a lane ends up with four neighbouring floats of one slice.
+template <int PM, int RB_, int MROWS, int KTMAX, int PD>
+__device__ __forceinline__ void tt_sweep_bwd_stream(const WsView& w, const TableDesc& td, uint32_t g1, float* gk, float* Cs4,
+                                                    uint32_t* next, int lane)
+{
+    constexpr int COLS = PM / MROWS * RB_, NG = 16 / MROWS, CS = RB_ + 4;
+    constexpr bool TR = PM < 16;                  // dC transposed: M = b, N = p
+    constexpr bool KHALF = PM == 4;               // p = 4..7 of the one dG k step do not exist: zero operands
+    constexpr int MT = TR ? 1 : PM / 16, NT = RB_ / 8;
+    constexpr int MT2 = RB_ / 16, KT2 = KHALF ? 1 : PM / 8;
+    constexpr int DM = TR ? MT2 : MT, DN = TR ? 1 : NT;
+    using Stream = RowStream<PM, RB_, NG, PD>;
+    constexpr int EP = Stream::EP, DP = Stream::DP;
+    const int K = w.K, km = K - 2, g = lane >> 2, t = lane & 3;
+    const int ra = td.r[km];
+    const uint32_t nK = (uint32_t)td.n[K - 1];
+    const int rn = tt_stream_row(g >> 1), rc = tt_stream_row(t);   // dG: row of this lane's column n = g of dE; of its columns 2t, 2t + 1 of the result
+    Stream rs(w.val[K], td.core[K - 1], Cs4 + NG * PM * CS, lane);
+    uint32_t nbase = 0;
+    if (lane == 0) nbase = atomicAdd(next, (uint32_t)NG);
+    nbase = __shfl_sync(0xffffffffu, nbase, 0);
+    uint32_t gq = lane < NG && nbase + lane < g1 ? w.tnode[K - 1][nbase + lane] : 0u;   // lane k: group k of the batch
+    while (nbase < g1) {
+        const int cnt = (int)min((uint32_t)NG, g1 - nbase);
+        uint32_t valq = 0, imq = 0, u0q = 0, u1q = 0;
+        const float* srcq = nullptr;
+        if (lane < cnt) {
+            valq = w.val[K - 1][gq];
+            imq = valq % (uint32_t)td.n[km];
+            srcq = tt_left_operand(w, td, K - 1, gq);
+            u0q = w.cstart[K - 1][gq];
+            u1q = w.cstart[K - 1][gq + 1];
+        }
+        rs.begin(gq, u0q, u1q, valq * nK, lane);
+        tt_quad_mid<COLS, MROWS, KTMAX, RB_>(td.core[km], td.slice_floats[km], ra, cnt, imq, srcq, Cs4, lane, [&]() { rs.fill(w.E, lane); });
+        if (lane == 0) nbase = atomicAdd(next, (uint32_t)NG);
+        nbase = __shfl_sync(0xffffffffu, nbase, 0);
+        gq = lane < NG && nbase + lane < g1 ? w.tnode[K - 1][nbase + lane] : 0u;   // the next batch
+        __syncwarp();
+        Tf32Pair ct[MT2][KT2][4];   // A[m = b][k = p] = C[p][b] of the current group
+        float dc[DM][DN][4];
+        uint32_t cur = 0xffffffffu, chain = 0;
+        bool folded = false;
+        // dC of the group so far to dP (a chain of the tensor core's truncating additions ends here: the sum goes on in rounded fp32)
+        auto hand_over = [&](uint32_t q) {
+            float* dst = w.dP[K - 1] + (size_t)rs.groups()[32 + q] * w.stride[K - 1];
+            if constexpr (TR) {
+                if (2 * t < PM) {
+#pragma unroll
+                    for (int mt = 0; mt < DM; ++mt)
+#pragma unroll
+                        for (int x = 0; x < 4; ++x) {
+                            float* d = dst + (2 * t + (x & 1)) * RB_ + 16 * mt + g + 8 * (x >> 1);
+                            *d = folded ? *d + dc[mt][0][x] : dc[mt][0][x];
+                        }
+                }
+            } else {
+#pragma unroll
+                for (int mt = 0; mt < DM; ++mt)
+#pragma unroll
+                    for (int nt = 0; nt < DN; ++nt)
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            float2* d = reinterpret_cast<float2*>(dst + (16 * mt + 8 * h + g) * RB_ + 8 * nt + 2 * t);
+                            float2 v = make_float2(dc[mt][nt][2 * h], dc[mt][nt][2 * h + 1]);
+                            if (folded) { const float2 o = *d; v.x += o.x; v.y += o.y; }
+                            *d = v;
+                        }
+            }
+#pragma unroll
+            for (int mt = 0; mt < DM; ++mt)
+#pragma unroll
+                for (int nt = 0; nt < DN; ++nt)
+#pragma unroll
+                    for (int x = 0; x < 4; ++x) dc[mt][nt][x] = 0.f;
+            chain = 0;
+        };
+#pragma unroll
+        for (int mt = 0; mt < DM; ++mt)
+#pragma unroll
+            for (int nt = 0; nt < DN; ++nt)
+#pragma unroll
+                for (int x = 0; x < 4; ++x) dc[mt][nt][x] = 0.f;
+#pragma unroll 1
+        for (int q = 0; q < cnt; ++q)   // groups without rows (dropped at the row capacity)
+            if (rs.groups()[8 + q] == rs.groups()[16 + q]) hand_over(q);
+        int slot = 0;
+#pragma unroll 1
+        for (uint32_t s = 0; s <= rs.steps; ++s) {
+            const uint32_t qn = s < rs.steps ? *rs.group_rows(s) : 0xffu, q = qn & 255u, nr = qn >> 8;
+            if (q != cur || chain >= 16) {
+                if (cur != 0xffffffffu) hand_over(cur);
+                if (s == rs.steps) break;
+                folded = q == cur;
+                if (q != cur) {
+                    cur = q;
+                    const float* Cs = Cs4 + q * (PM * CS);
+#pragma unroll
+                    for (int mt = 0; mt < MT2; ++mt)
+#pragma unroll
+                        for (int kt = 0; kt < KT2; ++kt) {
+                            ct[mt][kt][0] = tt_split_tf32(Cs[(8 * kt + t) * CS + 16 * mt + g]);
+                            ct[mt][kt][1] = tt_split_tf32(Cs[(8 * kt + t) * CS + 16 * mt + g + 8]);
+                            ct[mt][kt][2] = tt_split_tf32(KHALF ? 0.f : Cs[(8 * kt + t + 4) * CS + 16 * mt + g]);
+                            ct[mt][kt][3] = tt_split_tf32(KHALF ? 0.f : Cs[(8 * kt + t + 4) * CS + 16 * mt + g + 8]);
+                        }
+                }
+            }
+            const float* st = rs.wait(slot);
+            // ---- dG_K[i_K] += C^T . dE
+            float acc[2][MT2][4];
+#pragma unroll
+            for (int tile = 0; tile < 2; ++tile)
+#pragma unroll
+                for (int mt = 0; mt < MT2; ++mt)
+#pragma unroll
+                    for (int x = 0; x < 4; ++x) acc[tile][mt][x] = 0.f;
+            const float* El = st + rn * EP + 4 * t + 2 * (g & 1);
+#pragma unroll
+            for (int kt = 0; kt < KT2; ++kt) {
+                const float2 e0 = *reinterpret_cast<const float2*>(El + 32 * kt);
+                const float2 e1 = KHALF ? make_float2(0.f, 0.f) : *reinterpret_cast<const float2*>(El + 32 * kt + 16);
+                const Tf32Pair b0[2] = {tt_split_tf32(e0.x), tt_split_tf32(e1.x)}, b1[2] = {tt_split_tf32(e0.y), tt_split_tf32(e1.y)};
+#pragma unroll
+                for (int mt = 0; mt < MT2; ++mt) {
+                    tt_mma_3xtf32(acc[0][mt], ct[mt][kt], b0);
+                    tt_mma_3xtf32(acc[1][mt], ct[mt][kt], b1);
+                }
+            }
+            // ---- dC += dE . D^T
+            const float* Et = st + t * EP + 4 * g;
+            const float* Dt = st + 4 * EP + t * DP + 4 * g;
+            auto split4 = [](Tf32Pair (&d)[4], const float4& v) { d[0] = tt_split_tf32(v.x); d[1] = tt_split_tf32(v.y); d[2] = tt_split_tf32(v.z); d[3] = tt_split_tf32(v.w); };
+            if constexpr (TR) {
+                Tf32Pair e[4];   // dE[p = g] of row t, j = 0..3
+                split4(e, PM == 8 || g < PM ? *reinterpret_cast<const float4*>(Et) : make_float4(0.f, 0.f, 0.f, 0.f));
+                const Tf32Pair b0[2] = {e[0], e[1]}, b1[2] = {e[2], e[3]};
+#pragma unroll
+                for (int mt = 0; mt < MT2; ++mt) {
+                    Tf32Pair x[4], y[4];
+                    split4(x, *reinterpret_cast<const float4*>(Dt + 64 * mt));
+                    split4(y, *reinterpret_cast<const float4*>(Dt + 64 * mt + 32));
+                    const Tf32Pair a0[4] = {x[0], y[0], x[1], y[1]}, a1[4] = {x[2], y[2], x[3], y[3]};
+                    tt_mma_3xtf32(dc[mt][0], a0, b0);
+                    tt_mma_3xtf32(dc[mt][0], a1, b1);
+                }
+            } else {
+#pragma unroll
+                for (int mt = 0; mt < MT; ++mt) {
+                    Tf32Pair x[4], y[4];
+                    split4(x, *reinterpret_cast<const float4*>(Et + 64 * mt));
+                    split4(y, *reinterpret_cast<const float4*>(Et + 64 * mt + 32));
+                    const Tf32Pair a0[4] = {x[0], y[0], x[1], y[1]}, a1[4] = {x[2], y[2], x[3], y[3]};
+#pragma unroll
+                    for (int nt = 0; nt < NT; ++nt) {
+                        Tf32Pair d[4];
+                        split4(d, *reinterpret_cast<const float4*>(Dt + 32 * nt));
+                        const Tf32Pair b0[2] = {d[0], d[1]}, b1[2] = {d[2], d[3]};
+                        tt_mma_3xtf32(dc[mt][nt], a0, b0);
+                        tt_mma_3xtf32(dc[mt][nt], a1, b1);
+                    }
+                }
+            }
+            float* dst = gk + (size_t)rs.ids(s)[rc] * (RB_ * 4) + 4 * g;
+#pragma unroll
+            for (int mt = 0; mt < MT2; ++mt)
+#pragma unroll
+                for (int h = 0; h < 2; ++h)
+                    tt_red_v4_if((uint32_t)rc < nr, dst + (16 * mt + 8 * h) * 4, acc[0][mt][2 * h], acc[1][mt][2 * h], acc[0][mt][2 * h + 1], acc[1][mt][2 * h + 1]);
+            chain += 2;
+            __syncwarp();
+            rs.stage(slot, w.E, lane);
+            slot = slot + 1 == PD ? 0 : slot + 1;
+        }
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        __syncwarp();
+    }
+}
+#define BWD_RING 2   // steps in a warp's ring
+template <int PM, int RB_, int MROWS>
+struct BwdStream { static constexpr int FLOATS = 16 / MROWS * PM * (RB_ + 4) + RowStream<PM, RB_, 16 / MROWS, BWD_RING>::FLOATS; };   // per warp
+
 // rank-64 four-core shape (wide.cuh).  dG_K: a warp takes one row, a lane two values of b over the 32 rows of C and dE.  dC (32 x
 // 64) = sum over the group's rows of dE . D^T: two warps per group, half the columns each, as 3xTF32 tiles whose k is two rows
 // by four columns, every pair of rows added in rounded fp32 (a group has up to n_K rows).
@@ -1418,7 +1608,7 @@ __global__ void __launch_bounds__(WIDE_THREADS, 2) k_sweep_bwd_wide(WsView w, in
 // One CTA (4 warps) per work unit (table, q); last-core gradients go to one of TT_STRIPES L2-resident partial
 // copies with vector reductions, added up in fixed stripe order by k_reduce_gpart.
 template <int V>
-__global__ void __launch_bounds__(128, (V == 5 || V == 6 || V == 8 || V == 9 || V == 1) ? 6 : 0) k_sweep_bwd(WsView w, int pl_floats, int c_floats, int vbase)
+__global__ void __launch_bounds__(128, V == 5 ? 6 : V == 1 || V == 8 ? 4 : V == 6 || V == 9 ? 5 : 0) k_sweep_bwd(WsView w, int pl_floats, int c_floats, int vbase)
 {
     tt_pdl_enter();
     extern __shared__ __align__(16) float sm[];
@@ -1435,14 +1625,14 @@ __global__ void __launch_bounds__(128, (V == 5 || V == 6 || V == 8 || V == 9 || 
     float* As = sm + (size_t)wid * (pl_floats + c_floats);
     float* Cs = As + pl_floats;
     if (V == 0) tt_sweep_bwd_fast<16, 32, 4, 4, 1, true>(w, td, g1, gk, As, Cs, &next, lane);
-    if (V == 1) tt_sweep_bwd_quad<16, 16, 4, 4>(w, td, g1, gk, sm + (size_t)wid * (4 * 16 * 20), &next, lane);
+    if (V == 1) tt_sweep_bwd_stream<16, 16, 4, 4, BWD_RING>(w, td, g1, gk, sm + wid * BwdStream<16, 16, 4>::FLOATS, &next, lane);
     if (V == 2) tt_sweep_bwd_fast<16, 8, 4, 4, 1, true>(w, td, g1, gk, As, Cs, &next, lane);
     if (V == 3) tt_sweep_bwd_fast<32, 32, 4, 4, 2, true>(w, td, g1, gk, As, Cs, &next, lane);
     if (V == 5) tt_sweep_bwd_quad<8, 32, 2, 4>(w, td, g1, gk, sm + (size_t)wid * (8 * 8 * 36), &next, lane);
-    if (V == 6) tt_sweep_bwd_quad<8, 16, 2, 4>(w, td, g1, gk, sm + (size_t)wid * (8 * 8 * 20), &next, lane);
+    if (V == 6) tt_sweep_bwd_stream<8, 16, 2, 4, BWD_RING>(w, td, g1, gk, sm + wid * BwdStream<8, 16, 2>::FLOATS, &next, lane);
     if (V == 7) tt_sweep_bwd_fast<8, 8, 2, 2, 1, false>(w, td, g1, gk, As, Cs, &next, lane);   // 8 x 8: the FP32 pipe wins (0.39 against 0.41 ms)
-    if (V == 8) tt_sweep_bwd_quad<4, 32, 2, 4>(w, td, g1, gk, sm + (size_t)wid * (8 * 4 * 36), &next, lane);
-    if (V == 9) tt_sweep_bwd_quad<4, 16, 2, 4>(w, td, g1, gk, sm + (size_t)wid * (8 * 4 * 20), &next, lane);
+    if (V == 8) tt_sweep_bwd_stream<4, 32, 2, 4, BWD_RING>(w, td, g1, gk, sm + wid * BwdStream<4, 32, 2>::FLOATS, &next, lane);
+    if (V == 9) tt_sweep_bwd_stream<4, 16, 2, 4, BWD_RING>(w, td, g1, gk, sm + wid * BwdStream<4, 16, 2>::FLOATS, &next, lane);
     if (V == 10) tt_sweep_bwd_fast<4, 8, 2, 2, 1, false>(w, td, g1, gk, As, Cs, &next, lane);
 }
 
@@ -1471,19 +1661,14 @@ static cudaError_t launch_sweep_bwd(tt_emb* h, int max_pl, int max_c, cudaStream
     if (n == 0) return cudaSuccess;
     // tensor-core variants keep C with padded rows (stride r_{K-1} + 8 floats)
     if (V == 0) max_c = 16 * (32 + 8);
-    if (V == 1) max_c = 16 * (16 + 8);
     if (V == 2) max_c = 16 * (8 + 8);
     if (V == 3) max_c = 32 * (32 + 8);
-    if (V == 5) max_c = 8 * (32 + 8);
-    if (V == 6) max_c = 8 * (16 + 8);
-    if (V == 8) max_c = 4 * (32 + 8);
-    if (V == 9) max_c = 4 * (16 + 8);
     size_t smem = (size_t)4 * (max_pl + max_c) * sizeof(float);
     if (V == 5) smem = (size_t)4 * 8 * 8 * 36 * sizeof(float);    // eight C tiles per warp, rows padded by four floats
-    if (V == 6) smem = (size_t)4 * 8 * 8 * 20 * sizeof(float);
-    if (V == 8) smem = (size_t)4 * 8 * 4 * 36 * sizeof(float);
-    if (V == 9) smem = (size_t)4 * 8 * 4 * 20 * sizeof(float);
-    if (V == 1) smem = (size_t)4 * 4 * 16 * 20 * sizeof(float);   // four C tiles per warp
+    if (V == 6) smem = (size_t)4 * BwdStream<8, 16, 2>::FLOATS * sizeof(float);
+    if (V == 8) smem = (size_t)4 * BwdStream<4, 32, 2>::FLOATS * sizeof(float);
+    if (V == 9) smem = (size_t)4 * BwdStream<4, 16, 2>::FLOATS * sizeof(float);
+    if (V == 1) smem = (size_t)4 * BwdStream<16, 16, 4>::FLOATS * sizeof(float);
     cudaError_t e;
     if ((e = tt_stage_begin(h, 9 + TT_NUM_VARIANTS + 1 + V + 1, s)) != cudaSuccess) return e;
     if constexpr (V < 0) {

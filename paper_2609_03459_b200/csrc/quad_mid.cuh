@@ -11,6 +11,10 @@
 #pragma once
 #include "mma.cuh"
 
+// `hook` runs once per batch after its first block of columns: loads that the caller has under way by then are waited for
+// under the products of the other blocks.
+struct QuadNothing { __device__ __forceinline__ void operator()() const {} };
+
 // One pass.  Lane (g = lane / 4, t = lane % 4) feeds rows g and g + 8 of the stacked operand: row g belongs to group
 // g / MROWS (source srcA, taken when selA), row g + 8 to group (8 + g) / MROWS (srcB, selB); m = g % MROWS is the row
 // of P inside the group.  src points at P (MROWS x ra, row-major).  ra <= 8 * KTMAX, any value (the k range is padded
@@ -20,9 +24,9 @@
 // Column mapping: a block of 32 columns is one float4 load per lane and k row (8 lanes x 16 bytes = 128 bytes per
 // row); tile j of the block takes component j, i.e. tile column n' stands for slice column 32 * block + 4 n' + j, so
 // that a lane ends up with 8 consecutive columns of each of its two rows (two float4 stores per row).
-template <int COLS, int MROWS, int KTMAX, int RB>
+template <int COLS, int MROWS, int KTMAX, int RB, class Hook>
 __device__ __forceinline__ void tt_quad_mid_mma(const float* __restrict__ B, int ra, const float* __restrict__ srcA,
-                                                const float* __restrict__ srcB, bool selA, bool selB, float* Cs4, int lane)
+                                                const float* __restrict__ srcB, bool selA, bool selB, float* Cs4, int lane, Hook& hook)
 {
     static_assert((MROWS == 2 || MROWS == 4) && KTMAX % 2 == 0, "stacking of 8 or 4 groups");
     const int g = lane >> 2, t = lane & 3, m = g & (MROWS - 1);
@@ -81,6 +85,7 @@ __device__ __forceinline__ void tt_quad_mid_mma(const float* __restrict__ B, int
                 }
             }
         }
+        if (nb == 0) hook();
         if (selA) {
             *reinterpret_cast<float4*>(dstA + coff(nb)) = make_float4(acc[0][0], acc[1][0], acc[2][0], acc[3][0]);
             *reinterpret_cast<float4*>(dstA + coff(nb) + 4) = make_float4(acc[0][1], acc[1][1], acc[2][1], acc[3][1]);
@@ -94,10 +99,12 @@ __device__ __forceinline__ void tt_quad_mid_mma(const float* __restrict__ B, int
 
 // All passes of one batch of cnt <= 16 / MROWS groups.  Lane q < cnt holds group q's slice index (imq) and operand
 // pointer (srcq).
-template <int COLS, int MROWS, int KTMAX, int RB>
+template <int COLS, int MROWS, int KTMAX, int RB, class Hook = QuadNothing>
 __device__ __forceinline__ void tt_quad_mid(const float* __restrict__ core_mid, size_t slice_floats, int ra, int cnt, uint32_t imq,
-                                            const float* srcq, float* Cs4, int lane)
+                                            const float* srcq, float* Cs4, int lane, Hook hook = Hook())
 {
+    bool pending = true;
+    auto once = [&]() { if (pending) hook(); pending = false; };
     const int g = lane >> 2;
     const int qA = g / MROWS, qB = (8 + g) / MROWS;
     const unsigned long long sp = (unsigned long long)reinterpret_cast<uintptr_t>(srcq);
@@ -109,7 +116,7 @@ __device__ __forceinline__ void tt_quad_mid(const float* __restrict__ core_mid, 
         const uint32_t im = __shfl_sync(0xffffffffu, imq, first);
         const unsigned sel = __ballot_sync(0xffffffffu, lane < 16 / MROWS && ((remaining >> lane) & 1u) && imq == im) & ((1u << (16 / MROWS)) - 1u);
         const bool selA = (sel >> qA) & 1u, selB = (sel >> qB) & 1u;
-        tt_quad_mid_mma<COLS, MROWS, KTMAX, RB>(core_mid + (size_t)im * slice_floats, ra, srcA, srcB, selA, selB, Cs4, lane);
+        tt_quad_mid_mma<COLS, MROWS, KTMAX, RB>(core_mid + (size_t)im * slice_floats, ra, srcA, srcB, selA, selB, Cs4, lane, once);
         remaining &= ~sel;
     }
 }

@@ -1,0 +1,76 @@
+"""Backward sweeps that stream the rows of a batch of groups (ranks 16 with C of 16, 8 and 4 rows, rank 32 with C of 4 rows):
+groups of 1 to 5 rows (a step holds four), around 32 rows (a block of steps, where sums of dC are handed over) and of several
+hundred rows, in ranks that are no multiple of eight before them, three and four cores, and rows dropped at the row capacity.
+
+Bar: max|err| <= 1e-5 * max|ref|, the bound of the other parity tests (fp32 sums, 3xTF32 products)."""
+import numpy as np
+import pytest
+
+import oracle
+import workloads
+from test_gpu_parity import assert_close, binding, dev  # noqa: F401  (binding: fixture)
+from workloads import TableSpec
+
+pytestmark = pytest.mark.gpu
+
+SHAPES = [((4, 4, 4), (16, 16)), ((4, 4, 4), (5, 16)), ((2, 4, 4), (16, 16)), ((2, 4, 4), (3, 16)), ((2, 2, 4), (32, 32)), ((2, 2, 4), (16, 16))]
+
+
+def ids_with_groups(n, sizes, rng):
+    """Row ids whose length-2 prefixes hold sizes[i % len] rows each."""
+    rows = []
+    for i, p in enumerate(rng.permutation(n[0] * n[1])):
+        rows.append(p * n[2] + rng.choice(n[2], min(sizes[i % len(sizes)], n[2]), replace=False))
+    return np.concatenate(rows)
+
+
+@pytest.mark.parametrize("d,r", SHAPES)
+@pytest.mark.parametrize("n,sizes", [((3, 7, 9), (1, 2, 3, 4, 5)), ((2, 9, 140), (31, 32, 33, 1, 35, 64, 128, 140)), ((1, 1, 700), (700,)), ((37, 5, 6), (1, 6))])
+def test_gradients(binding, d, r, n, sizes):  # noqa: F811
+    spec = TableSpec(N=int(np.prod(n)), n=n, d=d, r=(1,) + r + (1,), alpha=1.0, core_dist="normal", core_scale=0.3)
+    rng = np.random.default_rng(len(sizes) + n[2])
+    T, B = 2, 50
+    wl = workloads.custom([spec] * T, B, 1, seed=1, with_grad=True)
+    per_table = [np.concatenate([x, rng.choice(x, 40)]) for x in (ids_with_groups(n, sizes, rng) for _ in range(T))]
+    per_table = [rng.permutation(x) for x in per_table]
+    wl.indices = np.concatenate(per_table).astype(np.int64)
+    cuts, at = [], 0
+    for x in per_table:
+        cuts += [at + c for c in [0] + sorted(rng.integers(0, len(x) + 1, B - 1).tolist())]
+        at += len(x)
+    wl.offsets = np.array(cuts + [at], dtype=np.int64)
+    emb = binding.from_workload(wl, enable_backward=True)
+    assert emb.table_variant(0) >= 0
+    ref = oracle.backward_workload(wl)
+    for rep in range(2):
+        out = emb.forward(dev(wl.indices), dev(wl.offsets), B)
+        assert_close(out.cpu().numpy(), oracle.forward_workload(wl), "out")
+        emb.backward(dev(wl.grad_out))
+        grads = emb.get_grads()
+        for t in range(T):
+            for k in range(3):
+                assert_close(grads[t][k], ref[t][k], f"dG[{t}][{k}]")
+    assert emb.status() == 0 and emb.check_guards() is None
+
+
+@pytest.mark.parametrize("d,r", SHAPES)
+def test_rows_dropped_at_the_capacity(binding, d, r):  # noqa: F811
+    # the last groups keep some or none of their rows; what is left is the gradient of the rows that were kept
+    n = (6, 8, 40)
+    spec = TableSpec(N=1920, n=n, d=d, r=(1,) + r + (1,), alpha=1.0, core_dist="normal", core_scale=0.3)
+    wl = workloads.custom([spec], 60, 12, seed=4, with_grad=True)
+    rng = np.random.default_rng(2)
+    wl.indices = rng.integers(0, 1920, wl.L).astype(np.int64)
+    kept = np.unique(wl.indices)[:301]
+    emb = binding.from_workload(wl, enable_backward=True, max_unique_rows=301)
+    emb.forward(dev(wl.indices), dev(wl.offsets), 60)
+    assert emb.status() == binding.STATUS_OVERFLOW
+    emb.backward(dev(wl.grad_out))
+    grads = emb.get_grads()
+    keep = np.isin(wl.indices, kept)
+    wl.offsets = np.concatenate([[0], np.cumsum(keep)])[wl.offsets].astype(np.int64)
+    wl.indices = wl.indices[keep]
+    ref = oracle.backward_workload(wl)
+    for k in range(3):
+        assert_close(grads[0][k], ref[0][k], f"dG[0][{k}]")
+    assert emb.check_guards() is None
