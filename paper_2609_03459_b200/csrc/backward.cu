@@ -509,15 +509,22 @@ __global__ void __launch_bounds__(256, 5) k_dE_fast(WsView w, const float* __res
 // order owning two of the 64 columns: one shared-memory load and two adds per row, a coalesced 256-byte store when a
 // segment ends, and no shuffles to combine partial sums.  About half the instructions per lookup of k_dE_fast, which
 // was bound by instruction issue.  Chunks, carries and the fix-up pass are those of k_dE / k_dE_fast.
+#define DE_ODD_MOST 61   // with the up to three floats before it, a row fits sixteen pieces
 #define DE_WARPS 7   // 4 CTAs x 7 warps x 8 KB of staging per SM
-template <int DD, bool WT>   // DD = D: 64 (two columns per lane), 32 (one) or 16 (one, lanes 0..15)
-__global__ void __launch_bounds__(32 * DE_WARPS, 4) k_dE_stage(WsView w, const float* __restrict__ grad_out)
+// DD = 128: rows of 512 bytes, two CTAs per SM (65 k lookups: dE with its fix-up 38 -> 29 us against k_dE_fast).
+// DD = 0: rows of any other length up to 61 floats.  A row starts anywhere in its first 16-byte piece; the pieces that it touches
+// are staged as they lie (the last ones of grad_out cut to its end), and a lane picks columns lane and lane + 32 behind the row's
+// shift.  1 M lookups of 45 floats: 112 -> 84 us against k_dE.
+template <int DD, bool WT>   // DD = D: 128 (four columns per lane), 64 (two), 32 (one), 16 (one, lanes 0..15) or 0
+__global__ void __launch_bounds__(32 * DE_WARPS, DD == 128 ? 2 : 4) k_dE_stage(WsView w, const float* __restrict__ grad_out)
 {
     tt_pdl_enter();
-    static_assert(DD == 64 || DD == 32 || DD == 16, "a lane owns DD / 32 columns (one column on the first DD lanes below 32)");
-    constexpr int R4 = DD / 4;          // float4 pieces per row
-    constexpr int RPI = 32 / R4;        // rows per cp.async instruction
-    constexpr int VPL = DD >= 32 ? DD / 32 : 1;   // columns per lane
+    static_assert(DD == 128 || DD == 64 || DD == 32 || DD == 16 || DD == 0, "a lane owns DD / 32 columns (one column on the first DD lanes below 32)");
+    constexpr bool ODD = DD == 0;
+    constexpr int R4 = ODD ? 16 : DD / 4;         // float4 pieces per staged row
+    constexpr int RPI = 32 / R4;                  // rows per cp.async instruction
+    constexpr int VPL = ODD ? 2 : DD >= 32 ? DD / 32 : 1;   // columns per lane
+    const int D = ODD ? w.D : DD;
     extern __shared__ __align__(16) float4 de_buf[];   // [DE_WARPS][32 rows][R4 float4]
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, sub = lane / R4, lr = lane % R4;
     float4* buf = de_buf + (size_t)wid * 32 * R4;
@@ -532,7 +539,7 @@ __global__ void __launch_bounds__(32 * DE_WARPS, 4) k_dE_stage(WsView w, const f
     const uint32_t prev = a > 0 ? w.pairs[a - 1].x : HT_EMPTY;
     const uint32_t next = b < Ltot ? w.pairs[b].x : HT_EMPTY;
     const float4* __restrict__ G4 = reinterpret_cast<const float4*>(grad_out);
-    float* carry = w.carry + (size_t)chunk * 2 * DD;
+    float* carry = w.carry + (size_t)chunk * 2 * D;
     const uint32_t* __restrict__ tbK = w.tb[w.K];
     float acc[VPL], part[VPL];
 #pragma unroll
@@ -546,11 +553,17 @@ __global__ void __launch_bounds__(32 * DE_WARPS, 4) k_dE_stage(WsView w, const f
     // two-level sum: rows are added into a per-batch partial (at most 32 terms) which is added to the segment's sum at
     // the end of the batch, so the rounding error of a long segment grows with sqrt(length / 32), not sqrt(length)
     auto store_row = [&](float* dst, bool with_part) {
-        if (VPL == 2) reinterpret_cast<float2*>(dst)[lane] = make_float2(acc[0] + (with_part ? part[0] : 0.f), acc[VPL - 1] + (with_part ? part[VPL - 1] : 0.f));
+        if (ODD) {
+            if (lane < D) dst[lane] = acc[0] + (with_part ? part[0] : 0.f);
+            if (lane + 32 < D) dst[lane + 32] = acc[VPL - 1] + (with_part ? part[VPL - 1] : 0.f);
+        } else if (VPL == 4)
+            reinterpret_cast<float4*>(dst)[lane] = make_float4(acc[0] + (with_part ? part[0] : 0.f), acc[1 % VPL] + (with_part ? part[1 % VPL] : 0.f),
+                                                               acc[2 % VPL] + (with_part ? part[2 % VPL] : 0.f), acc[VPL - 1] + (with_part ? part[VPL - 1] : 0.f));
+        else if (VPL == 2) reinterpret_cast<float2*>(dst)[lane] = make_float2(acc[0] + (with_part ? part[0] : 0.f), acc[VPL - 1] + (with_part ? part[VPL - 1] : 0.f));
         else if (lane < DD) dst[lane] = acc[0] + (with_part ? part[0] : 0.f);
     };
     auto close_segment = [&]() {
-        store_row((seg_first && prev == cur) ? carry : w.E + (size_t)cur * DD, true);   // head piece or whole segment
+        store_row((seg_first && prev == cur) ? carry : w.E + (size_t)cur * D, true);   // head piece or whole segment
 #pragma unroll
         for (int x = 0; x < VPL; ++x) { acc[x] = 0.f; part[x] = 0.f; }
         seg_first = false;
@@ -571,7 +584,17 @@ __global__ void __launch_bounds__(32 * DE_WARPS, 4) k_dE_stage(WsView w, const f
         if (lane == 0) before = last_slot;
         const unsigned starts = __ballot_sync(0xffffffffu, lane < n && mine.x != before);   // bit j: position j opens a segment
         last_slot = __shfl_sync(0xffffffffu, mine.x, n - 1);
-        if (n == 32) {   // all windows of a chunk but its last: no per-row test
+        const uint32_t shift = (grow * (uint32_t)D) & 3u;   // (ODD) floats before the row in its first piece
+        if constexpr (ODD) {
+            const uint64_t all = (uint64_t)w.B * w.T * D;
+#pragma unroll 4
+            for (int jj = 0; jj < 32 / RPI; ++jj) {
+                if (RPI * jj >= n) break;
+                const int j = RPI * jj + sub;
+                const uint64_t start = (uint64_t)__shfl_sync(0xffffffffu, grow, j) * (uint32_t)D, at = (start & ~(uint64_t)3) + 4 * lr;
+                if (j < n && at < start + D) tt_cp_async16_cut(buf + j * R4 + lr, grad_out + at, all - at);
+            }
+        } else if (n == 32) {   // all windows of a chunk but its last: no per-row test
 #pragma unroll
             for (int jj = 0; jj < 32 / RPI; ++jj) {
                 const int j = RPI * jj + sub;
@@ -598,7 +621,14 @@ __global__ void __launch_bounds__(32 * DE_WARPS, 4) k_dE_stage(WsView w, const f
         __syncwarp();
         auto add_row = [&](int j) {
             float x[VPL];
-            if (VPL == 2) {
+            if (ODD) {
+                const float* src = bufv + j * 64 + __shfl_sync(0xffffffffu, shift, j) + lane;
+                x[0] = lane < D ? src[0] : 0.f;
+                x[VPL - 1] = lane + 32 < D ? src[32] : 0.f;
+            } else if (VPL == 4) {
+                const float4 v = buf[j * 32 + lane];
+                x[0] = v.x; x[1 % VPL] = v.y; x[2 % VPL] = v.z; x[VPL - 1] = v.w;
+            } else if (VPL == 2) {
                 const float2 v = reinterpret_cast<const float2*>(bufv)[j * 32 + lane];
                 x[0] = v.x; x[VPL - 1] = v.y;
             } else x[0] = bufv[j * DD + (lane & (DD - 1))];
@@ -624,8 +654,12 @@ __global__ void __launch_bounds__(32 * DE_WARPS, 4) k_dE_stage(WsView w, const f
                 for (int jj = 0; jj < 7; ++jj) {
                     const uint32_t sj = __shfl_sync(0xffffffffu, cur_pairs.x, j0 + jj);
                     add_row(j0 + jj);
-                    float* dst = w.E + (size_t)sj * DD;
-                    if (VPL == 2) reinterpret_cast<float2*>(dst)[lane] = make_float2(part[0], part[VPL - 1]);
+                    float* dst = w.E + (size_t)sj * D;
+                    if (ODD) {
+                        if (lane < D) dst[lane] = part[0];
+                        if (lane + 32 < D) dst[lane + 32] = part[VPL - 1];
+                    } else if (VPL == 4) reinterpret_cast<float4*>(dst)[lane] = make_float4(part[0], part[1 % VPL], part[2 % VPL], part[VPL - 1]);
+                    else if (VPL == 2) reinterpret_cast<float2*>(dst)[lane] = make_float2(part[0], part[VPL - 1]);
                     else if (lane < DD) dst[lane] = part[0];
 #pragma unroll
                     for (int c = 0; c < VPL; ++c) part[c] = 0.f;
@@ -649,7 +683,7 @@ __global__ void __launch_bounds__(32 * DE_WARPS, 4) k_dE_stage(WsView w, const f
     }
     {   // last segment of the chunk: tail / head / whole
         const bool open_start = seg_first && prev == cur;
-        store_row(next == cur ? carry + DD : (open_start ? carry : w.E + (size_t)cur * DD), false);
+        store_row(next == cur ? carry + D : (open_start ? carry : w.E + (size_t)cur * D), false);
     }
 }
 
@@ -681,9 +715,12 @@ static cudaError_t launch_dE_t(tt_emb* h, const float* grad_out, cudaStream_t s)
     if (grid > 0) {
         const int D4 = h->D / 4;
         const bool wt = h->v.wsorted && (h->v.psw || h->v.pool_mean);
-        if (VEC && (h->D == 64 || h->D == 32 || h->D == 16)) {
-            const size_t smem = (size_t)DE_WARPS * 32 * (h->D / 4) * sizeof(float4);
-            auto kern = h->D == 64 ? (wt ? k_dE_stage<64, true> : k_dE_stage<64, false>)
+        const bool odd = !VEC && h->D <= DE_ODD_MOST && (reinterpret_cast<uintptr_t>(grad_out) & 15) == 0;
+        if (odd || (VEC && (h->D == 128 || h->D == 64 || h->D == 32 || h->D == 16))) {
+            const size_t smem = (size_t)DE_WARPS * 32 * (odd ? 16 : h->D / 4) * sizeof(float4);
+            auto kern = odd ? (wt ? k_dE_stage<0, true> : k_dE_stage<0, false>)
+                      : h->D == 128 ? (wt ? k_dE_stage<128, true> : k_dE_stage<128, false>)
+                      : h->D == 64 ? (wt ? k_dE_stage<64, true> : k_dE_stage<64, false>)
                       : h->D == 32 ? (wt ? k_dE_stage<32, true> : k_dE_stage<32, false>) : (wt ? k_dE_stage<16, true> : k_dE_stage<16, false>);
             cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             if (e != cudaSuccess) return e;

@@ -312,6 +312,13 @@ __device__ __forceinline__ void tt_cp_async16(void* smem_dst, const void* gsrc)
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(gsrc) : "memory");
 }
 
+// ... of the first `floats` of the 16 bytes only (at least one float), the others zero
+__device__ __forceinline__ void tt_cp_async16_cut(void* smem_dst, const void* gsrc, uint64_t floats)
+{
+    const unsigned d = (unsigned)__cvta_generic_to_shared(smem_dst);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(gsrc), "r"(floats < 4 ? (unsigned)floats * 4u : 16u) : "memory");
+}
+
 // left operand of level k (2..K-1) for node v: P_{k-1} of its parent (k = 2: the slice of the first core)
 __device__ __forceinline__ const float* tt_left_operand(const WsView& w, const TableDesc& td, int k, uint32_t v)
 {

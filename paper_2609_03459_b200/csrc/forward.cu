@@ -1429,6 +1429,129 @@ static cudaError_t launch_pool_vec(tt_emb* h, float* out, bool plan, cudaStream_
     return cudaGetLastError();
 }
 
+// Rows whose length is no multiple of four floats (or an `out` that is not 16-byte aligned), D <= 4 R4 - 3: a row starts anywhere
+// in its first 16-byte piece, so the R4 or fewer aligned pieces that it touches are staged as they lie and every lane picks its
+// columns (lane, lane + 32) behind the row's shift.  Same shares, windows and look-ahead as k_pool_async; the pieces past the last row
+// of the row buffer lie in its guard bytes.  1 M lookups of 45 floats: 101 us with a row per pair of 4-byte loads and a warp per bag,
+// 66 us now (2.7 TB/s of rows; the window's chain row id -> rank word -> rows, as in k_pool_async).
+template <int R4, bool WT>
+__global__ void __launch_bounds__(32 * POOL_WARPS, 4) k_pool_odd(WsView w, float* __restrict__ out)
+{
+    tt_pdl_enter();
+    static_assert(R4 == 16 || R4 == 8, "two or four rows per cp.async instruction");
+    constexpr int RPI = 32 / R4, P = 4 * R4;             // pitch of a staged row in floats
+    extern __shared__ __align__(16) float4 pool_buf[];   // [POOL_WARPS][32 rows][R4 float4]
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int sub = lane / R4, lr = lane % R4;
+    float4* buf = pool_buf + (size_t)wid * 32 * R4;
+    const float* bufv = reinterpret_cast<const float*>(buf);
+    const uint32_t D = (uint32_t)w.D;
+    const bool on0 = lane < (int)D, on1 = R4 == 16 && lane + 32 < (int)D;
+    const uint32_t capK = w.cap[w.K];
+    const int64_t C = w.pool_shares;
+    typedef int32_t pos_t;
+    auto clampL = [&](int64_t x) { return x < 0 ? (pos_t)0 : (x > w.L ? (pos_t)w.L : (pos_t)x); };
+    for (;;) {
+    int64_t ci = 0;     // shares are handed out in order through a counter (see k_pool_async)
+    if (lane == 0) ci = (int64_t)atomicAdd(&w.counters[CTR_POOL_NEXT], 1u);
+    ci = __shfl_sync(0xffffffffu, ci, 0);
+    if (ci >= C) break;
+    const pos_t b0 = (pos_t)__ldg(w.pool_bounds + ci), b1 = (pos_t)__ldg(w.pool_bounds + ci + 1);
+    if (b0 >= b1) continue;
+    pos_t o_lo = clampL(__ldg(w.offsets + b0)), o_next = clampL(__ldg(w.offsets + b0 + 1));
+    pos_t o_hi = o_next < o_lo ? o_lo : o_next;
+    int t = (int)(b0 / w.B);
+    uint32_t slot_next;
+    float wt_next = 1.f;
+    auto fetch = [&](pos_t base, pos_t lim, int tt) {   // rank look-up (and weight) of lookup base + lane
+        slot_next = (base + lane < lim) ? tt_lookup_slot(w, w.tdesc[tt], base + lane, capK) : 0xffffffffu;
+        if (WT) wt_next = (w.psw && base + lane < lim) ? __ldg(w.psw + base + lane) : 1.f;
+    };
+    fetch(o_lo, o_hi, t);
+    for (pos_t bag = b0; bag < b1; ++bag) {
+        const pos_t b = bag - (pos_t)t * w.B;
+        const bool has_next = bag + 1 < b1;
+        const pos_t n_lo = o_next;
+        const pos_t n_next = has_next ? clampL(__ldg(w.offsets + bag + 2)) : o_next;
+        const pos_t n_hi = n_next < n_lo ? n_lo : n_next;
+        const int tn = (has_next && b + 1 == w.B) ? t + 1 : t;
+        float acc0 = 0.f, acc1 = 0.f;
+        if (o_lo >= o_hi && has_next) fetch(n_lo, n_hi, tn);
+        for (pos_t l0 = o_lo; l0 < o_hi; l0 += 32) {
+            const uint32_t slot = slot_next;
+            const float wt = wt_next;
+            if (w.upairs && l0 + lane < o_hi) __stcs(&w.upairs[l0 + lane], make_uint2(slot, (uint32_t)b));
+            const int n = (int)min((pos_t)32, o_hi - l0);
+            const unsigned valid = __ballot_sync(0xffffffffu, lane < n && slot != 0xffffffffu);
+#pragma unroll 4
+            for (int jq = 0; jq < 32 / RPI; ++jq) {
+                if (RPI * jq >= n) break;
+                const int j = RPI * jq + sub;
+                const uint32_t sl = __shfl_sync(0xffffffffu, slot, j);
+                const uint64_t start = (uint64_t)sl * D;
+                if (((valid >> j) & 1u) && 4u * lr < (uint32_t)(start & 3) + D) tt_cp_async16(buf + j * R4 + lr, w.E + (start & ~(uint64_t)3) + 4 * lr);
+            }
+            asm volatile("cp.async.commit_group;" ::: "memory");
+            // the rank look-ups of the next batch (or of the next bag) overlap the gather
+            if (l0 + 32 < o_hi) fetch(l0 + 32, o_hi, t);
+            else if (has_next) fetch(n_lo, n_hi, tn);
+            const uint32_t shift = (slot * D) & 3u;
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+            __syncwarp();
+            float part0 = 0.f, part1 = 0.f;   // two-level sum: added to the bag's sum once per batch
+            for (int j0 = 0; j0 < n; j0 += 8) {
+#pragma unroll
+                for (int jj = 0; jj < 8; ++jj) {
+                    const int j = j0 + jj;
+                    const float* src = bufv + j * P + __shfl_sync(0xffffffffu, shift, j) + lane;
+                    const float wj = WT ? __shfl_sync(0xffffffffu, wt, j) : 1.f;
+                    const bool ok = (valid >> j) & 1u;
+                    const float x0 = ok && on0 ? src[0] : 0.f;
+                    part0 = WT ? fmaf(wj, x0, part0) : part0 + x0;
+                    if (R4 == 16) {
+                        const float x1 = ok && on1 ? src[32] : 0.f;
+                        part1 = WT ? fmaf(wj, x1, part1) : part1 + x1;
+                    }
+                }
+            }
+            acc0 += part0;
+            acc1 += part1;
+            __syncwarp();
+        }
+        if (WT && w.pool_mean && o_hi > o_lo) {
+            const float inv = 1.f / (float)(o_hi - o_lo);
+            acc0 *= inv;
+            acc1 *= inv;
+        }
+        float* o = out + ((size_t)b * w.T + t) * D + lane;
+        if (on0) __stcs(o, acc0);
+        if (on1) __stcs(o + 32, acc1);
+        o_lo = n_lo;
+        o_hi = n_hi;
+        o_next = n_next;
+        t = tn;
+    }
+    }
+}
+
+template <int R4, bool WT>
+static cudaError_t launch_pool_odd(tt_emb* h, float* out, bool plan, cudaStream_t s)
+{
+    const size_t smem = (size_t)POOL_WARPS * 32 * R4 * sizeof(float4);
+    cudaError_t e = cudaFuncSetAttribute(k_pool_odd<R4, WT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    if (plan) {
+        int per_sm = 0;
+        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_pool_odd<R4, WT>, 32 * POOL_WARPS, smem)) != cudaSuccess) return e;
+        const int64_t need = ((int64_t)h->v.T * h->v.B + POOL_WARPS - 1) / POOL_WARPS, most = (int64_t)(per_sm < 1 ? 1 : per_sm) * h->sm_count;
+        tt_pool_set(h, need < 1 ? 1 : (need < most ? need : most), POOL_WARPS);
+        return cudaSuccess;
+    }
+    if ((e = tt_launch_pdl(k_pool_odd<R4, WT>, dim3(h->pool_grid), dim3(32 * POOL_WARPS), smem, s, h->v, out)) != cudaSuccess) return e;
+    tt_note_launch();
+    return cudaGetLastError();
+}
+
 // any D (scalar path): lane handles elements lane, lane + 32, ... (NC of them per pass over the bag); 32 / NC rows in flight
 template <int NC>
 __global__ void __launch_bounds__(256) k_pool_scalar(WsView w, float* __restrict__ out)
@@ -1495,12 +1618,19 @@ static cudaError_t launch_pool_sized(tt_emb* h, int D4, float* out, bool plan, c
     if (D4 > 8 && D4 <= 16) return launch_pool_async<16, WT>(h, out, plan, s);
     if (D4 > 4 && D4 <= 8) return launch_pool_async<8, WT>(h, out, plan, s);
     if (D4 <= 4) return launch_pool_vec<4, 1, WT>(h, out, plan, s);
-    if (D4 <= 8) return launch_pool_vec<8, 1, WT>(h, out, plan, s);
-    if (D4 <= 16) return launch_pool_vec<16, 1, WT>(h, out, plan, s);
     if (D4 <= 32) return launch_pool_vec<32, 1, WT>(h, out, plan, s);
     if (D4 <= 64) return launch_pool_vec<32, 2, WT>(h, out, plan, s);
     if (D4 <= 128) return launch_pool_vec<32, 4, WT>(h, out, plan, s);
     return launch_pool_vec<32, 8, WT>(h, out, plan, s);
+}
+
+// rows that k_pool_odd stages (with the up to three floats before a row, its pieces fit the staging row)
+#define TT_POOL_ODD_MOST 61
+#define TT_POOL_ODD_NARROW 29
+template <bool WT>
+static cudaError_t launch_pool_unaligned(tt_emb* h, float* out, bool plan, cudaStream_t s)
+{
+    return h->D <= TT_POOL_ODD_NARROW ? launch_pool_odd<8, WT>(h, out, plan, s) : launch_pool_odd<16, WT>(h, out, plan, s);
 }
 
 static bool tt_pool_vectors(const tt_emb* h, const float* out)
@@ -1511,7 +1641,10 @@ static bool tt_pool_vectors(const tt_emb* h, const float* out)
 cudaError_t tt_plan_pooling(tt_emb* h, const float* out)
 {
     h->v.pool_shares = 0;
-    if (!tt_pool_vectors(h, out)) return cudaSuccess;   // a warp takes bags, not shares
+    if (!tt_pool_vectors(h, out)) {
+        if (h->D > TT_POOL_ODD_MOST) return cudaSuccess;   // a warp takes bags, not shares
+        return (h->v.psw || h->v.pool_mean) ? launch_pool_unaligned<true>(h, nullptr, true, nullptr) : launch_pool_unaligned<false>(h, nullptr, true, nullptr);
+    }
     return (h->v.psw || h->v.pool_mean) ? launch_pool_sized<true>(h, h->D / 4, nullptr, true, nullptr)
                                         : launch_pool_sized<false>(h, h->D / 4, nullptr, true, nullptr);
 }
@@ -1520,12 +1653,13 @@ cudaError_t tt_launch_pooling(tt_emb* h, float* out, cudaStream_t s)
 {
     WsView& w = h->v;
     const int D = w.D;
+    if (!tt_pool_vectors(h, out) && D <= TT_POOL_ODD_MOST)
+        return (w.psw || w.pool_mean) ? launch_pool_unaligned<true>(h, out, false, s) : launch_pool_unaligned<false>(h, out, false, s);
     if (!tt_pool_vectors(h, out)) {
         const int64_t want = ((int64_t)w.T * w.B + 7) / 8;  // 8 warps per CTA, one warp per bag
         int pgrid = (int)(want < (int64_t)h->sm_count * 8 ? want : (int64_t)h->sm_count * 8);
         const dim3 pg(pgrid < 1 ? 1 : pgrid);
-        cudaError_t e0 = D <= 32 ? tt_launch_pdl(k_pool_scalar<1>, pg, dim3(256), 0, s, w, out)
-                       : D <= 64 ? tt_launch_pdl(k_pool_scalar<2>, pg, dim3(256), 0, s, w, out)
+        cudaError_t e0 = D <= 64 ? tt_launch_pdl(k_pool_scalar<2>, pg, dim3(256), 0, s, w, out)
                        : D <= 128 ? tt_launch_pdl(k_pool_scalar<4>, pg, dim3(256), 0, s, w, out)
                                   : tt_launch_pdl(k_pool_scalar<8>, pg, dim3(256), 0, s, w, out);
         if (e0 != cudaSuccess) return e0;
