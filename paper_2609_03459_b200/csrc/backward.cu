@@ -1004,11 +1004,9 @@ template <int PM, int RB_>
 __device__ __forceinline__ void tt_warp_rows_dC_mma(const WsView& w, const TableDesc& td, uint32_t u0, uint32_t u1, uint32_t row_base,
                                                     float* dPdst, int lane)
 {
-    static_assert(PM == 4 || PM == 8 || PM % 16 == 0, "4 or 8 rows of dC fill the first rows of one row tile, else whole tiles");
-    constexpr bool HALF = PM < 16;   // rows PM..15 of the tile stay zero and are not stored
-    constexpr int MT = HALF ? 1 : PM / 16, NT = RB_ / 8;
+    static_assert(PM % 16 == 0, "whole row tiles");
+    constexpr int MT = PM / 16, NT = RB_ / 8;
     const int g = lane >> 2, t = lane & 3;
-    const bool rowok = !HALF || g < PM;
     const int K = w.K;
     const float* __restrict__ GK = td.core[K - 1];
     const uint32_t* __restrict__ rows = w.val[K];
@@ -1034,10 +1032,10 @@ __device__ __forceinline__ void tt_warp_rows_dC_mma(const WsView& w, const Table
         Tf32Pair a[MT][4];
 #pragma unroll
         for (int mt = 0; mt < MT; ++mt) {
-            a[mt][0] = tt_split_tf32(rowok ? __ldg(Ea + (16 * mt + g) * 4) : 0.f);
-            a[mt][1] = tt_split_tf32(HALF ? 0.f : __ldg(Ea + (16 * mt + g + 8) * 4));
-            a[mt][2] = tt_split_tf32(two && rowok ? __ldg(Ec + (16 * mt + g) * 4) : 0.f);
-            a[mt][3] = tt_split_tf32(two && !HALF ? __ldg(Ec + (16 * mt + g + 8) * 4) : 0.f);
+            a[mt][0] = tt_split_tf32(__ldg(Ea + (16 * mt + g) * 4));
+            a[mt][1] = tt_split_tf32(__ldg(Ea + (16 * mt + g + 8) * 4));
+            a[mt][2] = tt_split_tf32(two ? __ldg(Ec + (16 * mt + g) * 4) : 0.f);
+            a[mt][3] = tt_split_tf32(two ? __ldg(Ec + (16 * mt + g + 8) * 4) : 0.f);
         }
         float bv[NT][2];
 #pragma unroll
@@ -1065,8 +1063,8 @@ __device__ __forceinline__ void tt_warp_rows_dC_mma(const WsView& w, const Table
     for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
         for (int nt = 0; nt < NT; ++nt) {
-            if (rowok) *reinterpret_cast<float2*>(dPdst + (16 * mt + g) * RB_ + 8 * nt + 2 * t) = make_float2(tot[mt][nt][0], tot[mt][nt][1]);
-            if (!HALF) *reinterpret_cast<float2*>(dPdst + (16 * mt + g + 8) * RB_ + 8 * nt + 2 * t) = make_float2(tot[mt][nt][2], tot[mt][nt][3]);
+            *reinterpret_cast<float2*>(dPdst + (16 * mt + g) * RB_ + 8 * nt + 2 * t) = make_float2(tot[mt][nt][0], tot[mt][nt][1]);
+            *reinterpret_cast<float2*>(dPdst + (16 * mt + g + 8) * RB_ + 8 * nt + 2 * t) = make_float2(tot[mt][nt][2], tot[mt][nt][3]);
         }
 }
 
@@ -1074,9 +1072,7 @@ template <int PM, int RB_>
 __device__ __forceinline__ void tt_warp_rows_dG_mma(const float* Cs, const WsView& w, uint32_t u0, uint32_t u1, uint32_t row_base,
                                                     float* gk, int lane)
 {
-    constexpr bool KHALF = PM == 4;   // p = 4..7 of the one k step do not exist: zero operands
-    constexpr bool BHALF = RB_ == 8;  // b = 8..15 of the one row tile do not exist: zero operands, not reduced
-    constexpr int MT = BHALF ? 1 : RB_ / 16, KT = KHALF ? 1 : PM / 8;
+    constexpr int MT = RB_ / 16, KT = PM / 8;
     const int g = lane >> 2, t = lane & 3;
     const uint32_t* __restrict__ rows = w.val[w.K];
     Tf32Pair a[MT][KT][4];   // A[m = b][k = p] = C[p][b]
@@ -1085,9 +1081,9 @@ __device__ __forceinline__ void tt_warp_rows_dG_mma(const float* Cs, const WsVie
 #pragma unroll
         for (int kt = 0; kt < KT; ++kt) {
             a[mt][kt][0] = tt_split_tf32(Cs[(8 * kt + t) * (RB_ + 8) + 16 * mt + g]);
-            a[mt][kt][1] = tt_split_tf32(BHALF ? 0.f : Cs[(8 * kt + t) * (RB_ + 8) + 16 * mt + g + 8]);
-            a[mt][kt][2] = tt_split_tf32(KHALF ? 0.f : Cs[(8 * kt + t + 4) * (RB_ + 8) + 16 * mt + g]);
-            a[mt][kt][3] = tt_split_tf32(KHALF || BHALF ? 0.f : Cs[(8 * kt + t + 4) * (RB_ + 8) + 16 * mt + g + 8]);
+            a[mt][kt][1] = tt_split_tf32(Cs[(8 * kt + t) * (RB_ + 8) + 16 * mt + g + 8]);
+            a[mt][kt][2] = tt_split_tf32(Cs[(8 * kt + t + 4) * (RB_ + 8) + 16 * mt + g]);
+            a[mt][kt][3] = tt_split_tf32(Cs[(8 * kt + t + 4) * (RB_ + 8) + 16 * mt + g + 8]);
         }
     const int rb_ = g >> 2, jb = g & 3;       // B fragment: row rb_ of the pair, column jb of dE
     const int rc = t >> 1, jc = 2 * (t & 1);  // C fragment: row rc of the pair, columns jc, jc+1
@@ -1103,7 +1099,7 @@ __device__ __forceinline__ void tt_warp_rows_dG_mma(const float* Cs, const WsVie
 #pragma unroll
         for (int kt = 0; kt < KT; ++kt) {
             bv[kt][0] = valid ? __ldg(El + (8 * kt + t) * 4) : 0.f;
-            bv[kt][1] = valid && !KHALF ? __ldg(El + (8 * kt + t + 4) * 4) : 0.f;
+            bv[kt][1] = valid ? __ldg(El + (8 * kt + t + 4) * 4) : 0.f;
         }
 #pragma unroll
         for (int kt = 0; kt < KT; ++kt) {
@@ -1119,52 +1115,38 @@ __device__ __forceinline__ void tt_warp_rows_dG_mma(const float* Cs, const WsVie
 #pragma unroll
             for (int mt = 0; mt < MT; ++mt) {
                 tt_red_v2(dst + (16 * mt + g) * 4, acc[mt][0], acc[mt][1]);
-                if (!BHALF) tt_red_v2(dst + (16 * mt + g + 8) * 4, acc[mt][2], acc[mt][3]);
+                tt_red_v2(dst + (16 * mt + g + 8) * 4, acc[mt][2], acc[mt][3]);
             }
         }
     }
 }
 
-// Both row passes in one loop over the group's row pairs: the row ids and the dE rows come from memory once (the
-// second fragment layout of dE is served by L1), dC accumulates across the loop, dG_K tiles leave per pair.
-template <int PM, int RB_, int CS = RB_ + 8>   // CS: row stride of C in shared memory
+// Both row passes in one loop over the group's row pairs, for C of 8 rows: the row ids and the dE rows come from memory once (the
+// second fragment layout of dE is served by L1), dC accumulates across the loop, dG_K tiles leave per pair.  C of 8 rows would fill half
+// of the row tiles of dC, so that product runs transposed, dC^T[b][p] += sum_{(row, j)} D_row[b][j] * dE_row[p][j], M = b, N = 8
+// columns p, K = 8 = two rows x 4 columns j.
+template <int RB_, int CS>   // CS: row stride of C in shared memory
 __device__ __forceinline__ void tt_warp_rows_bwd_mma(const float* Cs, const WsView& w, const TableDesc& td, uint32_t u0, uint32_t u1,
                                                      uint32_t row_base, float* dPdst, float* gk, int lane)
 {
-    static_assert(PM == 4 || PM == 8 || PM % 16 == 0, "4 or 8 rows of dC fill the first rows of one row tile, else whole tiles");
-    constexpr bool HALF = PM < 16;                // rows PM..15 of the dC tile stay zero and are not stored
-    constexpr bool KHALF = PM == 4;               // p = 4..7 of the one dG k step do not exist: zero operands
-    constexpr int MT = HALF ? 1 : PM / 16, NT = RB_ / 8;     // dC tiles: rows p, columns b
-    constexpr bool BHALF = RB_ == 8;              // b = 8..15 of the one dG row tile do not exist: zero operands, not reduced
-    constexpr int MT2 = BHALF ? 1 : RB_ / 16, KT2 = KHALF ? 1 : PM / 8;   // dG tiles: rows b, k = p
+    constexpr int PM = 8, MT = RB_ / 16, NT = RB_ / 8;
     const int g = lane >> 2, t = lane & 3;
-    const bool rowok = !HALF || g < PM;
     const int K = w.K;
     const float* __restrict__ GK = td.core[K - 1];
     const uint32_t* __restrict__ rows = w.val[K];
-    Tf32Pair ct[MT2][KT2][4];   // A[m = b][k = p] = C[p][b]
+    Tf32Pair ct[MT][4];         // A[m = b][k = p] = C[p][b]
 #pragma unroll
-    for (int mt = 0; mt < MT2; ++mt)
+    for (int mt = 0; mt < MT; ++mt) {
+        ct[mt][0] = tt_split_tf32(Cs[t * CS + 16 * mt + g]);
+        ct[mt][1] = tt_split_tf32(Cs[t * CS + 16 * mt + g + 8]);
+        ct[mt][2] = tt_split_tf32(Cs[(t + 4) * CS + 16 * mt + g]);
+        ct[mt][3] = tt_split_tf32(Cs[(t + 4) * CS + 16 * mt + g + 8]);
+    }
+    float dc[MT][4], dct[MT][4];   // tensor-core accumulators and their rounded running sums (see tt_warp_rows_dC_mma)
 #pragma unroll
-        for (int kt = 0; kt < KT2; ++kt) {
-            ct[mt][kt][0] = tt_split_tf32(Cs[(8 * kt + t) * CS + 16 * mt + g]);
-            ct[mt][kt][1] = tt_split_tf32(BHALF ? 0.f : Cs[(8 * kt + t) * CS + 16 * mt + g + 8]);
-            ct[mt][kt][2] = tt_split_tf32(KHALF ? 0.f : Cs[(8 * kt + t + 4) * CS + 16 * mt + g]);
-            ct[mt][kt][3] = tt_split_tf32(KHALF || BHALF ? 0.f : Cs[(8 * kt + t + 4) * CS + 16 * mt + g + 8]);
-        }
-    // C of 8 or 4 rows would fill half or a quarter of the row tiles of dC: there the product runs transposed,
-    // dC^T[b][p] += sum_{(row, j)} D_row[b][j] * dE_row[p][j], M = b, N = 8 columns p (PM = 4: four of them zero), K = 8 =
-    // two rows x 4 columns j: RB_/16 tiles per pair instead of RB_/8
-    constexpr bool TR = HALF && RB_ >= 16;
-    constexpr int MTT = RB_ / 16;
-    constexpr int DM = TR ? MTT : MT, DN = TR ? 1 : NT;
-    float dc[DM][DN][4], dct[DM][DN][4];   // tensor-core accumulators and their rounded running sums (see tt_warp_rows_dC_mma)
+    for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
-    for (int mt = 0; mt < DM; ++mt)
-#pragma unroll
-        for (int nt = 0; nt < DN; ++nt)
-#pragma unroll
-            for (int x = 0; x < 4; ++x) { dc[mt][nt][x] = 0.f; dct[mt][nt][x] = 0.f; }
+        for (int x = 0; x < 4; ++x) { dc[mt][x] = 0.f; dct[mt][x] = 0.f; }
     const int rb_ = g >> 2, jb = g & 3;       // dG B fragment: row rb_ of the pair, column jb of dE
     const int rc = t >> 1, jc = 2 * (t & 1);  // dG C fragment: row rc of the pair, columns jc, jc+1
     for (uint32_t ub0 = u0; ub0 < u1; ub0 += 32) {
@@ -1178,109 +1160,60 @@ __device__ __forceinline__ void tt_warp_rows_bwd_mma(const float* Cs, const WsVi
         const uint32_t iKa = __shfl_sync(0xffffffffu, ids, ua - ub0), iKc = __shfl_sync(0xffffffffu, ids, uc - ub0);
         const float* __restrict__ Ea = w.E + (size_t)ua * (PM * 4);
         const float* __restrict__ Ec = w.E + (size_t)uc * (PM * 4);
-        // ---- loads: dE as A fragments (dC), slices as B fragments (dC), dE as B fragments (dG)
-        float av[MT][4], bv[NT][2], ev[KT2][2];
-#pragma unroll
-        for (int mt = 0; mt < MT; ++mt) {
-            // (transposed: av[0][0], av[0][2] are the B fragment dE_a[p = g][j = t], dE_c[g][t])
-            av[mt][0] = rowok ? __ldg(Ea + (16 * mt + g) * 4 + t) : 0.f;
-            av[mt][1] = HALF ? 0.f : __ldg(Ea + (16 * mt + g + 8) * 4 + t);
-            av[mt][2] = two && rowok ? __ldg(Ec + (16 * mt + g) * 4 + t) : 0.f;
-            av[mt][3] = two && !HALF ? __ldg(Ec + (16 * mt + g + 8) * 4 + t) : 0.f;
-        }
+        // ---- loads: dE as B fragment (dC), slices as A fragments (dC), dE as B fragment (dG)
+        const float e0 = __ldg(Ea + g * 4 + t), e1 = two ? __ldg(Ec + g * 4 + t) : 0.f;   // dE_a[p = g][j = t], dE_c[g][t]
         const float* __restrict__ Da = GK + (size_t)iKa * (RB_ * 4) + t;
         const float* __restrict__ Dc = GK + (size_t)iKc * (RB_ * 4) + t;
+        float dv[NT][2];
 #pragma unroll
         for (int nt = 0; nt < NT; ++nt) {
-            // (transposed: bv[2 mt][.], bv[2 mt + 1][.] are the A fragment rows b = 16 mt + g and + 8 of D_a, D_c)
-            bv[nt][0] = __ldg(Da + (8 * nt + g) * 4);
-            bv[nt][1] = two || !TR ? __ldg(Dc + (8 * nt + g) * 4) : 0.f;
+            // (dv[2 mt][.], dv[2 mt + 1][.] are the A fragment rows b = 16 mt + g and + 8 of D_a, D_c)
+            dv[nt][0] = __ldg(Da + (8 * nt + g) * 4);
+            dv[nt][1] = two ? __ldg(Dc + (8 * nt + g) * 4) : 0.f;
         }
         const bool valid = rb_ == 0 || two;
         const float* __restrict__ El = (rb_ == 0 ? Ea : Ec) + jb;
-#pragma unroll
-        for (int kt = 0; kt < KT2; ++kt) {
-            ev[kt][0] = valid ? __ldg(El + (8 * kt + t) * 4) : 0.f;
-            ev[kt][1] = valid && !KHALF ? __ldg(El + (8 * kt + t + 4) * 4) : 0.f;
-        }
+        const float v0 = valid ? __ldg(El + t * 4) : 0.f, v1 = valid ? __ldg(El + (t + 4) * 4) : 0.f;
         // ---- dC += dE . D^T
-        if constexpr (TR) {
-            Tf32Pair b[2];
-            b[0] = tt_split_tf32(av[0][0]);
-            b[1] = tt_split_tf32(av[0][2]);
+        {
+            const Tf32Pair b[2] = {tt_split_tf32(e0), tt_split_tf32(e1)};
 #pragma unroll
-            for (int mt = 0; mt < MTT; ++mt) {
-                Tf32Pair a[4];
-                a[0] = tt_split_tf32(bv[2 * mt][0]);
-                a[1] = tt_split_tf32(bv[2 * mt + 1][0]);
-                a[2] = tt_split_tf32(bv[2 * mt][1]);
-                a[3] = tt_split_tf32(bv[2 * mt + 1][1]);
-                tt_mma_3xtf32(dc[mt][0], a, b);
-            }
-        } else {
-            Tf32Pair a[MT][4];
-#pragma unroll
-            for (int mt = 0; mt < MT; ++mt)
-#pragma unroll
-                for (int x = 0; x < 4; ++x) a[mt][x] = tt_split_tf32(av[mt][x]);
-#pragma unroll
-            for (int nt = 0; nt < NT; ++nt) {
-                Tf32Pair b[2];
-                b[0] = tt_split_tf32(bv[nt][0]);
-                b[1] = tt_split_tf32(bv[nt][1]);
-#pragma unroll
-                for (int mt = 0; mt < MT; ++mt) tt_mma_3xtf32(dc[mt][nt], a[mt], b);
+            for (int mt = 0; mt < MT; ++mt) {
+                const Tf32Pair a[4] = {tt_split_tf32(dv[2 * mt][0]), tt_split_tf32(dv[2 * mt + 1][0]), tt_split_tf32(dv[2 * mt][1]), tt_split_tf32(dv[2 * mt + 1][1])};
+                tt_mma_3xtf32(dc[mt], a, b);
             }
         }
         // ---- dG_K[i_K] += C^T . dE
         {
-            float acc[MT2][4];
+            const Tf32Pair b[2] = {tt_split_tf32(v0), tt_split_tf32(v1)};
+            float acc[MT][4];
 #pragma unroll
-            for (int mt = 0; mt < MT2; ++mt) { acc[mt][0] = 0.f; acc[mt][1] = 0.f; acc[mt][2] = 0.f; acc[mt][3] = 0.f; }
-#pragma unroll
-            for (int kt = 0; kt < KT2; ++kt) {
-                Tf32Pair b[2];
-                b[0] = tt_split_tf32(ev[kt][0]);
-                b[1] = tt_split_tf32(ev[kt][1]);
-#pragma unroll
-                for (int mt = 0; mt < MT2; ++mt) tt_mma_3xtf32(acc[mt], ct[mt][kt], b);
+            for (int mt = 0; mt < MT; ++mt) {
+                acc[mt][0] = 0.f; acc[mt][1] = 0.f; acc[mt][2] = 0.f; acc[mt][3] = 0.f;
+                tt_mma_3xtf32(acc[mt], ct[mt], b);
             }
             if (rc == 0 || two) {
                 float* dst = gk + (size_t)(rc == 0 ? iKa : iKc) * (RB_ * 4) + jc;
 #pragma unroll
-                for (int mt = 0; mt < MT2; ++mt) {
+                for (int mt = 0; mt < MT; ++mt) {
                     tt_red_v2(dst + (16 * mt + g) * 4, acc[mt][0], acc[mt][1]);
-                    if (!BHALF) tt_red_v2(dst + (16 * mt + g + 8) * 4, acc[mt][2], acc[mt][3]);
+                    tt_red_v2(dst + (16 * mt + g + 8) * 4, acc[mt][2], acc[mt][3]);
                 }
             }
         }
     }
 #pragma unroll
-    for (int mt = 0; mt < DM; ++mt)
+    for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
-        for (int nt = 0; nt < DN; ++nt)
-#pragma unroll
-            for (int x = 0; x < 4; ++x) { dct[mt][nt][x] += dc[mt][nt][x]; dc[mt][nt][x] = 0.f; }
+        for (int x = 0; x < 4; ++x) { dct[mt][x] += dc[mt][x]; dc[mt][x] = 0.f; }
     }
-    if constexpr (TR) {
-        // the lane holds dC[p = 2t][b], dC[2t + 1][b] for b = 16 mt + g and b + 8
-        if (2 * t < PM) {
+    // the lane holds dC[p = 2t][b], dC[2t + 1][b] for b = 16 mt + g and b + 8
 #pragma unroll
-            for (int mt = 0; mt < MTT; ++mt) {
-                dPdst[(2 * t) * RB_ + 16 * mt + g] = dct[mt][0][0];
-                dPdst[(2 * t + 1) * RB_ + 16 * mt + g] = dct[mt][0][1];
-                dPdst[(2 * t) * RB_ + 16 * mt + g + 8] = dct[mt][0][2];
-                dPdst[(2 * t + 1) * RB_ + 16 * mt + g + 8] = dct[mt][0][3];
-            }
-        }
-    } else {
-#pragma unroll
-        for (int mt = 0; mt < MT; ++mt)
-#pragma unroll
-            for (int nt = 0; nt < NT; ++nt) {
-                if (rowok) *reinterpret_cast<float2*>(dPdst + (16 * mt + g) * RB_ + 8 * nt + 2 * t) = make_float2(dct[mt][nt][0], dct[mt][nt][1]);
-                if (!HALF) *reinterpret_cast<float2*>(dPdst + (16 * mt + g + 8) * RB_ + 8 * nt + 2 * t) = make_float2(dct[mt][nt][2], dct[mt][nt][3]);
-            }
+    for (int mt = 0; mt < MT; ++mt) {
+        dPdst[(2 * t) * RB_ + 16 * mt + g] = dct[mt][0];
+        dPdst[(2 * t + 1) * RB_ + 16 * mt + g] = dct[mt][1];
+        dPdst[(2 * t) * RB_ + 16 * mt + g + 8] = dct[mt][2];
+        dPdst[(2 * t + 1) * RB_ + 16 * mt + g + 8] = dct[mt][3];
     }
 }
 
@@ -1309,14 +1242,9 @@ __device__ __forceinline__ void tt_sweep_bwd_fast(const WsView& w, const TableDe
         __syncwarp();
         const uint32_t u0 = w.cstart[K - 1][g], u1 = w.cstart[K - 1][g + 1];
         if constexpr (MMA) {
-            // small C (rank 16): one fused loop over the row pairs is faster; larger C: two passes keep the register
-            // footprint low enough for twice the resident warps (measured on the 60-table configuration)
-            if constexpr (PM * RB_ <= 256) {
-                tt_warp_rows_bwd_mma<PM, RB_>(Cs, w, td, u0, u1, val * nK, w.dP[K - 1] + (size_t)g * w.stride[K - 1], gk, lane);
-            } else {
-                tt_warp_rows_dC_mma<PM, RB_>(w, td, u0, u1, val * nK, w.dP[K - 1] + (size_t)g * w.stride[K - 1], lane);
-                tt_warp_rows_dG_mma<PM, RB_>(Cs, w, u0, u1, val * nK, gk, lane);
-            }
+            // two passes keep the register footprint low enough for twice the resident warps of one fused loop
+            tt_warp_rows_dC_mma<PM, RB_>(w, td, u0, u1, val * nK, w.dP[K - 1] + (size_t)g * w.stride[K - 1], lane);
+            tt_warp_rows_dG_mma<PM, RB_>(Cs, w, u0, u1, val * nK, gk, lane);
         } else {
             tt_warp_rows_dC<PM, RB_, TP>(w, td, u0, u1, val * nK, w.dP[K - 1] + (size_t)g * w.stride[K - 1], lane);
             tt_warp_rows_dG<PM, RB_, TP>(Cs, w, u0, u1, val * nK, gk, lane);
@@ -1358,7 +1286,8 @@ __device__ __forceinline__ void tt_sweep_bwd_quad(const WsView& w, const TableDe
         for (int q = 0; q < cnt; ++q) {
             const uint32_t g = __shfl_sync(0xffffffffu, gq, q), val = __shfl_sync(0xffffffffu, valq, q);
             const uint32_t u0 = __shfl_sync(0xffffffffu, u0q, q), u1 = __shfl_sync(0xffffffffu, u1q, q);
-            tt_warp_rows_bwd_mma<PM, RB_, RB_ + 4>(Cs4 + (size_t)q * (PM * (RB_ + 4)), w, td, u0, u1, val * nK,
+            static_assert(PM == 8, "the fused loop takes C of 8 rows");
+            tt_warp_rows_bwd_mma<RB_, RB_ + 4>(Cs4 + (size_t)q * (PM * (RB_ + 4)), w, td, u0, u1, val * nK,
                                                    w.dP[K - 1] + (size_t)g * w.stride[K - 1], gk, lane);
         }
         __syncwarp();
@@ -1378,7 +1307,8 @@ __device__ __forceinline__ void tt_sweep_bwd_stream(const WsView& w, const Table
     constexpr bool TR = PM < 16;                  // dC transposed: M = b, N = p
     constexpr bool KHALF = PM == 4;               // p = 4..7 of the one dG k step do not exist: zero operands
     constexpr int MT = TR ? 1 : PM / 16, NT = RB_ / 8;
-    constexpr int MT2 = RB_ / 16, KT2 = KHALF ? 1 : PM / 8;
+    constexpr bool BHALF = RB_ == 8;              // b = 8..15 of the one row tile over b do not exist: zero operands, not stored
+    constexpr int MT2 = BHALF ? 1 : RB_ / 16, KT2 = KHALF ? 1 : PM / 8;
     constexpr int DM = TR ? MT2 : MT, DN = TR ? 1 : NT;
     using Stream = RowStream<PM, RB_, NG, PD>;
     constexpr int EP = Stream::EP, DP = Stream::DP;
@@ -1420,7 +1350,7 @@ __device__ __forceinline__ void tt_sweep_bwd_stream(const WsView& w, const Table
 #pragma unroll
                     for (int mt = 0; mt < DM; ++mt)
 #pragma unroll
-                        for (int x = 0; x < 4; ++x) {
+                        for (int x = 0; x < (BHALF ? 2 : 4); ++x) {
                             float* d = dst + (2 * t + (x & 1)) * RB_ + 16 * mt + g + 8 * (x >> 1);
                             *d = folded ? *d + dc[mt][0][x] : dc[mt][0][x];
                         }
@@ -1471,9 +1401,9 @@ __device__ __forceinline__ void tt_sweep_bwd_stream(const WsView& w, const Table
 #pragma unroll
                         for (int kt = 0; kt < KT2; ++kt) {
                             ct[mt][kt][0] = tt_split_tf32(Cs[(8 * kt + t) * CS + 16 * mt + g]);
-                            ct[mt][kt][1] = tt_split_tf32(Cs[(8 * kt + t) * CS + 16 * mt + g + 8]);
+                            ct[mt][kt][1] = tt_split_tf32(BHALF ? 0.f : Cs[(8 * kt + t) * CS + 16 * mt + g + 8]);
                             ct[mt][kt][2] = tt_split_tf32(KHALF ? 0.f : Cs[(8 * kt + t + 4) * CS + 16 * mt + g]);
-                            ct[mt][kt][3] = tt_split_tf32(KHALF ? 0.f : Cs[(8 * kt + t + 4) * CS + 16 * mt + g + 8]);
+                            ct[mt][kt][3] = tt_split_tf32(KHALF || BHALF ? 0.f : Cs[(8 * kt + t + 4) * CS + 16 * mt + g + 8]);
                         }
                 }
             }
@@ -1510,7 +1440,7 @@ __device__ __forceinline__ void tt_sweep_bwd_stream(const WsView& w, const Table
                 for (int mt = 0; mt < MT2; ++mt) {
                     Tf32Pair x[4], y[4];
                     split4(x, *reinterpret_cast<const float4*>(Dt + 64 * mt));
-                    split4(y, *reinterpret_cast<const float4*>(Dt + 64 * mt + 32));
+                    split4(y, BHALF ? make_float4(0.f, 0.f, 0.f, 0.f) : *reinterpret_cast<const float4*>(Dt + 64 * mt + 32));
                     const Tf32Pair a0[4] = {x[0], y[0], x[1], y[1]}, a1[4] = {x[2], y[2], x[3], y[3]};
                     tt_mma_3xtf32(dc[mt][0], a0, b0);
                     tt_mma_3xtf32(dc[mt][0], a1, b1);
@@ -1536,7 +1466,7 @@ __device__ __forceinline__ void tt_sweep_bwd_stream(const WsView& w, const Table
 #pragma unroll
             for (int mt = 0; mt < MT2; ++mt)
 #pragma unroll
-                for (int h = 0; h < 2; ++h)
+                for (int h = 0; h < (BHALF ? 1 : 2); ++h)
                     tt_red_v4_if((uint32_t)rc < nr, dst + (16 * mt + 8 * h) * 4, acc[0][mt][2 * h], acc[1][mt][2 * h], acc[0][mt][2 * h + 1], acc[1][mt][2 * h + 1]);
             chain += 2;
             __syncwarp();
@@ -1645,7 +1575,7 @@ __global__ void __launch_bounds__(WIDE_THREADS, 2) k_sweep_bwd_wide(WsView w, in
 // One CTA (4 warps) per work unit (table, q); last-core gradients go to one of TT_STRIPES L2-resident partial
 // copies with vector reductions, added up in fixed stripe order by k_reduce_gpart.
 template <int V>
-__global__ void __launch_bounds__(128, V == 5 ? 6 : V == 1 || V == 8 ? 4 : V == 6 || V == 9 ? 5 : 0) k_sweep_bwd(WsView w, int pl_floats, int c_floats, int vbase)
+__global__ void __launch_bounds__(128, V == 5 ? 6 : V == 1 || V == 8 ? 4 : V == 2 || V == 6 || V == 9 ? 5 : 0) k_sweep_bwd(WsView w, int pl_floats, int c_floats, int vbase)
 {
     tt_pdl_enter();
     extern __shared__ __align__(16) float sm[];
@@ -1663,11 +1593,11 @@ __global__ void __launch_bounds__(128, V == 5 ? 6 : V == 1 || V == 8 ? 4 : V == 
     float* Cs = As + pl_floats;
     if (V == 0) tt_sweep_bwd_fast<16, 32, 4, 4, 1, true>(w, td, g1, gk, As, Cs, &next, lane);
     if (V == 1) tt_sweep_bwd_stream<16, 16, 4, 4, BWD_RING>(w, td, g1, gk, sm + wid * BwdStream<16, 16, 4>::FLOATS, &next, lane);
-    if (V == 2) tt_sweep_bwd_fast<16, 8, 4, 4, 1, true>(w, td, g1, gk, As, Cs, &next, lane);
+    if (V == 2) tt_sweep_bwd_stream<16, 8, 4, 4, BWD_RING>(w, td, g1, gk, sm + wid * BwdStream<16, 8, 4>::FLOATS, &next, lane);
     if (V == 3) tt_sweep_bwd_fast<32, 32, 4, 4, 2, true>(w, td, g1, gk, As, Cs, &next, lane);
     if (V == 5) tt_sweep_bwd_quad<8, 32, 2, 4>(w, td, g1, gk, sm + (size_t)wid * (8 * 8 * 36), &next, lane);
     if (V == 6) tt_sweep_bwd_stream<8, 16, 2, 4, BWD_RING>(w, td, g1, gk, sm + wid * BwdStream<8, 16, 2>::FLOATS, &next, lane);
-    if (V == 7) tt_sweep_bwd_fast<8, 8, 2, 2, 1, false>(w, td, g1, gk, As, Cs, &next, lane);   // 8 x 8: the FP32 pipe wins (0.39 against 0.41 ms)
+    if (V == 7) tt_sweep_bwd_fast<8, 8, 2, 2, 1, false>(w, td, g1, gk, As, Cs, &next, lane);   // 8 x 8: the FP32 pipe wins (51 us against 57 with streamed rows; 8 tables, 5 M lookups 172 / 184)
     if (V == 8) tt_sweep_bwd_stream<4, 32, 2, 4, BWD_RING>(w, td, g1, gk, sm + wid * BwdStream<4, 32, 2>::FLOATS, &next, lane);
     if (V == 9) tt_sweep_bwd_stream<4, 16, 2, 4, BWD_RING>(w, td, g1, gk, sm + wid * BwdStream<4, 16, 2>::FLOATS, &next, lane);
     if (V == 10) tt_sweep_bwd_fast<4, 8, 2, 2, 1, false>(w, td, g1, gk, As, Cs, &next, lane);
@@ -1698,7 +1628,6 @@ static cudaError_t launch_sweep_bwd(tt_emb* h, int max_pl, int max_c, cudaStream
     if (n == 0) return cudaSuccess;
     // tensor-core variants keep C with padded rows (stride r_{K-1} + 8 floats)
     if (V == 0) max_c = 16 * (32 + 8);
-    if (V == 2) max_c = 16 * (8 + 8);
     if (V == 3) max_c = 32 * (32 + 8);
     size_t smem = (size_t)4 * (max_pl + max_c) * sizeof(float);
     if (V == 5) smem = (size_t)4 * 8 * 8 * 36 * sizeof(float);    // eight C tiles per warp, rows padded by four floats
@@ -1706,6 +1635,7 @@ static cudaError_t launch_sweep_bwd(tt_emb* h, int max_pl, int max_c, cudaStream
     if (V == 8) smem = (size_t)4 * BwdStream<4, 32, 2>::FLOATS * sizeof(float);
     if (V == 9) smem = (size_t)4 * BwdStream<4, 16, 2>::FLOATS * sizeof(float);
     if (V == 1) smem = (size_t)4 * BwdStream<16, 16, 4>::FLOATS * sizeof(float);
+    if (V == 2) smem = (size_t)4 * BwdStream<16, 8, 4>::FLOATS * sizeof(float);
     cudaError_t e;
     if ((e = tt_stage_begin(h, 9 + TT_NUM_VARIANTS + 1 + V + 1, s)) != cudaSuccess) return e;
     if constexpr (V < 0) {

@@ -3,7 +3,7 @@
 // A warp that loads a pair of rows (last digits, then slices of the last core and rows of dE), multiplies them and goes on to
 // the next pair waits for a chain of L2 round trips per pair; registers for a pair of look-ahead cost more warps than they save.  Here the
 // rows come through a ring in shared memory (cp.async, no registers), across the groups of the batch, and the last digits eight steps
-// ahead of that.  Backward sweeps, before / after, us: rank 16, C of 16 rows: 8 tables x 0.47 M rows 190 / 166, x 2.06 M rows 430 / 377,
+// ahead of that.  Backward sweeps, before / after, us: rank 16, C of 16 rows: 8 tables x 0.47 M rows 190 / 166, x 2.06 M rows 430 / 377, rank 8 (5 M lookups) 221 / 190,
 // the rank-16 tables of the 60-table step 2320 / 2240; 8 rows, rank 16 (8 tables, 5 M lookups) 328 / 212; 4 rows, rank 32 380 / 332;
 // 4 rows, rank 16 245 / 175 (weighted, 4 M lookups).  Bound by instruction latency at 16 to 20 warps per SM (issue slots 47 %, LSU 56 %,
 // tensor pipe 31 %; the intermediate products take a fifth, the reductions 6 %).  A ring of three steps is no faster, more warps at the

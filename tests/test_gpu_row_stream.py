@@ -1,4 +1,4 @@
-"""Backward sweeps that stream the rows of a batch of groups (ranks 16 with C of 16, 8 and 4 rows, rank 32 with C of 4 rows):
+"""Backward sweeps that stream the rows of a batch of groups (ranks 8 and 16 with C of 16, 8 and 4 rows, rank 32 with C of 4 rows):
 groups of 1 to 5 rows (a step holds four), around 32 rows (a block of steps, where sums of dC are handed over) and of several
 hundred rows, in ranks that are no multiple of eight before them, three and four cores, and rows dropped at the row capacity.
 
@@ -13,7 +13,7 @@ from workloads import TableSpec
 
 pytestmark = pytest.mark.gpu
 
-SHAPES = [((4, 4, 4), (16, 16)), ((4, 4, 4), (5, 16)), ((2, 4, 4), (16, 16)), ((2, 4, 4), (3, 16)), ((2, 2, 4), (32, 32)), ((2, 2, 4), (16, 16))]
+SHAPES = [((4, 4, 4), (8, 8)), ((2, 4, 4), (5, 8)), ((4, 4, 4), (16, 16)), ((4, 4, 4), (5, 16)), ((2, 4, 4), (16, 16)), ((2, 4, 4), (3, 16)), ((2, 2, 4), (32, 32)), ((2, 2, 4), (16, 16))]
 
 
 def ids_with_groups(n, sizes, rng):
@@ -54,15 +54,15 @@ def test_gradients(binding, d, r, n, sizes):  # noqa: F811
 
 
 @pytest.mark.parametrize("d,r", SHAPES)
-def test_rows_dropped_at_the_capacity(binding, d, r):  # noqa: F811
+@pytest.mark.parametrize("n,cap", [((6, 8, 40), 301), ((30, 32, 2), 77)])     # fewer groups than rows kept; more
+def test_rows_dropped_at_the_capacity(binding, d, r, n, cap):  # noqa: F811
     # the last groups keep some or none of their rows; what is left is the gradient of the rows that were kept
-    n = (6, 8, 40)
     spec = TableSpec(N=1920, n=n, d=d, r=(1,) + r + (1,), alpha=1.0, core_dist="normal", core_scale=0.3)
     wl = workloads.custom([spec], 60, 12, seed=4, with_grad=True)
     rng = np.random.default_rng(2)
     wl.indices = rng.integers(0, 1920, wl.L).astype(np.int64)
-    kept = np.unique(wl.indices)[:301]
-    emb = binding.from_workload(wl, enable_backward=True, max_unique_rows=301)
+    kept = np.unique(wl.indices)[:cap]
+    emb = binding.from_workload(wl, enable_backward=True, max_unique_rows=cap)
     emb.forward(dev(wl.indices), dev(wl.offsets), 60)
     assert emb.status() == binding.STATUS_OVERFLOW
     emb.backward(dev(wl.grad_out))
