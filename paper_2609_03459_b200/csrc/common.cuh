@@ -210,7 +210,7 @@ cudaError_t tt_stage_end(tt_emb* h, int stage, cudaStream_t s);
 
 // ---- launchers implemented in the .cu files (all enqueue on `s`, return cudaGetLastError()) ----
 cudaError_t tt_launch_grouping(tt_emb* h, cudaStream_t s);
-cudaError_t tt_launch_group_cluster(tt_emb* h, bool rows, cudaStream_t s);
+cudaError_t tt_launch_group_cluster(tt_emb* h, bool rows, int level, cudaStream_t s);
 int tt_group_cluster_ok();
 cudaError_t tt_launch_schedule(tt_emb* h, cudaStream_t s);
 cudaError_t tt_launch_tlist(tt_emb* h, int k, cudaStream_t s);   // digit-major list of the level-k nodes (backward, k < K-1)

@@ -190,9 +190,21 @@ __device__ __forceinline__ void tt_emit_set_bits(uint32_t* __restrict__ val, uin
 
 // ---- level K: rows
 
+__device__ __forceinline__ void tt_level_words(const WsView& w, int k, uint32_t warp, uint32_t warps);
+// side: CTAs at the end of both grids that write the bitmaps of levels K-1 (first kernel) and K-2 (second) from the bits alone, so that
+// these steps run beside the scan on the whole chip instead of after it in the cluster
 template <int TILE, class View = WsView>
 struct PopScan {
     View w;
+    uint32_t side = 0;
+    __device__ bool beside(uint32_t cta, uint32_t ctas, bool apply) const
+    {
+        if (cta + side < ctas) return false;
+        const int k = w.K - (apply ? 2 : 1);
+        const uint32_t per = TT_SCAN_THREADS / 32, warp = (cta + side - ctas) * per + (threadIdx.x >> 5);
+        if (k >= 1) tt_level_words(w, k, warp, side * per);
+        return true;
+    }
     __device__ uint32_t size() const { return w.total_words; }
     // every table starts on a scan-tile boundary: the table of a tile's first word is the table of all its words
     __device__ int locate(uint32_t i0) const
@@ -294,6 +306,33 @@ __device__ __forceinline__ bool tt_prefix_present(const WsView& w, const TableDe
     return tt_rank_incl(w, td, c, (uint32_t)hi - 1u) != tt_rank_excl(w, td, c, (uint32_t)lo);
 }
 
+// ... and from the level's bits alone, before it is scanned: some bit of [p n_{k+1}, (p + 1) n_{k+1}) is set.  One load per word, so
+// for radices of up to TT_BITS_RADIX only
+#define TT_BITS_RADIX 512
+__device__ __forceinline__ bool tt_prefix_any(const WsView& w, const TableDesc& td, int k, uint32_t p)
+{
+    const int c = k + 1;
+    const uint32_t radix = (uint32_t)td.n[k], space_c = c == w.K ? (uint32_t)td.N : td.prefix_space[c];
+    const uint64_t lo = (uint64_t)p * radix;
+    if (p >= td.prefix_space[k] || lo >= space_c) return false;
+    const uint32_t first = (uint32_t)lo, last = (uint32_t)(lo + radix < space_c ? lo + radix : space_c) - 1u;
+    const uint2* words = c == w.K ? w.bm + td.word_base : w.bml[c] + td.lword_base[c];
+    const uint32_t i0 = first >> 5, i1 = last >> 5;
+    uint32_t found = 0;
+    for (uint32_t i = i0; i <= i1; i += 4) {
+        uint32_t x[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) x[j] = i + j <= i1 ? words[i + j].x : 0u;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            if (i + j == i0) x[j] &= 0xffffffffu << (first & 31);
+            if (i + j == i1) x[j] &= 0xffffffffu >> (31 - (last & 31));
+            found |= x[j];
+        }
+    }
+    return found != 0;
+}
+
 // Level k < K from its own presence bitmap: the ascending distinct prefixes of every table.  Runs after the scan of
 // level k + 1 and k_prefix_bits, which sets this level's bits.
 template <class View = WsView>
@@ -370,10 +409,33 @@ __device__ __forceinline__ uint32_t tt_tkey(const TableDesc& td, int k, uint32_t
     return (val % nk) * td.prefix_space[k - 1] + val / nk;
 }
 
-__device__ __forceinline__ void tt_tmark_node(const WsView& w, const TableDesc& td, int k, uint32_t v)
+__device__ __forceinline__ void tt_tmark_value(const WsView& w, const TableDesc& td, int k, uint32_t val)
 {
-    const uint32_t key = tt_tkey(td, k, w.val[k][v]);
+    const uint32_t key = tt_tkey(td, k, val);
     atomicOr(&w.tbm[k][td.tword_base[k] + (key >> 5)].x, 1u << (key & 31));
+}
+__device__ __forceinline__ void tt_tmark_node(const WsView& w, const TableDesc& td, int k, uint32_t v) { tt_tmark_value(w, td, k, w.val[k][v]); }
+
+// Presence bitmap of level k from the bits of level k + 1, and the marks of the digit-major order of level K-1, by warps `warp`,
+// warp + warps, .. of a kernel that scans level k + 1 or one further down
+__device__ __forceinline__ void tt_level_words(const WsView& w, int k, uint32_t warp, uint32_t warps)
+{
+    const int lane = threadIdx.x & 31;
+    const bool mark = k == w.K - 1 && tt_digit_major(w);
+    const uint32_t n = w.total_words_l[k];
+    for (uint32_t i = warp; i < n; i += warps) {
+        int lo = 0, hi = w.T;
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if (w.tdesc[mid].lword_base[k] <= i) lo = mid; else hi = mid;
+        }
+        const TableDesc& td = w.tdesc[lo];
+        const uint32_t p = ((i - td.lword_base[k]) << 5) + lane;
+        const bool present = tt_prefix_any(w, td, k, p);
+        if (mark && present) tt_tmark_value(w, td, k, p);
+        const unsigned bits = __ballot_sync(0xffffffffu, present);
+        if (lane == 0) w.bml[k][i] = make_uint2(bits, 0u);
+    }
 }
 
 template <class View = WsView>

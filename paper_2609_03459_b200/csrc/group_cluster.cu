@@ -3,7 +3,7 @@
 //
 // The steps of grouping.cu are a chain of fifteen dependent kernels (marks, a scan per level, links, the digit-major list,
 // costs, boundaries), 3 to 5 us each however little they do.  Sixteen SMs do the same work on a few thousand lookups in
-// less than the launches cost: 1 k lookups, one table, grouping and schedule 74 -> 34 us, now bound by the latency of the
+// less than the launches cost: 1 k lookups, one table, grouping and schedule 74 -> 33 us, now bound by the latency of the
 // dependent loads in each step (one to three L2 round trips between two barriers).  The step functions are those of
 // group.cuh; only the distribution over threads differs.
 // Where every table is swept by warps that take one batch of groups at a time, the units hold equal group counts instead of
@@ -20,6 +20,7 @@
 
 #define GC_THREADS 1024
 #define GC_CTAS 16
+#define GC_NODES 4     // nodes that a thread links at a time
 
 // all writes of the cluster's threads before the barrier are visible to all of them after it
 __device__ __forceinline__ void gc_sync()
@@ -129,81 +130,242 @@ __device__ __forceinline__ void gc_scan(const F& f, uint32_t n, uint32_t* sums, 
         }
 }
 
+// The same for several scans at once, with one barrier for all of them (gc_scan pays one or two per scan, and each costs a round
+// trip through L2 besides the barrier itself).  First gc_amount for every scan, then gc_exchange, then gc_emit for every scan, whose
+// values come from L1 the second time.
+template <class F>
+__device__ __forceinline__ void gc_amount(const F& f, uint32_t n, uint32_t* warp_sums /* [32] */)
+{
+    const uint32_t per = gc_run(n), lo = min(n, blockIdx.x * per), hi = min(n, lo + per);
+    uint32_t amount = 0;
+#pragma unroll 4
+    for (uint32_t i = lo + threadIdx.x; i < hi; i += GC_THREADS) amount += tt_scan_amount(f, f.value(i, 0), 0);   // (no functor's value asks for the hint)
+    amount = __reduce_add_sync(0xffffffffu, amount);
+    if ((threadIdx.x & 31) == 0) warp_sums[threadIdx.x >> 5] = amount;
+}
+__device__ __forceinline__ void gc_exchange(uint32_t (*warp_sums)[GC_THREADS / 32], uint32_t (*sums)[GC_CTAS], int scans)
+{
+    const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    __syncthreads();
+    if (wid < (uint32_t)scans) {
+        const uint32_t tot = __reduce_add_sync(0xffffffffu, warp_sums[wid][lane]);
+        if (lane < GC_CTAS) {
+            uint32_t remote;
+            const uint32_t local = (uint32_t)__cvta_generic_to_shared(&sums[wid][blockIdx.x]);
+            asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(local), "r"(lane));
+            asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(remote), "r"(tot) : "memory");
+        }
+    }
+    gc_sync();
+}
+template <class F>
+__device__ __forceinline__ void gc_emit(const F& f, uint32_t n, const uint32_t* sums, uint32_t* sm)
+{
+    const uint32_t rank = blockIdx.x, tid = threadIdx.x, per = gc_run(n), lo = min(n, rank * per), hi = min(n, lo + per);
+    const int lane = tid & 31, wid = tid >> 5;
+    uint32_t carry = 0, all = 0;
+#pragma unroll
+    for (uint32_t i = 0; i < GC_CTAS; ++i) {
+        const uint32_t x = sums[i];
+        carry += i < rank ? x : 0u;
+        all += x;
+    }
+    if (rank == 0 && tid == 0) f.total(all);
+    int hint = lo < hi ? f.locate(lo) : 0;
+    for (uint32_t base = lo; base < hi; base += GC_TILE) {
+        uint32_t v[GC_IT], ex[GC_IT];
+        int at[GC_IT];
+#pragma unroll
+        for (int j = 0; j < GC_IT; ++j) {
+            const uint32_t i = base + (uint32_t)j * GC_THREADS + tid;
+            v[j] = 0;
+            if (i < hi) {
+                hint = f.locate_from(i, hint);
+                v[j] = f.value(i, hint);
+            }
+            at[j] = hint;
+        }
+        __syncthreads();        // the warps' sums of the tile (or scan) before are read
+#pragma unroll
+        for (int j = 0; j < GC_IT; ++j) {
+            const uint32_t a = base + (uint32_t)j * GC_THREADS + tid < hi ? tt_scan_amount(f, v[j], 0) : 0u;
+            uint32_t incl = a;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += y;
+            }
+            ex[j] = incl - a;
+            if (lane == 31) sm[j * (GC_THREADS / 32) + wid] = incl;   // element order: stripe j, then warp
+        }
+        __syncthreads();
+        if (wid == 0) {   // exclusive scan of the warps' sums, GC_IT per lane
+            uint32_t x[GC_IT], s = 0;
+#pragma unroll
+            for (int j = 0; j < GC_IT; ++j) { x[j] = sm[lane * GC_IT + j]; s += x[j]; }
+            uint32_t incl = s;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += y;
+            }
+            uint32_t run = incl - s;
+#pragma unroll
+            for (int j = 0; j < GC_IT; ++j) { sm[lane * GC_IT + j] = run; run += x[j]; }
+            if (lane == 31) sm[GC_THREADS / 32 * GC_IT] = run;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < GC_IT; ++j) {
+            const uint32_t i = base + (uint32_t)j * GC_THREADS + tid;
+            if (i < hi) f.emit(i, carry + sm[j * (GC_THREADS / 32) + wid] + ex[j], v[j], at[j]);
+        }
+        carry += sm[GC_THREADS / 32 * GC_IT];
+    }
+}
+
+// presence bits of the words of level k that this CTA scans, a warp per word, four words at a time; from the level below once it is
+// scanned, or (BITS) from its bits, and then with the marks of the digit-major order of level K-1
+template <bool BITS>
+__device__ __forceinline__ void gc_level_bits(const WsView& w, int k, bool mark)
+{
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const uint32_t n = w.total_words_l[k], per = gc_run(n), lo = min(n, blockIdx.x * per), hi = min(n, lo + per);
+    const LevelScan<const WsView&> ls{w, k};
+    int t = lo < hi ? ls.locate(lo) : 0;
+    for (uint32_t i0 = lo + wid; i0 < hi; i0 += GC_THREADS / 32 * 4) {
+        bool present[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const uint32_t i = i0 + (uint32_t)j * (GC_THREADS / 32);
+            present[j] = false;
+            if (i < hi) {
+                t = ls.locate_from(i, t);
+                const TableDesc& td = w.tdesc[t];
+                const uint32_t p = ((i - td.lword_base[k]) << 5) + lane;
+                present[j] = BITS ? tt_prefix_any(w, td, k, p) : tt_prefix_present(w, td, k, p);
+                if (mark && present[j]) tt_tmark_value(w, td, k, p);
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const uint32_t i = i0 + (uint32_t)j * (GC_THREADS / 32);
+            const unsigned bits = __ballot_sync(0xffffffffu, present[j]);
+            if (lane == 0 && i < hi) w.bml[k][i] = make_uint2(bits, 0u);
+        }
+    }
+}
+
+
 // rows: from the row ids on (workspace regions cleared here); otherwise the row bitmap is scanned already
-__global__ void __launch_bounds__(GC_THREADS) k_group_cluster(const __grid_constant__ WsView w, int rows)
+// level: 0, or one more than the highest level whose bitmap this kernel writes from the bits of the level below; all bitmaps are written before
+// any of them is scanned, and all are scanned at once.  (0: a radix is past TT_BITS_RADIX; level by level, each from the ranks of the one below)
+__global__ void __launch_bounds__(GC_THREADS) k_group_cluster(const __grid_constant__ WsView w, int rows, int level)
 {
     tt_pdl_enter();
     __shared__ uint32_t sm[GC_THREADS / 32 * GC_IT + 1];
-    __shared__ uint32_t sums[TT_MAXK + 1][GC_CTAS];   // [k]: the scan of level k, [K] later that of the costs; [0]: of the digit-major bitmap
+    __shared__ uint32_t sums[TT_MAXK + 1][GC_CTAS];   // a slot for every scan; [0]: of the digit-major bitmap, [K]: of the costs, where these are scanned late
     const int K = w.K;
     const uint32_t tid = threadIdx.x, first = blockIdx.x * GC_THREADS + tid, step = GC_CTAS * GC_THREADS;
-    const int lane = tid & 31, wid = tid >> 5;
     const bool digit_major = tt_digit_major(w);
     if (rows) {
         if (first < 16 + 64) reinterpret_cast<uint32_t*>(w.status)[first] = 0u;   // status and counters are adjacent
         uint4* bm4 = reinterpret_cast<uint4*>(w.bm);                             // a whole number of scan tiles
         for (uint32_t i = first; i < w.total_words / 2; i += step) bm4[i] = make_uint4(0u, 0u, 0u, 0u);
     }
-    if (digit_major)
+    if (digit_major && (rows || level == 0))   // (otherwise k_mark has cleared it)
         for (uint32_t i = first; i < w.ttotal_words[K - 1]; i += step) w.tbm[K - 1][i] = make_uint2(0u, 0u);
     gc_sync();   // also: every CTA runs before another writes into its shared memory
     if (rows) {
         tt_check_offsets(w, first, step);
         tt_mark_rows<false>(w, first, step, (int64_t)step * 4);
         gc_sync();
-        gc_scan(PopScan<TT_SCAN_TILE, const WsView&>{w}, w.total_words, sums[K], sm);
-        gc_sync();
     }
-    for (int k = K - 1; k >= 1; --k) {
-        // presence bits of the words that this CTA scans, a warp per word, four words at a time
-        const uint32_t n = w.total_words_l[k], per = gc_run(n), lo = min(n, blockIdx.x * per), hi = min(n, lo + per);
-        const LevelScan<const WsView&> ls{w, k};
-        int t = lo < hi ? ls.locate(lo) : 0;
-        for (uint32_t i0 = lo + wid; i0 < hi; i0 += GC_THREADS / 32 * 4) {
-            bool present[4];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const uint32_t i = i0 + (uint32_t)j * (GC_THREADS / 32);
-                present[j] = false;
-                if (i < hi) {
-                    t = ls.locate_from(i, t);
-                    const TableDesc& td = w.tdesc[t];
-                    present[j] = tt_prefix_present(w, td, k, ((i - td.lword_base[k]) << 5) + lane);
-                }
-            }
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const uint32_t i = i0 + (uint32_t)j * (GC_THREADS / 32);
-                const unsigned bits = __ballot_sync(0xffffffffu, present[j]);
-                if (lane == 0 && i < hi) w.bml[k][i] = make_uint2(bits, 0u);
+    const uint32_t twords = digit_major ? w.ttotal_words[K - 1] : 0u;
+    bool listed = level != 0;     // the digit-major bitmap is marked and scanned
+    if (level != 0) {
+        __shared__ uint32_t warp_sums[TT_MAXK + 1][GC_THREADS / 32];
+        for (int k = level - 1; k >= 1; --k) {
+            gc_level_bits<true>(w, k, digit_major && k == K - 1);
+            if (k > 1) gc_sync();
+            else __syncthreads();   // the words of level 1 are scanned by the CTA that has written them
+        }
+        // scans 0 .. K - 2: levels 1 .. K - 1; K - 1: the digit-major bitmap; K: the rows
+        const PopScan<TT_SCAN_TILE, const WsView&> ps{w};
+        const TPopScan<const WsView&> ts{w, K - 1};
+        for (int k = 1; k < K; ++k) gc_amount(LevelScan<const WsView&>{w, k}, w.total_words_l[k], warp_sums[k - 1]);
+        gc_amount(ts, twords, warp_sums[K - 1]);
+        gc_amount(ps, rows ? w.total_words : 0u, warp_sums[K]);
+        gc_exchange(warp_sums, sums, K + 1);
+        if (rows) gc_emit(ps, w.total_words, sums[K], sm);
+        for (int k = 1; k < K; ++k) gc_emit(LevelScan<const WsView&>{w, k}, w.total_words_l[k], sums[k - 1], sm);
+        if (digit_major) gc_emit(ts, twords, sums[K - 1], sm);
+        gc_sync();
+        if (digit_major) {   // more nodes than there is room for: the marks are those of the nodes that are kept
+            uint32_t all = 0;
+            for (int i = 0; i < GC_CTAS; ++i) all += sums[K - 2][i];
+            if (all > w.cap[K - 1]) {
+                listed = false;
+                for (uint32_t i = first; i < twords; i += step) w.tbm[K - 1][i] = make_uint2(0u, 0u);
+                gc_sync();
             }
         }
-        __syncthreads();
-        gc_scan(ls, n, sums[k], sm);
-        gc_sync();
+    } else {
+        if (rows) {
+            gc_scan(PopScan<TT_SCAN_TILE, const WsView&>{w}, w.total_words, sums[K], sm);
+            gc_sync();
+        }
+        for (int k = K - 1; k >= 1; --k) {
+            gc_level_bits<false>(w, k, false);
+            __syncthreads();
+            gc_scan(LevelScan<const WsView&>{w, k}, w.total_words_l[k], sums[k], sm);
+            gc_sync();
+        }
     }
-    // links of all levels in one pass over their nodes, unit boundaries by the threads that come last
-    uint32_t nodes = 0;
-    for (int k = K - 1; k >= 1; --k) nodes += w.counters[CTR_LEVEL0 + k];
+    // links of all levels, a level at a time, and the digit-major list; unit boundaries by the threads that come last
     if (first < (uint32_t)(K - 1)) tt_link_end(w, (int)first + 1);
-    for (uint32_t x = first; x < nodes; x += step) {
-        uint32_t v = x;
-        int k = K - 1;
-        while (v >= w.counters[CTR_LEVEL0 + k]) v -= w.counters[CTR_LEVEL0 + k--];
-        const TableDesc& td = w.tdesc[tt_find_table(w.tb[k], w.T, v)];
-        if (digit_major && k == K - 1) tt_tmark_node(w, td, k, v);
-        tt_link_node(w, td, k, v);
+    for (int k = K - 1; k >= 1; --k) {
+        const uint32_t count = w.counters[CTR_LEVEL0 + k];
+        const bool top = digit_major && k == K - 1, fill = top && listed && w.equal_units;
+        int t = 0;
+        for (uint32_t v0 = first; v0 < count; v0 += GC_NODES * step) {   // GC_NODES nodes at a time: their look-ups overlap
+            uint32_t val[GC_NODES], at[GC_NODES], up[GC_NODES], rank[GC_NODES];
+#pragma unroll
+            for (int j = 0; j < GC_NODES; ++j) val[j] = v0 + j * step < count ? w.val[k][v0 + j * step] : 0u;
+#pragma unroll
+            for (int j = 0; j < GC_NODES; ++j) {
+                const uint32_t v = v0 + j * step;
+                if (v >= count) break;
+                t = j == 0 ? tt_find_table(w.tb[k], w.T, v) : tt_find_table_from(w.tb[k], w.T, v, t);
+                const TableDesc& td = w.tdesc[t];
+                at[j] = tt_rank_at(w, td, k + 1, val[j] * (uint32_t)td.n[k]);
+                if (w.parent[k]) up[j] = tt_rank_at(w, td, k - 1, val[j] / (uint32_t)td.n[k - 1]);
+                if (fill) rank[j] = tt_trank(w, td, k, tt_tkey(td, k, val[j]));
+                else if (top && !listed) tt_tmark_value(w, td, k, val[j]);
+            }
+#pragma unroll
+            for (int j = 0; j < GC_NODES; ++j) {
+                const uint32_t v = v0 + j * step;
+                if (v >= count) break;
+                w.cstart[k][v] = at[j];
+                if (w.parent[k]) w.parent[k][v] = up[j];
+                if (fill) w.tnode[k][rank[j]] = v;
+            }
+        }
     }
     if (tt_pool_bounds_missing(w))
         for (int64_t ci = step - 1 - first; ci <= w.pool_shares; ci += step) tt_pool_bound(w, ci);
     const int64_t units = (int64_t)w.T * w.units_per_table;
     if (w.equal_units)
         for (int64_t u = step - 1 - first; u < units; u += step) tt_unit_bounds(w, (int)u);
+    if ((listed || !digit_major) && w.equal_units) return;
     gc_sync();
     const uint32_t groups = w.counters[CTR_LEVEL0 + K - 1];
     if (digit_major) {
-        gc_scan(TPopScan<const WsView&>{w, K - 1}, w.ttotal_words[K - 1], sums[0], sm);
-        gc_sync();
+        if (!listed) {
+            gc_scan(TPopScan<const WsView&>{w, K - 1}, twords, sums[0], sm);
+            gc_sync();
+        }
         for (uint32_t v = first; v < groups; v += step)
             tt_tfill_node(w, w.tdesc[tt_find_table(w.tb[K - 1], w.T, v)], K - 1, v, !w.equal_units);
     } else if (!w.equal_units) {
@@ -217,7 +379,7 @@ __global__ void __launch_bounds__(GC_THREADS) k_group_cluster(const __grid_const
     for (int64_t u = first; u < units; u += step) tt_unit_bounds(w, (int)u);
 }
 
-cudaError_t tt_launch_group_cluster(tt_emb* h, bool rows, cudaStream_t s)
+cudaError_t tt_launch_group_cluster(tt_emb* h, bool rows, int level, cudaStream_t s)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(GC_CTAS);
@@ -232,7 +394,7 @@ cudaError_t tt_launch_group_cluster(tt_emb* h, bool rows, cudaStream_t s)
     at[1].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 2;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, k_group_cluster, h->v, rows ? 1 : 0);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, k_group_cluster, h->v, rows ? 1 : 0, level);
     if (e == cudaSuccess) tt_note_launch();
     return e;
 }

@@ -32,10 +32,13 @@ __global__ void __launch_bounds__(256) k_check_offsets(WsView w)
 // 32: 102 / 103 / 107 / 115 for 103 us (one table of 16 M rows, 0.5 M lookups).  A second test of the word past L1 before the
 // atomic (the copy in L1 is often an old one) costs more than the requests it saves: 8 tables 124 us, 60 tables 950.
 #define TT_MARK_SEEDS_FROM (1 << 16)   // 8 k lookups: call 78.5 us with them, 78.0 without
+// clear: also clears the digit-major bitmap
 template <bool FUSED>
-__global__ void __launch_bounds__(256, 8) k_mark(WsView w)
+__global__ void __launch_bounds__(256, 8) k_mark(WsView w, int clear)
 {
     tt_pdl_enter();
+    if (clear)
+        for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < w.ttotal_words[w.K - 1]; i += gridDim.x * blockDim.x) w.tbm[w.K - 1][i] = make_uint2(0u, 0u);
     // one warp's lookups first: the popular rows are marked by then, and the other warps find their bits set
     if (w.L >= TT_MARK_SEEDS_FROM) {
         if (threadIdx.x < 32) tt_mark_rows<!FUSED>(w, (int64_t)blockIdx.x * blockDim.x * 4 + threadIdx.x, w.L, w.L);
@@ -171,7 +174,21 @@ cudaError_t tt_launch_grouping(tt_emb* h, cudaStream_t s)
     cudaError_t e;
     const int cluster = tt_use_cluster(h);
     w.equal_units = (cluster != 0 && (h->warp_groups || w.K == 2)) || (w.ablation & 2) ? 1 : 0;   // (units of K = 2 are ranges of rows)
-    if (cluster == 2) return tt_launch_group_cluster(h, true, s);
+    // Prefix bitmaps from the bits of the level below, before any scan.  With the row scan as kernels of their own, the two longest are written
+    // by CTAs beside it: in the cluster, sixteen SMs took 9 us for the 9 k words of 8 tables, all on the way of what follows.  Calls,
+    // before / after, us: 8 tables, 8 k lookups 78 / 63, 1.6 M 618 / 602 (training); one table, 0.7 M lookups 231 / 222, four cores 342 / 329;
+    // at most one / two / four such CTAs per SM: 65.7 / 63.6 / 62.8 and 604.7 / 602.2 / 601.8.
+    bool bits = true;
+    for (int t = 0; t < h->T; ++t)
+        for (int k = 1; k < w.K; ++k) bits = bits && h->tab[t].n[k] <= TT_BITS_RADIX;
+    if (cluster == 2) return tt_launch_group_cluster(h, true, bits ? w.K : 0, s);
+    unsigned side = 0;           // a warp per word of the largest of the bitmaps that are written beside the row scan
+    if (cluster == 1 && bits) {
+        uint32_t words = w.total_words_l[w.K - 1];
+        if (w.K >= 3 && w.total_words_l[w.K - 2] > words) words = w.total_words_l[w.K - 2];
+        side = (words + TT_SCAN_THREADS / 32 - 1) / (TT_SCAN_THREADS / 32);
+        if (side > (unsigned)h->sm_count * 4) side = (unsigned)h->sm_count * 4;
+    }
     // status word + counters are adjacent; bitmap follows its own region
     if ((e = cudaMemsetAsync(w.status, 0, (16 + 64) * sizeof(uint32_t), s)) != cudaSuccess) return e;
     const int64_t nb = (int64_t)w.T * w.B + 1;
@@ -195,20 +212,20 @@ cudaError_t tt_launch_grouping(tt_emb* h, cudaStream_t s)
             if ((e = tt_launch_pdl(k_check_offsets, dim3(g0), dim3(256), 0, s, w)) != cudaSuccess) return e;
             tt_note_launch();
         }
-        if ((e = tt_launch_pdl(fused ? k_mark<true> : k_mark<false>, dim3((unsigned)want), dim3(256), 0, s, w)) != cudaSuccess) return e;
+        if ((e = tt_launch_pdl(fused ? k_mark<true> : k_mark<false>, dim3((unsigned)want), dim3(256), 0, s, w, side && tt_digit_major(w) ? 1 : 0)) != cudaSuccess) return e;
         tt_note_launch();
     }
     // short bitmaps in finer tiles, so that they spread over the SMs
     const unsigned ptiles = (unsigned)(TT_HEAD_TILES * w.T) + w.rest_tiles;
     if (w.total_words <= TT_PSCAN_WORDS) {
-        PopScan<TT_SCAN_THREADS * TT_PSCAN_ITEMS> ps{w};
-        e = tt_scan<decltype(ps), TT_PSCAN_ITEMS>(ps, w.total_words, w.scan_tmp, s, ptiles * (TT_SCAN_ITEMS / TT_PSCAN_ITEMS));
+        PopScan<TT_SCAN_THREADS * TT_PSCAN_ITEMS> ps{w, side};
+        e = tt_scan<decltype(ps), TT_PSCAN_ITEMS>(ps, w.total_words, w.scan_tmp, s, ptiles * (TT_SCAN_ITEMS / TT_PSCAN_ITEMS), side);
     } else {
-        PopScan<TT_SCAN_TILE> ps{w};
-        e = tt_scan(ps, w.total_words, w.scan_tmp, s, ptiles);
+        PopScan<TT_SCAN_TILE> ps{w, side};
+        e = tt_scan(ps, w.total_words, w.scan_tmp, s, ptiles, side);
     }
     if (e != cudaSuccess) return e;
-    if (cluster == 1) return tt_launch_group_cluster(h, false, s);
+    if (cluster == 1) return tt_launch_group_cluster(h, false, side ? (w.K >= 4 ? w.K - 2 : 1) : 0, s);
     for (int k = w.K - 1; k >= 1; --k) {
         {
             const uint32_t want = (w.total_words_l[k] + 7u) / 8u;   // a warp per word

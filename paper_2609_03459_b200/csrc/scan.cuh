@@ -14,6 +14,8 @@
 //   __device__ uint32_t tile_of(uint32_t cta) const;        optional: the tile that CTA `cta` of the apply pass takes
 //                                                           (0xffffffff: none), for an order other than ascending,
 //                                                           e.g. the tiles with the most output first
+//   __device__ bool beside(uint32_t cta, uint32_t ctas, bool apply) const;   optional: whether CTA `cta` of the grid does other
+//                                                           work (and does it) instead of a tile
 //   WsView w;                                               w.counters[CTR_SCAN_TICKET] is the ticket (zero between scans)
 // ITEMS = elements per thread (tile = TT_SCAN_THREADS * ITEMS): the default for long inputs, fewer for short ones whose
 // tiles should still spread over the SMs.
@@ -24,6 +26,10 @@ template <class F>
 __device__ __forceinline__ auto tt_scan_amount(const F& f, uint32_t v, int) -> decltype(f.weight(v)) { return f.weight(v); }
 template <class F>
 __device__ __forceinline__ uint32_t tt_scan_amount(const F&, uint32_t v, long) { return v; }
+template <class F>
+__device__ __forceinline__ auto tt_scan_beside(const F& f, bool apply, int) -> decltype(f.beside(0u, 0u, apply)) { return f.beside(blockIdx.x, gridDim.x, apply); }
+template <class F>
+__device__ __forceinline__ bool tt_scan_beside(const F&, bool, long) { return false; }
 template <class F>
 __device__ __forceinline__ auto tt_scan_tile(const F& f, uint32_t cta, int) -> decltype(f.tile_of(cta)) { return f.tile_of(cta); }
 template <class F>
@@ -80,6 +86,7 @@ __global__ void __launch_bounds__(TT_SCAN_THREADS) tt_scan_reduce(F f, uint32_t*
     constexpr int TILE = TT_SCAN_THREADS * ITEMS;
     __shared__ uint32_t sm[34];
     __shared__ uint32_t ticket;
+    if (tt_scan_beside(f, false, 0)) return;
     const uint32_t n = f.size();
     const uint32_t ntiles = (uint32_t)(((uint64_t)n + TILE - 1) / TILE);
     if (ntiles == 0) {   // nothing to scan: the first CTA still reports the total
@@ -123,6 +130,7 @@ __global__ void __launch_bounds__(TT_SCAN_THREADS, 4) tt_scan_apply(F f, const u
     constexpr int TILE = TT_SCAN_THREADS * ITEMS;
     __shared__ uint32_t sm[34];
     __shared__ uint32_t sv[TILE + TILE / 32];
+    if (tt_scan_beside(f, true, 0)) return;
     const uint32_t n = f.size();
     const uint32_t tile = tt_scan_tile(f, blockIdx.x, 0);
     if (tile == 0xffffffffu) return;
@@ -159,18 +167,18 @@ __global__ void __launch_bounds__(TT_SCAN_THREADS, 4) tt_scan_apply(F f, const u
     }
 }
 
-// capacity = host-known upper bound of f.size(); tmp must hold ceil(capacity / tile) + 1 words; apply_ctas: size of the
+// capacity = host-known upper bound of f.size(); tmp must hold ceil(capacity / tile) + 1 words; side: CTAs of f.beside; apply_ctas: size of the
 // apply grid for a functor with tile_of (default: one CTA per tile)
 template <class F, int ITEMS = TT_SCAN_ITEMS>
-static inline cudaError_t tt_scan(const F& f, uint64_t capacity, uint32_t* tmp, cudaStream_t s, unsigned apply_ctas = 0)
+static inline cudaError_t tt_scan(const F& f, uint64_t capacity, uint32_t* tmp, cudaStream_t s, unsigned apply_ctas = 0, unsigned side = 0)
 {
     constexpr int TILE = TT_SCAN_THREADS * ITEMS;
     unsigned tiles = (unsigned)((capacity + TILE - 1) / TILE);
     if (tiles == 0) tiles = 1;
-    cudaError_t e = tt_launch_pdl(tt_scan_reduce<F, ITEMS>, dim3(tiles), dim3(TT_SCAN_THREADS), 0, s, f, tmp);
+    cudaError_t e = tt_launch_pdl(tt_scan_reduce<F, ITEMS>, dim3(tiles + side), dim3(TT_SCAN_THREADS), 0, s, f, tmp);
     if (e != cudaSuccess) return e;
     tt_note_launch();
-    if ((e = tt_launch_pdl(tt_scan_apply<F, ITEMS>, dim3(apply_ctas ? apply_ctas : tiles), dim3(TT_SCAN_THREADS), 0, s, f, (const uint32_t*)tmp)) != cudaSuccess) return e;
+    if ((e = tt_launch_pdl(tt_scan_apply<F, ITEMS>, dim3((apply_ctas ? apply_ctas : tiles) + side), dim3(TT_SCAN_THREADS), 0, s, f, (const uint32_t*)tmp)) != cudaSuccess) return e;
     tt_note_launch();
     return cudaGetLastError();
 }
