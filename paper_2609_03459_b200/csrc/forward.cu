@@ -1015,13 +1015,13 @@ __global__ void __launch_bounds__(32 * POOL_WARPS, 4) k_pool_async(WsView w, flo
 // window with one boundary is summed into two partial sums in one unrolled pass; a window with several bags in it is
 // summed by the whole warp at once, each sub-warp taking consecutive rows and the pieces of a bag that crosses
 // sub-warps being joined afterwards (from two boundaries on for rows of up to 128 bytes, from five on for wider rows,
-// where a sub-warp has sixteen rows to walk); a window with empty bags in it is summed bag by bag.  Weights and
+// where a sub-warp has sixteen rows to walk); a window with empty bags in it deals its bags out to the sub-warps.  Weights and
 // mean pooling take the same ways (the factor with the row, 1 / length where a bag is written): 131 k bags of 1 to 30 weighted
 // rows of 128 bytes 73 -> 63 us, of 1 to 8 rows of 256 bytes with mean 51 -> 41 us, of one weighted row 33 -> 17 us against
 // bag by bag.
 // 2 million bags of 128-byte rows, stream against one bag per window: 2 / 4 / 8 lookups each 0.20 / 0.28 / 0.51 ms
 // against 0.82; 1 to 15 lookups 0.54 against 0.83, 1 to 31 0.83 against 0.91, 1 to 63 1.22 against 1.27, 1 to 100 1.69
-// against 1.72, 1 to 200 3.09 against 3.00 ms.  256-byte rows: 2 / 4 / 8 lookups 0.29 / 0.44 / 0.74 ms against 0.88-0.92;
+// against 1.72, 1 to 200 3.09 against 3.00 ms; 262 k bags of 0 to 4 rows, mean, 67 us bag by bag, 39 with the bags dealt out.  256-byte rows: 2 / 4 / 8 lookups 0.29 / 0.44 / 0.74 ms against 0.88-0.92;
 // 1 to 15 lookups 0.78 against 0.95; 1 to 31 1.11-1.19 against 1.10; on the benchmark configuration (1 to 100 lookups)
 // 2.34-2.36 against 2.39 ms.  Hence the thresholds (the benchmark configuration stays with the per-bag kernel).  A
 // window ends early only at the end of the share or of a table (the rank look-up of a window uses one table).  With
@@ -1204,9 +1204,51 @@ __global__ void __launch_bounds__(32 * POOL_WARPS, 4) k_pool_stream(WsView w, fl
                 seek_bag(bag + n, pos);
                 continue;
             }
-            // no empty bag among those that start inside the window (an empty bag needs a row of zeros: left to the
-            // bag-by-bag loop below)
             const pos_t e_prev = __shfl_up_sync(0xffffffffu, e_mine, 1);
+            // empty bags among those that start inside the window: the bags that end in it (32 at most, of this table) and the one
+            // that goes on are dealt out to the sub-warps, an empty one as a sum of no rows
+            if (__any_sync(0xffffffffu, lane >= 1 && e_prev < wend && e_mine == e_prev)) {
+                const int nc = __popc(__ballot_sync(0xffffffffu, e_mine <= wend && bag + lane < (pos_t)(t + 1) * w.B));   // the first nc bags
+                const pos_t last = __shfl_sync(0xffffffffu, e_mine, nc - 1), upto = nc < 32 ? wend : last;   // rows past `upto` are fetched again
+                const int nb = nc + (last < upto ? 1 : 0);
+                const pos_t bt = bag - (pos_t)t * w.B;
+                if (w.upairs) {
+                    int k = 0;          // bags that end before or at this lane's row
+#pragma unroll
+                    for (int step = 16; step > 0; step >>= 1)
+                        if (__shfl_sync(0xffffffffu, e_mine, k + step - 1) <= pos + lane) k += step;
+                    if (pos + lane < upto) __stcs(&w.upairs[pos + lane], make_uint2(slot, (uint32_t)(bt + k)));
+                }
+                float4 carry = acc;     // the open bag's sum so far, the same in every sub-warp
+#pragma unroll
+                for (int o = R4; o < 32; o <<= 1) {
+                    carry.x += __shfl_xor_sync(0xffffffffu, carry.x, o); carry.y += __shfl_xor_sync(0xffffffffu, carry.y, o);
+                    carry.z += __shfl_xor_sync(0xffffffffu, carry.z, o); carry.w += __shfl_xor_sync(0xffffffffu, carry.w, o);
+                }
+                float4 keep = make_float4(0.f, 0.f, 0.f, 0.f);
+                for (int i0 = 0; i0 < nb; i0 += RPI) {
+                    const int i = i0 + sub, ii = i < nb ? i : nb - 1;
+                    const pos_t hi = __shfl_sync(0xffffffffu, e_mine, ii & 31), before = __shfl_sync(0xffffffffu, e_mine, (ii - 1) & 31);
+                    const pos_t lo = ii > 0 ? before : o_lo;
+                    if (i >= nb || !lane_on) continue;
+                    float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
+                    const int j1 = (int)((hi < upto ? hi : upto) - pos);
+                    for (int j = lo > pos ? (int)(lo - pos) : 0; j < j1; ++j)
+                        if ((valid >> j) & 1u) pool_add<WT>(sum, buf[j * R4 + lr], WT && w.psw ? __ldg(w.psw + pos + j) : 1.f);
+                    if (i == 0) tt_add4(sum, carry);
+                    if (i >= nc) { keep = sum; continue; }
+                    if (WT && w.pool_mean && hi > lo) {
+                        const float inv = 1.f / (float)(hi - lo);
+                        sum = make_float4(sum.x * inv, sum.y * inv, sum.z * inv, sum.w * inv);
+                    }
+                    __stcs(reinterpret_cast<float4*>(out + (size_t)(bt + i) * w.T * w.D + (size_t)t * w.D) + lr, sum);
+                }
+                __syncwarp();
+                pos = upto;
+                seek_bag(bag + nc, last);
+                acc = keep;
+                continue;
+            }
             const int inside = __popc(__ballot_sync(0xffffffffu, e_mine > pos && e_mine < wend));   // bag ends inside the window
             if (inside == 1 && plain && n == 32) {
                 // one boundary, at row c: the rows before it complete the open bag, the others start the next one
@@ -1228,7 +1270,7 @@ __global__ void __launch_bounds__(32 * POOL_WARPS, 4) k_pool_stream(WsView w, fl
                 continue;
             }
             const bool many = inside >= (R4 == 16 ? 5 : 2);   // fewer: cheaper bag by bag
-            if (many && !__any_sync(0xffffffffu, lane >= 1 && e_prev < wend && e_mine == e_prev)) {
+            if (many) {
                 // starts: bit j = row j is the first of its bag; closes: bit j = row j is the last of its bag
                 const unsigned starts = __reduce_or_sync(0xffffffffu, (e_mine > pos && e_mine < wend) ? 1u << (int)(e_mine - pos) : 0u)
                                       | (o_lo == pos ? 1u : 0u);
