@@ -321,12 +321,13 @@ extern "C" int tt_emb_create(const tt_emb_config_t* cfg, tt_emb_t* out_handle)
         return o;
     };
 #define TAKE(name, bytes) (rname = name, take(bytes))
-    h->off_status = TAKE("status", (16 + 64) * sizeof(uint32_t));
-    h->off_counters = h->off_status + 16 * sizeof(uint32_t);
     h->off_tdesc = TAKE("tdesc", (size_t)T * sizeof(TableDesc));
     h->off_tlstart = TAKE("tlstart", (size_t)(T + 1) * sizeof(int64_t));
     h->off_vlist = TAKE("vlist", (size_t)(2 + TT_MAXK + 1) * T * sizeof(int32_t));
-    h->off_bm = TAKE("bm", (size_t)words * sizeof(uint2));
+    // status, counters and row bitmap side by side: one memset clears them at the start of a forward
+    h->off_status = TAKE("status and bm", TT_STATUS_BYTES + (size_t)words * sizeof(uint2));
+    h->off_counters = h->off_status + 16 * sizeof(uint32_t);
+    h->off_bm = h->off_status + TT_STATUS_BYTES;
     for (int k = 1; k <= K - 1; ++k) h->off_bml[k] = TAKE("bml", (size_t)lwords[k] * sizeof(uint2));
     uint64_t scan_max = words;
     for (int k = 1; k <= K - 1; ++k) if (lwords[k] > scan_max) scan_max = lwords[k];

@@ -35,6 +35,7 @@
 // ... and of the any-shape sweeps, whose CTAs take a batch of groups at a time (3x3x5, 29 k groups, forward + backward sweep
 // with at least 1 / 4 / 8 / 16 groups: 332 / 285 / 252 / 253 us; 8x8 with K = 2, 420 k lookups, whole call 1.16 ms with 8, 1.68 with 16)
 #define TT_UNIT_GROUPS_ANY 8
+#define TT_STATUS_BYTES 512   // status word and counters (16 + 64 words), up to the row bitmap behind them
 #define TT_UNIT_ROWS 64   // fewest rows of a unit of a K = 2 table
 #define TT_DE_CHUNK 1024                                  // most sorted lookups per warp in the dE segment reduction
 #define TT_NUM_STAGES 33                                // 0..8 pipeline stages, 9..20 forward sweep variants -1..10, 21..32 backward sweep variants

@@ -189,8 +189,8 @@ cudaError_t tt_launch_grouping(tt_emb* h, cudaStream_t s)
         side = (words + TT_SCAN_THREADS / 32 - 1) / (TT_SCAN_THREADS / 32);
         if (side > (unsigned)h->sm_count * 4) side = (unsigned)h->sm_count * 4;
     }
-    // status word + counters are adjacent; bitmap follows its own region
-    if ((e = cudaMemsetAsync(w.status, 0, (16 + 64) * sizeof(uint32_t), s)) != cudaSuccess) return e;
+    // status word, counters and row bitmap lie side by side (with a memset each: 8 tables, 8 k lookups, call 63.1 us instead of 60.8)
+    if ((e = cudaMemsetAsync(w.status, 0, TT_STATUS_BYTES + (w.ablation & 4 ? 0 : (size_t)w.total_words * sizeof(uint2)), s)) != cudaSuccess) return e;
     const int64_t nb = (int64_t)w.T * w.B + 1;
     int g0 = (int)((nb + 255) / 256);
     if (g0 > h->sm_count * 8) g0 = h->sm_count * 8;
@@ -201,7 +201,6 @@ cudaError_t tt_launch_grouping(tt_emb* h, cudaStream_t s)
         tt_note_launch();
         return cudaGetLastError();
     }
-    if ((e = cudaMemsetAsync(w.bm, 0, (size_t)w.total_words * sizeof(uint2), s)) != cudaSuccess) return e;
     if (cluster == 0 && tt_digit_major(w) && (e = cudaMemsetAsync(w.tbm[w.K - 1], 0, (size_t)w.ttotal_words[w.K - 1] * sizeof(uint2), s)) != cudaSuccess) return e;
     {
         int64_t want = (w.L + 1023) / 1024;
