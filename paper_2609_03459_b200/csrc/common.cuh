@@ -17,6 +17,12 @@
 #define TT_CSCAN_ITEMS 4                                // the scan of the group costs
 #define TT_PSCAN_ITEMS 4                                // the scan of row bitmaps of up to TT_PSCAN_WORDS words
 #define TT_PSCAN_WORDS (1u << 21)
+// up to so many words, from so many lookups and from one per word on, tiles of half that size: the densest tile, whose rows one CTA
+// lists, takes half as long, and there are twice as many others.  Calls with tiles of 1024 / 512 words, us: 4 M lookups 772 / 763, 1.6 M
+// 591 / 586, one table, 0.7 M 216 / 212, 0.5 M 327 / 325; 65 k 408.7 / 410.1, 8 k 60.8 / 64.3 (all in 0.26 M to 0.57 M words); 0.94 M words, 0.7 M
+// lookups 193 / 191, of spread rows 184.6 / 188.4
+#define TT_PSCAN_FINE_WORDS 655360u
+#define TT_PSCAN_FINE_LOOKUPS (1 << 18)
 // most lookups whose marking pass also checks the offsets: one launch less, but the tables' ranges come from all over the
 // offsets (99 M lookups, 60 tables: grouping 0.76 ms with two kernels, 0.81 ms with one; 0.5 M, 8 tables: 3 us shorter)
 #define TT_FUSED_INGEST (1 << 22)

@@ -216,7 +216,10 @@ cudaError_t tt_launch_grouping(tt_emb* h, cudaStream_t s)
     }
     // short bitmaps in finer tiles, so that they spread over the SMs
     const unsigned ptiles = (unsigned)(TT_HEAD_TILES * w.T) + w.rest_tiles;
-    if (w.total_words <= TT_PSCAN_WORDS) {
+    if (w.total_words <= TT_PSCAN_FINE_WORDS && w.L >= TT_PSCAN_FINE_LOOKUPS && w.L >= (int64_t)w.total_words) {
+        PopScan<TT_SCAN_THREADS * 2> ps{w, side};
+        e = tt_scan<decltype(ps), 2>(ps, w.total_words, w.scan_tmp, s, ptiles * (TT_SCAN_ITEMS / 2), side);
+    } else if (w.total_words <= TT_PSCAN_WORDS) {
         PopScan<TT_SCAN_THREADS * TT_PSCAN_ITEMS> ps{w, side};
         e = tt_scan<decltype(ps), TT_PSCAN_ITEMS>(ps, w.total_words, w.scan_tmp, s, ptiles * (TT_SCAN_ITEMS / TT_PSCAN_ITEMS), side);
     } else {
