@@ -554,7 +554,7 @@ def main():
     # DRAM traffic per lookup / per distinct row of the top kernels comes from the tracked ncu summary of a reduced case
     # and is scaled by the units this launch processes; it is reported only for the shape the capture was taken on.
     ncu_traffic, capture = dram_traffic_per_unit()
-    pool_kernel = "k_pool_async" if 16 < D <= 64 and D % 4 == 0 else ("k_pool_vec" if D % 4 == 0 else "k_pool_scalar")
+    pool_kernel = "k_pool_async" if 16 < D <= 64 and D % 4 == 0 else ("k_pool_vec" if D % 4 == 0 else "k_pool_odd" if D <= 61 else "k_pool_scalar")
     if pool_kernel == "k_pool_async" and L < (12 if D > 32 else 33) * T * B:
         pool_kernel = "k_pool_stream"   # the library's choice for short bags (windows of lookups across bags)
     same_shape = capture.get("capture_D") == str(D) and capture.get("capture_recipe") in ("cfg3", "cfg5") and cfg_id in (3, 5)
@@ -600,7 +600,7 @@ def main():
     if train and "bwd_dE" in stage_ms:
         ms = stage_ms["bwd_dE"]
         ach = work["dE_kernel_bytes"] / (ms * 1e-3) / 1e9
-        de_kernel = "k_dE_stage" if D in (16, 32, 64) else "k_dE_fast"
+        de_kernel = "k_dE_stage" if D in (16, 32, 64, 128) or (D % 4 and D <= 61) else "k_dE_fast"
         kernels[de_kernel] = (ms, {"kernel": de_kernel + " (+k_dE_fix)", "bound": "hbm", "achieved": ach, "peak": hbm_gbs,
                                      "unit": "GB/s", "frac": ach / hbm_gbs, "traffic": traffic_of("k_dE"),
                                      "peak_source": peak_src})
