@@ -343,10 +343,15 @@ __global__ void __launch_bounds__(256) k_dE(WsView w, const float* __restrict__ 
 // slots-th piece, then the slots in order.  (One warp per row: 4 M lookups,
 // D = 16, dE 187 us in chunks of 512 and 302 us in chunks of 128; now 142 and 121 us.)
 #define DE_FIX_OWN 8    // pieces that a warp adds by itself
+// No launch_dependents: the CTAs of the sweep that follows are placed when these are done.  Let in earlier, a grid of less than a
+// wave went to the few SMs that had room by then and left the others idle.  Training calls, early / now, us: tables of 20 k rows: eight,
+// 4x8x4, rank 32, 0.66 M lookups 818 / 677; one, 2x4x4, rank 32, 82 k lookups 264 / 223; one of four cores, rank 64, 447 / 421; larger
+// grids lose the overlap of one launch: 8 tables, rank 16, 1.6 M lookups 588 / 591, 1 k lookups 103 / 104; four tables of 200 k
+// rows, 4x4x4, rank 32, whose sweep is just a wave, 359 / 373 (neighbouring units on one SM share their slices).
 template <bool VEC, int CPL>
 __global__ void __launch_bounds__(256) k_dE_fix(WsView w)
 {
-    tt_pdl_enter();
+    tt_pdl_wait();
     using piece_t = typename std::conditional<VEC, float4, float>::type;
     __shared__ piece_t s_part[256];
     __shared__ uint32_t s_chunk[8], s_slot[8], s_pieces[8];

@@ -238,9 +238,10 @@ cudaError_t tt_launch_pack(const TableDesc& td, int core, const float* src, floa
 // running and wait (griddepcontrol.wait) until that grid has completed and its writes are visible, so the launch
 // latency of a chain of short kernels overlaps the previous kernel instead of following it.  Without the attribute
 // (or after a non-kernel operation in the stream) the wait returns at once.
+__device__ __forceinline__ void tt_pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void tt_pdl_enter()
 {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    tt_pdl_wait();
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
