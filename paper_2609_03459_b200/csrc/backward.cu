@@ -1343,7 +1343,9 @@ __device__ __forceinline__ void tt_sweep_bwd_stream(const WsView& w, const Table
             u1q = w.cstart[K - 1][gq + 1];
         }
         rs.begin(gq, u0q, u1q, valq * nK, lane);
-        tt_quad_mid<COLS, MROWS, KTMAX, RB_>(td.core[km], td.slice_floats[km], ra, cnt, imq, srcq, Cs4, lane, [&]() { rs.fill(w.E, lane); });
+        auto fill = [&]() { rs.fill(w.E, lane); };
+        if constexpr (RB_ == 8) tt_quad_mid_fp32<RB_>(td.core[km], td.slice_floats[km], ra, cnt, imq, srcq, Cs4, lane, fill);
+        else tt_quad_mid<COLS, MROWS, KTMAX, RB_>(td.core[km], td.slice_floats[km], ra, cnt, imq, srcq, Cs4, lane, fill);
         if (lane == 0) nbase = atomicAdd(next, (uint32_t)NG);
         nbase = __shfl_sync(0xffffffffu, nbase, 0);
         gq = lane < NG && nbase + lane < g1 ? w.tnode[K - 1][nbase + lane] : 0u;   // the next batch

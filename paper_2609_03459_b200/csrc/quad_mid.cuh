@@ -120,3 +120,55 @@ __device__ __forceinline__ void tt_quad_mid(const float* __restrict__ core_mid, 
         remaining &= ~sel;
     }
 }
+
+// The same in fp32 for slices of 32 columns (rank 8, C of 16 rows), of up to four groups with any slices: eight lanes per group, each
+// with four columns of its four rows.  The backward rebuilds C from these: its sums are those that it had before the products of
+// neighbouring groups were formed together, four terms apart, then pairwise.
+template <int RB, class Hook>
+__device__ __forceinline__ void tt_quad_mid_fp32(const float* __restrict__ core_mid, size_t slice_floats, int ra, int cnt, uint32_t imq,
+                                                 const float* srcq, float* Cs4, int lane, Hook hook)
+{
+    static_assert(RB == 8, "a group's 32 columns are eight float4s");
+    const int q = lane >> 3, c4 = lane & 7;
+    const bool on = q < cnt;
+    const uint32_t im = __shfl_sync(0xffffffffu, imq, q);
+    const float* src = reinterpret_cast<const float*>((uintptr_t)__shfl_sync(0xffffffffu, (unsigned long long)reinterpret_cast<uintptr_t>(srcq), q));
+    const float4* __restrict__ B4 = reinterpret_cast<const float4*>(core_mid + (size_t)im * slice_floats) + c4;
+    float4 acc[4];
+#pragma unroll
+    for (int m = 0; m < 4; ++m) acc[m] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 1
+    for (int a0 = 0; a0 < ra; a0 += 8) {
+        float4 b[8];
+#pragma unroll
+        for (int a = 0; a < 8; ++a) b[a] = on && a0 + a < ra ? __ldg(B4 + (size_t)(a0 + a) * 8) : make_float4(0.f, 0.f, 0.f, 0.f);
+        if (a0 == 0) hook();
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+            float x[8];
+            const float* __restrict__ row = src + m * ra + a0;
+            if ((ra & 3) == 0) {
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const float4 v = on && a0 + 4 * h < ra ? __ldg(reinterpret_cast<const float4*>(row) + h) : make_float4(0.f, 0.f, 0.f, 0.f);
+                    x[4 * h] = v.x; x[4 * h + 1] = v.y; x[4 * h + 2] = v.z; x[4 * h + 3] = v.w;
+                }
+            } else {
+#pragma unroll
+                for (int a = 0; a < 8; ++a) x[a] = on && a0 + a < ra ? __ldg(row + a) : 0.f;
+            }
+            auto sum = [&](float b0, float b1, float b2, float b3, float b4, float b5, float b6, float b7) {
+                return (fmaf(x[4], b4, x[0] * b0) + fmaf(x[5], b5, x[1] * b1)) + (fmaf(x[6], b6, x[2] * b2) + fmaf(x[7], b7, x[3] * b3));
+            };
+            acc[m].x += sum(b[0].x, b[1].x, b[2].x, b[3].x, b[4].x, b[5].x, b[6].x, b[7].x);
+            acc[m].y += sum(b[0].y, b[1].y, b[2].y, b[3].y, b[4].y, b[5].y, b[6].y, b[7].y);
+            acc[m].z += sum(b[0].z, b[1].z, b[2].z, b[3].z, b[4].z, b[5].z, b[6].z, b[7].z);
+            acc[m].w += sum(b[0].w, b[1].w, b[2].w, b[3].w, b[4].w, b[5].w, b[6].w, b[7].w);
+        }
+    }
+    if (on) {
+        float* dst = Cs4 + (size_t)q * (16 * (RB + 4)) + (c4 >> 1) * (RB + 4) + 4 * (c4 & 1);   // columns 4 c4 .. of row m: row 4 m + c4 / 2 of C
+#pragma unroll
+        for (int m = 0; m < 4; ++m) *reinterpret_cast<float4*>(dst + (size_t)m * (4 * (RB + 4))) = acc[m];
+    }
+}

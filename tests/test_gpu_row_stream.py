@@ -74,3 +74,25 @@ def test_rows_dropped_at_the_capacity(binding, d, r, n, cap):  # noqa: F811
     for k in range(3):
         assert_close(grads[0][k], ref[0][k], f"dG[0][{k}]")
     assert emb.check_guards() is None
+
+
+@pytest.mark.parametrize("ra,b", [(8, 1), (8, 4), (5, 4), (16, 12), (7, 2), (32, 31)])
+def test_rebuilt_products_of_rank_8_in_fp32(binding, ra, b):  # noqa: F811
+    # C = x * 1 + 1 * (-1) with x = 1 + 2^-11 + 2^-23: both products and their sum are exact in fp32, while an operand split into two
+    # TF32 values has lost the last bit of x, 2^-12 of C.  Everything after C is exact: dG_K = 16 C * lookups of the row.
+    x = 1.0 + 2.0 ** -11 + 2.0 ** -23
+    spec = TableSpec(N=60, n=(3, 4, 5), d=(4, 4, 4), r=(1, ra, 8, 1), alpha=1.0, core_dist="normal", core_scale=0.3)
+    wl = workloads.custom([spec], 40, 3, seed=ra, with_grad=True)
+    g0, g1, g2 = (np.zeros_like(c) for c in wl.cores[0])
+    g0[0, :, :, 0], g0[0, :, :, b] = 1.0, 1.0
+    g1[0], g1[b] = x, -1.0
+    g2[:] = 1.0
+    wl.cores = [[g0, g1, g2]]
+    emb = binding.from_workload(wl, enable_backward=True)
+    assert emb.table_variant(0) == 2
+    emb.forward(dev(wl.indices), dev(wl.offsets), wl.B)
+    emb.backward(dev(np.ones((wl.B, 64), dtype=np.float32)))
+    got = emb.get_grads()[0][2].astype(np.float64)
+    lookups = np.bincount(wl.indices % 5, minlength=5)
+    ref = np.broadcast_to((16.0 * (x - 1.0) * lookups)[None, :, None, None], got.shape)
+    assert np.max(np.abs(got - ref)) <= 2.0 ** -21 * np.max(ref)   # sums of at most 120 exact terms of 13 bits
