@@ -309,25 +309,33 @@ extern "C" int tt_emb_create(const tt_emb_config_t* cfg, tt_emb_t* out_handle)
     size_t off = 0;
     h->num_regions = 0;
     const char* rname = "";
-    auto take = [&](size_t bytes) {
-        const size_t o = off, end = off + bytes;
-        off = align_up(end + 64, 256);
+    auto guard = [&](size_t from, size_t to, unsigned char value) {
         if (h->num_regions < 96) {
-            h->guard_off[h->num_regions] = end;
-            h->guard_len[h->num_regions] = off - end;
+            h->guard_off[h->num_regions] = from;
+            h->guard_len[h->num_regions] = to - from;
+            h->guard_value[h->num_regions] = value;
             h->region_name[h->num_regions] = rname;
             ++h->num_regions;
         }
+    };
+    auto take = [&](size_t bytes) {
+        const size_t o = off, end = off + bytes;
+        off = align_up(end + 64, 256);
+        guard(end, off, TT_GUARD);
         return o;
     };
 #define TAKE(name, bytes) (rname = name, take(bytes))
     h->off_tdesc = TAKE("tdesc", (size_t)T * sizeof(TableDesc));
     h->off_tlstart = TAKE("tlstart", (size_t)(T + 1) * sizeof(int64_t));
     h->off_vlist = TAKE("vlist", (size_t)(2 + TT_MAXK + 1) * T * sizeof(int32_t));
-    // status, counters and row bitmap side by side: one memset clears them at the start of a forward
-    h->off_status = TAKE("status and bm", TT_STATUS_BYTES + (size_t)words * sizeof(uint2));
+    // status, counters and row bitmap side by side: one memset clears them at the start of a forward, and the guard bytes behind the
+    // counters with them
+    h->off_status = off;
     h->off_counters = h->off_status + 16 * sizeof(uint32_t);
-    h->off_bm = h->off_status + TT_STATUS_BYTES;
+    off += TT_STATUS_BYTES;
+    rname = "status";
+    guard(h->off_status + (16 + 64) * sizeof(uint32_t), off, 0);
+    h->off_bm = TAKE("bm", (size_t)words * sizeof(uint2));
     for (int k = 1; k <= K - 1; ++k) h->off_bml[k] = TAKE("bml", (size_t)lwords[k] * sizeof(uint2));
     uint64_t scan_max = words;
     for (int k = 1; k <= K - 1; ++k) if (lwords[k] > scan_max) scan_max = lwords[k];
@@ -475,9 +483,9 @@ extern "C" int tt_emb_bind(tt_emb_t h, float* const* core_ptrs, void* workspace,
     {
         uint64_t list[2 * 96 + 2];
         for (int i = 0; i < h->num_regions; ++i) {
-            TT_CUDA(cudaMemsetAsync(base + h->guard_off[i], 0xA5, h->guard_len[i], s));
+            TT_CUDA(cudaMemsetAsync(base + h->guard_off[i], h->guard_value[i], h->guard_len[i], s));
             list[2 * i] = (uint64_t)h->guard_off[i];
-            list[2 * i + 1] = (uint64_t)h->guard_len[i];
+            list[2 * i + 1] = (uint64_t)h->guard_len[i] | (uint64_t)h->guard_value[i] << 56;
         }
         list[2 * 96] = 0; list[2 * 96 + 1] = 0;
         // the list's own guard was just written; the list itself is uploaded after it (pageable source: staged before return)
@@ -925,10 +933,11 @@ extern "C" int tt_emb_probe_gather(const void* buffer, size_t bytes, int32_t* sc
 __global__ void k_check_guards(const unsigned char* base, const uint64_t* list, int n, int* first_bad)
 {
     for (int i = 0; i < n; ++i) {
-        const uint64_t off = list[2 * i], len = list[2 * i + 1];
+        const uint64_t off = list[2 * i], len = list[2 * i + 1] & 0xffffffull;
+        const unsigned char value = (unsigned char)(list[2 * i + 1] >> 56);
         bool bad = false;
         for (uint64_t b = threadIdx.x; b < len; b += blockDim.x)
-            if (base[off + b] != 0xA5) bad = true;
+            if (base[off + b] != value) bad = true;
         if (bad) atomicMin(first_bad, i);
     }
 }

@@ -41,7 +41,8 @@
 // ... and of the any-shape sweeps, whose CTAs take a batch of groups at a time (3x3x5, 29 k groups, forward + backward sweep
 // with at least 1 / 4 / 8 / 16 groups: 332 / 285 / 252 / 253 us; 8x8 with K = 2, 420 k lookups, whole call 1.16 ms with 8, 1.68 with 16)
 #define TT_UNIT_GROUPS_ANY 8
-#define TT_STATUS_BYTES 512   // status word and counters (16 + 64 words), up to the row bitmap behind them
+#define TT_STATUS_BYTES 512   // status word and counters (16 + 64 words) with their guard bytes, up to the row bitmap behind them
+#define TT_GUARD 0xA5         // guard bytes behind the other workspace regions
 #define TT_UNIT_ROWS 64   // fewest rows of a unit of a K = 2 table
 #define TT_DE_CHUNK 1024                                  // most sorted lookups per warp in the dE segment reduction
 #define TT_NUM_STAGES 33                                // 0..8 pipeline stages, 9..20 forward sweep variants -1..10, 21..32 backward sweep variants
@@ -178,6 +179,7 @@ struct tt_emb {
     // guard bytes after every workspace region (tt_emb_check_guards): [guard_off[i], guard_off[i] + guard_len[i])
     int num_regions;
     size_t guard_off[96], guard_len[96];
+    unsigned char guard_value[96];
     const char* region_name[96];
     size_t off_guard_list;      // device copy of the (offset, length) pairs + the check's result word
     void* ws_base;
