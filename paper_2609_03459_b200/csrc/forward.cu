@@ -1021,7 +1021,7 @@ __global__ void __launch_bounds__(32 * POOL_WARPS, 4) k_pool_async(WsView w, flo
 // bag by bag.
 // 2 million bags of 128-byte rows, stream against one bag per window: 2 / 4 / 8 lookups each 0.20 / 0.28 / 0.51 ms
 // against 0.82; 1 to 15 lookups 0.54 against 0.83, 1 to 31 0.83 against 0.91, 1 to 63 1.22 against 1.27, 1 to 100 1.69
-// against 1.72, 1 to 200 3.09 against 3.00 ms; 262 k bags of 0 to 4 rows, mean, 67 us bag by bag, 39 with the bags dealt out.  256-byte rows: 2 / 4 / 8 lookups 0.29 / 0.44 / 0.74 ms against 0.88-0.92;
+// against 1.72, 1 to 200 3.09 against 3.00 ms; 262 k bags of 0 to 4 rows, mean, 67 us bag by bag, 34 with the bags dealt out.  256-byte rows: 2 / 4 / 8 lookups 0.29 / 0.44 / 0.74 ms against 0.88-0.92;
 // 1 to 15 lookups 0.78 against 0.95; 1 to 31 1.11-1.19 against 1.10; on the benchmark configuration (1 to 100 lookups)
 // 2.34-2.36 against 2.39 ms.  Hence the thresholds (the benchmark configuration stays with the per-bag kernel).  A
 // window ends early only at the end of the share or of a table (the rank look-up of a window uses one table).  With
@@ -1205,48 +1205,77 @@ __global__ void __launch_bounds__(32 * POOL_WARPS, 4) k_pool_stream(WsView w, fl
                 continue;
             }
             const pos_t e_prev = __shfl_up_sync(0xffffffffu, e_mine, 1);
-            // empty bags among those that start inside the window: the bags that end in it (32 at most, of this table) and the one
-            // that goes on are dealt out to the sub-warps, an empty one as a sum of no rows
-            if (__any_sync(0xffffffffu, lane >= 1 && e_prev < wend && e_mine == e_prev)) {
-                const int nc = __popc(__ballot_sync(0xffffffffu, e_mine <= wend && bag + lane < (pos_t)(t + 1) * w.B));   // the first nc bags
-                const pos_t last = __shfl_sync(0xffffffffu, e_mine, nc - 1), upto = nc < 32 ? wend : last;   // rows past `upto` are fetched again
-                const int nb = nc + (last < upto ? 1 : 0);
-                const pos_t bt = bag - (pos_t)t * w.B;
-                if (w.upairs) {
-                    int k = 0;          // bags that end before or at this lane's row
+            // Empty bags among those that start inside the window: the bags that end in it and the one that goes on are dealt out to the
+            // sub-warps, 32 at a time, an empty one as a sum of no rows.  Row r of a bag goes to partial sum r % RPI: as many partial
+            // sums as where the sub-warps share a bag.  Bag by bag / dealt out, 131 k bags, us: 128-byte rows: half of the bags empty,
+            // the others of 4, 10, 20 and 40 rows 33 / 21, 41 / 29, 49 / 41, 66 / 59 (weighted 35 / 22, 43 / 33, 54 / 47, 76 / 70), 30 %
+            // empty, the others of 30 rows 68 / 63 (79 / 74); 256-byte rows: 35 / 27, 45 / 37, 61 / 53, 84 / 84 (39 / 29, 51 / 41, 70 / 61,
+            // 93 / 92), 80 / 83 (86 / 86).  With at least 3, 5 or 9 bags in the window only: never faster, 43 / 50 at 20 rows with 5.
+            const bool empties = __any_sync(0xffffffffu, lane >= 1 && e_prev < wend && e_mine == e_prev);
+            if (empties) {
+                const pos_t base = pos;
+                const int t0 = t;
+                for (pos_t e = e_mine;;) {
+                    const int nc = __popc(__ballot_sync(0xffffffffu, e <= wend && bag + lane < (pos_t)(t + 1) * w.B));   // of this table
+                    const pos_t ended = __shfl_sync(0xffffffffu, e, (nc - 1) & 31), last = nc > 0 ? ended : o_lo, upto = nc < 32 ? wend : last;
+                    const int nb = nc + (last < upto ? 1 : 0);
+                    const pos_t bt = bag - (pos_t)t * w.B;
+                    if (w.upairs) {
+                        int k = 0;          // bags that end before or at this lane's row
 #pragma unroll
-                    for (int step = 16; step > 0; step >>= 1)
-                        if (__shfl_sync(0xffffffffu, e_mine, k + step - 1) <= pos + lane) k += step;
-                    if (pos + lane < upto) __stcs(&w.upairs[pos + lane], make_uint2(slot, (uint32_t)(bt + k)));
-                }
-                float4 carry = acc;     // the open bag's sum so far, the same in every sub-warp
-#pragma unroll
-                for (int o = R4; o < 32; o <<= 1) {
-                    carry.x += __shfl_xor_sync(0xffffffffu, carry.x, o); carry.y += __shfl_xor_sync(0xffffffffu, carry.y, o);
-                    carry.z += __shfl_xor_sync(0xffffffffu, carry.z, o); carry.w += __shfl_xor_sync(0xffffffffu, carry.w, o);
-                }
-                float4 keep = make_float4(0.f, 0.f, 0.f, 0.f);
-                for (int i0 = 0; i0 < nb; i0 += RPI) {
-                    const int i = i0 + sub, ii = i < nb ? i : nb - 1;
-                    const pos_t hi = __shfl_sync(0xffffffffu, e_mine, ii & 31), before = __shfl_sync(0xffffffffu, e_mine, (ii - 1) & 31);
-                    const pos_t lo = ii > 0 ? before : o_lo;
-                    if (i >= nb || !lane_on) continue;
-                    float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
-                    const int j1 = (int)((hi < upto ? hi : upto) - pos);
-                    for (int j = lo > pos ? (int)(lo - pos) : 0; j < j1; ++j)
-                        if ((valid >> j) & 1u) pool_add<WT>(sum, buf[j * R4 + lr], WT && w.psw ? __ldg(w.psw + pos + j) : 1.f);
-                    if (i == 0) tt_add4(sum, carry);
-                    if (i >= nc) { keep = sum; continue; }
-                    if (WT && w.pool_mean && hi > lo) {
-                        const float inv = 1.f / (float)(hi - lo);
-                        sum = make_float4(sum.x * inv, sum.y * inv, sum.z * inv, sum.w * inv);
+                        for (int step = 16; step > 0; step >>= 1)
+                            if (__shfl_sync(0xffffffffu, e, k + step - 1) <= base + lane) k += step;
+                        if (base + lane >= pos && base + lane < upto) __stcs(&w.upairs[base + lane], make_uint2(slot, (uint32_t)(bt + k)));
                     }
-                    __stcs(reinterpret_cast<float4*>(out + (size_t)(bt + i) * w.T * w.D + (size_t)t * w.D) + lr, sum);
+                    float4 carry = acc;     // the open bag's sum so far, the same in every sub-warp
+#pragma unroll
+                    for (int o = R4; o < 32; o <<= 1) {
+                        carry.x += __shfl_xor_sync(0xffffffffu, carry.x, o); carry.y += __shfl_xor_sync(0xffffffffu, carry.y, o);
+                        carry.z += __shfl_xor_sync(0xffffffffu, carry.z, o); carry.w += __shfl_xor_sync(0xffffffffu, carry.w, o);
+                    }
+                    float4 keep = make_float4(0.f, 0.f, 0.f, 0.f);
+                    for (int i0 = 0; i0 < nb; i0 += RPI) {
+                        const int i = i0 + sub, ii = i < nb ? i : nb - 1;
+                        const pos_t hi = __shfl_sync(0xffffffffu, e, ii & 31), before = __shfl_sync(0xffffffffu, e, (ii - 1) & 31);
+                        const pos_t lo = ii > 0 ? before : o_lo;
+                        const int j0 = (int)((lo > pos ? lo : pos) - base), len = i < nb ? (int)((hi < upto ? hi : upto) - base) - j0 : 0;
+                        const int steps = __reduce_max_sync(0xffffffffu, (len + RPI - 1) / RPI);   // (weights come by shuffle)
+                        unsigned rows = len > 0 ? (valid >> j0) & (0xffffffffu >> (32 - len)) : 0u;
+                        const float4* src = buf + j0 * R4 + lr;
+                        float4 part[RPI];
+#pragma unroll
+                        for (int c = 0; c < RPI; ++c) part[c] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 1
+                        for (int st = 0; st < steps; ++st, rows >>= RPI, src += RPI * R4) {
+#pragma unroll
+                            for (int c = 0; c < RPI; ++c) {
+                                const float wj = WT ? __shfl_sync(0xffffffffu, wt, (j0 + st * RPI + c) & 31) : 1.f;
+                                if (rows & (1u << c)) pool_add<WT>(part[c], src[c * R4], wj);
+                            }
+                        }
+#pragma unroll
+                        for (int o = 1; o < RPI; o <<= 1)
+#pragma unroll
+                            for (int c = 0; c < RPI; c += 2 * o) tt_add4(part[c], part[c + o]);
+                        float4 sum = part[0];
+                        if (i >= nb || !lane_on) continue;
+                        if (i == 0) tt_add4(sum, carry);
+                        if (i >= nc) { keep = sum; continue; }
+                        if (WT && w.pool_mean && hi > lo) {
+                            const float inv = 1.f / (float)(hi - lo);
+                            sum = make_float4(sum.x * inv, sum.y * inv, sum.z * inv, sum.w * inv);
+                        }
+                        __stcs(reinterpret_cast<float4*>(out + (size_t)(bt + i) * w.T * w.D + (size_t)t * w.D) + lr, sum);
+                    }
+                    pos = upto;
+                    seek_bag(bag + nc, last);
+                    acc = keep;
+                    if (nc < 32 || bag >= b1 || t != t0) break;
+                    const int ei = (int)(bag - ebase) + lane;
+                    const pos_t x0 = __shfl_sync(0xffffffffu, ends_reg, ei & 31), x1 = __shfl_sync(0xffffffffu, ends_nx, ei & 31);
+                    e = ei < 32 ? x0 : x1;
                 }
                 __syncwarp();
-                pos = upto;
-                seek_bag(bag + nc, last);
-                acc = keep;
                 continue;
             }
             const int inside = __popc(__ballot_sync(0xffffffffu, e_mine > pos && e_mine < wend));   // bag ends inside the window

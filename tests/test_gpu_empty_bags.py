@@ -53,3 +53,27 @@ def test_out_and_gradients(binding, d, kind, T, B):  # noqa: F811
             for k in range(3):
                 assert_close(grads[t][k], ref[t][k], f"dG[{t}][{k}] {mode}")
     assert emb.check_guards() is None
+
+
+@pytest.mark.parametrize("d,sums", [((4, 4, 4), 2), ((2, 4, 4), 4)])
+@pytest.mark.parametrize("weighted", [False, True])
+def test_rows_of_a_bag_in_several_partial_sums(binding, d, sums, weighted):  # noqa: F811
+    # Bags of 31 rows, the first of 2^24 and the others of 1, between empty ones: a partial sum that holds the first row loses its ones, the
+    # other partial sums keep theirs, and the last additions round to multiples of 2.  One chain would lose all thirty.
+    spec = TableSpec(N=40, n=(1, 1, 40), d=d, r=(1, 8, 8, 1), alpha=1.0, core_dist="normal", core_scale=0.3)
+    B, T = 30_000, 2          # enough bags that a warp's share holds several
+    wl = workloads.custom([spec] * T, B, 1, seed=2)
+    g = [np.zeros_like(c) for c in wl.cores[0]]
+    g[0][0, :, :, 0], g[1][0, :, :, 0], g[2][0] = 1.0, 1.0, 1.0
+    g[2][0, 0] = 2.0 ** 24
+    wl.cores = [g] * T
+    lens = np.tile([31, 0, 0, 1], T * B // 4)
+    wl.offsets = np.concatenate([[0], np.cumsum(lens)]).astype(np.int64)
+    wl.indices = np.tile(np.concatenate([np.arange(31), [39]]), T * B // 4).astype(np.int64)
+    emb = binding.from_workload(wl, enable_weighted=True)
+    emb.set_pooling("sum", dev(np.ones(wl.L, dtype=np.float32)) if weighted else None)
+    out = emb.forward(dev(wl.indices), dev(wl.offsets), B).cpu().numpy().astype(np.float64)
+    ref = np.tile([2.0 ** 24 + 30, 0.0, 0.0, 1.0], B // 4)[:, None]
+    assert emb.status() == 0
+    assert np.max(np.abs(out - ref)) <= -(-31 // sums)   # the ones beside the first row (one less than its rows) and half a unit
+    assert np.all(out[1::4] == 0.0) and np.all(out[3::4] == 1.0)
