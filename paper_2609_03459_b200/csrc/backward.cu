@@ -1441,67 +1441,116 @@ __device__ __forceinline__ void tt_sweep_bwd_stream(const WsView& w, const Table
                 }
             }
             const float* st = rs.wait(slot);
-            // ---- dG_K[i_K] += C^T . dE
-            float acc[2][MT2][4];
-#pragma unroll
-            for (int tile = 0; tile < 2; ++tile)
+            if (nr <= 2) {
+                // a step of one or two rows: half of the products, k = (row, j) and n = (row, j) in the order row, j.  (As four rows, two
+                // of them zeros, a row's four terms went into dC as two sums, each truncated: gradients of the first core with one to
+                // three rows per group 6 to 10 % further from 64 bits, 3.43e-7 instead of 3.13e-7 with C of 4 rows, rank 16.)
+                float acc[MT2][4];
 #pragma unroll
                 for (int mt = 0; mt < MT2; ++mt)
 #pragma unroll
-                    for (int x = 0; x < 4; ++x) acc[tile][mt][x] = 0.f;
-            const float* El = st + rn * EP + 4 * t + 2 * (g & 1);
+                    for (int x = 0; x < 4; ++x) acc[mt][x] = 0.f;
+                const float* El = st + (g >> 2) * EP + 4 * t + (g & 3);
 #pragma unroll
-            for (int kt = 0; kt < KT2; ++kt) {
-                const float2 e0 = *reinterpret_cast<const float2*>(El + 32 * kt);
-                const float2 e1 = KHALF ? make_float2(0.f, 0.f) : *reinterpret_cast<const float2*>(El + 32 * kt + 16);
-                const Tf32Pair b0[2] = {tt_split_tf32(e0.x), tt_split_tf32(e1.x)}, b1[2] = {tt_split_tf32(e0.y), tt_split_tf32(e1.y)};
+                for (int kt = 0; kt < KT2; ++kt) {
+                    const Tf32Pair b[2] = {tt_split_tf32(El[32 * kt]), tt_split_tf32(KHALF ? 0.f : El[32 * kt + 16])};
 #pragma unroll
-                for (int mt = 0; mt < MT2; ++mt) {
-                    tt_mma_3xtf32(acc[0][mt], ct[mt][kt], b0);
-                    tt_mma_3xtf32(acc[1][mt], ct[mt][kt], b1);
+                    for (int mt = 0; mt < MT2; ++mt) tt_mma_3xtf32(acc[mt], ct[mt][kt], b);
                 }
-            }
-            // ---- dC += dE . D^T
-            const float* Et = st + t * EP + 4 * g;
-            const float* Dt = st + 4 * EP + t * DP + 4 * g;
-            auto split4 = [](Tf32Pair (&d)[4], const float4& v) { d[0] = tt_split_tf32(v.x); d[1] = tt_split_tf32(v.y); d[2] = tt_split_tf32(v.z); d[3] = tt_split_tf32(v.w); };
-            if constexpr (TR) {
-                Tf32Pair e[4];   // dE[p = g] of row t, j = 0..3
-                split4(e, PM == 8 || g < PM ? *reinterpret_cast<const float4*>(Et) : make_float4(0.f, 0.f, 0.f, 0.f));
-                const Tf32Pair b0[2] = {e[0], e[1]}, b1[2] = {e[2], e[3]};
+                const float* Et = st + 4 * g + t;
+                const float* Dt = st + 4 * EP + 4 * g + t;
+                if constexpr (TR) {
+                    const bool on = PM == 8 || g < PM;
+                    const Tf32Pair b[2] = {tt_split_tf32(on ? Et[0] : 0.f), tt_split_tf32(on ? Et[EP] : 0.f)};
 #pragma unroll
-                for (int mt = 0; mt < MT2; ++mt) {
-                    Tf32Pair x[4], y[4];
-                    split4(x, *reinterpret_cast<const float4*>(Dt + 64 * mt));
-                    split4(y, BHALF ? make_float4(0.f, 0.f, 0.f, 0.f) : *reinterpret_cast<const float4*>(Dt + 64 * mt + 32));
-                    const Tf32Pair a0[4] = {x[0], y[0], x[1], y[1]}, a1[4] = {x[2], y[2], x[3], y[3]};
-                    tt_mma_3xtf32(dc[mt][0], a0, b0);
-                    tt_mma_3xtf32(dc[mt][0], a1, b1);
-                }
-            } else {
+                    for (int mt = 0; mt < MT2; ++mt) {
+                        const Tf32Pair a[4] = {tt_split_tf32(Dt[64 * mt]), tt_split_tf32(BHALF ? 0.f : Dt[64 * mt + 32]),
+                                               tt_split_tf32(Dt[DP + 64 * mt]), tt_split_tf32(BHALF ? 0.f : Dt[DP + 64 * mt + 32])};
+                        tt_mma_3xtf32(dc[mt][0], a, b);
+                    }
+                } else {
 #pragma unroll
-                for (int mt = 0; mt < MT; ++mt) {
-                    Tf32Pair x[4], y[4];
-                    split4(x, *reinterpret_cast<const float4*>(Et + 64 * mt));
-                    split4(y, *reinterpret_cast<const float4*>(Et + 64 * mt + 32));
-                    const Tf32Pair a0[4] = {x[0], y[0], x[1], y[1]}, a1[4] = {x[2], y[2], x[3], y[3]};
+                    for (int mt = 0; mt < MT; ++mt) {
+                        const Tf32Pair a[4] = {tt_split_tf32(Et[64 * mt]), tt_split_tf32(Et[64 * mt + 32]), tt_split_tf32(Et[EP + 64 * mt]), tt_split_tf32(Et[EP + 64 * mt + 32])};
 #pragma unroll
-                    for (int nt = 0; nt < NT; ++nt) {
-                        Tf32Pair d[4];
-                        split4(d, *reinterpret_cast<const float4*>(Dt + 32 * nt));
-                        const Tf32Pair b0[2] = {d[0], d[1]}, b1[2] = {d[2], d[3]};
-                        tt_mma_3xtf32(dc[mt][nt], a0, b0);
-                        tt_mma_3xtf32(dc[mt][nt], a1, b1);
+                        for (int nt = 0; nt < NT; ++nt) {
+                            const Tf32Pair b[2] = {tt_split_tf32(Dt[32 * nt]), tt_split_tf32(Dt[DP + 32 * nt])};
+                            tt_mma_3xtf32(dc[mt][nt], a, b);
+                        }
                     }
                 }
+                if ((uint32_t)(t >> 1) < nr) {
+                    float* dst = gk + (size_t)rs.ids(s)[t >> 1] * (RB_ * 4) + 4 * g + 2 * (t & 1);
+#pragma unroll
+                    for (int mt = 0; mt < MT2; ++mt) {
+                        tt_red_v2(dst + 64 * mt, acc[mt][0], acc[mt][1]);
+                        if (!BHALF) tt_red_v2(dst + 64 * mt + 32, acc[mt][2], acc[mt][3]);
+                    }
+                }
+                chain += 1;
+            } else {
+                // ---- dG_K[i_K] += C^T . dE
+                float acc[2][MT2][4];
+    #pragma unroll
+                for (int tile = 0; tile < 2; ++tile)
+    #pragma unroll
+                    for (int mt = 0; mt < MT2; ++mt)
+    #pragma unroll
+                        for (int x = 0; x < 4; ++x) acc[tile][mt][x] = 0.f;
+                const float* El = st + rn * EP + 4 * t + 2 * (g & 1);
+    #pragma unroll
+                for (int kt = 0; kt < KT2; ++kt) {
+                    const float2 e0 = *reinterpret_cast<const float2*>(El + 32 * kt);
+                    const float2 e1 = KHALF ? make_float2(0.f, 0.f) : *reinterpret_cast<const float2*>(El + 32 * kt + 16);
+                    const Tf32Pair b0[2] = {tt_split_tf32(e0.x), tt_split_tf32(e1.x)}, b1[2] = {tt_split_tf32(e0.y), tt_split_tf32(e1.y)};
+    #pragma unroll
+                    for (int mt = 0; mt < MT2; ++mt) {
+                        tt_mma_3xtf32(acc[0][mt], ct[mt][kt], b0);
+                        tt_mma_3xtf32(acc[1][mt], ct[mt][kt], b1);
+                    }
+                }
+                // ---- dC += dE . D^T
+                const float* Et = st + t * EP + 4 * g;
+                const float* Dt = st + 4 * EP + t * DP + 4 * g;
+                auto split4 = [](Tf32Pair (&d)[4], const float4& v) { d[0] = tt_split_tf32(v.x); d[1] = tt_split_tf32(v.y); d[2] = tt_split_tf32(v.z); d[3] = tt_split_tf32(v.w); };
+                if constexpr (TR) {
+                    Tf32Pair e[4];   // dE[p = g] of row t, j = 0..3
+                    split4(e, PM == 8 || g < PM ? *reinterpret_cast<const float4*>(Et) : make_float4(0.f, 0.f, 0.f, 0.f));
+                    const Tf32Pair b0[2] = {e[0], e[1]}, b1[2] = {e[2], e[3]};
+    #pragma unroll
+                    for (int mt = 0; mt < MT2; ++mt) {
+                        Tf32Pair x[4], y[4];
+                        split4(x, *reinterpret_cast<const float4*>(Dt + 64 * mt));
+                        split4(y, BHALF ? make_float4(0.f, 0.f, 0.f, 0.f) : *reinterpret_cast<const float4*>(Dt + 64 * mt + 32));
+                        const Tf32Pair a0[4] = {x[0], y[0], x[1], y[1]}, a1[4] = {x[2], y[2], x[3], y[3]};
+                        tt_mma_3xtf32(dc[mt][0], a0, b0);
+                        tt_mma_3xtf32(dc[mt][0], a1, b1);
+                    }
+                } else {
+    #pragma unroll
+                    for (int mt = 0; mt < MT; ++mt) {
+                        Tf32Pair x[4], y[4];
+                        split4(x, *reinterpret_cast<const float4*>(Et + 64 * mt));
+                        split4(y, *reinterpret_cast<const float4*>(Et + 64 * mt + 32));
+                        const Tf32Pair a0[4] = {x[0], y[0], x[1], y[1]}, a1[4] = {x[2], y[2], x[3], y[3]};
+    #pragma unroll
+                        for (int nt = 0; nt < NT; ++nt) {
+                            Tf32Pair d[4];
+                            split4(d, *reinterpret_cast<const float4*>(Dt + 32 * nt));
+                            const Tf32Pair b0[2] = {d[0], d[1]}, b1[2] = {d[2], d[3]};
+                            tt_mma_3xtf32(dc[mt][nt], a0, b0);
+                            tt_mma_3xtf32(dc[mt][nt], a1, b1);
+                        }
+                    }
+                }
+                float* dst = gk + (size_t)rs.ids(s)[rc] * (RB_ * 4) + 4 * g;
+    #pragma unroll
+                for (int mt = 0; mt < MT2; ++mt)
+    #pragma unroll
+                    for (int h = 0; h < (BHALF ? 1 : 2); ++h)
+                        tt_red_v4_if((uint32_t)rc < nr, dst + (16 * mt + 8 * h) * 4, acc[0][mt][2 * h], acc[1][mt][2 * h], acc[0][mt][2 * h + 1], acc[1][mt][2 * h + 1]);
+                chain += 2;
             }
-            float* dst = gk + (size_t)rs.ids(s)[rc] * (RB_ * 4) + 4 * g;
-#pragma unroll
-            for (int mt = 0; mt < MT2; ++mt)
-#pragma unroll
-                for (int h = 0; h < (BHALF ? 1 : 2); ++h)
-                    tt_red_v4_if((uint32_t)rc < nr, dst + (16 * mt + 8 * h) * 4, acc[0][mt][2 * h], acc[1][mt][2 * h], acc[0][mt][2 * h + 1], acc[1][mt][2 * h + 1]);
-            chain += 2;
             __syncwarp();
             rs.stage(slot, w.E, lane);
             slot = slot + 1 == PD ? 0 : slot + 1;

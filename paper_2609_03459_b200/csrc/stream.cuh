@@ -13,11 +13,7 @@
 #pragma once
 #include "common.cuh"
 
-// 16-byte asynchronous copy global -> shared (32-bit address), past L1; _or_zero: zeros instead of the source where !some
-__device__ __forceinline__ void tt_cp_async16_s(uint32_t smem_dst, const void* gsrc)
-{
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_dst), "l"(gsrc) : "memory");
-}
+// 16-byte asynchronous copy global -> shared (32-bit address), past L1; zeros instead of the source where !some
 __device__ __forceinline__ void tt_cp_async16_or_zero(uint32_t smem_dst, const void* gsrc, bool some)
 {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_dst), "l"(gsrc), "r"(some ? 16u : 0u) : "memory");
@@ -117,7 +113,9 @@ struct RowStream {
 #pragma unroll
             for (int x = 0; x < 4 * RB / 32; ++x) {
                 const int r = lane / RB + x * (32 / RB);
-                tt_cp_async16_s(dst + (4 * EP + r * DP + 4 * (lane % RB)) * 4, GK + (size_t)id[x * (32 / RB)] * (RB * 4));
+                const uint32_t to = dst + (4 * EP + r * DP + 4 * (lane % RB)) * 4;
+                const float* from = GK + (size_t)id[x * (32 / RB)] * (RB * 4);
+                tt_cp_async16_or_zero(to, from, (uint32_t)r < nr);
             }
             ++next;
         }

@@ -96,3 +96,23 @@ def test_rebuilt_products_of_rank_8_in_fp32(binding, ra, b):  # noqa: F811
     lookups = np.bincount(wl.indices % 5, minlength=5)
     ref = np.broadcast_to((16.0 * (x - 1.0) * lookups)[None, :, None, None], got.shape)
     assert np.max(np.abs(got - ref)) <= 2.0 ** -21 * np.max(ref)   # sums of at most 120 exact terms of 13 bits
+
+
+@pytest.mark.parametrize("d,r", [s for s in SHAPES if s != ((2, 4, 4), (5, 8))])   # (8 x 8 is left to fp32 multiply-adds)
+@pytest.mark.parametrize("rows", [1, 2, 5])
+def test_gradient_of_a_product_in_one_sum_per_pair_of_rows(binding, d, r, rows):  # noqa: F811
+    # A row's part of dC is 1 + 2^-24 + 2^-24 + 0: one sum of four terms gives 1 + 2^-23 (the tensor core keeps bits below the last one
+    # until it truncates the result), two terms and then two give 1.  Rows of zeros beside it must not split it.
+    n = (1, 1, 8)
+    spec = TableSpec(N=8, n=n, d=d, r=(1,) + r + (1,), alpha=1.0, core_dist="normal", core_scale=0.3)
+    wl = workloads.custom([spec], rows, 1, seed=1, with_grad=True)
+    wl.indices = np.arange(rows, dtype=np.int64)
+    g = [np.zeros_like(c) for c in wl.cores[0]]
+    g[0][0, 0, 0, 0] = 1.0                                  # P_1: one row, one column
+    g[2][:, rows - 1, :, 0] = [1.0, 2.0 ** -24, 2.0 ** -24, 0.0]
+    wl.cores = [g]
+    emb = binding.from_workload(wl, enable_backward=True)
+    emb.forward(dev(wl.indices), dev(wl.offsets), wl.B)
+    emb.backward(dev(np.ones((wl.B, int(np.prod(d))), dtype=np.float32)))
+    got = emb.get_grads()[0][1][0, 0].astype(np.float64)    # [d_2, r_2]: dC of the first row of P_1
+    assert np.all(got == 1.0 + 2.0 ** -23)
