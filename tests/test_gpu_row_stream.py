@@ -1,6 +1,7 @@
 """Backward sweeps that stream the rows of a batch of groups (ranks 8 and 16 with C of 16, 8 and 4 rows, rank 32 with C of 4 rows):
 groups of 1 to 5 rows (a step holds four), around 32 rows (a block of steps, where sums of dC are handed over) and of several
-hundred rows, in ranks that are no multiple of eight before them, three and four cores, and rows dropped at the row capacity.
+hundred rows, in ranks that are no multiple of eight before them, three and four cores (the left operand through the parent),
+rows and prefixes dropped at the row capacity; rebuilt products of rank 8 and gradients of short groups as exact as without the stream.
 
 Bar: max|err| <= 1e-5 * max|ref|, the bound of the other parity tests (fp32 sums, 3xTF32 products)."""
 import numpy as np
@@ -116,3 +117,54 @@ def test_gradient_of_a_product_in_one_sum_per_pair_of_rows(binding, d, r, rows):
     emb.backward(dev(np.ones((wl.B, int(np.prod(d))), dtype=np.float32)))
     got = emb.get_grads()[0][1][0, 0].astype(np.float64)    # [d_2, r_2]: dC of the first row of P_1
     assert np.all(got == 1.0 + 2.0 ** -23)
+
+
+@pytest.mark.parametrize("d,r,variant", [((2, 2, 4, 4), (5, 16, 16), 1), ((2, 2, 4, 4), (3, 8, 8), 2), ((1, 4, 4, 4), (4, 5, 16), 1), ((1, 4, 4, 4), (3, 7, 8), 2),
+                                         ((2, 1, 4, 4), (3, 16, 16), 6), ((2, 1, 2, 4), (4, 32, 32), 8), ((2, 1, 2, 4), (4, 16, 16), 9)])
+@pytest.mark.parametrize("n,sizes", [((3, 2, 7, 9), (1, 2, 3, 4, 5)), ((2, 2, 5, 140), (31, 32, 33, 1, 34, 64, 128, 140)), ((7, 5, 5, 6), (1, 6, 2))])
+def test_four_cores(binding, d, r, variant, n, sizes):  # noqa: F811
+    spec = TableSpec(N=int(np.prod(n)), n=n, d=d, r=(1,) + r + (1,), alpha=1.0, core_dist="normal", core_scale=0.3)
+    rng = np.random.default_rng(len(sizes) + n[3])
+    T, B = 2, 50
+    wl = workloads.custom([spec] * T, B, 1, seed=1, with_grad=True)
+    per_table = [ids_with_groups((n[0] * n[1], n[2], n[3]), sizes, rng) for _ in range(T)]
+    per_table = [rng.permutation(np.concatenate([x, rng.choice(x, 40)])) for x in per_table]
+    wl.indices = np.concatenate(per_table).astype(np.int64)
+    starts = np.concatenate([[0], np.cumsum([len(x) for x in per_table])])
+    cuts = [np.sort(rng.integers(a, b + 1, B - 1)) for a, b in zip(starts, starts[1:])]
+    wl.offsets = np.concatenate([np.concatenate([[a], c]) for a, c in zip(starts, cuts)] + [starts[-1:]]).astype(np.int64)
+    emb = binding.from_workload(wl, enable_backward=True)
+    assert emb.table_variant(0) == variant
+    out = emb.forward(dev(wl.indices), dev(wl.offsets), B)
+    assert_close(out.cpu().numpy(), oracle.forward_workload(wl), "out")
+    emb.backward(dev(wl.grad_out))
+    grads, ref = emb.get_grads(), oracle.backward_workload(wl)
+    for t in range(T):
+        for k in range(4):
+            assert_close(grads[t][k], ref[t][k], f"dG[{t}][{k}]")
+    assert emb.status() == 0 and emb.check_guards() is None
+
+
+@pytest.mark.parametrize("d,r", [((4, 4, 4), (16, 16)), ((2, 2, 4), (32, 32)), ((4, 8, 4), (32, 32)), ((3, 4, 5), (4, 3))])   # units of equal group counts; the last by cost
+@pytest.mark.parametrize("L", [700, 40_000])     # one cluster; marks of the digit-major order beside the row scan
+def test_prefixes_dropped_at_the_capacity(binding, d, r, L):  # noqa: F811
+    # 900 prefixes and more in a batch with room for 77 nodes: the marks made from all prefixes are made again from those that are kept
+    spec = TableSpec(N=1920, n=(30, 32, 2), d=d, r=(1,) + r + (1,), alpha=1.0, core_dist="normal", core_scale=0.3)
+    B, cap = 60, 77
+    wl = workloads.custom([spec], B, 1, seed=4, with_grad=True)
+    rng = np.random.default_rng(L)
+    wl.indices = rng.integers(0, 1920, L).astype(np.int64)
+    wl.offsets = np.concatenate([[0], np.sort(rng.integers(0, L + 1, B - 1)), [L]]).astype(np.int64)
+    kept = np.unique(wl.indices)[:cap]
+    emb = binding.from_workload(wl, enable_backward=True, max_unique_rows=cap)
+    emb.forward(dev(wl.indices), dev(wl.offsets), B)
+    assert emb.status() == binding.STATUS_OVERFLOW
+    emb.backward(dev(wl.grad_out))
+    grads = emb.get_grads()
+    keep = np.isin(wl.indices, kept)
+    wl.offsets = np.concatenate([[0], np.cumsum(keep)])[wl.offsets].astype(np.int64)
+    wl.indices = wl.indices[keep]
+    ref = oracle.backward_workload(wl)
+    for k in range(3):
+        assert_close(grads[0][k], ref[0][k], f"dG[0][{k}]")
+    assert emb.check_guards() is None
