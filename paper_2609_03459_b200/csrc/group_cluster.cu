@@ -31,102 +31,118 @@ __device__ __forceinline__ void gc_sync()
 // elements that each CTA takes
 __device__ __forceinline__ uint32_t gc_run(uint32_t n) { return (n + GC_CTAS - 1) / GC_CTAS; }
 
-// Exclusive scan of f over n elements: every CTA takes a run of them.  The CTAs' sums go straight into the shared memory of
-// all sixteen (`sums`, a slot of its own for every scan of the kernel); a run of up to GC_TILE elements stays in registers
-// between the sum and the second pass.  One barrier inside, none at the end.
 #define GC_IT 4
 #define GC_TILE (GC_THREADS * GC_IT)
+// Values of one tile of the CTA's run [.., hi): ex holds their exclusive prefixes inside their warps, sm the warps' (element order: stripe j,
+// then warp); the tile's sum comes back.
 template <class F>
-__device__ __forceinline__ void gc_scan(const F& f, uint32_t n, uint32_t* sums, uint32_t* sm)
+__device__ __forceinline__ uint32_t gc_load(const F& f, uint32_t base, uint32_t hi, int& hint, uint32_t (&v)[GC_IT], uint32_t (&ex)[GC_IT], int (&at)[GC_IT], uint32_t* sm)
 {
-    const uint32_t rank = blockIdx.x, tid = threadIdx.x;
-    const uint32_t per = gc_run(n);
-    const uint32_t lo = min(n, rank * per), hi = min(n, lo + per);
+    const uint32_t tid = threadIdx.x;
     const int lane = tid & 31, wid = tid >> 5;
-    int hint = lo < hi ? f.locate(lo) : 0;
-    uint32_t v[GC_IT], ex[GC_IT];
-    int at[GC_IT];
-    uint32_t carry = 0, tot = 0;
-    // values of one tile; exclusive prefixes of its elements inside their warps, the warps' in sm
-    auto load = [&](uint32_t base) {
 #pragma unroll
-        for (int j = 0; j < GC_IT; ++j) {
-            const uint32_t i = base + (uint32_t)j * GC_THREADS + tid;
-            v[j] = 0;
-            if (i < hi) {
-                hint = f.locate_from(i, hint);
-                v[j] = f.value(i, hint);
-            }
-            at[j] = hint;
+    for (int j = 0; j < GC_IT; ++j) {
+        const uint32_t i = base + (uint32_t)j * GC_THREADS + tid;
+        v[j] = 0;
+        if (i < hi) {
+            hint = f.locate_from(i, hint);
+            v[j] = f.value(i, hint);
         }
-#pragma unroll
-        for (int j = 0; j < GC_IT; ++j) {
-            const uint32_t a = base + (uint32_t)j * GC_THREADS + tid < hi ? tt_scan_amount(f, v[j], 0) : 0u;
-            uint32_t incl = a;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
-                if (lane >= o) incl += y;
-            }
-            ex[j] = incl - a;
-            if (lane == 31) sm[j * (GC_THREADS / 32) + wid] = incl;   // element order: stripe j, then warp
-        }
-        __syncthreads();
-        if (wid == 0) {   // exclusive scan of the warps' sums, GC_IT per lane
-            uint32_t x[GC_IT], s = 0;
-#pragma unroll
-            for (int j = 0; j < GC_IT; ++j) { x[j] = sm[lane * GC_IT + j]; s += x[j]; }
-            uint32_t incl = s;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
-                if (lane >= o) incl += y;
-            }
-            uint32_t run = incl - s;
-#pragma unroll
-            for (int j = 0; j < GC_IT; ++j) { sm[lane * GC_IT + j] = run; run += x[j]; }
-            if (lane == 31) sm[GC_THREADS / 32 * GC_IT] = run;
-        }
-        __syncthreads();
-        tot = sm[GC_THREADS / 32 * GC_IT];
-    };
-    auto emit = [&](uint32_t base) {
-#pragma unroll
-        for (int j = 0; j < GC_IT; ++j) {
-            const uint32_t i = base + (uint32_t)j * GC_THREADS + tid;
-            if (i < hi) f.emit(i, carry + sm[j * (GC_THREADS / 32) + wid] + ex[j], v[j], at[j]);
-        }
-        carry += tot;
-    };
-    const bool one = per <= GC_TILE;
-    if (one) load(lo);
-    else {
-        uint32_t amount = 0;
-        for (uint32_t i = lo + tid; i < hi; i += GC_THREADS) amount += tt_scan_amount(f, f.value(i, hint), 0);
-        tt_block_excl_scan(amount, sm, tot);
+        at[j] = hint;
     }
-    if (tid < GC_CTAS) {   // this CTA's sum to every CTA
+    __syncthreads();        // the warps' sums of the tile (or scan) before are read
+#pragma unroll
+    for (int j = 0; j < GC_IT; ++j) {
+        const uint32_t a = base + (uint32_t)j * GC_THREADS + tid < hi ? tt_scan_amount(f, v[j], 0) : 0u;
+        uint32_t incl = a;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += y;
+        }
+        ex[j] = incl - a;
+        if (lane == 31) sm[j * (GC_THREADS / 32) + wid] = incl;
+    }
+    __syncthreads();
+    if (wid == 0) {   // exclusive scan of the warps' sums, GC_IT per lane
+        uint32_t x[GC_IT], s = 0;
+#pragma unroll
+        for (int j = 0; j < GC_IT; ++j) { x[j] = sm[lane * GC_IT + j]; s += x[j]; }
+        uint32_t incl = s;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += y;
+        }
+        uint32_t run = incl - s;
+#pragma unroll
+        for (int j = 0; j < GC_IT; ++j) { sm[lane * GC_IT + j] = run; run += x[j]; }
+        if (lane == 31) sm[GC_THREADS / 32 * GC_IT] = run;
+    }
+    __syncthreads();
+    return sm[GC_THREADS / 32 * GC_IT];
+}
+template <class F>
+__device__ __forceinline__ void gc_store(const F& f, uint32_t base, uint32_t hi, uint32_t carry, const uint32_t (&v)[GC_IT], const uint32_t (&ex)[GC_IT], const int (&at)[GC_IT], const uint32_t* sm)
+{
+#pragma unroll
+    for (int j = 0; j < GC_IT; ++j) {
+        const uint32_t i = base + (uint32_t)j * GC_THREADS + threadIdx.x;
+        if (i < hi) f.emit(i, carry + sm[j * (GC_THREADS / 32) + (threadIdx.x >> 5)] + ex[j], v[j], at[j]);
+    }
+}
+// this CTA's sum into the shared memory of all sixteen, by their first GC_CTAS threads (or those of a warp)
+__device__ __forceinline__ void gc_tell(uint32_t* sums, uint32_t tot, uint32_t thread)
+{
+    if (thread < GC_CTAS) {
         uint32_t remote;
-        const uint32_t local = (uint32_t)__cvta_generic_to_shared(sums + rank);
-        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(local), "r"(tid));
+        const uint32_t local = (uint32_t)__cvta_generic_to_shared(sums + blockIdx.x);
+        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(local), "r"(thread));
         asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(remote), "r"(tot) : "memory");
     }
-    gc_sync();
-    uint32_t all = 0;
+}
+// sum of the CTAs before this one; the first CTA reports that of all
+template <class F>
+__device__ __forceinline__ uint32_t gc_carry(const F& f, const uint32_t* sums)
+{
+    uint32_t carry = 0, all = 0;
 #pragma unroll
     for (uint32_t i = 0; i < GC_CTAS; ++i) {
         const uint32_t x = sums[i];
-        carry += i < rank ? x : 0u;
+        carry += i < blockIdx.x ? x : 0u;
         all += x;
     }
-    if (rank == 0 && tid == 0) f.total(all);
-    if (one) emit(lo);
+    if (blockIdx.x == 0 && threadIdx.x == 0) f.total(all);
+    return carry;
+}
+
+// Exclusive scan of f over n elements: every CTA takes a run of them.  The CTAs' sums go straight into the shared memory of
+// all sixteen (`sums`, a slot of its own for every scan of the kernel); a run of up to GC_TILE elements stays in registers
+// between the sum and the second pass.  One barrier inside, none at the end.
+template <class F>
+__device__ __forceinline__ void gc_scan(const F& f, uint32_t n, uint32_t* sums, uint32_t* sm)
+{
+    const uint32_t per = gc_run(n), lo = min(n, blockIdx.x * per), hi = min(n, lo + per);
+    int hint = lo < hi ? f.locate(lo) : 0;
+    uint32_t v[GC_IT], ex[GC_IT], tot = 0;
+    int at[GC_IT];
+    const bool one = per <= GC_TILE;
+    if (one) tot = gc_load(f, lo, hi, hint, v, ex, at, sm);
+    else {
+        uint32_t amount = 0;
+        for (uint32_t i = lo + threadIdx.x; i < hi; i += GC_THREADS) amount += tt_scan_amount(f, f.value(i, hint), 0);
+        tt_block_excl_scan(amount, sm, tot);
+    }
+    gc_tell(sums, tot, threadIdx.x);
+    gc_sync();
+    uint32_t carry = gc_carry(f, sums);
+    if (one) gc_store(f, lo, hi, carry, v, ex, at, sm);
     else
         for (uint32_t base = lo; base < hi; base += GC_TILE) {
             hint = base == lo ? f.locate(lo) : hint;
-            load(base);
-            emit(base);
-            __syncthreads();
+            tot = gc_load(f, base, hi, hint, v, ex, at, sm);
+            gc_store(f, base, hi, carry, v, ex, at, sm);
+            carry += tot;
         }
 }
 
@@ -147,80 +163,19 @@ __device__ __forceinline__ void gc_exchange(uint32_t (*warp_sums)[GC_THREADS / 3
 {
     const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     __syncthreads();
-    if (wid < (uint32_t)scans) {
-        const uint32_t tot = __reduce_add_sync(0xffffffffu, warp_sums[wid][lane]);
-        if (lane < GC_CTAS) {
-            uint32_t remote;
-            const uint32_t local = (uint32_t)__cvta_generic_to_shared(&sums[wid][blockIdx.x]);
-            asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(local), "r"(lane));
-            asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(remote), "r"(tot) : "memory");
-        }
-    }
+    if (wid < (uint32_t)scans) gc_tell(sums[wid], __reduce_add_sync(0xffffffffu, warp_sums[wid][lane]), lane);
     gc_sync();
 }
 template <class F>
 __device__ __forceinline__ void gc_emit(const F& f, uint32_t n, const uint32_t* sums, uint32_t* sm)
 {
-    const uint32_t rank = blockIdx.x, tid = threadIdx.x, per = gc_run(n), lo = min(n, rank * per), hi = min(n, lo + per);
-    const int lane = tid & 31, wid = tid >> 5;
-    uint32_t carry = 0, all = 0;
-#pragma unroll
-    for (uint32_t i = 0; i < GC_CTAS; ++i) {
-        const uint32_t x = sums[i];
-        carry += i < rank ? x : 0u;
-        all += x;
-    }
-    if (rank == 0 && tid == 0) f.total(all);
-    int hint = lo < hi ? f.locate(lo) : 0;
+    const uint32_t per = gc_run(n), lo = min(n, blockIdx.x * per), hi = min(n, lo + per);
+    uint32_t v[GC_IT], ex[GC_IT], carry = gc_carry(f, sums);
+    int at[GC_IT], hint = lo < hi ? f.locate(lo) : 0;
     for (uint32_t base = lo; base < hi; base += GC_TILE) {
-        uint32_t v[GC_IT], ex[GC_IT];
-        int at[GC_IT];
-#pragma unroll
-        for (int j = 0; j < GC_IT; ++j) {
-            const uint32_t i = base + (uint32_t)j * GC_THREADS + tid;
-            v[j] = 0;
-            if (i < hi) {
-                hint = f.locate_from(i, hint);
-                v[j] = f.value(i, hint);
-            }
-            at[j] = hint;
-        }
-        __syncthreads();        // the warps' sums of the tile (or scan) before are read
-#pragma unroll
-        for (int j = 0; j < GC_IT; ++j) {
-            const uint32_t a = base + (uint32_t)j * GC_THREADS + tid < hi ? tt_scan_amount(f, v[j], 0) : 0u;
-            uint32_t incl = a;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
-                if (lane >= o) incl += y;
-            }
-            ex[j] = incl - a;
-            if (lane == 31) sm[j * (GC_THREADS / 32) + wid] = incl;   // element order: stripe j, then warp
-        }
-        __syncthreads();
-        if (wid == 0) {   // exclusive scan of the warps' sums, GC_IT per lane
-            uint32_t x[GC_IT], s = 0;
-#pragma unroll
-            for (int j = 0; j < GC_IT; ++j) { x[j] = sm[lane * GC_IT + j]; s += x[j]; }
-            uint32_t incl = s;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
-                if (lane >= o) incl += y;
-            }
-            uint32_t run = incl - s;
-#pragma unroll
-            for (int j = 0; j < GC_IT; ++j) { sm[lane * GC_IT + j] = run; run += x[j]; }
-            if (lane == 31) sm[GC_THREADS / 32 * GC_IT] = run;
-        }
-        __syncthreads();
-#pragma unroll
-        for (int j = 0; j < GC_IT; ++j) {
-            const uint32_t i = base + (uint32_t)j * GC_THREADS + tid;
-            if (i < hi) f.emit(i, carry + sm[j * (GC_THREADS / 32) + wid] + ex[j], v[j], at[j]);
-        }
-        carry += sm[GC_THREADS / 32 * GC_IT];
+        const uint32_t tot = gc_load(f, base, hi, hint, v, ex, at, sm);
+        gc_store(f, base, hi, carry, v, ex, at, sm);
+        carry += tot;
     }
 }
 
