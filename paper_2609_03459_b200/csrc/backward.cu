@@ -514,8 +514,8 @@ __global__ void __launch_bounds__(256, 5) k_dE_fast(WsView w, const float* __res
     }
 }
 
-// D = 64 (256-byte rows): the 32 grad_out rows of a batch of sorted positions are fetched into an 8 KB per-warp
-// buffer with cp.async (all in flight at once, no staging registers), then every lane walks the batch in position
+// The 32 grad_out rows of a batch of sorted positions are fetched into a per-warp buffer (8 KB with D = 64) with
+// cp.async (all in flight at once, no staging registers), then every lane walks the batch in position
 // order owning two of the 64 columns: one shared-memory load and two adds per row, a coalesced 256-byte store when a
 // segment ends, and no shuffles to combine partial sums.  About half the instructions per lookup of k_dE_fast, which
 // was bound by instruction issue.  Chunks, carries and the fix-up pass are those of k_dE / k_dE_fast.
@@ -1471,7 +1471,8 @@ __device__ __forceinline__ void tt_sweep_bwd_stream(const WsView& w, const Table
                 } else {
 #pragma unroll
                     for (int mt = 0; mt < MT; ++mt) {
-                        const Tf32Pair a[4] = {tt_split_tf32(Et[64 * mt]), tt_split_tf32(Et[64 * mt + 32]), tt_split_tf32(Et[EP + 64 * mt]), tt_split_tf32(Et[EP + 64 * mt + 32])};
+                        const Tf32Pair a[4] = {tt_split_tf32(Et[64 * mt]), tt_split_tf32(Et[64 * mt + 32]),
+                                               tt_split_tf32(Et[EP + 64 * mt]), tt_split_tf32(Et[EP + 64 * mt + 32])};
 #pragma unroll
                         for (int nt = 0; nt < NT; ++nt) {
                             const Tf32Pair b[2] = {tt_split_tf32(Dt[32 * nt]), tt_split_tf32(Dt[DP + 32 * nt])};
@@ -1512,7 +1513,9 @@ __device__ __forceinline__ void tt_sweep_bwd_stream(const WsView& w, const Table
                 // ---- dC += dE . D^T
                 const float* Et = st + t * EP + 4 * g;
                 const float* Dt = st + 4 * EP + t * DP + 4 * g;
-                auto split4 = [](Tf32Pair (&d)[4], const float4& v) { d[0] = tt_split_tf32(v.x); d[1] = tt_split_tf32(v.y); d[2] = tt_split_tf32(v.z); d[3] = tt_split_tf32(v.w); };
+                auto split4 = [](Tf32Pair (&d)[4], const float4& v) {
+                    d[0] = tt_split_tf32(v.x); d[1] = tt_split_tf32(v.y); d[2] = tt_split_tf32(v.z); d[3] = tt_split_tf32(v.w);
+                };
                 if constexpr (TR) {
                     Tf32Pair e[4];   // dE[p = g] of row t, j = 0..3
                     split4(e, PM == 8 || g < PM ? *reinterpret_cast<const float4*>(Et) : make_float4(0.f, 0.f, 0.f, 0.f));
@@ -1548,7 +1551,8 @@ __device__ __forceinline__ void tt_sweep_bwd_stream(const WsView& w, const Table
                 for (int mt = 0; mt < MT2; ++mt)
     #pragma unroll
                     for (int h = 0; h < (BHALF ? 1 : 2); ++h)
-                        tt_red_v4_if((uint32_t)rc < nr, dst + (16 * mt + 8 * h) * 4, acc[0][mt][2 * h], acc[1][mt][2 * h], acc[0][mt][2 * h + 1], acc[1][mt][2 * h + 1]);
+                        tt_red_v4_if((uint32_t)rc < nr, dst + (16 * mt + 8 * h) * 4, acc[0][mt][2 * h], acc[1][mt][2 * h],
+                                     acc[0][mt][2 * h + 1], acc[1][mt][2 * h + 1]);
                 chain += 2;
             }
             __syncwarp();

@@ -18,9 +18,11 @@
 #define TT_PSCAN_ITEMS 4                                // the scan of row bitmaps of up to TT_PSCAN_WORDS words
 #define TT_PSCAN_WORDS (1u << 21)
 // up to so many words, from so many lookups and from one per word on, tiles of half that size: the densest tile, whose rows one CTA
-// lists, takes half as long, and there are twice as many others.  Calls with tiles of 1024 / 512 words, us: 4 M lookups 772 / 763, 1.6 M
-// 591 / 586, one table, 0.7 M 216 / 212, 0.5 M 327 / 325; 65 k 408.7 / 410.1, 8 k 60.8 / 64.3 (all in 0.26 M to 0.57 M words); 0.94 M words, 0.7 M
-// lookups 193 / 191, of spread rows 184.6 / 188.4
+// lists, takes half as long, and there are twice as many others.  Forward calls of 1, 2, 4 and 8 tables of 1 M to 40 M rows, D = 16, with
+// 512-word tiles relative to 1024: up to 0.5 M words, 0.26 to 4 M lookups, popular rows first 0.95 to 0.99 (one table of 31 k words, 1 M
+// lookups 144.4 / 138.4 us; 0.5 M words, 0.26 M lookups 111.6 / 105.5), spread rows 0.96 to 1.0; 16 k and 65 k lookups 0.97 to 1.03; 0.78 M
+// words 0.98 to 1.02 (spread 173 / 175); 1 M words and more 0.99 to 1.04, with 16 k to 65 k lookups 1.02 to 1.08 (81 / 85).  The line
+// lies between 0.5 and 0.78 M words.
 #define TT_PSCAN_FINE_WORDS 655360u
 #define TT_PSCAN_FINE_LOOKUPS (1 << 18)
 // most lookups whose marking pass also checks the offsets: one launch less, but the tables' ranges come from all over the
@@ -111,7 +113,7 @@ struct WsView {
     uint32_t* tb[TT_MAXK + 1];          // [T+1] node range of each table at level k
     uint32_t* cost;                     // [cap_{K-1}+1] exclusive scan of per-group cost (+ total)
     int64_t pool_shares;                // shares of the lookups in the pooling pass (0: it takes no shares)
-    int64_t* pool_bounds;               // [shares + 1] first bag of every share of the pooling pass (tt_pool_bound)
+    int64_t* pool_bounds;               // [shares + 1] first bag of every share of the pooling pass (group.cuh)
     uint2* unit_rng;                    // [T * units per table] group range of every work unit (tt_unit_bounds)
     int32_t units_per_table;
     float* pbuf[TT_MAXK + 1];           // partial products P_k of level-k nodes, 2 <= k <= K-2

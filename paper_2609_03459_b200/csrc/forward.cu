@@ -734,7 +734,7 @@ __device__ __forceinline__ uint32_t tt_lookup_slot(const WsView& w, const TableD
     return slot;
 }
 
-// Pooling partition: the lookups are cut into C = W * chunks equal shares of whole bags (tt_pool_bound), and the
+// Pooling partition: the lookups are cut into C = W * chunks equal shares of whole bags (boundaries: group.cuh), and the
 // warps take the shares in order from a counter.  All resident warps therefore work inside one moving window of
 // about W shares at a time - a few tables - so the rows that several bags share are still in L2 when the next
 // bag asks for them; one contiguous share per warp would spread the warps over all tables at once.  Equal lookups are
@@ -1019,14 +1019,14 @@ __global__ void __launch_bounds__(32 * POOL_WARPS, 4) k_pool_async(WsView w, flo
 // mean pooling take the same ways (the factor with the row, 1 / length where a bag is written): 131 k bags of 1 to 30 weighted
 // rows of 128 bytes 73 -> 63 us, of 1 to 8 rows of 256 bytes with mean 51 -> 41 us, of one weighted row 33 -> 17 us against
 // bag by bag.
-// 2 million bags of 128-byte rows, stream against one bag per window: 2 / 4 / 8 lookups each 0.20 / 0.28 / 0.51 ms
-// against 0.82; 1 to 15 lookups 0.54 against 0.83, 1 to 31 0.83 against 0.91, 1 to 63 1.22 against 1.27, 1 to 100 1.69
-// against 1.72, 1 to 200 3.09 against 3.00 ms; 262 k bags of 0 to 4 rows, mean, 67 us bag by bag, 34 with the bags dealt out.  256-byte rows: 2 / 4 / 8 lookups 0.29 / 0.44 / 0.74 ms against 0.88-0.92;
-// 1 to 15 lookups 0.78 against 0.95; 1 to 31 1.11-1.19 against 1.10; on the benchmark configuration (1 to 100 lookups)
-// 2.34-2.36 against 2.39 ms.  Hence the thresholds (the benchmark configuration stays with the per-bag kernel).  A
-// window ends early only at the end of the share or of a table (the rank look-up of a window uses one table).  With
-// malformed offsets (status bit set by the offsets check earlier in the stream) every bag is summed over its own
-// clamped (offsets[bag], offsets[bag + 1]) pair as the header promises, and windows stop at the end of their bag.
+// 2 million bags of 128-byte rows, stream against one bag per window: 2 / 4 / 8 lookups each 0.20 / 0.28 / 0.51 ms against 0.82; 1
+// to 15 lookups 0.54 against 0.83, 1 to 31 0.83 against 0.91, 1 to 63 1.22 against 1.27, 1 to 100 1.69 against 1.72, 1 to 200 3.09
+// against 3.00 ms; 262 k bags of 0 to 4 rows, mean, 67 us bag by bag, 34 with the bags dealt out.  256-byte rows: 2 / 4 / 8 lookups
+// 0.29 / 0.44 / 0.74 ms against 0.88-0.92; 1 to 15 lookups 0.78 against 0.95; 1 to 31 1.11-1.19 against 1.10; on the benchmark
+// configuration (1 to 100 lookups) 2.34-2.36 against 2.39 ms.  Hence the thresholds (the benchmark configuration stays with the
+// per-bag kernel).  A window ends early only at the end of the share or of a table (the rank look-up of a window uses one table).
+// With malformed offsets (status bit set by the offsets check earlier in the stream) every bag is summed over its own clamped
+// (offsets[bag], offsets[bag + 1]) pair as the header promises, and windows stop at the end of their bag.
 #define TT_POOL_STREAM_BELOW 33        // rows of up to 128 bytes
 #define TT_POOL_STREAM_BELOW_WIDE 12   // rows of up to 256 bytes
 // a += v, or a += f * v with weights

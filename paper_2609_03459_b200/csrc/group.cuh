@@ -333,8 +333,9 @@ __device__ __forceinline__ bool tt_prefix_any(const WsView& w, const TableDesc& 
     return found != 0;
 }
 
-// Level k < K from its own presence bitmap: the ascending distinct prefixes of every table.  Runs after the scan of
-// level k + 1 and k_prefix_bits, which sets this level's bits.
+// Level k < K from its own presence bitmap: the ascending distinct prefixes of every table.  The level's bits are set by then: from the
+// ranks of level k + 1 once that is scanned (k_prefix_bits, gc_level_bits<false>), or from its bits (tt_level_words,
+// gc_level_bits<true>).
 template <class View = WsView>
 struct LevelScan {
     View w;

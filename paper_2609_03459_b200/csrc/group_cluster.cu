@@ -33,10 +33,11 @@ __device__ __forceinline__ uint32_t gc_run(uint32_t n) { return (n + GC_CTAS - 1
 
 #define GC_IT 4
 #define GC_TILE (GC_THREADS * GC_IT)
-// Values of one tile of the CTA's run [.., hi): ex holds their exclusive prefixes inside their warps, sm the warps' (element order: stripe j,
-// then warp); the tile's sum comes back.
+// Values of one tile of the CTA's run [.., hi): ex holds their exclusive prefixes inside their warps, sm the warps' (element order:
+// stripe j, then warp); the tile's sum comes back.
 template <class F>
-__device__ __forceinline__ uint32_t gc_load(const F& f, uint32_t base, uint32_t hi, int& hint, uint32_t (&v)[GC_IT], uint32_t (&ex)[GC_IT], int (&at)[GC_IT], uint32_t* sm)
+__device__ __forceinline__ uint32_t gc_load(const F& f, uint32_t base, uint32_t hi, int& hint, uint32_t (&v)[GC_IT], uint32_t (&ex)[GC_IT],
+                                            int (&at)[GC_IT], uint32_t* sm)
 {
     const uint32_t tid = threadIdx.x;
     const int lane = tid & 31, wid = tid >> 5;
@@ -83,7 +84,8 @@ __device__ __forceinline__ uint32_t gc_load(const F& f, uint32_t base, uint32_t 
     return sm[GC_THREADS / 32 * GC_IT];
 }
 template <class F>
-__device__ __forceinline__ void gc_store(const F& f, uint32_t base, uint32_t hi, uint32_t carry, const uint32_t (&v)[GC_IT], const uint32_t (&ex)[GC_IT], const int (&at)[GC_IT], const uint32_t* sm)
+__device__ __forceinline__ void gc_store(const F& f, uint32_t base, uint32_t hi, uint32_t carry, const uint32_t (&v)[GC_IT], const uint32_t (&ex)[GC_IT],
+                                         const int (&at)[GC_IT], const uint32_t* sm)
 {
 #pragma unroll
     for (int j = 0; j < GC_IT; ++j) {

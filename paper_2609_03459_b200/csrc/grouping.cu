@@ -5,12 +5,13 @@
 // the 126 MB L2, so marking costs one L2 access per lookup, and an exclusive scan of the word popcounts
 // yields (a) the ascending list of distinct rows, (b) a rank structure {bits, base} that maps any row id
 // to its slot with one 8-byte load, so no per-lookup inverse map is ever written.  The prefix levels are
-// built the same way: the marking pass also sets one bit per length-k prefix (k < K) in a small bitmap over
-// the prefix space, and a scan of its word popcounts yields the ascending distinct prefixes; the first child of
-// a prefix is a rank look-up in the next level's bitmap, so the run-length encoding of the sorted rows is never
-// walked.  A prefix is present when the scanned bitmap of the level below counts at least one node in its range of
-// children (two rank look-ups per possible prefix, k_prefix_bits), so the cost of a prefix level is proportional
-// to the size of its prefix space, not to the lookups or the rows.  No kernel waits on another CTA.
+// built the same way: one bit per possible length-k prefix (k < K) in a small bitmap over the prefix space, and a scan of
+// its word popcounts yields the ascending distinct prefixes; the first child of a prefix is a rank look-up in the next
+// level's bitmap, so the run-length encoding of the sorted rows is never walked.  A prefix is present when the level below
+// has a node in its range of children: with a kernel per step the scanned bitmap of that level counts them (two rank
+// look-ups per possible prefix, k_prefix_bits), with the cluster its bits are looked at before it is scanned, as long as the range is
+// short (group.cuh).  The cost of a prefix level is proportional to the size of its prefix space, not to the
+// lookups or the rows.  No kernel waits on another CTA.
 #include "common.cuh"
 #include "scan.cuh"
 #include "group.cuh"
@@ -142,15 +143,18 @@ __global__ void __launch_bounds__(256) k_nodedup_levels(WsView w)
     }
 }
 
-// 0: a kernel per step; 1: one cluster of sixteen SMs (group_cluster.cu) from the prefix levels on; 2: one cluster for
-// everything.  The cluster saves a dozen launches and loses where a step has work for more SMs: scans and links of large
-// prefix spaces, marks and scan of long row bitmaps, checks of many offsets.  Whole call with 0 / 1 / 2, us: 1 table of 1 M
-// rows (33 k words), 1 k lookups 73 / 53 / 43; 2 tables, 98 k words, 18 k lookups (training) 254 / 229 / 228; 8 tables, 573 k
-// words, 8 k lookups 95 / 78 / 95; 16 tables, prefix bitmaps of 10 k words 127 / 115; of 30 k words 221 / 253.
-// Up to 8 k words whatever the batch (0 / 1: 1 table of 10 M rows, 2 M lookups 333 / 308, 10 M lookups 773 / 743; 2 of 40 M rows,
-// 8 k words, 4 M lookups 489 / 475, 20 M 2046 / 2046); between 8 k and 16 k words only with few lookups, which leave most
-// of the prefixes out (8 tables of 10 M rows, 12 k words, spread rows: 85 k lookups 167 / 164, 4 M 725 / 747, 16 M 1434 / 1464).
-// Offsets (20 k lookups, 1 / 2): 0.26 M 92 / 87 and 108 / 110, 1 M 189 / 203.
+// 0: a kernel per step; 1: one cluster of sixteen SMs (group_cluster.cu) from the prefix levels on; 2: one cluster for everything.
+// The cluster saves a dozen launches and loses where a step has work for more SMs: scans and links of large prefix spaces, marks
+// and scan of long row bitmaps, checks of many offsets.  Forward calls with 0 / 1 / 2, us (L2 flushed in between): row bitmap of 31
+// k words, one table, 1 k lookups 83 / 58 / 54, 16 k 94 / 69 / 60, 33 k 103 / 73 / 67; 125 k words, one table, 1 k 85 / 60 / 63, 16
+// k 96 / 73 / 73; two tables, 94 k words, 16 k 91 / 69 / 69; four, 125 k words, 16 k 91 / 65 / 71; eight, 125 k words, 33 k 102 /
+// 73 / 83; eight, 0.5 M words, 8 k 106 / 77 / 110; thirty small tables, 16 k 110 / 77 / 99: with several tables the line of mode 2
+// lies lower than it has been drawn. Prefix bitmaps (0 / 1), spread rows unless stated: up to 8 k words whatever the batch: two
+// tables of 40 M rows, popular rows first, 33 k lookups 136 / 118, 2 M 458 / 433, 8 M 888 / 888; between 8 k and 16 k words only
+// with few lookups, which leave most of the prefixes out: 12 k words, eight tables, 33 k 134 / 112, 2 M 475 / 470, 8 M 850 / 843;
+// 16 k words, four tables, 33 k 153 / 138, 2 M 553 / 566, 8 M 962 / 980; past it 20 k words, 33 k 157 / 134, 2 M 571 / 583; 46 k
+// words, 33 k 210 / 196, 0.26 M 335 / 333, 2 M 784 / 831. Offsets (20 k lookups, 0 / 1 / 2): 0.2 M 123 / 97 / 101, 1 M 258 / 230 /
+// 237.
 #define TT_CLUSTER_ANY_WORDS (1u << 13)
 #define TT_CLUSTER_LEVEL_WORDS (1u << 14)
 #define TT_CLUSTER_LEVEL_LOOKUPS (1 << 21)
@@ -299,7 +303,8 @@ __global__ void __launch_bounds__(256) k_costs(WsView w)
 // Partition of the sweeps and of the pooling pass, once per forward: the group range of every work unit (the sweeps of the
 // forward and of the backward read two words instead of bisecting the cost array at the start of every CTA, two chains of
 // ~20 dependent loads each: contraction 2.27 -> 2.16 ms, backward sweeps 4.49 -> 4.43 ms on the 60-table training step) and
-// the first bag of every share.  One thread each, so that the bisections run side by side.
+// the first bag of every share, where there are many bags per share or the offsets are flagged (otherwise the offsets check has written
+// it).  One thread each, so that the bisections run side by side.
 __global__ void __launch_bounds__(128) k_partition(WsView w)
 {
     tt_pdl_enter();

@@ -1,15 +1,21 @@
 // The rows of a batch of groups as one stream of steps (four rows of one group each) that a warp fetches ahead of its products.
 //
-// A warp that loads a pair of rows (last digits, then slices of the last core and rows of dE), multiplies them and goes on to
-// the next pair waits for a chain of L2 round trips per pair; registers for a pair of look-ahead cost more warps than they save.  Here the
-// rows come through a ring in shared memory (cp.async, no registers), across the groups of the batch, and the last digits eight steps
-// ahead of that.  Backward sweeps, before / after, us: rank 16, C of 16 rows: 8 tables x 0.47 M rows 190 / 166, x 2.06 M rows 430 / 377, rank 8 (5 M lookups) 221 / 190,
-// the rank-16 tables of the 60-table step 2320 / 2240; 8 rows, rank 16 (8 tables, 5 M lookups) 328 / 212; 4 rows, rank 32 380 / 332;
-// 4 rows, rank 16 245 / 175 (weighted, 4 M lookups).  Bound by instruction latency at 16 to 20 warps per SM (issue slots 47 %, LSU 56 %,
-// tensor pipe 31 %; the intermediate products take a fifth, the reductions 6 %).  A ring of three steps is no faster, more warps at the
-// price of spills are slower (rank 16 at 96 registers 404 against 377).  With C of 16 x 32 or 8 x 32 its 9 KB of C tiles per warp leave
-// twelve warps per SM: 685 against 668 and 567 against 522, so those shapes keep the loop without a ring, and so do all forward
-// sweeps, whose row stage has half the operands (rank 32 373 against 328, rank 16 232 against 176).
+// A warp that loads a pair of rows (last digits, then slices of the last core and rows of dE), multiplies them and goes on to the
+// next pair waits for a chain of L2 round trips per pair; registers for a pair of look-ahead cost more warps than they save.  Here
+// the rows come through a ring in shared memory (cp.async, no registers), across the groups of the batch, and the last digits eight
+// steps ahead of that.  Backward sweeps, loop over pairs / stream, us: rank 16, C of 16 rows: 8 tables x 0.47 M rows 190 / 166, x
+// 2.06 M rows 430 / 379; C of 16 rows, rank 8 (8 tables, 5 M lookups) 233 / 201; 8 rows, rank 16 328 / 217; 4 rows, rank 32 379 /
+// 326; 4 rows, rank 16 287 / 205, weighted, 4 M lookups 242 / 177; the sweeps of the 60-table step together 7.05 / 6.88 ms.  Bound
+// by instruction latency at 16 to 20 warps per SM (rank 16, 0.47 M rows: issue slots 40 %, LSU 43 %, L1 48 %, tensor pipe 20 %) and
+// by the end of the grid.  A ring of three steps is no faster, more warps at the price of spills are slower (rank 16 at 96
+// registers 404 against 377).  With C of 16 x 32 or 8 x 32 its 9 KB of C tiles per warp leave twelve warps per SM: 685 against 668
+// and 567 against 522, so those shapes keep the loop without a ring, and so do all forward sweeps, whose row stage has half the
+// operands (rank 32 373 against 328, rank 16 232 against 176). Where groups hold one to four rows each, the loop over pairs with
+// its 24 warps is the faster one (8 tables of 40 M rows, 0.66 M spread lookups: rank 16, C of 16 rows 404 / 498; 4 rows, rank 32
+// 386 / 496; 8 and 4 rows, rank 16 323 / 345, 249 / 283; training calls 1353 / 1444, 1353 / 1462, 1058 / 1070, 894 / 920).  As a
+// kernel of its own for tables of few and even rows it gave those calls 2 to 5 % and took up to 10 % of calls over tables of mixed
+// sizes, which the stream serves better than either (8 tables of 10 k to 40 M rows, 0.25 M spread lookups, call: pairs 347, stream
+// 328, both 346).
 #pragma once
 #include "common.cuh"
 
@@ -30,9 +36,9 @@ struct RowStream {
     static constexpr int FLOATS = PD * STEP + INFO;
 
     const uint32_t* __restrict__ rows;
-    const float* __restrict__ GK;      // with this lane's offset in a slice
+    const float* __restrict__ GK;      // last core, with this lane's offset in a slice
     float* ring;
-    uint32_t ring_s;                   // its shared address, with this lane's offset in a slot
+    uint32_t ring_s;                   // its shared address
     uint32_t steps, next;              // of the batch; the next one to stage
     uint32_t nid, nuf, nqn;            // lane: row slot of the block (eight steps) after the one that is being staged
 
