@@ -29,7 +29,7 @@ __global__ void __launch_bounds__(256) k_check_offsets(WsView w)
 // Bound by the requests of the lookups that find their bit not set: the lookups of a popular row that are in flight before
 // its first mark lands queue up on one word.  So a CTA marks 32 lookups, waits for them and then takes all of its share.  Grouping
 // without / with, us: one table, 0.5 M lookups (exponent 1.2, 1 M, 10 M, 40 M rows) 91 / 61, 95 / 63, 102 / 72, spread rows 67 / 47,
-// 72 / 52, 87 / 69; 8 tables, 1.6 M lookups 126 / 112; 60 tables, 99 M lookups 865 / 770.  8 / 16 / 64 / 128 lookups instead of
+// 72 / 52, 87 / 69; 8 tables, 1.6 M lookups 126 / 112; 60 tables, 99 M lookups 816 to 905 / 802 to 814 over runs.  8 / 16 / 64 / 128 lookups instead of
 // 32: 102 / 103 / 107 / 115 for 103 us (one table of 16 M rows, 0.5 M lookups).  A second test of the word past L1 before the
 // atomic (the copy in L1 is often an old one) costs more than the requests it saves: 8 tables 124 us, 60 tables 950.
 #define TT_MARK_SEEDS_FROM (1 << 16)   // 8 k lookups: call 78.5 us with them, 78.0 without
