@@ -145,10 +145,10 @@ __device__ __forceinline__ void tt_mark_rows(const WsView& w, int64_t first, int
 // val[excl ..] = v0 + (positions of the set bits of `bits`), clipped at `cap`.  Called by all lanes that emit a word
 // (also with bits == 0).  A lane writes the first bits of its own word; a word with more is handed to the whole warp,
 // one lane per bit: a densely set word then is one coalesced store instead of 32 stores that each touch another
-// sector (a tile of the popular first rows of a table took 80 us against 20 us for a sparse one), EMIT_WORDS such words at
-// a time, whose chains of shuffles overlap (8 tables, 1.6 M lookups: grouping 112 -> 109 us; eight words 110).
+// sector (a tile of the popular first rows of a table took 80 us against 20 us for a sparse one).  Four such words at a time, so that
+// their shuffles overlap, gained 1 to 2 % of a call with many dense words (24 tables, 1 M lookups 253 / 249 us) and lost 2 to 3 % with
+// few (12 tables, 78 k lookups 270 / 277; 22 tables, 73 k 159 / 163).
 #define EMIT_OWN 8
-#define EMIT_WORDS 4
 __device__ __forceinline__ void tt_emit_set_bits(uint32_t* __restrict__ val, uint32_t cap, unsigned bits, uint32_t excl, uint32_t v0)
 {
     const unsigned act = __activemask();
@@ -167,24 +167,15 @@ __device__ __forceinline__ void tt_emit_set_bits(uint32_t* __restrict__ val, uin
     }
     unsigned todo = __ballot_sync(act, dense);
     while (todo) {
-        unsigned wb[EMIT_WORDS];
-        uint32_t we[EMIT_WORDS], wv[EMIT_WORDS];
-#pragma unroll
-        for (int q = 0; q < EMIT_WORDS; ++q) {
-            const int src = todo ? __ffs(todo) - 1 : lane;
-            const bool some = todo != 0;
-            todo &= todo - 1;
-            wb[q] = __shfl_sync(act, bits, src);
-            we[q] = __shfl_sync(act, excl, src);
-            wv[q] = __shfl_sync(act, v0, src);
-            if (!some) wb[q] = 0u;
+        const int src = __ffs(todo) - 1;
+        todo &= todo - 1;
+        const unsigned wb = __shfl_sync(act, bits, src);
+        const uint32_t we = __shfl_sync(act, excl, src);
+        const uint32_t wv = __shfl_sync(act, v0, src);
+        if ((wb >> lane) & 1u) {
+            const uint32_t sl = we + __popc(wb & ((1u << lane) - 1u));
+            if (sl < cap) val[sl] = wv + lane;
         }
-#pragma unroll
-        for (int q = 0; q < EMIT_WORDS; ++q)
-            if ((wb[q] >> lane) & 1u) {
-                const uint32_t sl = we[q] + __popc(wb[q] & ((1u << lane) - 1u));
-                if (sl < cap) val[sl] = wv[q] + lane;
-            }
     }
 }
 
