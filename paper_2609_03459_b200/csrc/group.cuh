@@ -68,8 +68,9 @@ __device__ __forceinline__ int64_t tt_table_start(const WsView& w, int t)
     return o < 0 ? 0 : (o > w.L ? w.L : o);
 }
 
-// the offsets: non-decreasing, from 0 to L; first lookup of every table into tl_start, boundaries of the pooling shares.  Threads
-// first, first + step, ..
+// the offsets: non-decreasing, from 0 to L; first lookup of every table into tl_start and (SHARES) boundaries of the pooling shares.
+// Threads first, first + step, ..
+template <bool SHARES>
 __device__ __forceinline__ void tt_check_offsets(const WsView& w, int64_t first, int64_t step)
 {
     const int64_t nb = (int64_t)w.T * w.B;
@@ -79,7 +80,7 @@ __device__ __forceinline__ void tt_check_offsets(const WsView& w, int64_t first,
         if (i == 0 && o != 0) bad = true;
         if (i == nb && o != w.L) bad = true;
     };
-    if (tt_pool_bounds_by_bag(w)) {
+    if (SHARES && tt_pool_bounds_by_bag(w)) {
         const double invL = 1.0 / (double)w.L;
         for (int64_t i = first; i <= nb; i += step) {
             const int64_t o = __ldg(w.offsets + i), o_next = i < nb ? __ldg(w.offsets + i + 1) : o;

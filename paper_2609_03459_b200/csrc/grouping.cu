@@ -21,7 +21,7 @@
 __global__ void __launch_bounds__(256) k_check_offsets(WsView w)
 {
     tt_pdl_enter();
-    tt_check_offsets(w, (int64_t)blockIdx.x * blockDim.x + threadIdx.x, (int64_t)gridDim.x * blockDim.x);
+    tt_check_offsets<true>(w, (int64_t)blockIdx.x * blockDim.x + threadIdx.x, (int64_t)gridDim.x * blockDim.x);
 }
 
 // FUSED: offsets and row ids in one pass (the marks take the tables' ranges from the offsets themselves); otherwise
@@ -45,7 +45,7 @@ __global__ void __launch_bounds__(256, 8) k_mark(WsView w, int clear)
         if (threadIdx.x < 32) tt_mark_rows<!FUSED>(w, (int64_t)blockIdx.x * blockDim.x * 4 + threadIdx.x, w.L, w.L);
         __syncthreads();
     }
-    if (FUSED) tt_check_offsets(w, (int64_t)blockIdx.x * blockDim.x + threadIdx.x, (int64_t)gridDim.x * blockDim.x);
+    if (FUSED) tt_check_offsets<true>(w, (int64_t)blockIdx.x * blockDim.x + threadIdx.x, (int64_t)gridDim.x * blockDim.x);
     tt_mark_rows<!FUSED>(w, (int64_t)blockIdx.x * blockDim.x * 4 + threadIdx.x, blockDim.x, (int64_t)gridDim.x * blockDim.x * 4);
 }
 
