@@ -215,8 +215,11 @@ __device__ __forceinline__ void gc_level_bits(const WsView& w, int k, bool mark)
 
 
 // rows: from the row ids on (workspace regions cleared here); otherwise the row bitmap is scanned already
-// level: 0, or one more than the highest level whose bitmap this kernel writes from the bits of the level below; all bitmaps are written before
-// any of them is scanned, and all are scanned at once.  (0: a radix is past TT_BITS_RADIX; level by level, each from the ranks of the one below)
+// BITS: all bitmaps are written before any of them is scanned, and all are scanned at once; level: one more than the highest level
+// whose bitmap this kernel writes from the bits of the level below.  !BITS (level = 0; a radix is past TT_BITS_RADIX): level by level,
+// each from the ranks of the one below.  (One kernel for both was longer for each: two tables, two cores, 4.7 k lookups, call 89 us,
+// 85 apart.)
+template <bool BITS>
 __global__ void __launch_bounds__(GC_THREADS) k_group_cluster(const __grid_constant__ WsView w, int rows, int level)
 {
     tt_pdl_enter();
@@ -230,7 +233,7 @@ __global__ void __launch_bounds__(GC_THREADS) k_group_cluster(const __grid_const
         uint4* bm4 = reinterpret_cast<uint4*>(w.bm);                             // a whole number of scan tiles
         for (uint32_t i = first; i < w.total_words / 2; i += step) bm4[i] = make_uint4(0u, 0u, 0u, 0u);
     }
-    if (digit_major && (rows || level == 0))   // (otherwise k_mark has cleared it)
+    if (digit_major && (rows || !BITS))   // (otherwise k_mark has cleared it)
         for (uint32_t i = first; i < w.ttotal_words[K - 1]; i += step) w.tbm[K - 1][i] = make_uint2(0u, 0u);
     gc_sync();   // also: every CTA runs before another writes into its shared memory
     if (rows) {
@@ -239,8 +242,8 @@ __global__ void __launch_bounds__(GC_THREADS) k_group_cluster(const __grid_const
         gc_sync();
     }
     const uint32_t twords = digit_major ? w.ttotal_words[K - 1] : 0u;
-    bool listed = level != 0;     // the digit-major bitmap is marked and scanned
-    if (level != 0) {
+    bool listed = BITS;     // the digit-major bitmap is marked and scanned
+    if constexpr (BITS) {
         __shared__ uint32_t warp_sums[TT_MAXK + 1][GC_THREADS / 32];
         for (int k = level - 1; k >= 1; --k) {
             gc_level_bits<true>(w, k, digit_major && k == K - 1);
@@ -353,7 +356,7 @@ cudaError_t tt_launch_group_cluster(tt_emb* h, bool rows, int level, cudaStream_
     at[1].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 2;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, k_group_cluster, h->v, rows ? 1 : 0, level);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, level != 0 ? k_group_cluster<true> : k_group_cluster<false>, h->v, rows ? 1 : 0, level);
     if (e == cudaSuccess) tt_note_launch();
     return e;
 }
@@ -361,7 +364,8 @@ cudaError_t tt_launch_group_cluster(tt_emb* h, bool rows, int level, cudaStream_
 // whether the device takes the cluster (sixteen CTAs are past the portable eight): asked once per handle
 int tt_group_cluster_ok()
 {
-    if (cudaFuncSetAttribute(k_group_cluster, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) { cudaGetLastError(); return 0; }
+    if (cudaFuncSetAttribute(k_group_cluster<true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+        cudaFuncSetAttribute(k_group_cluster<false>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) { cudaGetLastError(); return 0; }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(GC_CTAS);
     cfg.blockDim = dim3(GC_THREADS);
@@ -372,7 +376,8 @@ int tt_group_cluster_ok()
     at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, k_group_cluster, &cfg) != cudaSuccess) { cudaGetLastError(); return 0; }
-    return n > 0;
+    int n = 0, m = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, k_group_cluster<true>, &cfg) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&m, k_group_cluster<false>, &cfg) != cudaSuccess) { cudaGetLastError(); return 0; }
+    return n > 0 && m > 0;
 }
