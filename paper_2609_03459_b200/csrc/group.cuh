@@ -11,9 +11,9 @@
 
 // Share ci starts with the first bag whose offset is >= L ci / C.  The pass that checks the offsets writes the boundaries as
 // it goes: bag i + 1 is the first bag of every share whose target lies in (offsets[i], offsets[i + 1]].  (A bisection of
-// the offsets per share, 15 dependent loads each, took 6 us of its step in the cluster: 8 tables, 33 k bags, 33 k shares, call 652 -> 646 us.  With
-// many bags per share the search is cheaper than two quotients per bag: 60 k shares of 2 M bags grouping and schedule 811 / 806
-// us, of 7.9 M bags 1024 / 1052.)
+// the offsets per share, 15 dependent loads each, took 6 us of its step in the cluster: 8 tables, 33 k bags, 33 k shares, call
+// 652 -> 646 us.  With many bags per share the search is cheaper than two quotients per bag: 60 k shares of 2 M bags grouping and
+// schedule 811 / 806 us, of 7.9 M bags 1024 / 1052.  Where one cluster does everything, it searches: k_group_cluster.)
 
 #define TT_POOL_BAGS_PER_SHARE 64
 __device__ __forceinline__ bool tt_pool_bounds_by_bag(const WsView& w)
