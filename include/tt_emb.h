@@ -115,6 +115,8 @@ int tt_emb_bind(tt_emb_t h, float* const* core_ptrs, void* workspace, size_t wor
  * freed or overwritten once the forward has completed.  `offsets` must stay valid and unchanged until the backward
  * has completed if mean pooling is selected (the bag lengths are re-read); the inspection calls
  * tt_emb_export_level (with lookup_counts) and tt_emb_export_inverse re-read both arrays.  Asynchronous.
+ * Small calls on a handle without the backward make their rows lookup by lookup, without the grouping (same results and
+ * status; the inspection calls make the grouping when they are asked for it).
  */
 int tt_emb_forward(tt_emb_t h, const int64_t* indices, const int64_t* offsets, int64_t batch,
                    int64_t num_lookups, float* out, tt_emb_stream_t stream);
@@ -243,7 +245,7 @@ int tt_emb_unpack_core(tt_emb_t h, int32_t table, int32_t core, const float* can
  * Device events: time of stage `stage` of the most recent call, in milliseconds, measured with CUDA
  * events recorded on the call's stream when timing is enabled.  SYNCHRONISES on the stage's end event.
  * Stages: 0 grouping, 1 schedule (empty where the prefix levels are small and one kernel makes them and the schedule:
- * then stage 0 is both), 2 contraction, 3 pooling, 4 backward sort, 5 backward dE,
+ * then stage 0 is both), 2 contraction, 3 pooling (a small call that makes no grouping is stage 2 alone), 4 backward sort, 5 backward dE,
  * 6 backward contraction, 7 backward middle cores + reductions, 8 sgd; 9..20 the forward sweep kernel of shape
  * variant -1 (generic), 0..10; 21..32 the backward sweep kernel of the same variants (TT_EMB_ERR_STATE for a
  * variant no table uses).

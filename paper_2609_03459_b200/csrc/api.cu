@@ -598,6 +598,15 @@ static int forward_any(tt_emb* h, const void* indices, bool idx32, const int64_t
     h->have_forward = false;
     for (int i = 0; i < 4; ++i) h->ev_valid[i] = false;
     for (int i = 9; i < 9 + TT_NUM_VARIANTS + 1; ++i) h->ev_valid[i] = false;
+    bool direct = false;
+    int r = stage_begin(h, 2, s);
+    if (r) return r;
+    TT_CUDA(tt_launch_direct(h, out, &direct, s));
+    if (direct) {
+        if ((r = stage_end(h, 2, s))) return r;
+        h->have_forward = true;
+        return TT_EMB_OK;
+    }
     TT_CUDA(tt_plan_pooling(h, out));
     TT_STAGE(h, 0, s, tt_launch_grouping(h, s));
     TT_STAGE(h, 1, s, tt_launch_schedule(h, s));
@@ -716,6 +725,7 @@ extern "C" int tt_emb_grouping_counts(tt_emb_t h, int64_t* counts_host, tt_emb_s
     if (!h->bound || !h->have_forward) return TT_EMB_ERR_STATE;
     cudaStream_t s = (cudaStream_t)stream;
     const int T = h->T, K = h->K;
+    TT_CUDA(tt_regroup(h, s));
     uint32_t* tmp = (uint32_t*)malloc((size_t)(T + 1) * sizeof(uint32_t));
     if (!tmp) return TT_EMB_ERR_ARG;
     for (int k = 1; k <= K; ++k) {
@@ -735,6 +745,7 @@ extern "C" int tt_emb_export_level(tt_emb_t h, int32_t table, int32_t level, int
     if (!h->bound || !h->have_forward) return TT_EMB_ERR_STATE;
     if (lookup_counts && !h->enable_backward) return TT_EMB_ERR_STATE;  // needs the cursor scratch array
     cudaStream_t s = (cudaStream_t)stream;
+    TT_CUDA(tt_regroup(h, s));
     TT_CUDA(tt_launch_export_level(h, table, level, vals, row_counts, lookup_counts, s));
     TT_CUDA(cudaStreamSynchronize(s));
     return TT_EMB_OK;
@@ -745,6 +756,7 @@ extern "C" int tt_emb_export_inverse(tt_emb_t h, int32_t table, int32_t* inv, tt
     if (!h || !inv || table < 0 || table >= h->T) return TT_EMB_ERR_ARG;
     if (!h->bound || !h->have_forward) return TT_EMB_ERR_STATE;
     cudaStream_t s = (cudaStream_t)stream;
+    TT_CUDA(tt_regroup(h, s));
     TT_CUDA(tt_launch_export_inverse(h, table, inv, s));
     TT_CUDA(cudaStreamSynchronize(s));
     return TT_EMB_OK;

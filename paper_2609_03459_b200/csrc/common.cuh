@@ -152,7 +152,8 @@ __device__ __forceinline__ int64_t tt_index(const WsView& w, int64_t l)
 }
 
 enum { CTR_LEVEL0 = 0 /* +k */, CTR_TLEVEL0 = 8 /* +k */, CTR_COST_TOTAL = 16, CTR_SCAN_TICKET = 32 /* tiles of the running scan that have reported */,
-       CTR_POOL_NEXT = 34 /* next share of the lookups to be pooled (shares are handed out in order) */ };
+       CTR_POOL_NEXT = 34 /* next share of the lookups to be pooled (shares are handed out in order) */,
+       CTR_DIRECT = 40 /* k_direct: CTAs that have reported, their status bits; 1 where the last forward made no grouping, its batch, lookups, idx32 */ };
 
 struct tt_emb {
     int T, K, D;
@@ -187,6 +188,7 @@ struct tt_emb {
     void* ws_base;
     bool warp_groups;     // every table is swept by warps that take groups one batch at a time (not by whole CTAs)
     int cluster_ok;       // the device takes the cluster of group_cluster.cu
+    int direct_ctas[2];   // resident CTAs per SM of k_direct without / with weights, 0: not asked yet
     int pool_grid;        // CTAs of the pooling kernel (tt_plan_pooling)
     float* carry;         // workspace region of v.carry for chunks of TT_DE_CHUNK lookups
     size_t scan_tmp_elems;
@@ -228,6 +230,8 @@ cudaError_t tt_launch_tlist(tt_emb* h, int k, cudaStream_t s);   // digit-major 
 cudaError_t tt_plan_pooling(tt_emb* h, const float* out);          // grid and shares of the pooling pass, before the schedule
 cudaError_t tt_launch_contraction(tt_emb* h, cudaStream_t s);
 cudaError_t tt_launch_pooling(tt_emb* h, float* out, cudaStream_t s);
+cudaError_t tt_launch_direct(tt_emb* h, float* out, bool* launched, cudaStream_t s);   // the forward without the grouping, where that is shorter
+cudaError_t tt_regroup(tt_emb* h, cudaStream_t s);                 // the grouping of such a forward, for the inspection calls
 cudaError_t tt_launch_bwd_sort(tt_emb* h, cudaStream_t s);
 cudaError_t tt_launch_bwd_dE(tt_emb* h, const float* grad_out, cudaStream_t s);
 cudaError_t tt_launch_bwd_contraction(tt_emb* h, cudaStream_t s);

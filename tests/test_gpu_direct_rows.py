@@ -1,0 +1,134 @@
+"""Small forward-only calls, whose rows are made lookup by lookup in one kernel: every kind of shape that it takes (three cores with a
+kernel of their own, ranks that are no multiple of eight or of four, two and four cores), one to eight warps per bag, more bags than
+warps, both id types, pooling modes, bad ids and offsets; against the oracle, against the grouped path (the forward of a handle with the
+backward), and the grouping that the inspection calls make afterwards against the integer oracle.
+
+Bar: max|err| <= 1e-5 * max|ref|, the bound of the other parity tests (fp32 sums)."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import workloads
+from test_gpu_parity import assert_close, binding, check_grouping, dev  # noqa: F401  (binding: fixture)
+from workloads import TableSpec
+
+pytestmark = pytest.mark.gpu
+
+SHAPES = [((4, 4, 4), (1, 16, 16, 1)), ((4, 4, 4), (1, 32, 8, 1)), ((4, 4, 4), (1, 4, 32, 1)), ((4, 4, 4), (1, 12, 16, 1)), ((4, 8, 4), (1, 32, 32, 1)),
+          ((2, 4, 4), (1, 16, 32, 1)), ((2, 4, 4), (1, 8, 16, 1)), ((2, 4, 4), (1, 20, 8, 1)), ((2, 2, 4), (1, 32, 32, 1)), ((2, 2, 4), (1, 8, 16, 1)),
+          ((2, 2, 4), (1, 64, 8, 1)),                                     # with a kernel of their own
+          ((4, 4, 4), (1, 6, 16, 1)), ((2, 2, 4), (1, 128, 8, 1)), ((4, 6, 4), (1, 16, 24, 1)), ((2, 8, 8), (1, 4, 4, 1)), ((3, 3, 5), (1, 6, 4, 1)),
+          ((5, 3, 7), (1, 3, 9, 1)), ((8, 8), (1, 24, 1)), ((3, 5), (1, 7, 1)), ((2, 4, 4, 4), (1, 64, 64, 64, 1)),
+          ((2, 2, 4, 4), (1, 8, 16, 16, 1)), ((2, 3, 2, 3), (1, 5, 3, 7, 1))]
+ROWS = {2: (45, 41), 3: (11, 13, 14), 4: (6, 5, 9, 7)}
+
+
+def build(d, r, B, lens, T, seed):
+    n = ROWS[len(d)]
+    spec = TableSpec(N=int(np.prod(n)) - 3, n=n, d=d, r=r, alpha=1.0, core_dist="normal", core_scale=0.4)
+    wl = workloads.custom([spec] * T, B, lens, seed=seed)
+    return wl
+
+
+def launches(binding, emb, *call):  # noqa: F811
+    binding.launch_count(reset=True)
+    out = emb.forward(*call)
+    return binding.launch_count(), out
+
+
+@pytest.mark.parametrize("d,r", SHAPES)
+@pytest.mark.parametrize("B,lens,T", [(64, 1, 1), (70, (0, 3), 2), (64, (0, 40), 1), (90, (3, 9), 2), (1200, (0, 2), 3)])
+def test_out_and_grouping(binding, d, r, B, lens, T):  # noqa: F811
+    wl = build(d, r, B, lens, T, seed=B)
+    emb = binding.from_workload(wl)
+    off = dev(wl.offsets)
+    n, out = launches(binding, emb, dev(wl.indices), off, B)
+    assert n == 1 or (len(d) == 4 and r[1] == 64 and n >= 4)     # rows of rank 64, one by one, take longer than the grouping
+    assert emb.status() == 0
+    ref = oracle.forward_workload(wl)
+    assert_close(out.cpu().numpy(), ref, "out")
+    grouped = binding.from_workload(wl, enable_backward=True)
+    m, again = launches(binding, grouped, dev(wl.indices), off, B)
+    assert m >= 3
+    assert_close(out.cpu().numpy(), again.cpu().numpy(), "grouped")
+    check_grouping(emb, wl)
+    assert emb.status() == 0 and emb.check_guards() is None
+    # 32-bit ids, an output that is not 16-byte aligned, and a call after the grouping of the one before was asked for
+    room = torch.full((B * T * emb.D + 1,), 7.0, device="cuda")
+    emb.forward(dev(wl.indices.astype(np.int32)), off, B, out=room[1:].view(B, T * emb.D))
+    assert float(room[0]) == 7.0
+    if n == 1:
+        assert torch.equal(room[1:].view_as(out), out)
+    check_grouping(emb, wl)
+
+
+@pytest.mark.parametrize("d,r", [SHAPES[0], SHAPES[8], SHAPES[11], SHAPES[15], SHAPES[18]])
+@pytest.mark.parametrize("mode", ["mean", "weights"])
+def test_pooling_modes(binding, d, r, mode):  # noqa: F811
+    wl = build(d, r, 80, (0, 30), 2, seed=4)
+    emb = binding.from_workload(wl, enable_weighted=True)
+    weights = np.random.default_rng(0).normal(size=wl.L).astype(np.float32) if mode == "weights" else None
+    emb.set_pooling("mean" if mode == "mean" else "sum", None if weights is None else dev(weights))
+    n, out = launches(binding, emb, dev(wl.indices), dev(wl.offsets), 80)
+    assert n == 1 and emb.status() == 0
+    assert_close(out.cpu().numpy(), oracle.forward_workload(wl, weights=weights, mode="mean" if mode == "mean" else "sum"), "out")
+
+
+@pytest.mark.parametrize("B,lens", [(64, 1), (64, (0, 40)), (2000, (0, 3))])
+def test_bad_ids_and_offsets(binding, B, lens):  # noqa: F811
+    wl = build((4, 4, 4), (1, 8, 8, 1), B, lens, 2, seed=7)
+    N = wl.tables[0].N
+    emb = binding.from_workload(wl)
+    idx, off = dev(wl.indices), dev(wl.offsets)
+    good = emb.forward(idx, off, B).clone()
+    for bad_id in (N, -1, 1 << 40):
+        ids = wl.indices.copy()
+        ids[wl.L // 3] = bad_id
+        keep = wl.indices
+        wl.indices = ids
+        n, out = launches(binding, emb, dev(ids), off, B)
+        assert n == 1 and emb.status() == binding.STATUS_INDEX
+        assert_close(out.cpu().numpy(), oracle.forward_workload(wl), "out")
+        emb.grouping_counts()
+        assert emb.status() == binding.STATUS_INDEX
+        wl.indices = keep
+    for at, value in ((0, 5), (3, 1 << 40), (B // 2, -9), (2 * B, wl.L - 1), (2 * B, wl.L + 1)):
+        keep = wl.offsets
+        wl.offsets = keep.copy()
+        wl.offsets[at] = value
+        n, out = launches(binding, emb, idx, dev(wl.offsets), B)
+        assert n == 1 and emb.status() == binding.STATUS_OFFSETS
+        emb.grouping_counts()
+        assert emb.status() == binding.STATUS_OFFSETS
+        wl.offsets = keep
+        assert torch.equal(emb.forward(idx, off, B), good) and emb.status() == 0
+    check_grouping(emb, wl)
+    assert emb.check_guards() is None
+
+
+def test_capacity_and_graph(binding):  # noqa: F811
+    wl = build((4, 4, 4), (1, 16, 16, 1), 128, (1, 4), 2, seed=11)
+    ref = oracle.forward_workload(wl)
+    # a row buffer for fewer rows: the grouped path, which drops the surplus
+    small = binding.from_workload(wl, max_unique_rows=50)
+    n, _ = launches(binding, small, dev(wl.indices), dev(wl.offsets), 128)
+    assert n >= 3 and small.status() == binding.STATUS_OVERFLOW
+    # replayed with other contents, and between calls of the same handle; the inspection calls see the replay's lookups
+    emb = binding.from_workload(wl)
+    idx, off, out = dev(wl.indices), dev(wl.offsets), torch.empty((128, 128), device="cuda")
+    graph = emb.capture_forward(idx, off, 128, out)
+    other = build((4, 4, 4), (1, 16, 16, 1), 64, 1, 2, seed=12)
+    for shift in (0, 5):
+        emb.forward(dev(other.indices), dev(other.offsets), 64)
+        ids = (wl.indices + shift) % wl.tables[0].N
+        idx.copy_(dev(ids))
+        graph.replay()
+        keep, wl.indices = wl.indices, ids
+        assert_close(out.cpu().numpy(), oracle.forward_workload(wl), "out")
+        counts = emb.grouping_counts()
+        for t in range(2):
+            lo, hi = wl.offsets[t * 128], wl.offsets[(t + 1) * 128]
+            assert counts[t, 2] == len(np.unique(ids[lo:hi]))
+        wl.indices = keep
+    assert_close(emb.forward(dev(wl.indices), off, 128).cpu().numpy(), ref, "out")
