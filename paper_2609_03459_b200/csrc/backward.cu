@@ -1,9 +1,9 @@
 // Backward path (paper Sec. 3.2 backward, Eq. 2) and SGD.
 //
-//   1. sort:  the forward left one (slot, bag) pair per lookup; a counting sort by slot (counts -> exclusive
-//             scan -> scatter) groups the lookups of every distinct row.  Hot rows would serialise global
-//             atomics, so each CTA first aggregates the duplicates of its tile in shared memory (owner tags) and
-//             issues one global atomic per aggregated row per tile.
+//   1. sort:  the forward left one (slot, bag) pair per lookup; a counting sort by slot (counts, which give every pair its
+//             rank in its row -> segment starts -> scatter of the bags) groups the lookups of every distinct row.  Hot rows
+//             would serialise global atomics, so each CTA first aggregates the duplicates of its tile in shared memory (owner
+//             tags) and issues one global atomic per aggregated row per tile.
 //   2. dE:    segmented sum of grad_out rows over the sorted pairs.  Fixed-size chunks of sorted positions per
 //             warp (skew-proof); segments that cross chunk borders leave partial sums which a second kernel
 //             adds in position order.
@@ -60,151 +60,246 @@ __global__ void __launch_bounds__(256) k_bwd_clear(WsView w)
     }
 }
 
+// Positions per warp (a power of two), and where the warps leave the pieces of segments that cross a chunk border.  A chunk is walked
+// serially, so short batches want short chunks (1024 positions: 65 thousand lookups kept 64 warps busy) and long ones
+// chunks that amortise the borders.  dE with 32 / 128 / 256 / 512 / 1024 positions per warp, us: 65 k lookups (D = 128,
+// at least 160 there) 39 / 39 / 60 / 101 / 185; 0.5 M (D = 32) 33 / 31 / 42 / 62 / 103; 1.6 M (D = 64) 72 / 70 / 70 / 85 /
+// 113; 4 M (D = 16) 173 / 122 / 121 / 142 / 173.
+static void tt_de_partition(tt_emb* h)
+{
+    WsView& w = h->v;
+    int64_t want = w.L / 2048 < 128 ? w.L / 2048 : 128;
+    if (want < w.L / 32768) want = w.L / 32768;
+    int log = 5;
+    while ((2LL << log) <= want && (1 << log) < TT_DE_CHUNK) ++log;
+    // the pieces of more than L / TT_DE_CHUNK chunks go where the unsorted pairs were (the sort has consumed them): 8 bytes
+    // per lookup, so a chunk holds at least about D positions
+    const uintptr_t u0 = (reinterpret_cast<uintptr_t>(w.upairs) + 15) & ~(uintptr_t)15;
+    const size_t room = reinterpret_cast<uintptr_t>(w.upairs + h->max_lookups + 1) - u0;
+    while ((1 << log) < TT_DE_CHUNK && (size_t)((w.L + (1LL << log) - 1) >> log) * 2 * h->D * sizeof(float) > room) ++log;
+    w.carry = (1 << log) < TT_DE_CHUNK ? reinterpret_cast<float*>(u0) : h->carry;
+    while (((w.L + (1LL << log) - 1) >> log) > 2 * TT_POOL_MAX_SHARES) ++log;   // the room for the chunks' first rows
+    w.de_chunk_log = (uint32_t)log;
+    w.chunk_slot = reinterpret_cast<uint32_t*>(w.pool_bounds);   // (the pooling is done with its boundaries)
+}
+
 // ---------------------------------------------------------------------------------------------- 1. sort by slot
 
-// MODE 0: cnt[slot] += occurrences.  MODE 1: pairs[seg_start[slot] + claimed position] = (slot, bag).
+// A pair's place among the pairs of its row: cnt[slot] += occurrences, rank[l] = occurrences claimed before this one.  With the ranks
+// from here the placing pass claims nothing.  (Two passes of claims, one to count and one to place: sort of 60 tables 2620 us, of 240
+// 1590, of 4 M weighted pairs 173, of 0.5 M 47; now 1825, 1236, 109, 30.)
 //
 // Aggregation of a tile's duplicates without a probing hash table (two shared-memory atomics per pair made the
-// shared-memory atomic unit the limit of both passes): every pair stores a tag (low key bits, its number in the tile)
+// shared-memory atomic unit the limit of the pass): every pair stores a tag (low key bits, its number in the tile)
 // into bucket h(key) with a plain store; after a barrier the bucket holds the tag of one of its writers.  That pair
 // owns the bucket.  A pair with the owner's key is a duplicate: it counts itself in extra[h] (the only shared-memory
 // atomic left, and only duplicates issue it) and the owner makes one global atomic for all of them.  A pair with another
 // key lost the bucket and goes to the global counter by itself.  h takes the key bits above bit 19 as they are, so that
 // bucket and the 20 low bits together identify the key and a 32-bit tag is enough.
-#define TT_SORT0_TILES 24
+#define TT_SORT0_TILES 8
 #define HT_LOW_BITS 20
 #define HT_ID_BITS 11
-template <int MODE>
-__global__ void __launch_bounds__(256) k_sort_pass(WsView w)
+__device__ __forceinline__ uint32_t* tt_sort_ranks(const WsView& w)
+{
+    return tt_weighted(w) ? reinterpret_cast<uint32_t*>(w.wsorted) : reinterpret_cast<uint32_t*>(w.pairs) + (w.upairs - w.pairs);
+}
+__global__ void __launch_bounds__(256) k_sort_count(WsView w)
 {
     tt_pdl_enter();
     static_assert(HT_TILE == (1 << HT_ID_BITS) && HT_SIZE == (1 << (32 - HT_LOW_BITS)) && HT_LOW_BITS + HT_ID_BITS <= 32, "tag layout");
     const uint2* __restrict__ upairs = w.upairs;
+    uint32_t* const rank = tt_sort_ranks(w);
     const uint32_t capK = w.cap[w.K];
     __shared__ uint32_t tag[HT_SIZE];
-    __shared__ uint32_t extra[HT_SIZE];   // duplicates of the owner's key; MODE 1: then the claimed base position
+    __shared__ uint32_t extra[HT_SIZE];   // duplicates of the owner's key, then the owner's rank
     const int64_t L = w.L;
     const int64_t ntiles = (L + HT_TILE - 1) / HT_TILE;
-    const bool weighted = MODE == 1 && w.wsorted && (w.psw || w.pool_mean);
     for (int i = threadIdx.x; i < HT_SIZE; i += blockDim.x) extra[i] = 0u;
     // the first barrier of the tile loop orders this before the first atomic on extra
-    auto emit = [&](uint32_t pos, const uint2& pr, int64_t l) {
-        w.pairs[pos] = pr;
-        if (weighted) {   // weighted / mean pooling: the pair's factor travels with it
-            float a = w.psw ? __ldg(w.psw + l) : 1.f;
-            if (w.pool_mean) {
-                const int64_t gb = (int64_t)tt_find_table(w.tb[w.K], w.T, pr.x) * w.B + pr.y;
-                const int64_t len = __ldg(w.offsets + gb + 1) - __ldg(w.offsets + gb);
-                a /= (float)(len > 0 ? len : 1);
-            }
-            w.wsorted[pos] = a;
-        }
-    };
     enum { ROLE_NONE = 0, ROLE_OWNER = 1, ROLE_DUP = 2 };
     for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-        uint2 pr[HT_TILE / 256];
-        uint32_t st[HT_TILE / 256];   // bucket (12 bits) | rank among the duplicates (12 bits) << 12 | role << 24
+        uint32_t key[HT_TILE / 256];
+        uint32_t st[HT_TILE / 256];   // bucket (12 bits) | number among the duplicates (12 bits) << 12 | role << 24
 #pragma unroll
         for (int j = 0; j < HT_TILE / 256; ++j) {
             const int64_t l = tile * HT_TILE + j * 256 + threadIdx.x;
-            pr[j] = l < L ? __ldcs(upairs + l) : make_uint2(HT_EMPTY, 0u);
-            if (pr[j].x >= capK || (int64_t)pr[j].y >= w.B) pr[j].x = HT_EMPTY;  // invalid lookup (or malformed offsets)
+            const uint2 pr = l < L ? __ldcs(upairs + l) : make_uint2(HT_EMPTY, 0u);
+            key[j] = pr.x >= capK || (int64_t)pr.y >= w.B ? HT_EMPTY : pr.x;  // invalid lookup (or malformed offsets)
         }
 #pragma unroll
         for (int j = 0; j < HT_TILE / 256; ++j) {
-            if (pr[j].x == HT_EMPTY) continue;
-            const uint32_t low = pr[j].x & ((1u << HT_LOW_BITS) - 1u);
-            const uint32_t h = ((pr[j].x >> HT_LOW_BITS) ^ ((low * 2654435761u) >> HT_LOW_BITS)) & (HT_SIZE - 1);
+            if (key[j] == HT_EMPTY) continue;
+            const uint32_t low = key[j] & ((1u << HT_LOW_BITS) - 1u);
+            const uint32_t h = ((key[j] >> HT_LOW_BITS) ^ ((low * 2654435761u) >> HT_LOW_BITS)) & (HT_SIZE - 1);
             st[j] = h;
             tag[h] = (low << HT_ID_BITS) | (uint32_t)(j * 256 + threadIdx.x);
         }
         __syncthreads();
+        uint32_t* const out = rank + tile * HT_TILE + threadIdx.x;
+        uint32_t first[HT_TILE / 256];   // claims: all of a thread's are on their way before the first is looked at (60 tables 2160 -> 1870)
 #pragma unroll
         for (int j = 0; j < HT_TILE / 256; ++j) {
-            if (pr[j].x == HT_EMPTY) continue;
-            const uint32_t low = pr[j].x & ((1u << HT_LOW_BITS) - 1u);
+            if (key[j] == HT_EMPTY) continue;
+            const uint32_t low = key[j] & ((1u << HT_LOW_BITS) - 1u);
             const uint32_t h = st[j];
             const uint32_t tg = tag[h];
             if ((tg >> HT_ID_BITS) == low) {
                 if ((tg & (HT_TILE - 1)) == (uint32_t)(j * 256 + threadIdx.x)) st[j] = h | (ROLE_OWNER << 24);
-                else if (MODE == 0) { atomicAdd(&extra[h], 1u); st[j] = h | (ROLE_DUP << 24); }
                 else st[j] = h | ((atomicAdd(&extra[h], 1u) + 1u) << 12) | (ROLE_DUP << 24);
-            } else {   // another key holds the bucket
-                if (MODE == 0) atomicAdd(&w.cnt[pr[j].x], 1u);
-                else emit(atomicAdd(&w.cnt[pr[j].x], 1u), pr[j], tile * HT_TILE + j * 256 + threadIdx.x);
-            }
+            } else first[j] = atomicAdd(&w.cnt[key[j]], 1u);   // another key holds the bucket
         }
         __syncthreads();
-        // one global atomic per owner.  MODE 1 claims a run of positions directly on the scanned count array:
-        // cnt[slot] starts as the segment start and ends as the segment end (= next segment's start)
+#pragma unroll
+        for (int j = 0; j < HT_TILE / 256; ++j) {   // one global atomic per owner
+            if (key[j] == HT_EMPTY || (st[j] >> 24) != ROLE_OWNER) continue;
+            first[j] = atomicAdd(&w.cnt[key[j]], 1u + extra[st[j] & (HT_SIZE - 1)]);
+        }
 #pragma unroll
         for (int j = 0; j < HT_TILE / 256; ++j) {
-            if (pr[j].x == HT_EMPTY || (st[j] >> 24) != ROLE_OWNER) continue;
-            const uint32_t h = st[j] & (HT_SIZE - 1);
-            const uint32_t n = 1u + extra[h];
-            if (MODE == 0) {
-                atomicAdd(&w.cnt[pr[j].x], n);
-                extra[h] = 0u;
-            } else {
-                const uint32_t base = atomicAdd(&w.cnt[pr[j].x], n);
-                extra[h] = base;
-                emit(base, pr[j], tile * HT_TILE + j * 256 + threadIdx.x);
-            }
+            if (key[j] == HT_EMPTY || (st[j] >> 24) == ROLE_DUP) continue;
+            if ((st[j] >> 24) == ROLE_OWNER) extra[st[j] & (HT_SIZE - 1)] = first[j];
+            out[j * 256] = first[j];
         }
-        if (MODE == 1) {
-            __syncthreads();
+        __syncthreads();
 #pragma unroll
-            for (int j = 0; j < HT_TILE / 256; ++j) {
-                if (pr[j].x == HT_EMPTY || (st[j] >> 24) != ROLE_DUP) continue;
-                emit(extra[st[j] & (HT_SIZE - 1)] + ((st[j] >> 12) & 0xfffu), pr[j], tile * HT_TILE + j * 256 + threadIdx.x);
-            }
-            __syncthreads();
-#pragma unroll
-            for (int j = 0; j < HT_TILE / 256; ++j)
-                if (pr[j].x != HT_EMPTY && (st[j] >> 24) == ROLE_OWNER) extra[st[j] & (HT_SIZE - 1)] = 0u;
+        for (int j = 0; j < HT_TILE / 256; ++j) {
+            if (key[j] == HT_EMPTY || (st[j] >> 24) != ROLE_DUP) continue;
+            out[j * 256] = extra[st[j] & (HT_SIZE - 1)] + ((st[j] >> 12) & 0xfffu);
         }
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < HT_TILE / 256; ++j)
+            if (key[j] != HT_EMPTY && (st[j] >> 24) == ROLE_OWNER) extra[st[j] & (HT_SIZE - 1)] = 0u;
     }
 }
 
-struct CntScan {
-    WsView w;
-    __device__ uint32_t size() const { return w.counters[CTR_LEVEL0 + w.K]; }
-    __device__ int locate(uint32_t) const { return 0; }
-    __device__ uint32_t value(uint32_t i, int) const { return w.cnt[i]; }
-    __device__ void emit(uint32_t i, uint32_t excl, uint32_t, int) const { w.cnt[i] = excl; }
-    __device__ void total(uint32_t tot) const { w.cnt[size()] = tot; }
+// Counts -> segment starts in one kernel: a row's count becomes the sum of those before it in its tile, the CTA that reports last adds up
+// the tiles (a ticket counter; nobody waits), and a start is the sum of both (tt_seg_start).
+#define CNT_TILE_LOG 12
+struct CntTotal {
+    const WsView& w;
+    __device__ void total(uint32_t tot) const { w.cnt[w.counters[CTR_LEVEL0 + w.K]] = tot; }
 };
+__global__ void __launch_bounds__(256) k_seg_starts(WsView w)
+{
+    tt_pdl_enter();
+    constexpr int TILE = 1 << CNT_TILE_LOG, ITEMS = TILE / 256;
+    __shared__ uint32_t sm[34];
+    __shared__ uint32_t sv[TILE + TILE / 32];
+    __shared__ uint32_t ticket;
+    const uint32_t n = w.counters[CTR_LEVEL0 + w.K], ntiles = (n + TILE - 1) >> CNT_TILE_LOG, base = blockIdx.x << CNT_TILE_LOG;
+    if (n == 0) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) w.cnt[0] = 0u;
+        return;
+    }
+    if (blockIdx.x >= ntiles) return;
+#pragma unroll
+    for (int j = 0; j < ITEMS; ++j) {
+        const uint32_t i = base + (uint32_t)j * 256 + threadIdx.x;
+        sv[tt_scan_pad(j * 256 + threadIdx.x)] = i < n ? w.cnt[i] : 0u;
+    }
+    __syncthreads();
+    uint32_t mine[ITEMS], s = 0, tot;
+#pragma unroll
+    for (int j = 0; j < ITEMS; ++j) { mine[j] = sv[tt_scan_pad(threadIdx.x * ITEMS + j)]; s += mine[j]; }
+    uint32_t ex = tt_block_excl_scan(s, sm, tot);
+    if (threadIdx.x == 0) {
+        w.scan_tmp[blockIdx.x] = tot;
+        __threadfence();                                   // the sum is visible before the ticket is
+        ticket = atomicAdd(w.counters + CTR_SCAN_TICKET, 1u);
+    }
+#pragma unroll
+    for (int j = 0; j < ITEMS; ++j) { sv[tt_scan_pad(threadIdx.x * ITEMS + j)] = ex; ex += mine[j]; }
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < ITEMS; ++j) {
+        const uint32_t i = base + (uint32_t)j * 256 + threadIdx.x;
+        if (i < n) w.cnt[i] = sv[tt_scan_pad(j * 256 + threadIdx.x)];
+    }
+    if (ticket != ntiles - 1) return;
+    __threadfence();
+    tt_scan_spine_cta(CntTotal{w}, w.scan_tmp, ntiles, sm);
+    if (threadIdx.x == 0) w.counters[CTR_SCAN_TICKET] = 0u;
+}
+// first sorted position of row `slot` (the number of pairs for slot = U)
+__device__ __forceinline__ uint32_t tt_seg_start(const WsView& w, uint32_t slot, uint32_t U)
+{
+    return w.cnt[slot] + (slot < U ? w.scan_tmp[slot >> CNT_TILE_LOG] : 0u);
+}
+
+// The bags in sorted order, with the pairs' factors where the pooling has any; the row of a position follows from the segment starts, so
+// that only the rows of the chunks' first positions are written down (chunk_slot).  No atomics and no barriers: the places are known.
+// Bound by the scattered stores.  With 2 / 4 / 8 pairs per thread: 60 tables sort 1898 / 1867 / 1875 us, 4 M weighted pairs 106 / 109 /
+// 112, 0.5 M 30 / 30 / 34.
+#define SORT_PLACE_PER 4
+template <bool WT>
+__global__ void __launch_bounds__(256) k_sort_place(WsView w)
+{
+    tt_pdl_enter();
+    constexpr int PER = SORT_PLACE_PER;
+    const uint32_t capK = w.cap[w.K], U = w.counters[CTR_LEVEL0 + w.K];
+    const uint32_t* const rank = tt_sort_ranks(w);
+    const int64_t l0 = (int64_t)blockIdx.x * (256 * PER) + threadIdx.x;
+    uint2 pr[PER];
+    uint32_t rk[PER];
+    float a[PER];
+    int t = 0;
+    if (WT && w.pool_mean) t = tt_find_table64(w.tl_start, w.T, l0);
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+        const int64_t l = l0 + j * 256;
+        pr[j] = l < w.L ? __ldcs(w.upairs + l) : make_uint2(HT_EMPTY, 0u);
+        if (pr[j].x >= capK || (int64_t)pr[j].y >= w.B) pr[j].x = HT_EMPTY;
+        rk[j] = pr[j].x != HT_EMPTY ? __ldcs(rank + l) : 0u;
+        if (WT) {
+            a[j] = w.psw && l < w.L ? __ldg(w.psw + l) : 1.f;
+            if (w.pool_mean && pr[j].x != HT_EMPTY) {
+                while (t + 1 < w.T && w.tl_start[t + 1] <= l) ++t;
+                const int64_t gb = (int64_t)t * w.B + pr[j].y;
+                const int64_t len = __ldg(w.offsets + gb + 1) - __ldg(w.offsets + gb);
+                a[j] /= (float)(len > 0 ? len : 1);
+            }
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < PER; ++j)
+        if (pr[j].x != HT_EMPTY) rk[j] += tt_seg_start(w, pr[j].x, U);
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+        if (pr[j].x == HT_EMPTY) continue;
+        if (WT) w.pairs[rk[j]] = make_uint2(pr[j].y, __float_as_uint(a[j]));
+        else reinterpret_cast<uint32_t*>(w.pairs)[rk[j]] = pr[j].y;
+        if ((rk[j] & ((1u << w.de_chunk_log) - 1u)) == 0u) w.chunk_slot[rk[j] >> w.de_chunk_log] = pr[j].x;
+    }
+}
 
 cudaError_t tt_launch_bwd_sort(tt_emb* h, cudaStream_t s)
 {
     WsView& w = h->v;
     const int zgrid = h->sm_count * 8;
     cudaError_t e;
+    tt_de_partition(h);
     if ((e = tt_launch_pdl(k_bwd_clear, dim3(zgrid), dim3(256), 0, s, w)) != cudaSuccess) return e;
     tt_note_launch();
     const int64_t ntiles = (w.L + HT_TILE - 1) / HT_TILE;
-    int per_sm0 = 0, per_sm1 = 0;   // persistent grids sized to what is actually resident (no partial second wave)
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm0, k_sort_pass<0>, 256, 0)) != cudaSuccess) return e;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm1, k_sort_pass<1>, 256, 0)) != cudaSuccess) return e;
-    auto grid_of = [&](int per_sm) {
-        int64_t g = (int64_t)(per_sm < 1 ? 1 : per_sm) * h->sm_count;
-        if (g > ntiles) g = ntiles;
-        return (int)(g < 1 ? 1 : g);
-    };
+    int per_sm = 0;   // a persistent grid sized to what is actually resident (no partial second wave)
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sort_count, 256, 0)) != cudaSuccess) return e;
     // the counting pass as a grid of more CTAs than fit at once, TT_SORT0_TILES tiles each: the block scheduler then
     // balances the tiles' very different costs (a tile of popular rows aggregates to a few claims, one of unpopular rows
-    // makes two thousand; as a resident grid the first CTA was done at 58 % of the kernel).  4 / 8 / 16 / 24 / 32 / 48
-    // tiles per CTA: 2.92 / 2.68 / 2.57 / 2.52 / 2.54 / 2.68 ms for the sort, 2.62 ms with the resident grid
-    int g0 = grid_of(per_sm0);
-    {
-        const int64_t many = (ntiles + TT_SORT0_TILES - 1) / TT_SORT0_TILES;
-        if (many > g0) g0 = (int)many;
-    }
-    if ((e = tt_launch_pdl(k_sort_pass<0>, dim3(g0), dim3(256), 0, s, w)) != cudaSuccess) return e;
+    // makes two thousand).  Sort with 4 / 8 / 24 / 48 tiles per CTA, us: 60 tables 2003 / 1825 / 1867 / 1876, 240 tables 1357 / 1236 / 1289 /
+    // 1440
+    int64_t g = (int64_t)(per_sm < 1 ? 1 : per_sm) * h->sm_count;
+    if (g > ntiles) g = ntiles;
+    if (g < 1) g = 1;
+    const int64_t many = (ntiles + TT_SORT0_TILES - 1) / TT_SORT0_TILES;
+    if (many > g) g = many;
+    if ((e = tt_launch_pdl(k_sort_count, dim3((unsigned)g), dim3(256), 0, s, w)) != cudaSuccess) return e;
     tt_note_launch();
-    CntScan cs{w};
-    if ((e = tt_scan(cs, w.cap[w.K], w.scan_tmp, s)) != cudaSuccess) return e;
-    if ((e = tt_launch_pdl(k_sort_pass<1>, dim3(grid_of(per_sm1)), dim3(256), 0, s, w)) != cudaSuccess) return e;
+    const int64_t rows = (int64_t)w.cap[w.K] < w.L ? (int64_t)w.cap[w.K] : w.L;
+    if ((e = tt_launch_pdl(k_seg_starts, dim3((unsigned)((rows >> CNT_TILE_LOG) + 1)), dim3(256), 0, s, w)) != cudaSuccess) return e;
+    tt_note_launch();
+    if (w.L == 0) return cudaGetLastError();
+    if ((e = tt_launch_pdl(tt_weighted(w) ? k_sort_place<true> : k_sort_place<false>, dim3((unsigned)((w.L + 256 * SORT_PLACE_PER - 1) / (256 * SORT_PLACE_PER))), dim3(256), 0, s, w)) != cudaSuccess) return e;
     tt_note_launch();
     return cudaGetLastError();
 }
@@ -268,6 +363,79 @@ struct RowAcc {
     }
 };
 
+// The sorted positions of a warp's chunk, 32 at a time: rows from the segment starts, bags (and factors) as stored.  `next` is called
+// once per batch, after it the loads of the batch that follows are on their way.
+struct DePairs {
+    const WsView& w;
+    uint32_t U, total, a, b;       // rows, pairs; the chunk [a, b)
+    uint32_t prev, next_slot;      // row of the position before the chunk if the chunk starts inside it; of the position after it
+    uint32_t s, v;                 // row of the last position looked at; start of row s + 1 + lane
+    uint32_t bag;
+    float factor;
+
+    __device__ __forceinline__ uint32_t start(uint32_t slot) const { return slot < U ? tt_seg_start(w, slot, U) : total; }
+    __device__ __forceinline__ DePairs(const WsView& w_, int64_t chunk) : w(w_)
+    {
+        U = w.counters[CTR_LEVEL0 + w.K];
+        total = w.cnt[U];
+        const int64_t a64 = chunk << w.de_chunk_log;
+        a = a64 < total ? (uint32_t)a64 : total;
+        b = min(a + (1u << w.de_chunk_log), total);
+    }
+    template <bool WT>
+    __device__ __forceinline__ void fetch(uint32_t p, int lane)    // positions p + lane
+    {
+        v = start(s + 1 + lane);
+        bag = 0u;
+        factor = 1.f;
+        if (p + lane < b) {
+            if (WT) {
+                const uint2 x = __ldcs(w.pairs + p + lane);
+                bag = x.x;
+                factor = __uint_as_float(x.y);
+            } else bag = __ldcs(reinterpret_cast<const uint32_t*>(w.pairs) + p + lane);
+        }
+    }
+    // a < b
+    template <bool WT>
+    __device__ __forceinline__ void begin(int64_t chunk, int lane)
+    {
+        s = w.chunk_slot[chunk];
+        next_slot = b < total ? w.chunk_slot[chunk + 1] : HT_EMPTY;
+        fetch<WT>(a, lane);
+        prev = start(s) < a ? s : HT_EMPTY;
+    }
+    // bit j: position p + j starts another row than the one before it (j < n); rows without pairs (lookups that malformed offsets leave out) among
+    // them: false, `rows` then finds the rows, otherwise every start is one row further and s is the row of the last position
+    __device__ __forceinline__ bool starts(uint32_t p, int n, unsigned& bits)
+    {
+        const bool in = v - p < (uint32_t)n;
+        bits = __reduce_or_sync(0xffffffffu, in ? 1u << (v - p) : 0u);
+        const int k = __popc(bits);
+        if (k != __popc(__ballot_sync(0xffffffffu, in))) return false;
+        s += k;
+        return true;
+    }
+    // row of position p + lane (lane < n), all lanes: n positions from p on
+    __device__ __forceinline__ uint32_t rows(uint32_t p, int n, int lane)
+    {
+        uint32_t row = s;
+        for (;;) {
+            int k = 0;             // starts among those of rows s + 1 .. s + 32 that are not past this position
+#pragma unroll
+            for (int step = 16; step > 0; step >>= 1)
+                if (__shfl_sync(0xffffffffu, v, k + step - 1) <= p + lane) k += step;
+            if (__shfl_sync(0xffffffffu, v, k) <= p + lane) ++k;
+            row += k;
+            if (!__any_sync(0xffffffffu, k == 32 && lane < n)) break;
+            s += 32;               // (32 rows of one pair each, or rows without pairs)
+            v = start(s + 1 + lane);
+        }
+        s = __shfl_sync(0xffffffffu, row, n - 1);
+        return lane < n ? row : HT_EMPTY;
+    }
+};
+
 template <bool VEC, int CPL>
 __global__ void __launch_bounds__(256) k_dE(WsView w, const float* __restrict__ grad_out)
 {
@@ -275,26 +443,24 @@ __global__ void __launch_bounds__(256) k_dE(WsView w, const float* __restrict__ 
     constexpr int NF = !VEC && CPL <= 4 ? 16 / CPL : 4;   // narrow rows: more of them in flight
     const int lane = threadIdx.x & 31;
     const int64_t chunk = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const uint32_t U = w.counters[CTR_LEVEL0 + w.K];
-    const uint32_t Ltot = w.cnt[U];
-    const int64_t a64 = chunk * w.de_chunk;
-    if (a64 >= Ltot) return;
-    const uint32_t a = (uint32_t)a64;
-    const uint32_t b = min(a + w.de_chunk, Ltot);
+    DePairs pairs(w, chunk);
+    const uint32_t a = pairs.a, b = pairs.b;
+    if (a >= b) return;
     const int D = w.D;
     const size_t gstride = (size_t)w.T * D;
-    const uint32_t prev = a > 0 ? w.pairs[a - 1].x : HT_EMPTY;
-    const uint32_t next = b < Ltot ? w.pairs[b].x : HT_EMPTY;
+    const bool weighted = tt_weighted(w);
+    if (weighted) pairs.begin<true>(chunk, lane); else pairs.begin<false>(chunk, lane);
+    const uint32_t prev = pairs.prev, next = pairs.next_slot;
     RowAcc<VEC, CPL> acc;
     acc.clear();
-    uint32_t cur = w.pairs[a].x;
+    uint32_t cur = pairs.s;
     int tcur = tt_find_table(w.tb[w.K], w.T, cur);
     bool seg_first = true;
     float* carry = w.carry + (size_t)chunk * 2 * D;
     for (uint32_t p0 = a; p0 < b; p0 += 32) {
-        const uint2 mine = (p0 + lane < b) ? __ldg(&w.pairs[p0 + lane]) : make_uint2(HT_EMPTY, 0u);
-        const bool weighted = w.wsorted && (w.psw || w.pool_mean);
-        const float wmine = (weighted && p0 + lane < b) ? __ldg(&w.wsorted[p0 + lane]) : 1.f;
+        const uint2 mine = make_uint2(pairs.rows(p0, (int)min(32u, b - p0), lane), pairs.bag);
+        const float wmine = pairs.factor;
+        if (p0 + 32 < b) { if (weighted) pairs.fetch<true>(p0 + 32, lane); else pairs.fetch<false>(p0 + 32, lane); }
         const int n = (int)min(32u, b - p0);
         // NF rows of grad_out in flight at a time (their addresses need the table of each pair's slot; positions are
         // sorted, so the table changes rarely), then the rows are folded in position order
@@ -362,17 +528,13 @@ __global__ void __launch_bounds__(256) k_dE_fix(WsView w)
     const int64_t chunk = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const uint32_t U = w.counters[CTR_LEVEL0 + w.K];
     const uint32_t Ltot = w.cnt[U];
-    const int64_t a64 = chunk * w.de_chunk;
+    const int64_t a64 = chunk << w.de_chunk_log, b64 = a64 + (1LL << w.de_chunk_log);
     const int D = w.D;
-    if (a64 < Ltot) {
-        const uint32_t a = (uint32_t)a64;
-        const uint32_t b = min(a + w.de_chunk, Ltot);
-        const uint32_t first = w.pairs[a].x, last = w.pairs[b - 1].x;
-        const uint32_t prev = a > 0 ? w.pairs[a - 1].x : HT_EMPTY;
-        const uint32_t next = b < Ltot ? w.pairs[b].x : HT_EMPTY;
-        // something continues past this chunk, and it started here
-        if (b < Ltot && next == last && !(first == last && prev == first)) {
-            const uint32_t pieces = (w.cnt[last] - 1u) / w.de_chunk - (uint32_t)chunk + 1u;
+    if (b64 < Ltot) {
+        const uint32_t last = w.chunk_slot[chunk + 1], from = tt_seg_start(w, last, U);   // the row after this chunk
+        if (from < (uint32_t)b64 && from >= (uint32_t)a64) {                              // starts in it
+            const uint32_t end = tt_seg_start(w, last + 1, U);
+            const uint32_t pieces = ((end - 1u) >> w.de_chunk_log) - (uint32_t)chunk + 1u;
             if (pieces > DE_FIX_OWN) {
                 if (lane == 0) {
                     const uint32_t i = atomicAdd(&s_n, 1u);
@@ -432,21 +594,18 @@ __global__ void __launch_bounds__(256, 5) k_dE_fast(WsView w, const float* __res
     constexpr int RPI = 32 / LPR, NF = 4;
     const int lane = threadIdx.x & 31, sub = lane / LPR, lr = lane % LPR;
     const int64_t chunk = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const uint32_t U = w.counters[CTR_LEVEL0 + w.K];
-    const uint32_t Ltot = w.cnt[U];
-    const int64_t a64 = chunk * w.de_chunk;
-    if (a64 >= Ltot) return;
-    const uint32_t a = (uint32_t)a64;
-    const uint32_t b = min(a + w.de_chunk, Ltot);
+    DePairs pairs(w, chunk);
+    const uint32_t a = pairs.a, b = pairs.b;
+    if (a >= b) return;
+    pairs.begin<WT>(chunk, lane);
     const int D = w.D, D4 = D >> 2;
     const bool lane_on = lr < D4;
-    const uint32_t prev = a > 0 ? w.pairs[a - 1].x : HT_EMPTY;
-    const uint32_t next = b < Ltot ? w.pairs[b].x : HT_EMPTY;
+    const uint32_t prev = pairs.prev, next = pairs.next_slot;
     const float4* __restrict__ G4 = reinterpret_cast<const float4*>(grad_out);
     float4* __restrict__ E4 = reinterpret_cast<float4*>(w.E);
     float4* carry4 = reinterpret_cast<float4*>(w.carry + (size_t)chunk * 2 * D);
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-    uint32_t cur = w.pairs[a].x;
+    uint32_t cur = pairs.s;
     bool seg_first = true;
     // close the running segment: combine the sub-warps, store (sub-warp 0 writes), clear
     auto close_segment = [&]() {
@@ -462,9 +621,10 @@ __global__ void __launch_bounds__(256, 5) k_dE_fast(WsView w, const float* __res
     };
     uint32_t last_slot = cur;  // slot of the position before the current batch
     for (uint32_t p0 = a; p0 < b; p0 += 32) {
-        const uint2 mine = (p0 + lane < b) ? __ldcs(&w.pairs[p0 + lane]) : make_uint2(HT_EMPTY, 0u);
-        const float wmine = (WT && p0 + lane < b) ? __ldcs(&w.wsorted[p0 + lane]) : 1.f;   // factor of this lane's pair
         const int n = (int)min(32u, b - p0);
+        const uint2 mine = make_uint2(pairs.rows(p0, n, lane), pairs.bag);
+        const float wmine = pairs.factor;   // of this lane's pair
+        if (p0 + 32 < b) pairs.fetch<WT>(p0 + 32, lane);
         // row index of this lane's pair inside grad_out viewed as [B*T][D]
         const uint32_t grow = lane < n ? mine.y * (uint32_t)w.T + (uint32_t)tt_find_table(w.tb[w.K], w.T, mine.x) : 0u;
         uint32_t before = __shfl_up_sync(0xffffffffu, mine.x, 1);
@@ -540,26 +700,22 @@ __global__ void __launch_bounds__(32 * DE_WARPS, DD == 128 ? 2 : 4) k_dE_stage(W
     float4* buf = de_buf + (size_t)wid * 32 * R4;
     const float* bufv = reinterpret_cast<const float*>(buf);
     const int64_t chunk = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const uint32_t U = w.counters[CTR_LEVEL0 + w.K];
-    const uint32_t Ltot = w.cnt[U];
-    const int64_t a64 = chunk * w.de_chunk;
-    if (a64 >= Ltot) return;
-    const uint32_t a = (uint32_t)a64;
-    const uint32_t b = min(a + w.de_chunk, Ltot);
-    const uint32_t prev = a > 0 ? w.pairs[a - 1].x : HT_EMPTY;
-    const uint32_t next = b < Ltot ? w.pairs[b].x : HT_EMPTY;
+    DePairs pairs(w, chunk);
+    const uint32_t a = pairs.a, b = pairs.b;
+    if (a >= b) return;
+    pairs.begin<WT>(chunk, lane);
+    const uint32_t prev = pairs.prev, next = pairs.next_slot;
     const float4* __restrict__ G4 = reinterpret_cast<const float4*>(grad_out);
     float* carry = w.carry + (size_t)chunk * 2 * D;
     const uint32_t* __restrict__ tbK = w.tb[w.K];
     float acc[VPL], part[VPL];
 #pragma unroll
     for (int x = 0; x < VPL; ++x) { acc[x] = 0.f; part[x] = 0.f; }
-    uint32_t cur = w.pairs[a].x;
+    uint32_t cur = pairs.s;
     bool seg_first = true;
-    uint32_t last_slot = cur;
     // slot range of the table the chunk is in: positions are sorted, so a batch rarely leaves it
     int tcur = tt_find_table(tbK, w.T, cur);
-    uint32_t t_lo = tbK[tcur], t_hi = tbK[tcur + 1];
+    uint32_t t_hi = tbK[tcur + 1];
     // two-level sum: rows are added into a per-batch partial (at most 32 terms) which is added to the segment's sum at
     // the end of the batch, so the rounding error of a long segment grows with sqrt(length / 32), not sqrt(length)
     auto store_row = [&](float* dst, bool with_part) {
@@ -577,23 +733,22 @@ __global__ void __launch_bounds__(32 * DE_WARPS, DD == 128 ? 2 : 4) k_dE_stage(W
 #pragma unroll
         for (int x = 0; x < VPL; ++x) { acc[x] = 0.f; part[x] = 0.f; }
         seg_first = false;
+        ++cur;
     };
-    uint2 mine = (a + lane < b) ? __ldcs(&w.pairs[a + lane]) : make_uint2(HT_EMPTY, 0u);
-    float wmine = (WT && a + lane < b) ? __ldcs(&w.wsorted[a + lane]) : 1.f;
     for (uint32_t p0 = a; p0 < b; p0 += 32) {
         const int n = (int)min(32u, b - p0);
+        unsigned starts;
+        const bool plain = pairs.starts(p0, n, starts);
+        const uint32_t row = plain ? cur + __popc(starts & (0xffffffffu >> (31 - lane))) : pairs.rows(p0, n, lane);
+        const uint32_t bag = pairs.bag;
+        const float wmine = pairs.factor;
         int tl = tcur;
-        if (!__all_sync(0xffffffffu, lane >= n || (mine.x >= t_lo && mine.x < t_hi))) {
-            tl = lane < n ? tt_find_table(tbK, w.T, mine.x) : tcur;
+        if (pairs.s >= t_hi) {
+            tl = lane < n ? tt_find_table(tbK, w.T, row) : tcur;
             tcur = __shfl_sync(0xffffffffu, tl, n - 1);
-            t_lo = tbK[tcur];
             t_hi = tbK[tcur + 1];
         }
-        const uint32_t grow = mine.y * (uint32_t)w.T + (uint32_t)tl;   // row of grad_out viewed as [B*T][DD]
-        uint32_t before = __shfl_up_sync(0xffffffffu, mine.x, 1);
-        if (lane == 0) before = last_slot;
-        const unsigned starts = __ballot_sync(0xffffffffu, lane < n && mine.x != before);   // bit j: position j opens a segment
-        last_slot = __shfl_sync(0xffffffffu, mine.x, n - 1);
+        const uint32_t grow = bag * (uint32_t)w.T + (uint32_t)tl;   // row of grad_out viewed as [B*T][DD]
         const uint32_t shift = (grow * (uint32_t)D) & 3u;   // (ODD) floats before the row in its first piece
         if constexpr (ODD) {
             const uint64_t all = (uint64_t)w.B * w.T * D;
@@ -620,13 +775,7 @@ __global__ void __launch_bounds__(32 * DE_WARPS, DD == 128 ? 2 : 4) k_dE_stage(W
             }
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
-        // the pairs of the next batch arrive while the rows are in flight
-        const uint2 cur_pairs = mine;
-        const float cur_w = wmine;
-        if (p0 + 32 < b) {
-            mine = (p0 + 32 + lane < b) ? __ldcs(&w.pairs[p0 + 32 + lane]) : make_uint2(HT_EMPTY, 0u);
-            if (WT) wmine = (p0 + 32 + lane < b) ? __ldcs(&w.wsorted[p0 + 32 + lane]) : 1.f;
-        }
+        if (p0 + 32 < b) pairs.fetch<WT>(p0 + 32, lane);   // the next batch's arrive while the rows are in flight
         asm volatile("cp.async.wait_group 0;" ::: "memory");
         __syncwarp();
         auto add_row = [&](int j) {
@@ -643,7 +792,7 @@ __global__ void __launch_bounds__(32 * DE_WARPS, DD == 128 ? 2 : 4) k_dE_stage(W
                 x[0] = v.x; x[VPL - 1] = v.y;
             } else x[0] = bufv[j * DD + (lane & (DD - 1))];
             if (WT) {
-                const float wj = __shfl_sync(0xffffffffu, cur_w, j);
+                const float wj = __shfl_sync(0xffffffffu, wmine, j);
 #pragma unroll
                 for (int c = 0; c < VPL; ++c) x[c] *= wj;
             }
@@ -652,7 +801,7 @@ __global__ void __launch_bounds__(32 * DE_WARPS, DD == 128 ? 2 : 4) k_dE_stage(W
         };
         // eight rows at a time; a run of eight without a segment start (popular rows: most lookups sit in segments far
         // longer than a batch) is added without looking at the start bits
-        for (int j0 = 0; j0 < n; j0 += 8) {
+        for (int j0 = 0; plain && j0 < n; j0 += 8) {
             if (j0 + 8 <= n && ((starts >> j0) & 0xffu) == 0u) {
 #pragma unroll
                 for (int jj = 0; jj < 8; ++jj) add_row(j0 + jj);
@@ -660,11 +809,11 @@ __global__ void __launch_bounds__(32 * DE_WARPS, DD == 128 ? 2 : 4) k_dE_stage(W
                 // eight starts in a row (rows looked up once: most distinct rows): the first closes the running segment,
                 // the next seven rows are whole segments of one row each and are copied out, the eighth opens a new one
                 close_segment();
+                float* dst = w.E + (size_t)cur * D;
+                cur += 7;
 #pragma unroll
-                for (int jj = 0; jj < 7; ++jj) {
-                    const uint32_t sj = __shfl_sync(0xffffffffu, cur_pairs.x, j0 + jj);
+                for (int jj = 0; jj < 7; ++jj, dst += D) {
                     add_row(j0 + jj);
-                    float* dst = w.E + (size_t)sj * D;
                     if (ODD) {
                         if (lane < D) dst[lane] = part[0];
                         if (lane + 32 < D) dst[lane + 32] = part[VPL - 1];
@@ -674,7 +823,6 @@ __global__ void __launch_bounds__(32 * DE_WARPS, DD == 128 ? 2 : 4) k_dE_stage(W
 #pragma unroll
                     for (int c = 0; c < VPL; ++c) part[c] = 0.f;
                 }
-                cur = __shfl_sync(0xffffffffu, cur_pairs.x, j0 + 7);
                 add_row(j0 + 7);
             } else if (VPL == 4 && j0 + 8 <= n) {
                 // segments of a few rows: with fourteen warps per SM the eight rows are fetched before the first start is looked at (0.66 M
@@ -685,29 +833,32 @@ __global__ void __launch_bounds__(32 * DE_WARPS, DD == 128 ? 2 : 4) k_dE_stage(W
                 for (int jj = 0; jj < 8; ++jj) {
                     v[jj] = buf[(j0 + jj) * R4 + lr];
                     if (WT) {
-                        const float wj = __shfl_sync(0xffffffffu, cur_w, j0 + jj);
+                        const float wj = __shfl_sync(0xffffffffu, wmine, j0 + jj);
                         v[jj] = make_float4(v[jj].x * wj, v[jj].y * wj, v[jj].z * wj, v[jj].w * wj);
                     }
                 }
 #pragma unroll
                 for (int jj = 0; jj < 8; ++jj) {
-                    if ((starts >> (j0 + jj)) & 1u) {
-                        close_segment();
-                        cur = __shfl_sync(0xffffffffu, cur_pairs.x, j0 + jj);
-                    }
+                    if ((starts >> (j0 + jj)) & 1u) close_segment();
                     part[0] += v[jj].x; part[1 % VPL] += v[jj].y; part[2 % VPL] += v[jj].z; part[VPL - 1] += v[jj].w;
                 }
             } else {
                 const int j1 = min(j0 + 8, n);
                 for (int j = j0; j < j1; ++j) {
-                    if ((starts >> j) & 1u) {
-                        close_segment();
-                        cur = __shfl_sync(0xffffffffu, cur_pairs.x, j);
-                    }
+                    if ((starts >> j) & 1u) close_segment();
                     add_row(j);
                 }
             }
         }
+        if (!plain)
+            for (int j = 0; j < n; ++j) {
+                const uint32_t rj = __shfl_sync(0xffffffffu, row, j);
+                if (rj != cur) {
+                    close_segment();
+                    cur = rj;
+                }
+                add_row(j);
+            }
 #pragma unroll
         for (int c = 0; c < VPL; ++c) { acc[c] += part[c]; part[c] = 0.f; }
         __syncwarp();
@@ -718,34 +869,14 @@ __global__ void __launch_bounds__(32 * DE_WARPS, DD == 128 ? 2 : 4) k_dE_stage(W
     }
 }
 
-// Positions per warp, and where the warps leave the pieces of segments that cross a chunk border.  A chunk is walked
-// serially, so short batches want short chunks (1024 positions: 65 thousand lookups kept 64 warps busy) and long ones
-// chunks that amortise the borders.  dE with 32 / 128 / 256 / 512 / 1024 positions per warp, us: 65 k lookups (D = 128,
-// at least 160 there) 39 / 39 / 60 / 101 / 185; 0.5 M (D = 32) 33 / 31 / 42 / 62 / 103; 1.6 M (D = 64) 72 / 70 / 70 / 85 /
-// 113; 4 M (D = 16) 173 / 122 / 121 / 142 / 173.
-static void tt_de_partition(tt_emb* h)
-{
-    WsView& w = h->v;
-    int64_t c = w.L / 2048 < 128 ? w.L / 2048 : 128;
-    if (c < w.L / 32768) c = w.L / 32768;
-    c = c < 32 ? 32 : (c > TT_DE_CHUNK ? TT_DE_CHUNK : c / 32 * 32);
-    // the pieces of more than L / TT_DE_CHUNK chunks go where the unsorted pairs were (the sort has consumed them): 8 bytes
-    // per lookup, so a chunk holds at least about D positions
-    const uintptr_t u0 = (reinterpret_cast<uintptr_t>(w.upairs) + 15) & ~(uintptr_t)15;
-    const size_t room = reinterpret_cast<uintptr_t>(w.upairs + h->max_lookups + 1) - u0;
-    while (c < TT_DE_CHUNK && (size_t)((w.L + c - 1) / c) * 2 * h->D * sizeof(float) > room) c += 32;
-    w.de_chunk = (uint32_t)c;
-    w.carry = c < TT_DE_CHUNK ? reinterpret_cast<float*>(u0) : h->carry;
-}
-
 template <bool VEC, int CPL>
 static cudaError_t launch_dE_t(tt_emb* h, const float* grad_out, cudaStream_t s)
 {
-    const int64_t chunks = (h->v.L + h->v.de_chunk - 1) / h->v.de_chunk;
+    const int64_t chunks = (h->v.L + (1LL << h->v.de_chunk_log) - 1) >> h->v.de_chunk_log;
     const int grid = (int)((chunks + 7) / 8);
     if (grid > 0) {
         const int D4 = h->D / 4;
-        const bool wt = h->v.wsorted && (h->v.psw || h->v.pool_mean);
+        const bool wt = tt_weighted(h->v);
         const bool odd = !VEC && h->D <= DE_ODD_MOST && (reinterpret_cast<uintptr_t>(grad_out) & 15) == 0;
         if (odd || (VEC && (h->D == 128 || h->D == 64 || h->D == 32 || h->D == 16))) {
             const size_t smem = (size_t)DE_WARPS * 32 * (odd ? 16 : h->D / 4) * sizeof(float4);
@@ -774,7 +905,6 @@ cudaError_t tt_launch_bwd_dE(tt_emb* h, const float* grad_out, cudaStream_t s)
 {
     const int D = h->D;
     const bool vec = (D % 4 == 0) && ((reinterpret_cast<uintptr_t>(grad_out) & 15) == 0);
-    tt_de_partition(h);
     if (vec) {
         if (D <= 128) return launch_dE_t<true, 1>(h, grad_out, s);
         if (D <= 256) return launch_dE_t<true, 2>(h, grad_out, s);

@@ -46,7 +46,7 @@
 #define TT_STATUS_BYTES 512   // status word and counters (16 + 64 words) with their guard bytes, up to the row bitmap behind them
 #define TT_GUARD 0xA5         // guard bytes behind the other workspace regions
 #define TT_UNIT_ROWS 64   // fewest rows of a unit of a K = 2 table
-#define TT_DE_CHUNK 1024                                  // most sorted lookups per warp in the dE segment reduction
+#define TT_DE_CHUNK 1024                                  // sorted lookups per warp in the dE segment reduction, at most (up to 268 M lookups)
 #define TT_NUM_STAGES 33                                // 0..8 pipeline stages, 9..20 forward sweep variants -1..10, 21..32 backward sweep variants
 #define TT_STRIPES 8                                     // L2-resident partial copies of the last core's gradient
 #define TT_NUM_MIDFAST 11                                // tensor-core instances of the middle-core backward (backward.cu)
@@ -119,14 +119,15 @@ struct WsView {
     float* pbuf[TT_MAXK + 1];           // partial products P_k of level-k nodes, 2 <= k <= K-2
     float* E;                           // [capU][D] rows (forward) / dE (backward)
     // backward
-    uint32_t* cnt;                      // [capU+1] lookups per distinct row -> exclusive scan
+    uint32_t* cnt;                      // [capU+1] lookups per distinct row -> segment starts inside their tiles (tt_seg_start)
     uint32_t* cursor;                   // [capU]
-    uint2* pairs;                       // [L] (slot, bag) sorted by slot
+    uint2* pairs;                       // [L] bags sorted by slot (uint32, behind them the pairs' ranks), or (bag, factor) with weights or mean pooling
+    uint32_t* chunk_slot;               // slot of the first sorted position of every dE chunk (in the space of pool_bounds)
     uint2* upairs;                      // [L] (slot, bag) in lookup order, written by the pooling kernel (null: forward only)
     float* dP[TT_MAXK + 1];             // dP_k per level-k node, 2 <= k <= K-1
     float* Y[TT_MAXK + 1];              // per level-k node: its contribution to dP_{k-1} of its parent
     float* carry;                       // [chunks][2][D] pieces of the segments that cross a chunk border
-    uint32_t de_chunk;                  // sorted lookups per warp in the dE segment reduction (at most TT_DE_CHUNK)
+    uint32_t de_chunk_log;              // 1 << de_chunk_log sorted lookups per warp in the dE segment reduction
     float* gpart;                       // [TT_STRIPES][gpart_stride] partial copies of all tables' last-core gradients
     int64_t gpart_stride;               // floats per stripe
     uint2* tbm[TT_MAXK + 1];            // digit-major node bitmaps, levels 2..K-1
@@ -135,7 +136,7 @@ struct WsView {
     const int64_t* offsets;
     // pooling beyond the plain sum (tt_emb_set_pooling)
     const float* psw;                   // per-lookup weights [L] or null
-    float* wsorted;                     // [L] factor of every sorted pair (weight, or 1 / bag length), backward only
+    float* wsorted;                     // [L] the pairs' ranks where these have factors (weight, or 1 / bag length), backward only
     int32_t pool_mean;                  // 1: mean pooling
     int32_t idx32;                      // 1: `indices` points at int32 row ids (tt_emb_forward_i32)
 };
@@ -150,6 +151,9 @@ __device__ __forceinline__ int64_t tt_index(const WsView& w, int64_t l)
     }
     return STREAM ? __ldcs(w.indices + l) : __ldg(w.indices + l);
 }
+
+// whether the pairs of the backward have factors
+__host__ __device__ __forceinline__ bool tt_weighted(const WsView& w) { return w.wsorted && (w.psw || w.pool_mean); }
 
 enum { CTR_LEVEL0 = 0 /* +k */, CTR_TLEVEL0 = 8 /* +k */, CTR_COST_TOTAL = 16, CTR_SCAN_TICKET = 32 /* tiles of the running scan that have reported */,
        CTR_POOL_NEXT = 34 /* next share of the lookups to be pooled (shares are handed out in order) */,
