@@ -5,8 +5,8 @@
 //             would serialise global atomics, so each CTA first aggregates the duplicates of its tile in shared memory (owner
 //             tags) and issues one global atomic per aggregated row per tile.
 //   2. dE:    segmented sum of grad_out rows over the sorted pairs.  Fixed-size chunks of sorted positions per
-//             warp (skew-proof); segments that cross chunk borders leave partial sums which a second kernel
-//             adds in position order.
+//             warp (skew-proof); segments that cross chunk borders leave partial sums, which the last warp to arrive,
+//             or with many chunks a second kernel, adds in position order.
 //   3. last level: per group, C is rebuilt in shared memory; every row contributes C^T.dE to the slice of
 //             the last core it selects and dE.D^T to the group's dC (summed over the rows sharing C before
 //             going up, Eq. 2; the sum is the k-loop of the tensor-core product, so dC is written once).
@@ -50,6 +50,7 @@ __global__ void __launch_bounds__(256) k_bwd_clear(WsView w)
     if (x < parts * w.T) { g0 = w.tdesc[x % w.T].grad[0]; floats = w.tdesc[x % w.T].core_floats[0]; }   // (on their way during the clears below)
     const uint32_t n = w.counters[CTR_LEVEL0 + w.K] + 1u;
     for (uint32_t i = first; i < n; i += step) w.cnt[i] = 0u;
+    for (uint32_t i = first; (uint64_t)i << w.de_chunk_log < (uint64_t)w.L; i += step) w.chunk_ctr[i] = 0u;
     float4* g4 = reinterpret_cast<float4*>(w.gpart);                 // every table's copy is a whole number of float4s
     const int64_t n4 = (int64_t)TT_STRIPES * w.gpart_stride / 4;
     for (int64_t i = first; i < n4; i += step) g4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -78,9 +79,10 @@ static void tt_de_partition(tt_emb* h)
     const size_t room = reinterpret_cast<uintptr_t>(w.upairs + h->max_lookups + 1) - u0;
     while ((1 << log) < TT_DE_CHUNK && (size_t)((w.L + (1LL << log) - 1) >> log) * 2 * h->D * sizeof(float) > room) ++log;
     w.carry = (1 << log) < TT_DE_CHUNK ? reinterpret_cast<float*>(u0) : h->carry;
-    while (((w.L + (1LL << log) - 1) >> log) > 2 * TT_POOL_MAX_SHARES) ++log;   // the room for the chunks' first rows
+    while (((w.L + (1LL << log) - 1) >> log) > TT_POOL_MAX_SHARES) ++log;   // the room for the chunks' first rows and counters
     w.de_chunk_log = (uint32_t)log;
     w.chunk_slot = reinterpret_cast<uint32_t*>(w.pool_bounds);   // (the pooling is done with its boundaries)
+    w.chunk_ctr = w.chunk_slot + TT_POOL_MAX_SHARES + 1;
 }
 
 // ---------------------------------------------------------------------------------------------- 1. sort by slot
@@ -363,12 +365,14 @@ struct RowAcc {
     }
 };
 
+#define DE_SPILL_LOG 1     // half a chunk
 // The sorted positions of a warp's chunk, 32 at a time: rows from the segment starts, bags (and factors) as stored.  `next` is called
 // once per batch, after it the loads of the batch that follows are on their way.
 struct DePairs {
     const WsView& w;
     uint32_t U, total, a, b;       // rows, pairs; the chunk [a, b)
     uint32_t prev, next_slot;      // row of the position before the chunk if the chunk starts inside it; of the position after it
+    uint32_t row0, from, till;     // row of the chunk's first position, its first position and the one after its last
     uint32_t s, v;                 // row of the last position looked at; start of row s + 1 + lane
     uint32_t bag;
     float factor;
@@ -396,14 +400,42 @@ struct DePairs {
             } else bag = __ldcs(reinterpret_cast<const uint32_t*>(w.pairs) + p + lane);
         }
     }
-    // a < b
-    template <bool WT>
+    // Positions that a chunk takes of the next one to end its last segment, instead of leaving a piece of it there
+    __device__ __forceinline__ uint32_t spill() const { return (1u << w.de_chunk_log) >> DE_SPILL_LOG; }
+    // a < b before; afterwards a = b where the chunk before has taken all of this one's positions
+    template <bool WT, bool JOIN>
     __device__ __forceinline__ void begin(int64_t chunk, int lane)
     {
         s = w.chunk_slot[chunk];
         next_slot = b < total ? w.chunk_slot[chunk + 1] : HT_EMPTY;
         fetch<WT>(a, lane);
-        prev = start(s) < a ? s : HT_EMPTY;
+        row0 = s;
+        from = start(s);
+        if (JOIN && b < total) {
+            const uint32_t end = start(next_slot + 1u);
+            if (start(next_slot) < b && end - b <= spill()) {
+                b = end;
+                next_slot = HT_EMPTY;
+            }
+        }
+        till = __shfl_sync(0xffffffffu, v, 0);
+        prev = HT_EMPTY;
+        if (from < a) {
+            if (JOIN && till - a <= spill()) {          // the chunk before ends it
+                a = till;
+                if (a >= b) return;
+                int k;
+                do {                            // (more than one: rows without pairs)
+                    k = __popc(__ballot_sync(0xffffffffu, v <= a));
+                    s += k;
+                    v = start(s + 1 + lane);
+                } while (k == 32);
+                fetch<WT>(a, lane);
+                row0 = s;
+                from = a;
+                till = __shfl_sync(0xffffffffu, v, 0);
+            } else prev = s;
+        }
     }
     // bit j: position p + j starts another row than the one before it (j < n); rows without pairs (lookups that malformed offsets leave out) among
     // them: false, `rows` then finds the rows, otherwise every start is one row further and s is the row of the last position
@@ -436,6 +468,89 @@ struct DePairs {
     }
 };
 
+// Segments that cross chunk borders leave a piece per chunk: the head of a chunk (its first row, begun in an earlier one) or the tail (goes
+// on in the next; a chunk inside one segment has a tail only).  With few chunks the warp whose piece arrives last adds them up, in order
+// (counters; nobody waits); a popular row spans hundreds of chunks, so that pieces are added 32 at a time, by the last of the 32, and
+// then those sums.  A short rest of a segment stays with the chunk before (DE_SPILL_LOG), which leaves the popular rows' pieces only.
+// With many chunks the wait for the stores at the end of every warp costs more than the kernel that adds the pieces up afterwards
+// (k_dE_fix).  dE, kernel afterwards / last arrival, us: 65 k lookups, D = 128 26 / 21; 0.5 M, D = 32 31 / 27; 1 M, D = 45 86 / 70; 1.6 M, D =
+// 64 69 / 60; 3.7 M, D = 64 (29 k chunks): call 1548 / 1500; 2.4 M, D = 16 (19 k chunks) call 711 / 718; 4 M, D = 16 (32 k chunks) 118 / 121;
+// 60 tables (97 k chunks) 2150 / 2235.  (Warps that take chunks from a counter, with the counts a chunk later: 60 tables 2640.)
+#define DE_JOIN_CHUNKS 16384      // twice as many for rows of more than 32 floats
+#define DE_JOIN 32
+// fields of a chunk's counter: pieces of 32 that start in it, of the first ones of a segment that does, sums of 32 of that segment
+#define DE_CTR_REST 0
+#define DE_CTR_FIRST 6
+#define DE_CTR_SUMS 12
+// dst = the pieces of chunks x, x + step, .. (m of them) of the segment that ends in chunk c1
+template <bool VEC>
+__device__ __forceinline__ void de_sum(const WsView& w, float* dst, uint32_t x, uint32_t m, uint32_t step, uint32_t c1, int lane)
+{
+    using piece_t = typename std::conditional<VEC, float4, float>::type;
+    constexpr int PF = VEC ? 4 : 1, NF = 8;
+    const int D = w.D, cols = D / PF;
+    int lpr = 32;
+    while (lpr > 1 && lpr / 2 >= cols) lpr >>= 1;
+    const uint32_t slots = 32u / lpr, slot = lane / lpr;
+    for (int c0 = 0; c0 < cols; c0 += lpr) {
+        const int c = c0 + lane % lpr;
+        RowAcc<VEC, 1> sum;
+        sum.clear();
+        for (uint32_t i0 = slot; i0 < m; i0 += NF * slots) {
+            piece_t v[NF];
+#pragma unroll
+            for (int k = 0; k < NF; ++k) {
+                const uint32_t i = i0 + k * slots, y = x + i * step;
+                v[k] = i < m && c < cols ? __ldcg(reinterpret_cast<const piece_t*>(w.carry) + ((size_t)y * 2 + (y < c1 ? 1 : 0)) * cols + c) : piece_t{};
+            }
+            RowAcc<VEC, 1> part;
+            part.clear();
+#pragma unroll
+            for (int k = 0; k < NF; ++k) part.add_shared(&v[k]);
+#pragma unroll
+            for (int k = 0; k < PF; ++k) sum.v[k] += part.v[k];
+        }
+        for (int o = lpr; o < 32; o <<= 1)
+#pragma unroll
+            for (int k = 0; k < PF; ++k) sum.v[k] += __shfl_xor_sync(0xffffffffu, sum.v[k], o);
+        if (slot == 0 && c < cols) sum.store(dst + PF * c, PF, 0);
+    }
+}
+template <bool VEC>
+__device__ __forceinline__ void de_arrive(const WsView& w, uint32_t chunk, uint32_t row, uint32_t from, uint32_t till, uint32_t spill, int lane)
+{
+    uint32_t c1 = (till - 1u) >> w.de_chunk_log;
+    if (till - (c1 << w.de_chunk_log) <= spill) --c1;     // (the segment goes on past a border: c1 > c0)
+    const uint32_t c0 = from >> w.de_chunk_log, pieces = c1 - c0 + 1u;
+    const uint32_t block = (chunk - c0) / DE_JOIN, x = c0 + block * DE_JOIN, m = min((uint32_t)DE_JOIN, pieces - block * DE_JOIN);
+    const int shift = block == 0 ? DE_CTR_FIRST : DE_CTR_REST;
+    uint32_t seen = 0;
+    if (lane == 0) seen = atomicAdd(w.chunk_ctr + x, 1u << shift) >> shift & 63u;
+    if (__shfl_sync(0xffffffffu, seen, 0) != m - 1u) return;
+    __threadfence();
+    float* const out = w.E + (size_t)row * w.D;
+    const uint32_t sums = (pieces + DE_JOIN - 1u) / DE_JOIN;
+    de_sum<VEC>(w, sums == 1 ? out : w.carry + ((size_t)x * 2 + (x < c1 ? 1 : 0)) * w.D, x, m, 1, c1, lane);
+    if (sums == 1) return;
+    __threadfence();
+    __syncwarp();
+    if (lane == 0) seen = atomicAdd(w.chunk_ctr + c0, 1u << DE_CTR_SUMS) >> DE_CTR_SUMS;
+    if (__shfl_sync(0xffffffffu, seen, 0) != sums - 1u) return;
+    __threadfence();
+    de_sum<VEC>(w, out, c0, sums, DE_JOIN, c1, lane);
+}
+// a chunk's pieces are stored; cur: row of its last position
+template <bool VEC>
+__device__ __forceinline__ void de_finish(const WsView& w, const DePairs& pairs, int64_t chunk, uint32_t cur, int lane)
+{
+    const bool begun = pairs.prev == pairs.row0, goes_on = pairs.next_slot == cur && !(begun && cur == pairs.row0);
+    if (!begun && !goes_on) return;
+    __threadfence();
+    __syncwarp();
+    if (begun) de_arrive<VEC>(w, (uint32_t)chunk, pairs.row0, pairs.from, pairs.till, pairs.spill(), lane);
+    if (goes_on) de_arrive<VEC>(w, (uint32_t)chunk, cur, (uint32_t)(chunk << w.de_chunk_log), pairs.start(cur + 1u), pairs.spill(), lane);
+}
+
 template <bool VEC, int CPL>
 __global__ void __launch_bounds__(256) k_dE(WsView w, const float* __restrict__ grad_out)
 {
@@ -444,12 +559,13 @@ __global__ void __launch_bounds__(256) k_dE(WsView w, const float* __restrict__ 
     const int lane = threadIdx.x & 31;
     const int64_t chunk = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     DePairs pairs(w, chunk);
-    const uint32_t a = pairs.a, b = pairs.b;
-    if (a >= b) return;
+    if (pairs.a >= pairs.b) return;
     const int D = w.D;
     const size_t gstride = (size_t)w.T * D;
     const bool weighted = tt_weighted(w);
-    if (weighted) pairs.begin<true>(chunk, lane); else pairs.begin<false>(chunk, lane);
+    if (weighted) pairs.begin<true, false>(chunk, lane); else pairs.begin<false, false>(chunk, lane);
+    const uint32_t a = pairs.a, b = pairs.b;
+    if (a >= b) return;
     const uint32_t prev = pairs.prev, next = pairs.next_slot;
     RowAcc<VEC, CPL> acc;
     acc.clear();
@@ -595,9 +711,10 @@ __global__ void __launch_bounds__(256, 5) k_dE_fast(WsView w, const float* __res
     const int lane = threadIdx.x & 31, sub = lane / LPR, lr = lane % LPR;
     const int64_t chunk = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     DePairs pairs(w, chunk);
+    if (pairs.a >= pairs.b) return;
+    pairs.begin<WT, false>(chunk, lane);
     const uint32_t a = pairs.a, b = pairs.b;
     if (a >= b) return;
-    pairs.begin<WT>(chunk, lane);
     const int D = w.D, D4 = D >> 2;
     const bool lane_on = lr < D4;
     const uint32_t prev = pairs.prev, next = pairs.next_slot;
@@ -681,14 +798,14 @@ __global__ void __launch_bounds__(256, 5) k_dE_fast(WsView w, const float* __res
 // was bound by instruction issue.  Chunks, carries and the fix-up pass are those of k_dE / k_dE_fast.
 #define DE_ODD_MOST 61   // with the up to three floats before it, a row fits sixteen pieces
 #define DE_WARPS 7   // 4 CTAs x 7 warps x 8 KB of staging per SM
-// DD = 128: rows of 512 bytes, two CTAs per SM (65 k lookups: dE with its fix-up 38 -> 29 us against k_dE_fast).
+// DD = 128: rows of 512 bytes, two CTAs per SM (65 k lookups: dE with the pieces added up 38 -> 29 us against k_dE_fast).
 // DD = 0: rows of any other length up to 61 floats.  A row starts anywhere in its first 16-byte piece; the pieces that it touches
 // are staged as they lie (the last ones of grad_out cut to its end), and a lane picks columns lane and lane + 32 behind the row's
 // shift.  1 M lookups of 45 floats: 112 -> 84 us against k_dE.
-template <int DD, bool WT>   // DD = D: 128 (four columns per lane), 64 (two), 32 (one), 16 (one, lanes 0..15) or 0
+template <int DD, bool WT, bool JOIN>   // DD = D: 128 (four columns per lane), 64 (two), 32 (one), 16 (one, lanes 0..15) or 0
 __global__ void __launch_bounds__(32 * DE_WARPS, DD == 128 ? 2 : 4) k_dE_stage(WsView w, const float* __restrict__ grad_out)
 {
-    tt_pdl_enter();
+    if (JOIN) tt_pdl_wait(); else tt_pdl_enter();   // (the sweep comes next: see k_dE_fix)
     static_assert(DD == 128 || DD == 64 || DD == 32 || DD == 16 || DD == 0, "a lane owns DD / 32 columns (one column on the first DD lanes below 32)");
     constexpr bool ODD = DD == 0;
     constexpr int R4 = ODD ? 16 : DD / 4;         // float4 pieces per staged row
@@ -701,9 +818,10 @@ __global__ void __launch_bounds__(32 * DE_WARPS, DD == 128 ? 2 : 4) k_dE_stage(W
     const float* bufv = reinterpret_cast<const float*>(buf);
     const int64_t chunk = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     DePairs pairs(w, chunk);
+    if (pairs.a >= pairs.b) return;
+    pairs.begin<WT, JOIN>(chunk, lane);
     const uint32_t a = pairs.a, b = pairs.b;
     if (a >= b) return;
-    pairs.begin<WT>(chunk, lane);
     const uint32_t prev = pairs.prev, next = pairs.next_slot;
     const float4* __restrict__ G4 = reinterpret_cast<const float4*>(grad_out);
     float* carry = w.carry + (size_t)chunk * 2 * D;
@@ -867,6 +985,14 @@ __global__ void __launch_bounds__(32 * DE_WARPS, DD == 128 ? 2 : 4) k_dE_stage(W
         const bool open_start = seg_first && prev == cur;
         store_row(next == cur ? carry + D : (open_start ? carry : w.E + (size_t)cur * D), false);
     }
+    if (JOIN) de_finish<!ODD>(w, pairs, chunk, cur, lane);
+}
+
+template <bool WT, bool JOIN>
+static auto de_stage_kernel(int D) -> void (*)(WsView, const float*)
+{
+    return D == 0 ? k_dE_stage<0, WT, JOIN> : D == 128 ? k_dE_stage<128, WT, JOIN> : D == 64 ? k_dE_stage<64, WT, JOIN>
+         : D == 32 ? k_dE_stage<32, WT, JOIN> : k_dE_stage<16, WT, JOIN>;
 }
 
 template <bool VEC, int CPL>
@@ -877,18 +1003,18 @@ static cudaError_t launch_dE_t(tt_emb* h, const float* grad_out, cudaStream_t s)
     if (grid > 0) {
         const int D4 = h->D / 4;
         const bool wt = tt_weighted(h->v);
+        const bool join = chunks <= (h->D > 32 ? 2 * DE_JOIN_CHUNKS : DE_JOIN_CHUNKS);
         const bool odd = !VEC && h->D <= DE_ODD_MOST && (reinterpret_cast<uintptr_t>(grad_out) & 15) == 0;
         if (odd || (VEC && (h->D == 128 || h->D == 64 || h->D == 32 || h->D == 16))) {
             const size_t smem = (size_t)DE_WARPS * 32 * (odd ? 16 : h->D / 4) * sizeof(float4);
-            auto kern = odd ? (wt ? k_dE_stage<0, true> : k_dE_stage<0, false>)
-                      : h->D == 128 ? (wt ? k_dE_stage<128, true> : k_dE_stage<128, false>)
-                      : h->D == 64 ? (wt ? k_dE_stage<64, true> : k_dE_stage<64, false>)
-                      : h->D == 32 ? (wt ? k_dE_stage<32, true> : k_dE_stage<32, false>) : (wt ? k_dE_stage<16, true> : k_dE_stage<16, false>);
+            auto kern = join ? (wt ? de_stage_kernel<true, true>(odd ? 0 : h->D) : de_stage_kernel<false, true>(odd ? 0 : h->D))
+                             : (wt ? de_stage_kernel<true, false>(odd ? 0 : h->D) : de_stage_kernel<false, false>(odd ? 0 : h->D));
             cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             if (e != cudaSuccess) return e;
             const int sgrid = (int)((chunks + DE_WARPS - 1) / DE_WARPS);
             if ((e = tt_launch_pdl(kern, dim3(sgrid), dim3(32 * DE_WARPS), smem, s, h->v, grad_out)) != cudaSuccess) return e;
             tt_note_launch();
+            if (join) return cudaGetLastError();
         } else
         if (VEC && D4 <= 8) { if (wt) k_dE_fast<8, true><<<grid, 256, 0, s>>>(h->v, grad_out); else k_dE_fast<8, false><<<grid, 256, 0, s>>>(h->v, grad_out); tt_note_launch(); }
         else if (VEC && D4 <= 16) { if (wt) k_dE_fast<16, true><<<grid, 256, 0, s>>>(h->v, grad_out); else k_dE_fast<16, false><<<grid, 256, 0, s>>>(h->v, grad_out); tt_note_launch(); }

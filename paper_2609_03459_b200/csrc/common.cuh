@@ -46,7 +46,7 @@
 #define TT_STATUS_BYTES 512   // status word and counters (16 + 64 words) with their guard bytes, up to the row bitmap behind them
 #define TT_GUARD 0xA5         // guard bytes behind the other workspace regions
 #define TT_UNIT_ROWS 64   // fewest rows of a unit of a K = 2 table
-#define TT_DE_CHUNK 1024                                  // sorted lookups per warp in the dE segment reduction, at most (up to 268 M lookups)
+#define TT_DE_CHUNK 1024                                  // sorted lookups per warp in the dE segment reduction, at most (up to 134 M lookups)
 #define TT_NUM_STAGES 33                                // 0..8 pipeline stages, 9..20 forward sweep variants -1..10, 21..32 backward sweep variants
 #define TT_STRIPES 8                                     // L2-resident partial copies of the last core's gradient
 #define TT_NUM_MIDFAST 11                                // tensor-core instances of the middle-core backward (backward.cu)
@@ -123,6 +123,7 @@ struct WsView {
     uint32_t* cursor;                   // [capU]
     uint2* pairs;                       // [L] bags sorted by slot (uint32, behind them the pairs' ranks), or (bag, factor) with weights or mean pooling
     uint32_t* chunk_slot;               // slot of the first sorted position of every dE chunk (in the space of pool_bounds)
+    uint32_t* chunk_ctr;                // pieces of the segments that cross chunk borders, counted as they arrive (behind them)
     uint2* upairs;                      // [L] (slot, bag) in lookup order, written by the pooling kernel (null: forward only)
     float* dP[TT_MAXK + 1];             // dP_k per level-k node, 2 <= k <= K-1
     float* Y[TT_MAXK + 1];              // per level-k node: its contribution to dP_{k-1} of its parent
