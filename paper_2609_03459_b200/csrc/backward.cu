@@ -2300,7 +2300,7 @@ __global__ void __launch_bounds__(128, 5) k_mid_mma(WsView w, int k, int variant
 // Bound by the operand path (16 fragment loads for 24 tensor instructions) and, for short node lists, by a CTA's look-ups.
 // Middle stage, 2x4x4x4 with rank 64 (65 536 lookups): 5.05 ms with one FP32 thread per output element over the whole
 // node list, 0.16 ms as tiles; 3x3x5 with ranks 6 and 4 (4 tables, 1 M lookups): 0.41 and 0.06 ms.
-template <bool FOLD>
+template <bool FOLD, bool WHOLE>
 __global__ void __launch_bounds__(128, 4) k_mid_tile(WsView w, int k, int lbase, int dgz, int yctas)
 {
     tt_pdl_enter();
@@ -2385,7 +2385,7 @@ __global__ void __launch_bounds__(128, 4) k_mid_tile(WsView w, int k, int lbase,
                     if (8 * p >= left) break;
                     const float* Aa = A + (8 * p + t) * MT_PA;
                     const float* Da = D + (8 * p + t) * MT_PA;
-                    tt_quarter_step(sum, Aa, Aa + 8, Aa + 4 * MT_PA, Aa + 4 * MT_PA + 8, 1, Da, Da + 4 * MT_PA, 1, mtl, ntl);
+                    tt_quarter_step<WHOLE>(sum, Aa, Aa + 8, Aa + 4 * MT_PA, Aa + 4 * MT_PA + 8, 1, Da, Da + 4 * MT_PA, 1, mtl, ntl);
                 }
             }
             if (wid == 0) { s_a[ring2][lane] = pa; s_d[ring2][lane] = pd; }   // the ring slot of the pass before
@@ -2473,7 +2473,7 @@ __global__ void __launch_bounds__(128, 4) k_mid_tile(WsView w, int k, int lbase,
                     if (c * MT_KROWS + 8 * p >= cols) break;
                     const float* Da = D + 8 * p;
                     const float* Ba = B + 8 * p;
-                    tt_quarter_step(sum, Da, Da + 8 * MT_PC, Da + 4, Da + 8 * MT_PC + 4, MT_PC, Ba, Ba + 4, MT_PC, mtl, ntl);
+                    tt_quarter_step<WHOLE>(sum, Da, Da + 8 * MT_PC, Da + 4, Da + 8 * MT_PC + 4, MT_PC, Ba, Ba + 4, MT_PC, mtl, ntl);
                 }
             }
             __syncthreads();
@@ -2595,12 +2595,14 @@ cudaError_t tt_launch_bwd_middle(tt_emb* h, cudaStream_t s)
         uint32_t sum_blocks = 1;
         int dgz = 1;                  // generic shapes: tiles of the slice gradient,
         int64_t ytiles = 1;           // most tiles of Y of a slice
+        bool whole = true;            // all shapes fill the quarters of their tiles
         for (int t = 0; t < h->T; ++t) {
             const TableDesc& td = h->tab[t];
             const int kc = k - 1;
             const uint32_t nout = (uint32_t)(td.P[kc] * td.r[kc]), pieces = (nout & 3) ? nout : nout / 4;
             if ((pieces + 31) / 32 > sum_blocks) sum_blocks = (pieces + 31) / 32;
             if (td.midfast[k] >= 0) { any_fast[td.midfast[k]] = true; continue; }
+            if (td.r[kc] % (MT_EDGE / 2) != 0 || td.d[kc] * td.r[kc + 1] % (MT_EDGE / 2) != 0) whole = false;
             const int tiles = ((td.r[kc] + MT_EDGE - 1) / MT_EDGE) * ((td.d[kc] * td.r[kc + 1] + MT_EDGE - 1) / MT_EDGE);
             if (tiles > dgz) dgz = tiles;
             const int64_t rows = (int64_t)(td.prefix_space[k - 1] < w.cap[k] ? td.prefix_space[k - 1] : w.cap[k]) * td.P[kc];
@@ -2637,7 +2639,8 @@ cudaError_t tt_launch_bwd_middle(tt_emb* h, cudaStream_t s)
             const int64_t slices = (int64_t)h->mmaxn[k][0] * ngen;
             const bool fold = slices >= 64 * h->sm_count;
             const int yctas = fold ? 0 : tt_ctas_per_slice(h->sm_count, slices, ytiles);
-            if ((e = tt_launch_pdl(fold ? k_mid_tile<true> : k_mid_tile<false>, dim3(h->mmaxn[k][0], ngen, dgz + yctas), dim3(128), 0, st(), w, k, mlist(-1), dgz, yctas)) != cudaSuccess) return e;
+            auto kern = whole ? (fold ? k_mid_tile<true, true> : k_mid_tile<false, true>) : (fold ? k_mid_tile<true, false> : k_mid_tile<false, false>);
+            if ((e = tt_launch_pdl(kern, dim3(h->mmaxn[k][0], ngen, dgz + yctas), dim3(128), 0, st(), w, k, mlist(-1), dgz, yctas)) != cudaSuccess) return e;
             tt_note_launch();
         }
         if (fork && (e = tt_join(h, s, 4)) != cudaSuccess) return e;
