@@ -2009,6 +2009,12 @@ cudaError_t tt_launch_bwd_contraction(tt_emb* h, cudaStream_t s)
         }
     }
     cudaError_t e;
+    // four cores: the digit-major list of level 2 is made beside the sweeps, as far as the scan's space is free (the segment starts are done
+    // with); the middle level waits for it.  Five short kernels on the way of the call otherwise: 65 k lookups, rank 64, call 380 to 367 us
+    if (h->K == 4 && !h->serial) {
+        if ((e = tt_fork(h, s, 1)) != cudaSuccess) return e;
+        if ((e = tt_launch_tlist(h, 2, h->side[0])) != cudaSuccess) return e;
+    }
     // P_k of the levels below K-1 are still in pbuf from the forward (K = 4 only)
     // tables of different shape variants are independent: their kernels run side by side on forked streams
     int nvar = 0;
@@ -2611,7 +2617,7 @@ cudaError_t tt_launch_bwd_middle(tt_emb* h, cudaStream_t s)
         }
         const int ngen = h->mcount[k][0];
         // level K-1's digit-major list already exists: the forward built it to order its sweep
-        if (k != h->K - 1 && (e = tt_launch_tlist(h, k, s)) != cudaSuccess) return e;
+        if (k != h->K - 1 && (e = h->serial ? tt_launch_tlist(h, k, s) : tt_join(h, s, 1)) != cudaSuccess) return e;
         // the shape variants are independent (different tables): run them side by side so that the tail of one
         // (a few long node lists) overlaps the others
         int nfast = 0;
