@@ -221,6 +221,7 @@ extern "C" int tt_emb_create(const tt_emb_config_t* cfg, tt_emb_t* out_handle)
 
     // work units: every table is cut into `units` equal-cost slices, one CTA each
     // about 8 waves of 8 resident CTAs per SM: fine enough that the last wave and table-size differences do not matter
+    int64_t few = 1;
     int Q = (64 * h->sm_count + T - 1) / T;   // (32 * and 128 * measured: 16.8 / 16.5 ms per training step against 16.4)
     {   // ... but not so fine that a unit holds only a few groups
         int unit_groups = h->tab[0].unit_groups;
@@ -229,9 +230,17 @@ extern "C" int tt_emb_create(const tt_emb_config_t* cfg, tt_emb_t* out_handle)
         uint64_t groups = level_space[K - 1] < (uint64_t)h->capU ? level_space[K - 1] : (uint64_t)h->capU;
         const int64_t by_groups = K == 2 ? h->capU / T / TT_UNIT_ROWS : (int64_t)(groups / (uint64_t)T / (uint64_t)unit_groups);
         if (Q > by_groups) Q = (int)by_groups;
+        few = groups / TT_FEW_GROUPS + 1;
     }
     if (Q < 8) Q = 8;
     if (Q > 16384) Q = 16384;
+    h->v.few_units = (uint32_t)(TT_FEW_UNITS * h->sm_count);
+    const int64_t share = (2 * (int64_t)h->v.few_units + T - 1) / T;
+    if (few > share) few = share;
+    if (few > h->v.few_units) few = h->v.few_units;
+    h->sweep_ctas = Q < few ? (int)few : Q;
+    h->v.few_share = 1.f / (float)h->v.few_units;
+    h->v.cta_share = 1.f / (float)h->sweep_ctas;
     int unit_base = 0;
     for (int t = 0; t < T; ++t) {
         h->tab[t].units = Q;

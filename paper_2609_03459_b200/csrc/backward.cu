@@ -1543,7 +1543,7 @@ __device__ __forceinline__ void tt_sweep_bwd_fast(const WsView& w, const TableDe
 // The fused-loop shapes with the intermediate products of NG = 16 / MROWS neighbouring groups formed together on the
 // tensor cores, as in the forward sweep (quad_mid.cuh): one group at a time, every group read its whole slice of core
 // K-1 (16 KB at rank 32) for a product of MROWS rows, which made the L1/L2 path the limit where groups hold few rows.
-template <int PM, int RB_, int MROWS, int KTMAX>
+template <int PM, int RB_, int MROWS, int KTMAX, bool FEW>
 __device__ __forceinline__ void tt_sweep_bwd_quad(const WsView& w, const TableDesc& td, uint32_t g1, float* gk, float* Cs4,
                                                   uint32_t* next, int lane)
 {
@@ -1554,10 +1554,10 @@ __device__ __forceinline__ void tt_sweep_bwd_quad(const WsView& w, const TableDe
     const uint32_t nK = (uint32_t)td.n[K - 1];
     for (;;) {
         uint32_t base = 0;
-        if (lane == 0) base = atomicAdd(next, (uint32_t)NG);
+        if (lane == 0) base = atomicAdd(next, FEW ? next[1] : (uint32_t)NG);
         base = __shfl_sync(0xffffffffu, base, 0);
         if (base >= g1) break;
-        const int cnt = (int)min((uint32_t)NG, g1 - base);
+        const int cnt = (int)min(FEW ? next[1] : (uint32_t)NG, g1 - base);
         uint32_t gq = 0, valq = 0, imq = 0, u0q = 0, u1q = 0;
         const float* srcq = nullptr;
         if (lane < cnt) {
@@ -1586,7 +1586,7 @@ __device__ __forceinline__ void tt_sweep_bwd_quad(const WsView& w, const TableDe
 //         the first step and 2, 3 in the second, so that a fragment is one 16-byte load.  C of 8 or 4 rows: transposed.
 //   dG_K[i_K] += C^T . dE: n = (row, j), two tiles: n / 2 is the row (tt_stream_row), j = 2 (n % 2) + tile, so that an operand of both
 //         tiles is one 8-byte load and a lane ends up with four neighbouring floats of one slice.
-template <int PM, int RB_, int MROWS, int KTMAX, int PD>
+template <int PM, int RB_, int MROWS, int KTMAX, int PD, bool FEW>
 __device__ __forceinline__ void tt_sweep_bwd_stream(const WsView& w, const TableDesc& td, uint32_t g1, float* gk, float* Cs4,
                                                     uint32_t* next, int lane)
 {
@@ -1605,11 +1605,11 @@ __device__ __forceinline__ void tt_sweep_bwd_stream(const WsView& w, const Table
     const int rn = tt_stream_row(g >> 1), rc = tt_stream_row(t);   // dG: row of this lane's column n = g of dE; of its columns 2t, 2t + 1 of the result
     Stream rs(w.val[K], td.core[K - 1], Cs4 + NG * PM * CS, lane);
     uint32_t nbase = 0;
-    if (lane == 0) nbase = atomicAdd(next, (uint32_t)NG);
+    if (lane == 0) nbase = atomicAdd(next, FEW ? next[1] : (uint32_t)NG);
     nbase = __shfl_sync(0xffffffffu, nbase, 0);
-    uint32_t gq = lane < NG && nbase + lane < g1 ? w.tnode[K - 1][nbase + lane] : 0u;   // lane k: group k of the batch
+    uint32_t gq = (uint32_t)lane < (FEW ? next[1] : (uint32_t)NG) && nbase + lane < g1 ? w.tnode[K - 1][nbase + lane] : 0u;   // lane k: group k of the batch
     while (nbase < g1) {
-        const int cnt = (int)min((uint32_t)NG, g1 - nbase);
+        const int cnt = (int)min(FEW ? next[1] : (uint32_t)NG, g1 - nbase);
         uint32_t valq = 0, imq = 0, u0q = 0, u1q = 0;
         const float* srcq = nullptr;
         if (lane < cnt) {
@@ -1623,9 +1623,9 @@ __device__ __forceinline__ void tt_sweep_bwd_stream(const WsView& w, const Table
         auto fill = [&]() { rs.fill(w.E, lane); };
         if constexpr (RB_ == 8) tt_quad_mid_fp32<RB_>(td.core[km], td.slice_floats[km], ra, cnt, imq, srcq, Cs4, lane, fill);
         else tt_quad_mid<COLS, MROWS, KTMAX, RB_>(td.core[km], td.slice_floats[km], ra, cnt, imq, srcq, Cs4, lane, fill);
-        if (lane == 0) nbase = atomicAdd(next, (uint32_t)NG);
+        if (lane == 0) nbase = atomicAdd(next, FEW ? next[1] : (uint32_t)NG);
         nbase = __shfl_sync(0xffffffffu, nbase, 0);
-        gq = lane < NG && nbase + lane < g1 ? w.tnode[K - 1][nbase + lane] : 0u;   // the next batch
+        gq = (uint32_t)lane < (FEW ? next[1] : (uint32_t)NG) && nbase + lane < g1 ? w.tnode[K - 1][nbase + lane] : 0u;   // the next batch
         __syncwarp();
         Tf32Pair ct[MT2][KT2][4];   // A[m = b][k = p] = C[p][b] of the current group
         float dc[DM][DN][4];
@@ -1826,6 +1826,7 @@ struct BwdStream { static constexpr int FLOATS = 16 / MROWS * PM * (RB_ + 4) + R
 // rank-64 four-core shape (wide.cuh).  dG_K: a warp takes one row, a lane two values of b over the 32 rows of C and dE.  dC (32 x
 // 64) = sum over the group's rows of dE . D^T: two warps per group, half the columns each, as 3xTF32 tiles whose k is two rows
 // by four columns, every pair of rows added in rounded fp32 (a group has up to n_K rows).
+template <bool FEW>
 __global__ void __launch_bounds__(WIDE_THREADS, 2) k_sweep_bwd_wide(WsView w, int vbase)
 {
     tt_pdl_enter();
@@ -1833,8 +1834,9 @@ __global__ void __launch_bounds__(WIDE_THREADS, 2) k_sweep_bwd_wide(WsView w, in
     __shared__ WideBatch batches[2];
     float *Bs = sm, *As = Bs + 64 * WIDE_BP, *Cs = As + 8 * WIDE_GROUPS * WIDE_AP;
     const int t = w.vlist[vbase + blockIdx.y], K = w.K, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const uint2 rng = w.unit_rng[t * w.units_per_table + blockIdx.x];
     const TableDesc& td = w.tdesc[t];
+    uint32_t step;
+    const uint2 rng = tt_sweep_unit<FEW>(w, t, WIDE_GROUPS, step);
     const int stripe = (blockIdx.x + blockIdx.y) % TT_STRIPES;
     float* gk = w.gpart + (size_t)stripe * w.gpart_stride + td.gpart_off;
     const uint32_t nK = (uint32_t)td.n[K - 1];
@@ -1916,33 +1918,34 @@ __global__ void __launch_bounds__(WIDE_THREADS, 2) k_sweep_bwd_wide(WsView w, in
 
 // One CTA (4 warps) per work unit (table, q); last-core gradients go to one of TT_STRIPES L2-resident partial
 // copies with vector reductions, added up in fixed stripe order by k_reduce_gpart.
-template <int V>
+template <int V, bool FEW>
 __global__ void __launch_bounds__(128, V == 5 ? 6 : V == 1 || V == 8 ? 4 : V == 2 || V == 6 || V == 9 ? 5 : 0) k_sweep_bwd(WsView w, int pl_floats, int c_floats, int vbase)
 {
     tt_pdl_enter();
     extern __shared__ __align__(16) float sm[];
-    const int t = w.vlist[vbase + blockIdx.y], q = blockIdx.x;
-    const uint2 rng = w.unit_rng[t * w.units_per_table + q];
-    const uint32_t g0 = rng.x, g1 = rng.y;
+    const int t = w.vlist[vbase + blockIdx.y];
     const TableDesc& td = w.tdesc[t];
     const int stripe = (blockIdx.x + blockIdx.y) % TT_STRIPES;
     float* gk = w.gpart + (size_t)stripe * w.gpart_stride + td.gpart_off;
-    __shared__ uint32_t next;
-    if (threadIdx.x == 0) next = g0;
+    __shared__ uint32_t next[2];   // the CTA's next group, groups that a warp takes at a time
+    uint32_t step;
+    const uint2 rng = tt_sweep_unit<FEW>(w, t, V < 5 ? 4 : 8, step);
+    const uint32_t g1 = rng.y;
+    if (threadIdx.x == 0) { next[0] = rng.x; next[1] = step; }
     __syncthreads();
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     float* As = sm + (size_t)wid * (pl_floats + c_floats);
     float* Cs = As + pl_floats;
-    if (V == 0) tt_sweep_bwd_fast<16, 32, 4, 4, 1, true>(w, td, g1, gk, As, Cs, &next, lane);
-    if (V == 1) tt_sweep_bwd_stream<16, 16, 4, 4, BWD_RING>(w, td, g1, gk, sm + wid * BwdStream<16, 16, 4>::FLOATS, &next, lane);
-    if (V == 2) tt_sweep_bwd_stream<16, 8, 4, 4, BWD_RING>(w, td, g1, gk, sm + wid * BwdStream<16, 8, 4>::FLOATS, &next, lane);
-    if (V == 3) tt_sweep_bwd_fast<32, 32, 4, 4, 2, true>(w, td, g1, gk, As, Cs, &next, lane);
-    if (V == 5) tt_sweep_bwd_quad<8, 32, 2, 4>(w, td, g1, gk, sm + (size_t)wid * (8 * 8 * 36), &next, lane);
-    if (V == 6) tt_sweep_bwd_stream<8, 16, 2, 4, BWD_RING>(w, td, g1, gk, sm + wid * BwdStream<8, 16, 2>::FLOATS, &next, lane);
-    if (V == 7) tt_sweep_bwd_fast<8, 8, 2, 2, 1, false>(w, td, g1, gk, As, Cs, &next, lane);   // 8 x 8: the FP32 pipe wins (51 us against 57 with streamed rows; 8 tables, 5 M lookups 172 / 184)
-    if (V == 8) tt_sweep_bwd_stream<4, 32, 2, 4, BWD_RING>(w, td, g1, gk, sm + wid * BwdStream<4, 32, 2>::FLOATS, &next, lane);
-    if (V == 9) tt_sweep_bwd_stream<4, 16, 2, 4, BWD_RING>(w, td, g1, gk, sm + wid * BwdStream<4, 16, 2>::FLOATS, &next, lane);
-    if (V == 10) tt_sweep_bwd_fast<4, 8, 2, 2, 1, false>(w, td, g1, gk, As, Cs, &next, lane);
+    if (V == 0) tt_sweep_bwd_fast<16, 32, 4, 4, 1, true>(w, td, g1, gk, As, Cs, next, lane);
+    if (V == 1) tt_sweep_bwd_stream<16, 16, 4, 4, BWD_RING, FEW>(w, td, g1, gk, sm + wid * BwdStream<16, 16, 4>::FLOATS, next, lane);
+    if (V == 2) tt_sweep_bwd_stream<16, 8, 4, 4, BWD_RING, FEW>(w, td, g1, gk, sm + wid * BwdStream<16, 8, 4>::FLOATS, next, lane);
+    if (V == 3) tt_sweep_bwd_fast<32, 32, 4, 4, 2, true>(w, td, g1, gk, As, Cs, next, lane);
+    if (V == 5) tt_sweep_bwd_quad<8, 32, 2, 4, FEW>(w, td, g1, gk, sm + (size_t)wid * (8 * 8 * 36), next, lane);
+    if (V == 6) tt_sweep_bwd_stream<8, 16, 2, 4, BWD_RING, FEW>(w, td, g1, gk, sm + wid * BwdStream<8, 16, 2>::FLOATS, next, lane);
+    if (V == 7) tt_sweep_bwd_fast<8, 8, 2, 2, 1, false>(w, td, g1, gk, As, Cs, next, lane);   // 8 x 8: the FP32 pipe wins (51 us against 57 with streamed rows; 8 tables, 5 M lookups 172 / 184)
+    if (V == 8) tt_sweep_bwd_stream<4, 32, 2, 4, BWD_RING, FEW>(w, td, g1, gk, sm + wid * BwdStream<4, 32, 2>::FLOATS, next, lane);
+    if (V == 9) tt_sweep_bwd_stream<4, 16, 2, 4, BWD_RING, FEW>(w, td, g1, gk, sm + wid * BwdStream<4, 16, 2>::FLOATS, next, lane);
+    if (V == 10) tt_sweep_bwd_fast<4, 8, 2, 2, 1, false>(w, td, g1, gk, As, Cs, next, lane);
 }
 
 // fixed-order sum of the partial copies of the last core's gradient
@@ -1968,6 +1971,7 @@ static cudaError_t launch_sweep_bwd(tt_emb* h, int max_pl, int max_c, cudaStream
 {
     const int n = h->vcount[V + 1];
     if (n == 0) return cudaSuccess;
+    [[maybe_unused]] const bool few = tt_few_groups(h);
     // tensor-core variants keep C with padded rows (stride r_{K-1} + 8 floats)
     if (V == 0) max_c = 16 * (32 + 8);
     if (V == 3) max_c = 32 * (32 + 8);
@@ -1985,11 +1989,13 @@ static cudaError_t launch_sweep_bwd(tt_emb* h, int max_pl, int max_c, cudaStream
         if ((e = cudaFuncSetAttribute(k_sweep_bwd_any, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
         if ((e = tt_launch_pdl(k_sweep_bwd_any, dim3(h->units_per_table, n), dim3(GEN_THREADS), smem, s, h->v, h->vbase[0])) != cudaSuccess) return e;
     } else if constexpr (V == 4) {
-        if ((e = cudaFuncSetAttribute(k_sweep_bwd_wide, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)WIDE_SMEM)) != cudaSuccess) return e;
-        if ((e = tt_launch_pdl(k_sweep_bwd_wide, dim3(h->units_per_table, n), dim3(WIDE_THREADS), WIDE_SMEM, s, h->v, h->vbase[V + 1])) != cudaSuccess) return e;
+        auto kern = few ? k_sweep_bwd_wide<true> : k_sweep_bwd_wide<false>;
+        if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)WIDE_SMEM)) != cudaSuccess) return e;
+        if ((e = tt_launch_pdl(kern, dim3(few ? h->sweep_ctas : h->units_per_table, n), dim3(WIDE_THREADS), WIDE_SMEM, s, h->v, h->vbase[V + 1])) != cudaSuccess) return e;
     } else {
-        if ((e = cudaFuncSetAttribute(k_sweep_bwd<V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
-        if ((e = tt_launch_pdl(k_sweep_bwd<V>, dim3(h->units_per_table, n), dim3(128), smem, s, h->v, max_pl, max_c, h->vbase[V + 1])) != cudaSuccess) return e;
+        auto kern = few ? k_sweep_bwd<V, true> : k_sweep_bwd<V, false>;
+        if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
+        if ((e = tt_launch_pdl(kern, dim3(few ? h->sweep_ctas : h->units_per_table, n), dim3(128), smem, s, h->v, max_pl, max_c, h->vbase[V + 1])) != cudaSuccess) return e;
     }
     tt_note_launch();
     if ((e = tt_stage_end(h, 9 + TT_NUM_VARIANTS + 1 + V + 1, s)) != cudaSuccess) return e;

@@ -43,6 +43,18 @@
 // ... and of the any-shape sweeps, whose CTAs take a batch of groups at a time (3x3x5, 29 k groups, forward + backward sweep
 // with at least 1 / 4 / 8 / 16 groups: 332 / 285 / 252 / 253 us; 8x8 with K = 2, 420 k lookups, whole call 1.16 ms with 8, 1.68 with 16)
 #define TT_UNIT_GROUPS_ANY 8
+// Batches of few groups: below TT_FEW_LIMIT groups per CTA of TT_FEW_UNITS on every SM, the sweeps cut the tables' groups into that many
+// equal parts of at least TT_FEW_GROUPS, and each of a CTA's warps takes a quarter.  A warp that takes its four or eight at once fetches
+// one slice after the other, 3 us each for 4 KB, 12 us for 32 KB, while most of the chip idles.  Forward / backward sweep, us, in the
+// schedule's units and so cut: D = 128, rank 32, 1.0 k groups 180 / 96 and 23 / 19; D = 32, rank 32, 0.8 k 52 / 59 and 19 / 23; rank 16,
+// 1.2 k 28 / 43 and 17 / 23; four cores, 0.5 k 56 / 70 and 29 / 37.  Limits of 4 / 8 / 12: 150 drawn calls 0.965 / 0.961 / 0.959 of
+// their time (geometric mean), but above 8 cheap and dear groups in equal parts cost some 3 %.  Six CTAs per SM: as four.
+// The kernels that can do this take 1 % longer where there are more groups after all (a step in shared memory, spills), so they are
+// launched where at most TT_FEW_MAYBE times as many are possible by the lookups and the tables.
+#define TT_FEW_UNITS 4
+#define TT_FEW_GROUPS 4
+#define TT_FEW_LIMIT 8
+#define TT_FEW_MAYBE 8
 #define TT_STATUS_BYTES 512   // status word and counters (16 + 64 words) with their guard bytes, up to the row bitmap behind them
 #define TT_GUARD 0xA5         // guard bytes behind the other workspace regions
 #define TT_UNIT_ROWS 64   // fewest rows of a unit of a K = 2 table
@@ -89,6 +101,8 @@ struct WsView {
                                         // one cluster for tables swept by warps, without the scan of the costs: group_cluster.cu)
     int32_t cost_shift;                 // cost unit of the schedule = 2^cost_shift FMAs
     uint32_t paired_groups;             // from this many groups on, units of shapes with eight groups per warp hold 2 * TT_UNIT_GROUPS
+    uint32_t few_units;                 // sweep CTAs that run at once: few groups are cut into about that many units (tt_sweep_unit)
+    float few_share, cta_share;         // 1 / few_units, 1 / CTAs of a table in the sweeps
     float fused_lr;                     // != 0: the kernels that finalise a gradient also apply G -= fused_lr * dG (cores in sgd_mask)
     int32_t stride[TT_MAXK + 1];        // floats per node of the level-k partial-product buffers (max over tables)
     int64_t B, L;                       // current batch / lookups
@@ -169,6 +183,7 @@ struct tt_emb {
     int sm_count;
     int units_total;
     int units_per_table;
+    int sweep_ctas;       // CTAs of a table in the sweeps: its units, or more where few groups are cut finer
     int vcount[TT_NUM_VARIANTS + 1];   // tables per variant, index 0 = generic (-1)
     int vbase[TT_NUM_VARIANTS + 1];    // first entry of each variant in vlist
     // middle-core kernels of level k: tables grouped by their variant (index 0 = generic), largest first, in
@@ -231,6 +246,12 @@ cudaError_t tt_launch_grouping(tt_emb* h, cudaStream_t s);
 cudaError_t tt_launch_group_cluster(tt_emb* h, bool rows, int level, cudaStream_t s);
 int tt_group_cluster_ok();
 cudaError_t tt_launch_schedule(tt_emb* h, cudaStream_t s);
+// whether the call may have so few groups that its sweeps cut them finer than the schedule's units (tt_sweep_unit)
+inline bool tt_few_groups(const tt_emb* h)
+{
+    const int64_t most = h->v.L < (int64_t)h->v.cap[h->K - 1] ? h->v.L : (int64_t)h->v.cap[h->K - 1];
+    return most <= (int64_t)h->v.few_units * TT_FEW_LIMIT * TT_FEW_MAYBE;
+}
 cudaError_t tt_launch_tlist(tt_emb* h, int k, cudaStream_t s);   // digit-major list of the level-k nodes (backward, k < K-1)
 cudaError_t tt_plan_pooling(tt_emb* h, const float* out);          // grid and shares of the pooling pass, before the schedule
 cudaError_t tt_launch_contraction(tt_emb* h, cudaStream_t s);
@@ -406,6 +427,23 @@ __device__ __forceinline__ void tt_unit_range(const WsView& w, int t, int q, uin
     };
     g0 = q == 0 ? a : lower(lo_c);
     g1 = q == Q - 1 ? b : lower(hi_c);
+}
+
+// Group range of a sweep's CTA, and how many of its groups a warp takes at a time (up to ng).  FEW: the batch may have few groups; without
+// branches, so that the loads of the table's descriptor that follow are issued with these (with them behind a branch 21 tables' backward
+// sweep of 14 k groups took 115 us instead of 100).
+template <bool FEW>
+__device__ __forceinline__ uint2 tt_sweep_unit(const WsView& w, int t, uint32_t ng, uint32_t& step)
+{
+    step = ng;
+    if (!FEW) return w.unit_rng[t * w.units_per_table + blockIdx.x];
+    const uint32_t q = blockIdx.x, Q = w.units_per_table, total = w.tb[w.K - 1][w.T], a = w.tb[w.K - 1][t], n = w.tb[w.K - 1][t + 1] - a;
+    const uint2 unit = w.unit_rng[t * Q + min(q, Q - 1)];
+    const bool few = total < w.few_units * TT_FEW_LIMIT, none = q >= Q;
+    const uint32_t per = max(max((uint32_t)TT_FEW_GROUPS, __float2uint_ru((float)total * w.few_share)), __float2uint_ru((float)n * w.cta_share) + 1);
+    const uint32_t lo = min(q * per, n), hi = min(lo + per, n);
+    if (few) step = min(ng, (per + 3) / 4);
+    return make_uint2(few ? a + lo : none ? 0u : unit.x, few ? a + hi : none ? 0u : unit.y);
 }
 
 __device__ __forceinline__ int tt_find_table64(const int64_t* __restrict__ tb, int T, int64_t v)

@@ -465,7 +465,7 @@ __device__ __forceinline__ void tt_sweep_fast(const WsView& w, const TableDesc& 
 // Tensor-core variants: a warp takes NG = 16 / MROWS consecutive groups of the digit-major order at a time; their
 // intermediate products are formed together (quad_mid.cuh), then each group's rows are produced from its C in shared
 // memory, on the tensor cores too.
-template <int PM, int RB, int MROWS, int KTMAX>
+template <int PM, int RB, int MROWS, int KTMAX, bool FEW>
 __device__ __forceinline__ void tt_sweep_quad(const WsView& w, const TableDesc& td, uint32_t g1, float* Cs4, uint32_t* next, int lane)
 {
     constexpr int COLS = PM / MROWS * RB;   // d_{K-1} * r_{K-1}
@@ -475,10 +475,10 @@ __device__ __forceinline__ void tt_sweep_quad(const WsView& w, const TableDesc& 
     const uint32_t nK = (uint32_t)td.n[K - 1];
     for (;;) {
         uint32_t base = 0;
-        if (lane == 0) base = atomicAdd(next, (uint32_t)NG);
+        if (lane == 0) base = atomicAdd(next, FEW ? next[1] : (uint32_t)NG);
         base = __shfl_sync(0xffffffffu, base, 0);
         if (base >= g1) break;
-        const int cnt = (int)min((uint32_t)NG, g1 - base);
+        const int cnt = (int)min(FEW ? next[1] : (uint32_t)NG, g1 - base);
         uint32_t valq = 0, imq = 0, u0q = 0, u1q = 0;
         const float* srcq = nullptr;
         if (lane < cnt) {
@@ -503,6 +503,7 @@ __device__ __forceinline__ void tt_sweep_quad(const WsView& w, const TableDesc& 
 }
 
 // rank-64 four-core shape (wide.cuh): a warp makes one row, a lane one of its 32 rows of C by the four columns of the slice
+template <bool FEW>
 __global__ void __launch_bounds__(WIDE_THREADS, 2) k_sweep_fwd_wide(WsView w, int vbase)
 {
     tt_pdl_enter();
@@ -510,8 +511,9 @@ __global__ void __launch_bounds__(WIDE_THREADS, 2) k_sweep_fwd_wide(WsView w, in
     __shared__ WideBatch batches[2];
     float *Bs = sm, *As = Bs + 64 * WIDE_BP, *Cs = As + 8 * WIDE_GROUPS * WIDE_AP;
     const int t = w.vlist[vbase + blockIdx.y], K = w.K, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const uint2 rng = w.unit_rng[t * w.units_per_table + blockIdx.x];
     const TableDesc& td = w.tdesc[t];
+    uint32_t step;
+    const uint2 rng = tt_sweep_unit<FEW>(w, t, WIDE_GROUPS, step);
     const uint32_t nK = (uint32_t)td.n[K - 1];
     WideLoop<false> loop(w, td, rng, batches, Bs, As, Cs);
     while (loop.next()) {
@@ -575,31 +577,32 @@ __global__ void __launch_bounds__(GEN_THREADS) k_sweep_fwd_any(WsView w, int vba
 // fused levels K-1 and K: C stays on chip, rows go to w.E.  One CTA (4 warps) per work unit (table, q);
 // one instantiation per shape variant V so that each gets its own register budget.  blockIdx.y walks the
 // tables of variant V (w.vlist), blockIdx.x the table's equal-cost slices.
-template <int V>
+template <int V, bool FEW>
 __global__ void __launch_bounds__(128, V != 3 ? 6 : 1) k_sweep_fwd(WsView w, int pl_floats, int c_floats, int vbase)
 {
     tt_pdl_enter();
     extern __shared__ __align__(16) float sm[];
-    __shared__ uint32_t next;
+    __shared__ uint32_t next[2];   // the CTA's next group, groups that a warp takes at a time
     const int t = w.vlist[vbase + blockIdx.y];
-    const uint2 rng = w.unit_rng[t * w.units_per_table + blockIdx.x];
-    const uint32_t g0 = rng.x, g1 = rng.y;
+    uint32_t step;
+    const uint2 rng = tt_sweep_unit<FEW>(w, t, V < 5 ? 4 : 8, step);
+    const uint32_t g1 = rng.y;
     const TableDesc& td = w.tdesc[t];
-    if (threadIdx.x == 0) next = g0;
+    if (threadIdx.x == 0) { next[0] = rng.x; next[1] = step; }
     __syncthreads();
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    if (V == 0) tt_sweep_quad<16, 32, 4, 4>(w, td, g1, sm + (size_t)wid * (4 * 16 * 36), &next, lane);
-    if (V == 1) tt_sweep_quad<16, 16, 4, 4>(w, td, g1, sm + (size_t)wid * (4 * 16 * 20), &next, lane);
-    if (V == 3) tt_sweep_quad<32, 32, 4, 4>(w, td, g1, sm + (size_t)wid * (4 * 32 * 36), &next, lane);
+    if (V == 0) tt_sweep_quad<16, 32, 4, 4, FEW>(w, td, g1, sm + (size_t)wid * (4 * 16 * 36), next, lane);
+    if (V == 1) tt_sweep_quad<16, 16, 4, 4, FEW>(w, td, g1, sm + (size_t)wid * (4 * 16 * 20), next, lane);
+    if (V == 3) tt_sweep_quad<32, 32, 4, 4, FEW>(w, td, g1, sm + (size_t)wid * (4 * 32 * 36), next, lane);
     float* As = sm + (size_t)wid * (pl_floats + c_floats);
     float* Cs = As + pl_floats;
-    if (V == 2) tt_sweep_quad<16, 8, 4, 4>(w, td, g1, sm + (size_t)wid * (4 * 16 * 12), &next, lane);
-    if (V == 5) tt_sweep_quad<8, 32, 2, 4>(w, td, g1, sm + (size_t)wid * (8 * 8 * 36), &next, lane);
-    if (V == 6) tt_sweep_quad<8, 16, 2, 4>(w, td, g1, sm + (size_t)wid * (8 * 8 * 20), &next, lane);
-    if (V == 7) tt_sweep_quad<8, 8, 2, 4>(w, td, g1, sm + (size_t)wid * (8 * 8 * 12), &next, lane);
-    if (V == 8) tt_sweep_quad<4, 32, 2, 4>(w, td, g1, sm + (size_t)wid * (8 * 4 * 36), &next, lane);
-    if (V == 9) tt_sweep_quad<4, 16, 2, 4>(w, td, g1, sm + (size_t)wid * (8 * 4 * 20), &next, lane);
-    if (V == 10) tt_sweep_fast<4, 8, 2, 2, 1, false>(w, td, g1, As, Cs, &next, lane);
+    if (V == 2) tt_sweep_quad<16, 8, 4, 4, FEW>(w, td, g1, sm + (size_t)wid * (4 * 16 * 12), next, lane);
+    if (V == 5) tt_sweep_quad<8, 32, 2, 4, FEW>(w, td, g1, sm + (size_t)wid * (8 * 8 * 36), next, lane);
+    if (V == 6) tt_sweep_quad<8, 16, 2, 4, FEW>(w, td, g1, sm + (size_t)wid * (8 * 8 * 20), next, lane);
+    if (V == 7) tt_sweep_quad<8, 8, 2, 4, FEW>(w, td, g1, sm + (size_t)wid * (8 * 8 * 12), next, lane);
+    if (V == 8) tt_sweep_quad<4, 32, 2, 4, FEW>(w, td, g1, sm + (size_t)wid * (8 * 4 * 36), next, lane);
+    if (V == 9) tt_sweep_quad<4, 16, 2, 4, FEW>(w, td, g1, sm + (size_t)wid * (8 * 4 * 20), next, lane);
+    if (V == 10) tt_sweep_fast<4, 8, 2, 2, 1, false>(w, td, g1, As, Cs, next, lane);
 }
 
 // dynamic shared memory of k_sweep_fwd<V> / k_sweep_bwd<V>: four C tiles per warp for the tensor-core variants
@@ -622,6 +625,7 @@ static cudaError_t launch_sweep_fwd(tt_emb* h, int max_pl, int max_c, cudaStream
 {
     const int n = h->vcount[V + 1];
     if (n == 0) return cudaSuccess;
+    [[maybe_unused]] const bool few = tt_few_groups(h);
     cudaError_t e;
     if ((e = tt_stage_begin(h, 9 + V + 1, s)) != cudaSuccess) return e;
     if constexpr (V < 0) {
@@ -629,12 +633,14 @@ static cudaError_t launch_sweep_fwd(tt_emb* h, int max_pl, int max_c, cudaStream
         if ((e = cudaFuncSetAttribute(k_sweep_fwd_any, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
         if ((e = tt_launch_pdl(k_sweep_fwd_any, dim3(h->units_per_table, n), dim3(GEN_THREADS), smem, s, h->v, h->vbase[0])) != cudaSuccess) return e;
     } else if constexpr (V == 4) {
-        if ((e = cudaFuncSetAttribute(k_sweep_fwd_wide, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)WIDE_SMEM)) != cudaSuccess) return e;
-        if ((e = tt_launch_pdl(k_sweep_fwd_wide, dim3(h->units_per_table, n), dim3(WIDE_THREADS), WIDE_SMEM, s, h->v, h->vbase[V + 1])) != cudaSuccess) return e;
+        auto kern = few ? k_sweep_fwd_wide<true> : k_sweep_fwd_wide<false>;
+        if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)WIDE_SMEM)) != cudaSuccess) return e;
+        if ((e = tt_launch_pdl(kern, dim3(few ? h->sweep_ctas : h->units_per_table, n), dim3(WIDE_THREADS), WIDE_SMEM, s, h->v, h->vbase[V + 1])) != cudaSuccess) return e;
     } else {
         const size_t smem = tt_sweep_smem(V, max_pl, max_c);
-        if ((e = cudaFuncSetAttribute(k_sweep_fwd<V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
-        if ((e = tt_launch_pdl(k_sweep_fwd<V>, dim3(h->units_per_table, n), dim3(128), smem, s, h->v, max_pl, max_c, h->vbase[V + 1])) != cudaSuccess) return e;
+        auto kern = few ? k_sweep_fwd<V, true> : k_sweep_fwd<V, false>;
+        if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
+        if ((e = tt_launch_pdl(kern, dim3(few ? h->sweep_ctas : h->units_per_table, n), dim3(128), smem, s, h->v, max_pl, max_c, h->vbase[V + 1])) != cudaSuccess) return e;
     }
     tt_note_launch();
     if ((e = tt_stage_end(h, 9 + V + 1, s)) != cudaSuccess) return e;
