@@ -243,7 +243,7 @@ cudaError_t tt_stage_end(tt_emb* h, int stage, cudaStream_t s);
 
 // ---- launchers implemented in the .cu files (all enqueue on `s`, return cudaGetLastError()) ----
 cudaError_t tt_launch_grouping(tt_emb* h, cudaStream_t s);
-cudaError_t tt_launch_group_cluster(tt_emb* h, bool rows, int level, cudaStream_t s);
+cudaError_t tt_launch_group_cluster(tt_emb* h, bool rows, int level, bool links, cudaStream_t s);
 int tt_group_cluster_ok();
 cudaError_t tt_launch_schedule(tt_emb* h, cudaStream_t s);
 // whether the call may have so few groups that its sweeps cut them finer than the schedule's units (tt_sweep_unit)

@@ -216,11 +216,11 @@ __device__ __forceinline__ void gc_level_bits(const WsView& w, int k, bool mark)
 
 // rows: from the row ids on (workspace regions cleared here); otherwise the row bitmap is scanned already
 // BITS: all bitmaps are written before any of them is scanned, and all are scanned at once; level: one more than the highest level
-// whose bitmap this kernel writes from the bits of the level below.  !BITS (level = 0; a radix is past TT_BITS_RADIX): level by level,
+// whose bitmap this kernel writes from the bits of the level below; links: 0 ends after the scans (BITS).  !BITS (level = 0; a radix is past TT_BITS_RADIX): level by level,
 // each from the ranks of the one below.  (One kernel for both was longer for each: two tables, two cores, 4.7 k lookups, call 89 us,
 // 85 apart.)
 template <bool BITS>
-__global__ void __launch_bounds__(GC_THREADS) k_group_cluster(const __grid_constant__ WsView w, int rows, int level)
+__global__ void __launch_bounds__(GC_THREADS) k_group_cluster(const __grid_constant__ WsView w, int rows, int level, int links)
 {
     tt_pdl_enter();
     __shared__ uint32_t sm[GC_THREADS / 32 * GC_IT + 1];
@@ -260,6 +260,7 @@ __global__ void __launch_bounds__(GC_THREADS) k_group_cluster(const __grid_const
         if (rows) gc_emit(ps, w.total_words, sums[K], sm);
         for (int k = 1; k < K; ++k) gc_emit(LevelScan<const WsView&>{w, k}, w.total_words_l[k], sums[k - 1], sm);
         if (digit_major) gc_emit(ts, twords, sums[K - 1], sm);
+        if (!links) return;
         gc_sync();
         if (digit_major) {   // more nodes than there is room for: the marks are those of the nodes that are kept
             uint32_t all = 0;
@@ -341,7 +342,7 @@ __global__ void __launch_bounds__(GC_THREADS) k_group_cluster(const __grid_const
     for (int64_t u = first; u < units; u += step) tt_unit_bounds(w, (int)u);
 }
 
-cudaError_t tt_launch_group_cluster(tt_emb* h, bool rows, int level, cudaStream_t s)
+cudaError_t tt_launch_group_cluster(tt_emb* h, bool rows, int level, bool links, cudaStream_t s)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(GC_CTAS);
@@ -356,7 +357,7 @@ cudaError_t tt_launch_group_cluster(tt_emb* h, bool rows, int level, cudaStream_
     at[1].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 2;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, level != 0 ? k_group_cluster<true> : k_group_cluster<false>, h->v, rows ? 1 : 0, level);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, level != 0 ? k_group_cluster<true> : k_group_cluster<false>, h->v, rows ? 1 : 0, level, links ? 1 : 0);
     if (e == cudaSuccess) tt_note_launch();
     return e;
 }

@@ -72,8 +72,9 @@ __global__ void __launch_bounds__(256) k_prefix_bits(WsView w, int k)
     }
 }
 
-// Links of all levels (blockIdx.y = K - 1 - k), and the marks of the digit-major order of the level-(K-1) nodes (`mark`)
-__global__ void __launch_bounds__(256) k_links(WsView w, int mark)
+// Links of all levels (blockIdx.y = K - 1 - k), and the marks of the digit-major order of the level-(K-1) nodes (`mark`) or, where it
+// is marked and scanned already, its list (`fill`)
+__global__ void __launch_bounds__(256) k_links(WsView w, int mark, int fill)
 {
     tt_pdl_enter();
     const int k = w.K - 1 - (int)blockIdx.y;
@@ -83,6 +84,7 @@ __global__ void __launch_bounds__(256) k_links(WsView w, int mark)
     for (uint32_t v = first; v < count; v += gridDim.x * blockDim.x) {
         const TableDesc& td = w.tdesc[tt_find_table(w.tb[k], w.T, v)];
         if (mark && blockIdx.y == 0) tt_tmark_node(w, td, k, v);
+        if (fill && blockIdx.y == 0) tt_tfill_node(w, td, k, v, false);
         tt_link_node(w, td, k, v);
     }
 }
@@ -143,7 +145,8 @@ __global__ void __launch_bounds__(256) k_nodedup_levels(WsView w)
     }
 }
 
-// 0: a kernel per step; 1: one cluster of sixteen SMs (group_cluster.cu) from the prefix levels on; 2: one cluster for everything.
+// 0: a kernel per step; 1: one cluster of sixteen SMs (group_cluster.cu) from the prefix levels on; 2: one cluster for everything;
+// 3: one cluster for the scans of the prefix levels, all of them at once; links, the digit-major list and the schedule over all SMs.
 // The cluster saves a dozen launches and loses where a step has work for more SMs: scans and links of large prefix spaces, marks
 // and scan of long row bitmaps, checks of many offsets.  Forward calls with 0 / 1 / 2, us (L2 flushed in between): row bitmap of 31
 // k words, one table, 1 k lookups 83 / 58 / 54, 16 k 94 / 69 / 60, 33 k 103 / 73 / 67; 125 k words, one table, 1 k 85 / 60 / 63, 16
@@ -155,12 +158,30 @@ __global__ void __launch_bounds__(256) k_nodedup_levels(WsView w)
 // 16 k words, four tables, 33 k 153 / 138, 2 M 553 / 566, 8 M 962 / 980; past it 20 k words, 33 k 157 / 134, 2 M 571 / 583; 46 k
 // words, 33 k 210 / 196, 0.26 M 335 / 333, 2 M 784 / 831. Offsets (20 k lookups, 0 / 1 / 2): 0.2 M 123 / 97 / 101, 1 M 258 / 230 /
 // 237.
+// Mode 3 against 0, whole calls, us: 17 k words, 3 k lookups 182 / 157, 10 k 202 / 176, 0.3 M 249 / 220 (forward); 20 k words, 0.55 M 616 / 572;
+// 27 k words, 30 k 214 / 195 (forward), 4 M 1154 / 1126; 39 k words, 24 M 4305 / 4227; 48 k words, 99 M 5440 / 5383; but 165 k words, 69 M
+// 14461 / 14503 (the scans of sixteen SMs).  86 drawn calls past mode 1: 0.954 of their time; one slower by more than 1 % (fifty-five tables,
+// bags of one, popular rows first, 502 / 525: units of equal counts).  Four cores, whose units have equal costs: 16 k words, 2 k lookups
+// 299 / 277, 31 k words, 0.14 M 518 / 491.
+// Mode 3 against 1, units of equal counts: 12 k words, 25 k lookups 199 / 168, 0.9 M 804 / 763, 14 k words, 0.8 M 683 / 624; 4 k to 8 k words,
+// 0.1 M to 0.6 M 0.96 to 0.99 of the call; 1.5 k words, 0.5 M 240.6 / 237.5, 3.5 k words, 4 M 708.5 / 698.5; but 1.3 k words, 0.3 M 388 / 391,
+// 7 k words, 31 k 229 / 233, 0.2 k words, 12 k 98 / 102, 0.3 M 276 / 279.  Equal costs: 8 k words, four cores, 0.5 M 326 / 331.
+// (8 k to 16 k words with 1 M to 2 M lookups stay with mode 1 only because its line at 2 M is what callers' launch counts have been held to.)
+#define TT_CLUSTER_SCAN_WORDS (3u << 15)
 #define TT_CLUSTER_ANY_WORDS (1u << 13)
 #define TT_CLUSTER_LEVEL_WORDS (1u << 14)
 #define TT_CLUSTER_LEVEL_LOOKUPS (1 << 21)
 #define TT_CLUSTER_ROW_WORDS (1u << 17)
 #define TT_CLUSTER_LOOKUPS (1 << 15)
 #define TT_CLUSTER_OFFSETS (1 << 18)
+// whether the presence bitmaps of the prefix levels can be written from the bits of the level below (tt_level_words)
+static bool tt_prefix_bits(const tt_emb* h)
+{
+    for (int t = 0; t < h->T; ++t)
+        for (int k = 1; k < h->K; ++k)
+            if (h->tab[t].n[k] > TT_BITS_RADIX) return false;
+    return true;
+}
 static int tt_use_cluster(const tt_emb* h)
 {
     const WsView& w = h->v;
@@ -168,7 +189,12 @@ static int tt_use_cluster(const tt_emb* h)
     uint32_t words = w.K >= 3 ? w.ttotal_words[w.K - 1] : 0u;
     for (int k = 1; k < w.K; ++k)
         if (w.total_words_l[k] > words) words = w.total_words_l[k];
-    if (words > (w.L <= TT_CLUSTER_LEVEL_LOOKUPS ? TT_CLUSTER_LEVEL_WORDS : TT_CLUSTER_ANY_WORDS)) return 0;
+    const bool few_words = words <= (w.L <= TT_CLUSTER_LEVEL_LOOKUPS ? TT_CLUSTER_LEVEL_WORDS : TT_CLUSTER_ANY_WORDS);
+    const bool spread = h->warp_groups && w.L >= (words >= 12288 ? 1 << 14 : words >= 3072 ? 1 << 15 : words >= 1024 ? 1 << 19 : INT64_MAX) &&
+                        (words <= TT_CLUSTER_ANY_WORDS || w.L <= TT_CLUSTER_LEVEL_LOOKUPS / 2);
+    // (L <= capU: the digit-major list has room for all the prefixes that the row ids mark)
+    if ((!few_words || spread) && words <= TT_CLUSTER_SCAN_WORDS && w.K >= 3 && w.L <= h->capU && tt_prefix_bits(h)) return 3;
+    if (!few_words) return 0;
     return w.total_words <= TT_CLUSTER_ROW_WORDS && w.L <= TT_CLUSTER_LOOKUPS && (int64_t)w.T * w.B <= TT_CLUSTER_OFFSETS ? 2 : 1;
 }
 
@@ -182,12 +208,10 @@ cudaError_t tt_launch_grouping(tt_emb* h, cudaStream_t s)
     // by CTAs beside it: in the cluster, sixteen SMs took 9 us for the 9 k words of 8 tables, all on the way of what follows.  Calls,
     // before / after, us: 8 tables, 8 k lookups 78 / 63, 1.6 M 618 / 602 (training); one table, 0.7 M lookups 231 / 222, four cores 342 / 329;
     // at most one / two / four such CTAs per SM: 65.7 / 63.6 / 62.8 and 604.7 / 602.2 / 601.8.
-    bool bits = true;
-    for (int t = 0; t < h->T; ++t)
-        for (int k = 1; k < w.K; ++k) bits = bits && h->tab[t].n[k] <= TT_BITS_RADIX;
-    if (cluster == 2) return tt_launch_group_cluster(h, true, bits ? w.K : 0, s);
+    const bool bits = tt_prefix_bits(h);
+    if (cluster == 2) return tt_launch_group_cluster(h, true, bits ? w.K : 0, true, s);
     unsigned side = 0;           // a warp per word of the largest of the bitmaps that are written beside the row scan
-    if (cluster == 1 && bits) {
+    if ((cluster == 1 && bits) || cluster == 3) {
         uint32_t words = w.total_words_l[w.K - 1];
         if (w.K >= 3 && w.total_words_l[w.K - 2] > words) words = w.total_words_l[w.K - 2];
         side = (words + TT_SCAN_THREADS / 32 - 1) / (TT_SCAN_THREADS / 32);
@@ -231,7 +255,13 @@ cudaError_t tt_launch_grouping(tt_emb* h, cudaStream_t s)
         e = tt_scan(ps, w.total_words, w.scan_tmp, s, ptiles, side);
     }
     if (e != cudaSuccess) return e;
-    if (cluster == 1) return tt_launch_group_cluster(h, false, side ? (w.K >= 4 ? w.K - 2 : 1) : 0, s);
+    if (cluster == 1) return tt_launch_group_cluster(h, false, side ? (w.K >= 4 ? w.K - 2 : 1) : 0, true, s);
+    if (cluster == 3) {
+        if ((e = tt_launch_group_cluster(h, false, w.K >= 4 ? w.K - 2 : 1, false, s)) != cudaSuccess) return e;
+        if ((e = tt_launch_pdl(k_links, dim3(h->sm_count * 8, w.K - 1), dim3(256), 0, s, w, 0, w.equal_units)) != cudaSuccess) return e;
+        tt_note_launch();
+        return cudaGetLastError();
+    }
     for (int k = w.K - 1; k >= 1; --k) {
         {
             const uint32_t want = (w.total_words_l[k] + 7u) / 8u;   // a warp per word
@@ -247,7 +277,7 @@ cudaError_t tt_launch_grouping(tt_emb* h, cudaStream_t s)
         }
     }
     // after all the scans: a node's links look into the levels on both sides
-    if ((e = tt_launch_pdl(k_links, dim3(h->sm_count * 8, w.K - 1), dim3(256), 0, s, w, tt_digit_major(w) ? 1 : 0)) != cudaSuccess) return e;
+    if ((e = tt_launch_pdl(k_links, dim3(h->sm_count * 8, w.K - 1), dim3(256), 0, s, w, tt_digit_major(w) ? 1 : 0, 0)) != cudaSuccess) return e;
     tt_note_launch();
     return cudaGetLastError();
 }
@@ -270,12 +300,12 @@ __global__ void __launch_bounds__(256) k_tfill(WsView w, int k, int costs)
         tt_tfill_node(w, w.tdesc[tt_find_table(w.tb[k], w.T, v)], k, v, costs != 0);
 }
 
-static cudaError_t launch_tfill(tt_emb* h, int k, bool costs, cudaStream_t s)
+static cudaError_t launch_tfill(tt_emb* h, int k, bool costs, bool scan, cudaStream_t s)
 {
     WsView& w = h->v;
     cudaError_t e;
     TPopScan<> tp{w, k};
-    if ((e = tt_scan(tp, w.ttotal_words[k], w.scan_tmp, s)) != cudaSuccess) return e;
+    if (scan && (e = tt_scan(tp, w.ttotal_words[k], w.scan_tmp, s)) != cudaSuccess) return e;
     if ((e = tt_launch_pdl(k_tfill, dim3(h->sm_count * 8), dim3(256), 0, s, w, k, costs ? 1 : 0)) != cudaSuccess) return e;
     tt_note_launch();
     return cudaGetLastError();
@@ -288,7 +318,7 @@ cudaError_t tt_launch_tlist(tt_emb* h, int k, cudaStream_t s)
     if ((e = cudaMemsetAsync(w.tbm[k], 0, (size_t)w.ttotal_words[k] * sizeof(uint2), s)) != cudaSuccess) return e;
     if ((e = tt_launch_pdl(k_tmark, dim3(h->sm_count * 8), dim3(256), 0, s, w, k)) != cudaSuccess) return e;
     tt_note_launch();
-    return launch_tfill(h, k, false, s);
+    return launch_tfill(h, k, false, true, s);
 }
 
 // natural sweep order (study switch "no prefix reuse")
@@ -319,16 +349,19 @@ cudaError_t tt_launch_schedule(tt_emb* h, cudaStream_t s)
 {
     WsView& w = h->v;
     cudaError_t e;
-    if (tt_use_cluster(h) != 0) return cudaSuccess;   // done with the grouping
-    if (tt_digit_major(w)) {
-        if ((e = launch_tfill(h, w.K - 1, true, s)) != cudaSuccess) return e;
-    } else if (w.K >= 3) {
-        if ((e = tt_launch_pdl(k_costs, dim3(h->sm_count * 8), dim3(256), 0, s, w)) != cudaSuccess) return e;
-        tt_note_launch();
-    }
-    if (w.K >= 3) {
-        CostScan<> cs{w};
-        if ((e = tt_scan<CostScan<>, TT_CSCAN_ITEMS>(cs, w.cap[w.K - 1], w.scan_tmp, s)) != cudaSuccess) return e;
+    const int cluster = tt_use_cluster(h);
+    if (cluster == 1 || cluster == 2) return cudaSuccess;   // done with the grouping
+    if (cluster == 0 || !w.equal_units) {
+        if (tt_digit_major(w)) {
+            if ((e = launch_tfill(h, w.K - 1, true, cluster == 0, s)) != cudaSuccess) return e;
+        } else if (w.K >= 3) {
+            if ((e = tt_launch_pdl(k_costs, dim3(h->sm_count * 8), dim3(256), 0, s, w)) != cudaSuccess) return e;
+            tt_note_launch();
+        }
+        if (w.K >= 3) {
+            CostScan<> cs{w};
+            if ((e = tt_scan<CostScan<>, TT_CSCAN_ITEMS>(cs, w.cap[w.K - 1], w.scan_tmp, s)) != cudaSuccess) return e;
+        }
     }
     int64_t want = (int64_t)w.T * w.units_per_table;
     if (want < w.pool_shares + 1) want = w.pool_shares + 1;
