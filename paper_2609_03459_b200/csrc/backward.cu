@@ -1047,6 +1047,21 @@ cudaError_t tt_launch_bwd_dE(tt_emb* h, const float* grad_out, cudaStream_t s)
 
 // ---------------------------------------------------------------------------------------------- 3. last level
 
+// dC of the batch's groups to the level above (K = 2: it is the gradient of the first core's slice itself); ends with a barrier
+template <int THREADS>
+__device__ __forceinline__ void gen_hand_up(const WsView& w, const TableDesc& td, int cnt, const GenBatch& b, const float* dCs)
+{
+    const int K = w.K, Pm = td.P[K - 1], rb = td.r[K - 1], pitch = gen_pitch(rb);
+    for (int it = threadIdx.x; it < cnt * Pm * rb; it += THREADS) {
+        const int q = it / (Pm * rb), e = it - q * (Pm * rb), p = e / rb;
+        float* dst = K >= 3 ? w.dP[K - 1] + (size_t)b.g[q] * w.stride[K - 1] : td.grad[0] + (size_t)b.val[q] * td.slice_floats[0];
+        const float x = dCs[q * (Pm * pitch) + p * pitch + (e - p * rb)];
+        if (b.part[q]) atomicAdd(dst + e, x);   // K = 2: the first core's gradient starts at zero
+        else dst[e] = x;
+    }
+    __syncthreads();
+}
+
 // any shape: batches of groups spread flat over the CTA (generic.cuh)
 __global__ void __launch_bounds__(GEN_THREADS, 3) k_sweep_bwd_any(WsView w, int vbase)
 {
@@ -1069,7 +1084,7 @@ __global__ void __launch_bounds__(GEN_THREADS, 3) k_sweep_bwd_any(WsView w, int 
         const int cnt = (int)min(ng, groups.y - base);
         for (int i = threadIdx.x; i < cnt * Pm * pitch; i += GEN_THREADS) dCs[i] = 0.f;
         gen_batch_begin(w, td, base, cnt, range, b);
-        gen_batch_c(w, td, cnt, b, Cs);
+        gen_batch_c<GEN_THREADS>(w, td, cnt, b, Cs);
         const uint32_t rows = b.row0[cnt];
         for (uint32_t r0 = 0; r0 < rows; r0 += GEN_ROWS) {
             const int n = (int)min((uint32_t)GEN_ROWS, rows - r0);
@@ -1083,15 +1098,43 @@ __global__ void __launch_bounds__(GEN_THREADS, 3) k_sweep_bwd_any(WsView w, int 
             }
             __syncthreads();
         }
-        // hand dC to the level above (K = 2: it is the gradient of the first core's slice itself)
-        for (int it = threadIdx.x; it < cnt * Pm * rb; it += GEN_THREADS) {
-            const int q = it / (Pm * rb), e = it - q * (Pm * rb), p = e / rb;
-            float* dst = K >= 3 ? w.dP[K - 1] + (size_t)b.g[q] * w.stride[K - 1] : td.grad[0] + (size_t)b.val[q] * td.slice_floats[0];
-            const float x = dCs[q * (Pm * pitch) + p * pitch + (e - p * rb)];
-            if (b.part[q]) atomicAdd(dst + e, x);   // K = 2: the first core's gradient starts at zero
-            else dst[e] = x;
+        gen_hand_up<GEN_THREADS>(w, td, cnt, b, dCs);
+    }
+}
+
+// the same for one last dim factor of 1, 2, 3, 5, 6 or 7
+template <int DK>
+__global__ void __launch_bounds__(GEN_ODD_THREADS, 6) k_sweep_bwd_odd(WsView w, int vbase, int c_floats)
+{
+    tt_pdl_enter();
+    extern __shared__ __align__(16) float sm[];
+    __shared__ GenBatch b;
+    __shared__ float s_part[4 * GEN_P * GEN_ODD_THREADS];
+    const int t = w.vlist[vbase + blockIdx.y], K = w.K;
+    const uint2 rng = w.unit_rng[t * w.units_per_table + blockIdx.x];
+    const TableDesc& td = w.tdesc[t];
+    const int stripe = (blockIdx.x + blockIdx.y) % TT_STRIPES;
+    float* gk = w.gpart + (size_t)stripe * w.gpart_stride + td.gpart_off;
+    float *Cs = sm, *dCs = sm + c_floats, *Es = dCs + c_floats;
+    const int Pm = td.P[K - 1], rb = td.r[K - 1], pitch = gen_pitch(rb);
+    const uint32_t ng = (uint32_t)gen_groups(td, K), chunk = (uint32_t)gen_stage_rows(w.D);
+    uint2 groups, range;
+    gen_unit(w, t, rng, groups, range);
+    for (uint32_t base = groups.x; base < groups.y; base += ng) {
+        const int cnt = (int)min(ng, groups.y - base);
+        for (int i = threadIdx.x; i < cnt * Pm * pitch; i += GEN_ODD_THREADS) dCs[i] = 0.f;
+        gen_batch_begin(w, td, base, cnt, range, b);
+        gen_batch_c<GEN_ODD_THREADS>(w, td, cnt, b, Cs);
+        const uint32_t rows = b.row0[cnt];
+        for (uint32_t r0 = 0; r0 < rows; r0 += chunk) {
+            const int n = (int)min(chunk, rows - r0);
+            gen_rows(w, td, cnt, r0, n, b);
+            gen_stage(w, n, b, Es);
+            gen_slice_odd<DK>(w, td, n, b, Cs, Es, gk);
+            gen_dc_odd<DK>(w, td, r0, n, b, Es, dCs, s_part);
+            __syncthreads();
         }
-        __syncthreads();
+        gen_hand_up<GEN_ODD_THREADS>(w, td, cnt, b, dCs);
     }
 }
 
@@ -1985,6 +2028,17 @@ static cudaError_t launch_sweep_bwd(tt_emb* h, int max_pl, int max_c, cudaStream
     cudaError_t e;
     if ((e = tt_stage_begin(h, 9 + TT_NUM_VARIANTS + 1 + V + 1, s)) != cudaSuccess) return e;
     if constexpr (V < 0) {
+        int c_floats;
+        if (const int dk = gen_odd_factor(h, c_floats)) {
+            auto kern = dk == 1 ? k_sweep_bwd_odd<1> : dk == 2 ? k_sweep_bwd_odd<2> : dk == 3 ? k_sweep_bwd_odd<3>
+                      : dk == 5 ? k_sweep_bwd_odd<5> : dk == 6 ? k_sweep_bwd_odd<6> : k_sweep_bwd_odd<7>;
+            smem = (size_t)(2 * c_floats + gen_stage_rows(h->D) * gen_stage_pitch(h->D)) * sizeof(float);
+            if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
+            if ((e = tt_launch_pdl(kern, dim3(h->units_per_table, n), dim3(GEN_ODD_THREADS), smem, s, h->v, h->vbase[0], c_floats)) != cudaSuccess) return e;
+            tt_note_launch();
+            if ((e = tt_stage_end(h, 9 + TT_NUM_VARIANTS + 1 + V + 1, s)) != cudaSuccess) return e;
+            return cudaGetLastError();
+        }
         smem = 2 * GEN_C_FLOATS * sizeof(float);
         if ((e = cudaFuncSetAttribute(k_sweep_bwd_any, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
         if ((e = tt_launch_pdl(k_sweep_bwd_any, dim3(h->units_per_table, n), dim3(GEN_THREADS), smem, s, h->v, h->vbase[0])) != cudaSuccess) return e;

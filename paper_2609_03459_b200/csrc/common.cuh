@@ -43,6 +43,11 @@
 // ... and of the any-shape sweeps, whose CTAs take a batch of groups at a time (3x3x5, 29 k groups, forward + backward sweep
 // with at least 1 / 4 / 8 / 16 groups: 332 / 285 / 252 / 253 us; 8x8 with K = 2, 420 k lookups, whole call 1.16 ms with 8, 1.68 with 16)
 #define TT_UNIT_GROUPS_ANY 8
+// ... and with last dim factors that are no multiples of four, whose threads take whole rows, at least TT_UNIT_ROWS_ODD rows too, up to 32
+// groups, where there are groups enough.  3x3x5, forward + backward sweep, us, units of 4 / 8 / 16 / 32 groups: 1.8 rows a group, 26 k groups
+// 119 / 91 / 79 / 92; 1.4 rows, 17 k groups 94 / 58 / 53 / 56; 8 rows, 29 k groups 168 / 161 / 179 / 226; with at least 24 / 32 / 48 rows the
+// first 77 / 69 / 72 (calls 259.9 / 252.6 / 255.7).
+#define TT_UNIT_ROWS_ODD 32
 // Batches of few groups: below TT_FEW_LIMIT groups per CTA of TT_FEW_UNITS on every SM, the sweeps cut the tables' groups into that many
 // equal parts of at least TT_FEW_GROUPS, and each of a CTA's warps takes a quarter.  A warp that takes its four or eight at once fetches
 // one slice after the other, 3 us each for 4 KB, 12 us for 32 KB, while most of the chip idles.  Forward / backward sweep, us, in the
@@ -407,6 +412,10 @@ __device__ __forceinline__ void tt_unit_range(const WsView& w, int t, int q, uin
         const bool pair = (td.fast == 5 || td.fast == 6 || td.fast == 8 || td.fast == 9) && w.tb[lvl][w.T] >= w.paired_groups;
         const int by_groups = (int)(pair ? (b - a + 2 * TT_UNIT_GROUPS - 1) / (2 * TT_UNIT_GROUPS) : (b - a) / (uint32_t)td.unit_groups);
         if (Q > by_groups) Q = by_groups < 1 ? 1 : by_groups;
+        if (td.fast < 0 && (td.d[w.K - 1] & 3) != 0 && w.tb[lvl][w.T] >= 2 * TT_UNIT_GROUPS_ANY * w.few_units) {
+            const int by_rows = (int)max((w.tb[w.K][t + 1] - w.tb[w.K][t]) / TT_UNIT_ROWS_ODD, (b - a) / 32u);
+            if (Q > by_rows) Q = by_rows < 1 ? 1 : by_rows;
+        }
     }
     if (q >= Q) { g0 = a; g1 = a; return; }
     if (w.equal_units) {   // equal group counts

@@ -9,6 +9,7 @@
 // 24 k lookups in 4 tables: the training call 1.43 -> 0.20 ms (few groups of up to 2000 rows each: units are ranges of rows).
 #pragma once
 #include "common.cuh"
+#include "tiles.cuh"
 
 #define GEN_THREADS 256
 #define GEN_GROUPS 32
@@ -83,13 +84,14 @@ __device__ __forceinline__ void gen_batch_begin(const WsView& w, const TableDesc
 }
 
 // C of every group of the batch into Cs (ends with a barrier)
+template <int THREADS>
 __device__ __forceinline__ void gen_batch_c(const WsView& w, const TableDesc& td, int cnt, const GenBatch& b, float* Cs)
 {
     const int K = w.K, km = K - 2, Pm = td.P[K - 1], rb = td.r[K - 1], pitch = gen_pitch(rb), tile = Pm * pitch;
     if (K >= 3) {
         constexpr int MB = 8;
         const int M = td.P[km], ra = td.r[km], dm = td.d[km], cols = dm * rb, mblocks = (M + MB - 1) / MB;
-        for (int it = threadIdx.x; it < cnt * mblocks * cols; it += GEN_THREADS) {
+        for (int it = threadIdx.x; it < cnt * mblocks * cols; it += THREADS) {
             const int c = it % cols, qm = it / cols, q = qm / mblocks, m0 = (qm - q * mblocks) * MB, mm = min(MB, M - m0);
             const float* P = b.left[q] + m0 * ra;
             const float* B = td.core[km] + (size_t)(b.val[q] % (uint32_t)td.n[km]) * td.slice_floats[km] + c;
@@ -109,7 +111,7 @@ __device__ __forceinline__ void gen_batch_c(const WsView& w, const TableDesc& td
                 if (i < mm) dst[i * dm * pitch] = acc[i];
         }
     } else {
-        for (int it = threadIdx.x; it < cnt * Pm * rb; it += GEN_THREADS) {
+        for (int it = threadIdx.x; it < cnt * Pm * rb; it += THREADS) {
             const int q = it / (Pm * rb), e = it - q * (Pm * rb), p = e / rb;
             Cs[q * tile + p * pitch + (e - p * rb)] = b.left[q][e];
         }
@@ -117,10 +119,9 @@ __device__ __forceinline__ void gen_batch_c(const WsView& w, const TableDesc& td
     __syncthreads();
 }
 
-// look up rows r0 .. r0 + n of the batch (ends with a barrier)
+// look up rows r0 .. r0 + n of the batch, at most one per thread (ends with a barrier)
 __device__ __forceinline__ void gen_rows(const WsView& w, const TableDesc& td, int cnt, uint32_t r0, int n, GenBatch& b)
 {
-    static_assert(GEN_ROWS == GEN_THREADS, "one row per thread");
     if ((int)threadIdx.x < n) {
         const uint32_t r = r0 + threadIdx.x;
         int lo = 0, hi = cnt;             // the group that holds row r
@@ -306,4 +307,240 @@ __device__ __forceinline__ void gen_backward_dc(const WsView& w, const TableDesc
             add((int)threadIdx.x, x);
         }
     }
+}
+
+// ---- last dim factors of 1, 2, 3, 5, 6 or 7 (DK) --------------------------------------------------------------------------------
+//
+// Rows of E and slices of the last core are no whole float4s there, and the items above take one load for every product or two, each of a
+// warp's lanes from another place.  Here a chunk's rows pass through shared memory (Es, odd pitch, read and written as whole lines), and a
+// thread holds four values of r_{K-1} by all of d_K, whose slice parts are whole float4s where the slice is: 9 loads for 20 products in
+// dG_K, 20 for 60 in dC, 17 for 60 in E at d_K = 5.  Bound by shared-memory loads and the scattered loads of the slices.
+// Chunks hold few rows (8 groups of 1 to 8 rows), so CTAs are small: with 256 / 128 / 96 / 64 threads the call of 4 tables with 3x3x5, ranks 6
+// and 4, 1 M lookups, takes 460 / 447 / 459 / 484 us, 473 with the items above; forward sweep 59 -> 64, backward 135 -> 99.  With units of
+// enough rows (TT_UNIT_ROWS_ODD): 3 tables, 0.14 M lookups 41 -> 29 and 76 -> 40, call 295 -> 252; 43 k lookups 27 -> 19, 50 -> 31.
+// Below GEN_ODD_LOOKUPS a unit's few rows leave most threads idle here too, and theirs is the longer chain: 0.9 k lookups, calls 109 above,
+// 111 here, 15 k 132 / 133, 36 k 189 / 165.
+#define GEN_ODD_LOOKUPS (1 << 14)
+#define GEN_ODD_THREADS 128
+#define GEN_STAGE_FLOATS 12288   // of the staged rows; fewer than GEN_STAGE_LEAST rows leave threads without one
+#define GEN_STAGE_LEAST 64
+#define GEN_P 3                  // rows of C that a thread takes at a time
+__host__ __device__ __forceinline__ int gen_stage_pitch(int D) { return D | 1; }
+__host__ __device__ __forceinline__ int gen_stage_rows(int D)
+{
+    const int n = GEN_STAGE_FLOATS / gen_stage_pitch(D);
+    return n < GEN_ODD_THREADS ? n : GEN_ODD_THREADS;
+}
+
+// f(row, element) for all of the chunk's rows, a warp per row
+template <class F>
+__device__ __forceinline__ void gen_each(int n, int D, const F& f)
+{
+    const int lane = threadIdx.x & 31;
+    for (int i = threadIdx.x >> 5; i < n; i += GEN_ODD_THREADS / 32)
+        for (int e = lane; e < D; e += 32) f(i, e);
+}
+
+// d = na x DK values of the slice part at p (VEC: four rows, 16-byte aligned)
+template <int DK>
+__device__ __forceinline__ void gen_part(float (&d)[4 * DK], const float* __restrict__ p, int na, bool vec)
+{
+    if (vec && na == 4) {
+#pragma unroll
+        for (int v = 0; v < DK; ++v) {
+            const float4 x = __ldg(reinterpret_cast<const float4*>(p) + v);
+            d[4 * v] = x.x; d[4 * v + 1] = x.y; d[4 * v + 2] = x.z; d[4 * v + 3] = x.w;
+        }
+    } else {
+#pragma unroll
+        for (int f = 0; f < 4 * DK; ++f) d[f] = f < na * DK ? __ldg(p + f) : 0.f;
+    }
+}
+
+// E = C . G_K[i_K] of the n looked-up rows, GEN_P rows of C to a thread
+template <int DK>
+__device__ __forceinline__ void gen_forward_odd(const WsView& w, const TableDesc& td, int n, const GenBatch& b, const float* Cs, float* Es)
+{
+    const int K = w.K, Pm = td.P[K - 1], rb = td.r[K - 1], pitch = gen_pitch(rb), slice = td.slice_floats[K - 1], ep = gen_stage_pitch(w.D);
+    for (int it = threadIdx.x; it < n * ((Pm + GEN_P - 1) / GEN_P); it += GEN_ODD_THREADS) {
+        const int i = it % n, p = it / n * GEN_P;
+        const float* D = td.core[K - 1] + (size_t)b.iK[i] * slice;
+        const float* c = Cs + b.q[i] * (Pm * pitch);
+        float x[GEN_P][DK];
+        int row[GEN_P];
+#pragma unroll
+        for (int k = 0; k < GEN_P; ++k) {
+            row[k] = min(p + k, Pm - 1) * pitch;
+#pragma unroll
+            for (int j = 0; j < DK; ++j) x[k][j] = 0.f;
+        }
+        for (int a0 = 0; a0 < rb; a0 += 4) {
+            float d[4 * DK];
+            gen_part<DK>(d, D + a0 * DK, min(4, rb - a0), (slice & 3) == 0);
+#pragma unroll
+            for (int a = 0; a < 4; ++a) {
+                if (a0 + a >= rb) break;
+#pragma unroll
+                for (int k = 0; k < GEN_P; ++k) {
+                    const float y = c[row[k] + a0 + a];
+#pragma unroll
+                    for (int j = 0; j < DK; ++j) x[k][j] = fmaf(y, d[a * DK + j], x[k][j]);
+                }
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < GEN_P; ++k)
+            if (p + k < Pm)
+#pragma unroll
+                for (int j = 0; j < DK; ++j) Es[i * ep + (p + k) * DK + j] = x[k][j];
+    }
+    __syncthreads();
+    gen_each(n, w.D, [&](int r, int e) { w.E[(size_t)b.u[r] * w.D + e] = Es[r * ep + e]; });
+}
+
+// the n looked-up rows of dE into Es (ends with a barrier)
+__device__ __forceinline__ void gen_stage(const WsView& w, int n, const GenBatch& b, float* Es)
+{
+    const int ep = gen_stage_pitch(w.D);
+    gen_each(n, w.D, [&](int r, int e) { tt_cp_async4(Es + r * ep + e, w.E + (size_t)b.u[r] * w.D + e); });
+    asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
+    __syncthreads();
+}
+
+// dG_K[i_K] += C^T . dE of the staged rows, a thread four rows of a slice
+template <int DK>
+__device__ __forceinline__ void gen_slice_odd(const WsView& w, const TableDesc& td, int n, const GenBatch& b, const float* Cs, const float* Es, float* gk)
+{
+    const int K = w.K, Pm = td.P[K - 1], rb = td.r[K - 1], pitch = gen_pitch(rb), slice = td.slice_floats[K - 1], ep = gen_stage_pitch(w.D);
+    for (int it = threadIdx.x; it < n * ((rb + 3) / 4); it += GEN_ODD_THREADS) {
+        const int i = it % n, a0 = it / n * 4, na = min(4, rb - a0);
+        const float* c = Cs + b.q[i] * (Pm * pitch) + a0;
+        const float* dE = Es + i * ep;
+        float x[4 * DK];
+#pragma unroll
+        for (int f = 0; f < 4 * DK; ++f) x[f] = 0.f;
+        for (int p = 0; p < Pm; ++p) {
+            float e[DK];
+#pragma unroll
+            for (int j = 0; j < DK; ++j) e[j] = dE[p * DK + j];
+#pragma unroll
+            for (int a = 0; a < 4; ++a) {
+                const float y = c[p * pitch + min(a, na - 1)];
+#pragma unroll
+                for (int j = 0; j < DK; ++j) x[a * DK + j] = fmaf(y, e[j], x[a * DK + j]);
+            }
+        }
+        float* dst = gk + (size_t)b.iK[i] * slice + a0 * DK;
+        if ((slice & 3) == 0 && na == 4) {
+#pragma unroll
+            for (int v = 0; v < DK; ++v) {
+                const float y[4] = {x[4 * v], x[4 * v + 1], x[4 * v + 2], x[4 * v + 3]};
+                gen_red4(dst + 4 * v, y);
+            }
+        } else {
+#pragma unroll
+            for (int f = 0; f < 4 * DK; ++f)
+                if (f < na * DK) atomicAdd(dst + f, x[f]);
+        }
+    }
+}
+
+// dC += dE . G_K[i_K]^T over the staged rows, r0 the first of them: GEN_P by four elements of one group's dC to a thread, otherwise as
+// gen_backward_dc; s_part [4 GEN_P][GEN_ODD_THREADS]
+template <int DK>
+__device__ __forceinline__ void gen_dc_odd(const WsView& w, const TableDesc& td, uint32_t r0, int n, const GenBatch& b, const float* Es, float* dCs, float* s_part)
+{
+    const int K = w.K, Pm = td.P[K - 1], rb = td.r[K - 1], pitch = gen_pitch(rb), slice = td.slice_floats[K - 1], ep = gen_stage_pitch(w.D);
+    const int q0 = (int)b.q[0], nq = (int)b.q[n - 1] - q0 + 1, ab = (rb + 3) / 4, per = (Pm + GEN_P - 1) / GEN_P * ab, items = nq * per;
+    const int parts = items < GEN_ODD_THREADS ? min(16, GEN_ODD_THREADS / items) : 1;
+    auto add = [&](int ie, const float (&x)[GEN_P][4]) {
+        const int qq = ie / per, e = ie - qq * per, p = e / ab * GEN_P, a0 = (e - e / ab * ab) * 4;
+        float* dst = dCs + (q0 + qq) * (Pm * pitch) + p * pitch + a0;
+#pragma unroll
+        for (int k = 0; k < GEN_P; ++k)
+#pragma unroll
+            for (int a = 0; a < 4; ++a)
+                if (p + k < Pm && a0 + a < rb) dst[k * pitch + a] += x[k][a];
+    };
+    for (int it = threadIdx.x; it < items * parts; it += GEN_ODD_THREADS) {
+        const int part = it / items, ie = it - part * items, qq = ie / per, e = ie - qq * per, p = e / ab * GEN_P, a0 = (e - e / ab * ab) * 4;
+        const int q = q0 + qq, na = min(4, rb - a0);
+        int i0 = b.row0[q] > r0 ? (int)(b.row0[q] - r0) : 0, i1 = min(n, (int)(b.row0[q + 1] - r0));
+        const int len = (i1 - i0 + parts - 1) / parts;
+        i0 += part * len;
+        i1 = min(i1, i0 + len);
+        int row[GEN_P];
+        float sum[GEN_P][4];
+#pragma unroll
+        for (int k = 0; k < GEN_P; ++k) {
+            row[k] = min(p + k, Pm - 1) * DK;
+#pragma unroll
+            for (int a = 0; a < 4; ++a) sum[k][a] = 0.f;
+        }
+        for (int ib = i0; ib < i1; ib += 8) {
+            float acc[GEN_P][4];
+#pragma unroll
+            for (int k = 0; k < GEN_P; ++k)
+#pragma unroll
+                for (int a = 0; a < 4; ++a) acc[k][a] = 0.f;
+            const int ie8 = min(i1, ib + 8);
+            for (int i = ib; i < ie8; ++i) {
+                float d[4 * DK];
+                gen_part<DK>(d, td.core[K - 1] + (size_t)b.iK[i] * slice + a0 * DK, na, (slice & 3) == 0);
+#pragma unroll
+                for (int k = 0; k < GEN_P; ++k) {
+                    const float* dE = Es + i * ep + row[k];
+#pragma unroll
+                    for (int j = 0; j < DK; ++j) {
+                        const float y = dE[j];
+#pragma unroll
+                        for (int a = 0; a < 4; ++a) acc[k][a] = fmaf(y, d[a * DK + j], acc[k][a]);
+                    }
+                }
+            }
+#pragma unroll
+            for (int k = 0; k < GEN_P; ++k)
+#pragma unroll
+                for (int a = 0; a < 4; ++a) sum[k][a] += acc[k][a];
+        }
+        if (parts > 1) {                             // then a thread has one item
+#pragma unroll
+            for (int k = 0; k < GEN_P; ++k)
+#pragma unroll
+                for (int a = 0; a < 4; ++a) s_part[(4 * k + a) * GEN_ODD_THREADS + it] = sum[k][a];
+        } else add(ie, sum);
+    }
+    if (parts > 1) {
+        __syncthreads();
+        if ((int)threadIdx.x < items) {
+            float x[GEN_P][4];
+#pragma unroll
+            for (int k = 0; k < GEN_P; ++k)
+#pragma unroll
+                for (int a = 0; a < 4; ++a) {
+                    const float* s = s_part + (4 * k + a) * GEN_ODD_THREADS + threadIdx.x;
+                    x[k][a] = s[0];
+                    for (int part = 1; part < parts; ++part) x[k][a] += s[part * items];
+                }
+            add((int)threadIdx.x, x);
+        }
+    }
+}
+
+// The last dim factor that all of the handle's any-shape tables have, where the call is for the code above (otherwise 0), and the floats of
+// their C tiles of a batch
+inline int gen_odd_factor(const tt_emb* h, int& c_floats)
+{
+    int dk = 0;
+    c_floats = 0;
+    for (int t = 0; t < h->T; ++t) {
+        const TableDesc& td = h->tab[t];
+        if (td.fast >= 0) continue;
+        const int d = td.d[h->K - 1], tile = td.P[h->K - 1] * gen_pitch(td.r[h->K - 1]);
+        const int n = GEN_C_FLOATS / tile < GEN_GROUPS ? GEN_C_FLOATS / tile : GEN_GROUPS;
+        if (dk != 0 && d != dk) return 0;
+        dk = d;
+        if (n * tile > c_floats) c_floats = n * tile;
+    }
+    return dk < 8 && dk % 4 != 0 && h->v.L >= GEN_ODD_LOOKUPS && gen_stage_rows(h->D) >= GEN_STAGE_LEAST ? dk : 0;
 }
