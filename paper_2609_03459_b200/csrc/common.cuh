@@ -43,10 +43,10 @@
 // ... and of the any-shape sweeps, whose CTAs take a batch of groups at a time (3x3x5, 29 k groups, forward + backward sweep
 // with at least 1 / 4 / 8 / 16 groups: 332 / 285 / 252 / 253 us; 8x8 with K = 2, 420 k lookups, whole call 1.16 ms with 8, 1.68 with 16)
 #define TT_UNIT_GROUPS_ANY 8
-// ... and with last dim factors that are no multiples of four, whose threads take whole rows, at least TT_UNIT_ROWS_ODD rows too, up to 32
-// groups, where there are groups enough.  3x3x5, forward + backward sweep, us, units of 4 / 8 / 16 / 32 groups: 1.8 rows a group, 26 k groups
-// 119 / 91 / 79 / 92; 1.4 rows, 17 k groups 94 / 58 / 53 / 56; 8 rows, 29 k groups 168 / 161 / 179 / 226; with at least 24 / 32 / 48 rows the
-// first 77 / 69 / 72 (calls 259.9 / 252.6 / 255.7).
+// ... and with last dim factors that are no multiples of four, whose backward takes rows to a thread, at least TT_UNIT_ROWS_ODD rows too, up
+// to 32 groups, where there are groups enough.  3x3x5, backward sweep, us, units of 4 / 8 / 16 / 32 groups: 1.8 rows a group, 26 k groups 76 /
+// 56 / 48 / 57; 1.4 rows, 17 k groups 59 / 35 / 31 / 32; 8 rows, 29 k groups 104 / 97 / 106 / 133; with at least 24 / 32 / 48 rows the first
+// 46 / 40 / 42 (forward sweep, with 8 groups and with 32 rows: 40 / 33).
 #define TT_UNIT_ROWS_ODD 32
 // Batches of few groups: below TT_FEW_LIMIT groups per CTA of TT_FEW_UNITS on every SM, the sweeps cut the tables' groups into that many
 // equal parts of at least TT_FEW_GROUPS, and each of a CTA's warps takes a quarter.  A warp that takes its four or eight at once fetches

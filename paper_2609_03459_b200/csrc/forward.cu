@@ -574,34 +574,6 @@ __global__ void __launch_bounds__(GEN_THREADS) k_sweep_fwd_any(WsView w, int vba
     }
 }
 
-// the same for one last dim factor of 1, 2, 3, 5, 6 or 7
-template <int DK>
-__global__ void __launch_bounds__(GEN_ODD_THREADS, 8) k_sweep_fwd_odd(WsView w, int vbase, int c_floats)
-{
-    tt_pdl_enter();
-    extern __shared__ __align__(16) float sm[];
-    __shared__ GenBatch b;
-    const int t = w.vlist[vbase + blockIdx.y];
-    const uint2 rng = w.unit_rng[t * w.units_per_table + blockIdx.x];
-    const TableDesc& td = w.tdesc[t];
-    const uint32_t ng = (uint32_t)gen_groups(td, w.K), chunk = (uint32_t)gen_stage_rows(w.D);
-    uint2 groups, range;
-    gen_unit(w, t, rng, groups, range);
-    for (uint32_t base = groups.x; base < groups.y; base += ng) {
-        const int cnt = (int)min(ng, groups.y - base);
-        gen_batch_begin(w, td, base, cnt, range, b);
-        gen_batch_c<GEN_ODD_THREADS>(w, td, cnt, b, sm);
-        const uint32_t rows = b.row0[cnt];
-        for (uint32_t r0 = 0; r0 < rows; r0 += chunk) {
-            const int n = (int)min(chunk, rows - r0);
-            gen_rows(w, td, cnt, r0, n, b);
-            gen_forward_odd<DK>(w, td, n, b, sm, sm + c_floats);
-            __syncthreads();
-        }
-        __syncthreads();
-    }
-}
-
 // fused levels K-1 and K: C stays on chip, rows go to w.E.  One CTA (4 warps) per work unit (table, q);
 // one instantiation per shape variant V so that each gets its own register budget.  blockIdx.y walks the
 // tables of variant V (w.vlist), blockIdx.x the table's equal-cost slices.
@@ -657,17 +629,6 @@ static cudaError_t launch_sweep_fwd(tt_emb* h, int max_pl, int max_c, cudaStream
     cudaError_t e;
     if ((e = tt_stage_begin(h, 9 + V + 1, s)) != cudaSuccess) return e;
     if constexpr (V < 0) {
-        int c_floats;
-        if (const int dk = gen_odd_factor(h, c_floats)) {
-            auto kern = dk == 1 ? k_sweep_fwd_odd<1> : dk == 2 ? k_sweep_fwd_odd<2> : dk == 3 ? k_sweep_fwd_odd<3>
-                      : dk == 5 ? k_sweep_fwd_odd<5> : dk == 6 ? k_sweep_fwd_odd<6> : k_sweep_fwd_odd<7>;
-            const size_t smem = (size_t)(c_floats + gen_stage_rows(h->D) * gen_stage_pitch(h->D)) * sizeof(float);
-            if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
-            if ((e = tt_launch_pdl(kern, dim3(h->units_per_table, n), dim3(GEN_ODD_THREADS), smem, s, h->v, h->vbase[0], c_floats)) != cudaSuccess) return e;
-            tt_note_launch();
-            if ((e = tt_stage_end(h, 9 + V + 1, s)) != cudaSuccess) return e;
-            return cudaGetLastError();
-        }
         const size_t smem = GEN_C_FLOATS * sizeof(float);
         if ((e = cudaFuncSetAttribute(k_sweep_fwd_any, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
         if ((e = tt_launch_pdl(k_sweep_fwd_any, dim3(h->units_per_table, n), dim3(GEN_THREADS), smem, s, h->v, h->vbase[0])) != cudaSuccess) return e;

@@ -309,17 +309,17 @@ __device__ __forceinline__ void gen_backward_dc(const WsView& w, const TableDesc
     }
 }
 
-// ---- last dim factors of 1, 2, 3, 5, 6 or 7 (DK) --------------------------------------------------------------------------------
+// ---- backward with last dim factors of 1, 2, 3, 5, 6 or 7 (DK) ---------------------------------------------------------------------
 //
-// Rows of E and slices of the last core are no whole float4s there, and the items above take one load for every product or two, each of a
-// warp's lanes from another place.  Here a chunk's rows pass through shared memory (Es, odd pitch, read and written as whole lines), and a
-// thread holds four values of r_{K-1} by all of d_K, whose slice parts are whole float4s where the slice is: 9 loads for 20 products in
-// dG_K, 20 for 60 in dC, 17 for 60 in E at d_K = 5.  Bound by shared-memory loads and the scattered loads of the slices.
-// Chunks hold few rows (8 groups of 1 to 8 rows), so CTAs are small: with 256 / 128 / 96 / 64 threads the call of 4 tables with 3x3x5, ranks 6
-// and 4, 1 M lookups, takes 460 / 447 / 459 / 484 us, 473 with the items above; forward sweep 59 -> 64, backward 135 -> 99.  With units of
-// enough rows (TT_UNIT_ROWS_ODD): 3 tables, 0.14 M lookups 41 -> 29 and 76 -> 40, call 295 -> 252; 43 k lookups 27 -> 19, 50 -> 31.
+// Rows of dE and slices of the last core are no whole float4s there, and the items above take one load for every product or two, each of a
+// warp's lanes from another place.  Here a chunk's rows pass through shared memory (Es, odd pitch, read as whole lines), and a thread holds
+// four values of r_{K-1} by all of d_K, whose slice parts are whole float4s where the slice is: 9 loads for 20 products in dG_K, 20 for 60
+// in dC at d_K = 5.  Bound by shared-memory loads and the scattered loads of the slices.  Chunks hold few rows (8 groups of 1 to 8 rows),
+// so CTAs are small: with 128 / 96 / 64 threads the sweep of 4 tables with 3x3x5, ranks 6 and 4, 1 M lookups, takes 97 / 106 / 125 us, 135
+// with the items above; with units of enough rows (TT_UNIT_ROWS_ODD) 3 tables, 0.14 M lookups 76 -> 40, one table, 43 k 50 -> 31.
 // Below GEN_ODD_LOOKUPS a unit's few rows leave most threads idle here too, and theirs is the longer chain: 0.9 k lookups, calls 109 above,
-// 111 here, 15 k 132 / 133, 36 k 189 / 165.
+// 111 here, 15 k 132 / 133, 36 k 189 / 165.  In the forward sweep, whose rows would be staged on their way out, the items above stay:
+// the first of these calls takes 439 us with them and 448 with staged rows, another with 0.19 M lookups 359 and 386.
 #define GEN_ODD_LOOKUPS (1 << 14)
 #define GEN_ODD_THREADS 128
 #define GEN_STAGE_FLOATS 12288   // of the staged rows; fewer than GEN_STAGE_LEAST rows leave threads without one
@@ -330,15 +330,6 @@ __host__ __device__ __forceinline__ int gen_stage_rows(int D)
 {
     const int n = GEN_STAGE_FLOATS / gen_stage_pitch(D);
     return n < GEN_ODD_THREADS ? n : GEN_ODD_THREADS;
-}
-
-// f(row, element) for all of the chunk's rows, a warp per row
-template <class F>
-__device__ __forceinline__ void gen_each(int n, int D, const F& f)
-{
-    const int lane = threadIdx.x & 31;
-    for (int i = threadIdx.x >> 5; i < n; i += GEN_ODD_THREADS / 32)
-        for (int e = lane; e < D; e += 32) f(i, e);
 }
 
 // d = na x DK values of the slice part at p (VEC: four rows, 16-byte aligned)
@@ -357,52 +348,12 @@ __device__ __forceinline__ void gen_part(float (&d)[4 * DK], const float* __rest
     }
 }
 
-// E = C . G_K[i_K] of the n looked-up rows, GEN_P rows of C to a thread
-template <int DK>
-__device__ __forceinline__ void gen_forward_odd(const WsView& w, const TableDesc& td, int n, const GenBatch& b, const float* Cs, float* Es)
-{
-    const int K = w.K, Pm = td.P[K - 1], rb = td.r[K - 1], pitch = gen_pitch(rb), slice = td.slice_floats[K - 1], ep = gen_stage_pitch(w.D);
-    for (int it = threadIdx.x; it < n * ((Pm + GEN_P - 1) / GEN_P); it += GEN_ODD_THREADS) {
-        const int i = it % n, p = it / n * GEN_P;
-        const float* D = td.core[K - 1] + (size_t)b.iK[i] * slice;
-        const float* c = Cs + b.q[i] * (Pm * pitch);
-        float x[GEN_P][DK];
-        int row[GEN_P];
-#pragma unroll
-        for (int k = 0; k < GEN_P; ++k) {
-            row[k] = min(p + k, Pm - 1) * pitch;
-#pragma unroll
-            for (int j = 0; j < DK; ++j) x[k][j] = 0.f;
-        }
-        for (int a0 = 0; a0 < rb; a0 += 4) {
-            float d[4 * DK];
-            gen_part<DK>(d, D + a0 * DK, min(4, rb - a0), (slice & 3) == 0);
-#pragma unroll
-            for (int a = 0; a < 4; ++a) {
-                if (a0 + a >= rb) break;
-#pragma unroll
-                for (int k = 0; k < GEN_P; ++k) {
-                    const float y = c[row[k] + a0 + a];
-#pragma unroll
-                    for (int j = 0; j < DK; ++j) x[k][j] = fmaf(y, d[a * DK + j], x[k][j]);
-                }
-            }
-        }
-#pragma unroll
-        for (int k = 0; k < GEN_P; ++k)
-            if (p + k < Pm)
-#pragma unroll
-                for (int j = 0; j < DK; ++j) Es[i * ep + (p + k) * DK + j] = x[k][j];
-    }
-    __syncthreads();
-    gen_each(n, w.D, [&](int r, int e) { w.E[(size_t)b.u[r] * w.D + e] = Es[r * ep + e]; });
-}
-
 // the n looked-up rows of dE into Es (ends with a barrier)
 __device__ __forceinline__ void gen_stage(const WsView& w, int n, const GenBatch& b, float* Es)
 {
     const int ep = gen_stage_pitch(w.D);
-    gen_each(n, w.D, [&](int r, int e) { tt_cp_async4(Es + r * ep + e, w.E + (size_t)b.u[r] * w.D + e); });
+    for (int i = threadIdx.x >> 5; i < n; i += GEN_ODD_THREADS / 32)
+        for (int e = threadIdx.x & 31; e < w.D; e += 32) tt_cp_async4(Es + i * ep + e, w.E + (size_t)b.u[i] * w.D + e);
     asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
     __syncthreads();
 }

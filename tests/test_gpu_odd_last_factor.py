@@ -1,4 +1,4 @@
-"""Any-shape sweeps with a last dim factor below eight that is no multiple of four: every factor, ranks below, at and above four, slices
+"""Any-shape backward with a last dim factor below eight that is no multiple of four: every factor, ranks below, at and above four, slices
 that are whole float4s and not, rows of C below and above what a thread takes, two to four cores, chunks of many rows and of few; and
 what keeps the general items: other last factors beside, rows past the staged ones, few lookups.
 
