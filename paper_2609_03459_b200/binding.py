@@ -132,8 +132,9 @@ def make_config(num_rows: Sequence[int], row_factors: Sequence[Sequence[int]], d
 
 def _stream_ptr(stream=None) -> int:
     import torch
-    s = torch.cuda.current_stream() if stream is None else stream
-    return int(s.cuda_stream)
+    if stream is None:   # without a Stream object, which took 3.6 of the 8.7 us that a small forward keeps the host
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    return int(stream.cuda_stream)
 
 
 class TTEmbeddingBag:

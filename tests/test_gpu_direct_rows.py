@@ -132,3 +132,11 @@ def test_capacity_and_graph(binding):  # noqa: F811
             assert counts[t, 2] == len(np.unique(ids[lo:hi]))
         wl.indices = keep
     assert_close(emb.forward(dev(wl.indices), off, 128).cpu().numpy(), ref, "out")
+
+
+def test_calls_go_to_the_current_stream(binding):  # noqa: F811
+    import torch
+    side = torch.cuda.Stream()
+    for stream in (torch.cuda.default_stream(), side, torch.cuda.ExternalStream(side.cuda_stream)):
+        with torch.cuda.stream(stream):
+            assert binding._stream_ptr() == binding._stream_ptr(stream) == stream.cuda_stream
