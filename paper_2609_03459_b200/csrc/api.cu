@@ -423,6 +423,18 @@ extern "C" int tt_emb_dim(tt_emb_t h, int32_t* D)
     return TT_EMB_OK;
 }
 
+static cudaError_t make_side_streams(tt_emb* h)
+{
+    cudaError_t e;
+    if (h->side_created) return cudaSuccess;
+    for (int i = 0; i < 4; ++i)
+        if ((e = cudaStreamCreateWithFlags(&h->side[i], cudaStreamNonBlocking)) != cudaSuccess) return e;
+    for (int i = 0; i < 5; ++i)
+        if ((e = cudaEventCreateWithFlags(&h->side_ev[i], cudaEventDisableTiming)) != cudaSuccess) return e;
+    h->side_created = true;
+    return cudaSuccess;
+}
+
 // ------------------------------------------------------------------------------------------------ bind
 
 extern "C" int tt_emb_bind(tt_emb_t h, float* const* core_ptrs, void* workspace, size_t workspace_bytes,
@@ -500,6 +512,8 @@ extern "C" int tt_emb_bind(tt_emb_t h, float* const* core_ptrs, void* workspace,
         // the list's own guard was just written; the list itself is uploaded after it (pageable source: staged before return)
         TT_CUDA(cudaMemcpyAsync(base + h->off_guard_list, list, sizeof(list), cudaMemcpyHostToDevice, s));
     }
+    // every backward of four cores forks (tt_launch_bwd_contraction): its first call took 120 us longer with the streams made there
+    if (K == 4 && h->enable_backward) TT_CUDA(make_side_streams(h));
     h->bound = true;
     h->have_forward = false;
     return TT_EMB_OK;
@@ -510,13 +524,7 @@ extern "C" int tt_emb_bind(tt_emb_t h, float* const* core_ptrs, void* workspace,
 cudaError_t tt_fork(tt_emb* h, cudaStream_t s, int n)
 {
     cudaError_t e;
-    if (!h->side_created) {
-        for (int i = 0; i < 4; ++i)
-            if ((e = cudaStreamCreateWithFlags(&h->side[i], cudaStreamNonBlocking)) != cudaSuccess) return e;
-        for (int i = 0; i < 5; ++i)
-            if ((e = cudaEventCreateWithFlags(&h->side_ev[i], cudaEventDisableTiming)) != cudaSuccess) return e;
-        h->side_created = true;
-    }
+    if ((e = make_side_streams(h)) != cudaSuccess) return e;
     if ((e = cudaEventRecord(h->side_ev[4], s)) != cudaSuccess) return e;
     for (int i = 0; i < n; ++i)
         if ((e = cudaStreamWaitEvent(h->side[i], h->side_ev[4], 0)) != cudaSuccess) return e;
