@@ -392,10 +392,11 @@ extern "C" int tt_emb_destroy(tt_emb_t h)
     if (!h) return TT_EMB_ERR_ARG;
     if (h->ev_created)
         for (int i = 0; i < TT_NUM_STAGES; ++i) { cudaEventDestroy(h->ev[i][0]); cudaEventDestroy(h->ev[i][1]); }
-    if (h->side_created) {
-        for (int i = 0; i < 4; ++i) cudaStreamDestroy(h->side[i]);
-        for (int i = 0; i < 5; ++i) cudaEventDestroy(h->side_ev[i]);
+    for (int i = 0; i < 4; ++i) {
+        if (h->side[i]) cudaStreamDestroy(h->side[i]);
+        if (h->side_ev[i]) cudaEventDestroy(h->side_ev[i]);
     }
+    if (h->fork_ev) cudaEventDestroy(h->fork_ev);
     free(h->tab);
     free(h->vlist_host);
     delete h;
@@ -423,15 +424,16 @@ extern "C" int tt_emb_dim(tt_emb_t h, int32_t* D)
     return TT_EMB_OK;
 }
 
-static cudaError_t make_side_streams(tt_emb* h)
+// the first n side streams, with their events, and the event that they wait for
+static cudaError_t make_side_streams(tt_emb* h, int n)
 {
     cudaError_t e;
-    if (h->side_created) return cudaSuccess;
-    for (int i = 0; i < 4; ++i)
-        if ((e = cudaStreamCreateWithFlags(&h->side[i], cudaStreamNonBlocking)) != cudaSuccess) return e;
-    for (int i = 0; i < 5; ++i)
+    if (!h->fork_ev && (e = cudaEventCreateWithFlags(&h->fork_ev, cudaEventDisableTiming)) != cudaSuccess) return e;
+    for (; h->side_made < n; ++h->side_made) {
+        const int i = h->side_made;
+        if (!h->side[i] && (e = cudaStreamCreateWithFlags(&h->side[i], cudaStreamNonBlocking)) != cudaSuccess) return e;
         if ((e = cudaEventCreateWithFlags(&h->side_ev[i], cudaEventDisableTiming)) != cudaSuccess) return e;
-    h->side_created = true;
+    }
     return cudaSuccess;
 }
 
@@ -512,8 +514,8 @@ extern "C" int tt_emb_bind(tt_emb_t h, float* const* core_ptrs, void* workspace,
         // the list's own guard was just written; the list itself is uploaded after it (pageable source: staged before return)
         TT_CUDA(cudaMemcpyAsync(base + h->off_guard_list, list, sizeof(list), cudaMemcpyHostToDevice, s));
     }
-    // every backward of four cores forks (tt_launch_bwd_contraction): its first call took 120 us longer with the streams made there
-    if (K == 4 && h->enable_backward) TT_CUDA(make_side_streams(h));
+    // every backward of four cores forks (tt_launch_bwd_contraction): its first call took 120 us longer with the stream made there
+    if (K == 4 && h->enable_backward) TT_CUDA(make_side_streams(h, 1));
     h->bound = true;
     h->have_forward = false;
     return TT_EMB_OK;
@@ -524,10 +526,10 @@ extern "C" int tt_emb_bind(tt_emb_t h, float* const* core_ptrs, void* workspace,
 cudaError_t tt_fork(tt_emb* h, cudaStream_t s, int n)
 {
     cudaError_t e;
-    if ((e = make_side_streams(h)) != cudaSuccess) return e;
-    if ((e = cudaEventRecord(h->side_ev[4], s)) != cudaSuccess) return e;
+    if ((e = make_side_streams(h, n)) != cudaSuccess) return e;
+    if ((e = cudaEventRecord(h->fork_ev, s)) != cudaSuccess) return e;
     for (int i = 0; i < n; ++i)
-        if ((e = cudaStreamWaitEvent(h->side[i], h->side_ev[4], 0)) != cudaSuccess) return e;
+        if ((e = cudaStreamWaitEvent(h->side[i], h->fork_ev, 0)) != cudaSuccess) return e;
     return cudaSuccess;
 }
 

@@ -225,10 +225,11 @@ struct tt_emb {
     cudaEvent_t ev[TT_NUM_STAGES][2];
     bool ev_valid[TT_NUM_STAGES];
     bool ev_created;
-    // side streams for kernels of different shape variants that may overlap (created on first use)
+    // side streams for kernels of different shape variants that may overlap (created on first use; the first at bind for training with
+    // four cores)
     cudaStream_t side[4];
-    cudaEvent_t side_ev[5];
-    bool side_created;
+    cudaEvent_t side_ev[4], fork_ev;
+    int side_made;
 };
 
 // every kernel launch of the library is noted here (api.cu); read with tt_emb_launch_count
