@@ -366,8 +366,8 @@ struct RowAcc {
 };
 
 #define DE_SPILL_LOG 1     // half a chunk
-// The sorted positions of a warp's chunk, 32 at a time: rows from the segment starts, bags (and factors) as stored.  `next` is called
-// once per batch, after it the loads of the batch that follows are on their way.
+// The sorted positions of a warp's chunk, 32 at a time: rows from the segment starts, bags (and factors) as stored.  `rows` and
+// then `fetch` are called once per batch; after them the loads of the batch that follows are on their way.
 struct DePairs {
     const WsView& w;
     uint32_t U, total, a, b;       // rows, pairs; the chunk [a, b)
@@ -619,7 +619,7 @@ __global__ void __launch_bounds__(256) k_dE(WsView w, const float* __restrict__ 
 }
 
 // The chunk in which a border-crossing segment starts adds up its pieces: its own tail, the tails of the chunks that the
-// segment fills, the head in the chunk where it ends (the sort has left the segment's end in cnt).  A warp adds a few
+// segment fills, the head in the chunk where it ends (the next row's start is the segment's end).  A warp adds a few
 // pieces by itself; a popular row spans hundreds of chunks, and one warp would walk them one memory round trip after the
 // other, so those are left to the whole CTA: 256 threads as 256 / (D / VEC) piece slots side by side, each with every
 // slots-th piece, then the slots in order.  (One warp per row: 4 M lookups,

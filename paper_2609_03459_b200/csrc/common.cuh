@@ -55,11 +55,12 @@
 // 1.2 k 28 / 43 and 17 / 23; four cores, 0.5 k 56 / 70 and 29 / 37.  Limits of 4 / 8 / 12: 150 drawn calls 0.965 / 0.961 / 0.959 of
 // their time (geometric mean), but above 8 cheap and dear groups in equal parts cost some 3 %.  Six CTAs per SM: as four.
 // The kernels that can do this take 1 % longer where there are more groups after all (a step in shared memory, spills), so they are
-// launched where at most TT_FEW_MAYBE times as many are possible by the lookups and the tables.
+// launched where at most TT_FEW_MAYBE times as many are possible by the lookups and the tables (8 times: 4 tables, D = 128, rank 32, 30 k
+// possible, 0.14 M lookups, training call 616 without, 638 with them; no drawn call with that many possible had few).
 #define TT_FEW_UNITS 4
 #define TT_FEW_GROUPS 4
 #define TT_FEW_LIMIT 8
-#define TT_FEW_MAYBE 8
+#define TT_FEW_MAYBE 4
 #define TT_STATUS_BYTES 512   // status word and counters (16 + 64 words) with their guard bytes, up to the row bitmap behind them
 #define TT_GUARD 0xA5         // guard bytes behind the other workspace regions
 #define TT_UNIT_ROWS 64   // fewest rows of a unit of a K = 2 table
