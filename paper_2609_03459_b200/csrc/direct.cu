@@ -156,8 +156,8 @@ __device__ __forceinline__ void direct_chunk(const TableDesc& td, float* sm, uns
     const Vec* const gB = reinterpret_cast<const Vec*>(td.core[1]) + (on_b ? lane : 0);
     auto stage = [&](int src, int buf) {
         const uint32_t x = __shfl_sync(0xffffffffu, i_first, src), y = __shfl_sync(0xffffffffu, i_last, src);
-        if (on_a) direct_cp16(sm + buf * DIRECT_SLICE + 4 * lane, gA + x * (uint32_t)an);
-        if (on_d) direct_cp16(sm + (2 + buf) * DIRECT_SLICE + 4 * lane, gD + y * (uint32_t)(4 * R));
+        if (on_a) direct_cp16(sm + buf * DIRECT_SLICE + 4 * lane, gA + (size_t)x * (uint32_t)an);
+        if (on_d) direct_cp16(sm + (2 + buf) * DIRECT_SLICE + 4 * lane, gD + (size_t)y * (uint32_t)(4 * R));
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
     Vec b[2][4];

@@ -140,3 +140,27 @@ def test_calls_go_to_the_current_stream(binding):  # noqa: F811
     for stream in (torch.cuda.default_stream(), side, torch.cuda.ExternalStream(side.cuda_stream)):
         with torch.cuda.stream(stream):
             assert binding._stream_ptr() == binding._stream_ptr(stream) == stream.cuda_stream
+
+
+@pytest.mark.parametrize("big", [0, 2])
+def test_cores_of_more_than_2_to_the_32_floats(binding, big):  # noqa: F811
+    # first and last core of (2^25 + 64) slices of 128 floats, 17 GB; digits whose slices lie 2^32 floats apart
+    n, r, most = [3, 2, 3], (1, 32, 8, 1) if big == 0 else (1, 8, 32, 1), (1 << 25) + 64
+    n[big] = most
+    used = [0, 5, 63, (1 << 25) - 1, 1 << 25, (1 << 25) + 5, most - 1]
+    g = torch.Generator(device="cuda")
+    g.manual_seed(big)
+    cores = [torch.zeros((r[k], n[k], 4, r[k + 1]), device="cuda") for k in range(3)]
+    for k in range(3):
+        for i in used if k == big else range(n[k]):
+            cores[k][:, i] = torch.randn((r[k], 4, r[k + 1]), generator=g, device="cuda")
+    B = 70
+    digits = [[used[b % len(used)] if k == big else (b + k) % n[k] for k in range(3)] for b in range(B)]
+    ids = torch.tensor([(i * n[1] + j) * n[2] + m for i, j, m in digits], device="cuda")
+    emb = binding.TTEmbeddingBag([int(np.prod(n, dtype=np.int64))], [n], [(4, 4, 4)], [r], B, B)
+    emb.set_cores([cores])
+    count, out = launches(binding, emb, ids, torch.arange(B + 1, device="cuda"), B)
+    assert count == 1 and emb.status() == 0
+    ref = torch.stack([torch.einsum("pa,aqb,bs->pqs", cores[0][0, i].double(), cores[1][:, j].double(), cores[2][:, m, :, 0].double()).reshape(-1)
+                       for i, j, m in digits])
+    assert_close(out.cpu().numpy(), ref.cpu().numpy(), "out")
