@@ -68,6 +68,21 @@ __device__ __forceinline__ int64_t tt_table_start(const WsView& w, int t)
     return o < 0 ? 0 : (o > w.L ? w.L : o);
 }
 
+// Lookups that may be in no bag, before the first offset and from the last one on, have no pair for the backward (what a call before
+// left in their place would be counted with rows and bags that this call may not have).  By the grid's first warp: such offsets are an
+// error of the caller's.
+__device__ __forceinline__ void tt_clear_pairs(const WsView& w)
+{
+    if (blockIdx.x != 0 || threadIdx.x >= 32 || !w.upairs) return;
+    const uint32_t L = (uint32_t)w.L;
+    auto clampL = [&](int64_t o) { return o < 0 ? 0u : o > w.L ? L : (uint32_t)o; };
+    uint32_t o0 = clampL(__ldg(w.offsets)), oL = clampL(__ldg(w.offsets + (int64_t)w.T * w.B));
+    if (o0 == 0 && oL == L) return;
+    if (o0 > oL) oL = 0u;      // bags that go up again may cover any part
+    for (uint32_t l = threadIdx.x; l < L; l += 32)
+        if (l < o0 || l >= oL) w.upairs[l] = make_uint2(0xffffffffu, 0u);
+}
+
 // the offsets: non-decreasing, from 0 to L; first lookup of every table into tl_start and (SHARES) boundaries of the pooling shares.
 // Threads first, first + step, ..
 template <bool SHARES>

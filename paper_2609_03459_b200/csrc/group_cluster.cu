@@ -238,6 +238,7 @@ __global__ void __launch_bounds__(GC_THREADS) k_group_cluster(const __grid_const
     gc_sync();   // also: every CTA runs before another writes into its shared memory
     if (rows) {
         tt_check_offsets<false>(w, first, step);
+        tt_clear_pairs(w);
         tt_mark_rows<false>(w, first, step, (int64_t)step * 4);
         gc_sync();
     }

@@ -21,6 +21,7 @@
 __global__ void __launch_bounds__(256) k_check_offsets(WsView w)
 {
     tt_pdl_enter();
+    tt_clear_pairs(w);
     tt_check_offsets<true>(w, (int64_t)blockIdx.x * blockDim.x + threadIdx.x, (int64_t)gridDim.x * blockDim.x);
 }
 
@@ -47,6 +48,7 @@ __global__ void __launch_bounds__(256, 8) k_mark(WsView w, int clear)
     }
     if (FUSED) tt_check_offsets<true>(w, (int64_t)blockIdx.x * blockDim.x + threadIdx.x, (int64_t)gridDim.x * blockDim.x);
     tt_mark_rows<!FUSED>(w, (int64_t)blockIdx.x * blockDim.x * 4 + threadIdx.x, blockDim.x, (int64_t)gridDim.x * blockDim.x * 4);
+    if (FUSED) tt_clear_pairs(w);
 }
 
 // ---------------------------------------------------------------------------------------------- prefix levels

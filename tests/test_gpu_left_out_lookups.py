@@ -1,0 +1,45 @@
+"""Lookups that malformed offsets leave out of every bag: they add nothing to the gradients, whatever the call before left in the workspace,
+for each way the offsets are checked (in one cluster, with the marks, in a kernel of its own).
+
+Bar: max|err| <= 1e-5 * max|ref| per tensor, the bound of the other parity tests (two-level fp32 sums)."""
+import numpy as np
+import pytest
+
+import oracle
+import workloads
+from test_gpu_parity import assert_close, binding, dev  # noqa: F401  (binding: fixture)
+from workloads import TableSpec
+
+pytestmark = pytest.mark.gpu
+
+
+def check_gradients(binding, emb, wl, offsets, what):  # noqa: F811
+    s = wl.tables[0]
+    emb.forward(dev(wl.indices), dev(offsets), wl.B)
+    assert emb.status() == (0 if what == "good" else binding.STATUS_OFFSETS)
+    emb.backward(dev(wl.grad_out))
+    # the lookups that are in bags, as a batch of their own
+    bags = [wl.indices[lo:hi] for lo, hi in zip(offsets[:-1], offsets[1:])]
+    kept = np.concatenate([[0], np.cumsum([len(b) for b in bags])]).astype(np.int64)
+    ref = oracle.backward(s.n, s.d, s.r, s.N, wl.cores[0], np.concatenate(bags), kept, wl.grad_out, memo=True)
+    for k, g in enumerate(emb.get_grads()[0]):
+        assert_close(g, ref[k], f"{what} dG[{k}]")
+    assert emb.check_guards() is None
+
+
+@pytest.mark.parametrize("L", [3000, 60_000, (1 << 22) + 1])
+def test_repeated_rows(binding, L):  # noqa: F811
+    # every row is looked up in a bag as well
+    spec = TableSpec(N=700, n=(9, 9, 9), d=(2, 2, 4), r=(1, 8, 8, 1), alpha=1.0, core_dist="normal", core_scale=0.3)
+    B = 120
+    rng = np.random.default_rng(L)
+    wl = workloads.custom([spec], B, 1, seed=3, with_grad=True)
+    wl.indices = np.resize(rng.permutation(700), L).astype(np.int64)
+    good = np.concatenate([[0], np.sort(rng.integers(0, L + 1, B - 1)), [L]]).astype(np.int64)
+    emb = binding.from_workload(wl, enable_backward=True)
+    check_gradients(binding, emb, wl, good, "good")
+    ends = L // 8 + np.sort(rng.integers(0, L // 2, B + 1))
+    falls = np.concatenate([[3 * L // 4], np.linspace(L // 4, L // 2, B // 2), np.linspace(L // 9, L // 5, B // 2)])   # two runs of bags
+    for what, offsets in (("ends", ends), ("falls", falls)):
+        check_gradients(binding, emb, wl, offsets.astype(np.int64), what)
+        check_gradients(binding, emb, wl, good, "good")
