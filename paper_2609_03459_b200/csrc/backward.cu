@@ -176,7 +176,8 @@ __global__ void __launch_bounds__(256) k_sort_count(WsView w)
 }
 
 // Counts -> segment starts in one kernel: a row's count becomes the sum of those before it in its tile, the CTA that reports last adds up
-// the tiles (a ticket counter; nobody waits), and a start is the sum of both (tt_seg_start).
+// the tiles (a ticket counter; nobody waits), and a start is the sum of both (tt_seg_start).  The row buffer still holds the rows: those
+// without pairs (malformed offsets leave all their lookups out) are set to zero, as nothing else writes their dE.
 #define CNT_TILE_LOG 12
 struct CntTotal {
     const WsView& w;
@@ -195,6 +196,7 @@ __global__ void __launch_bounds__(256) k_seg_starts(WsView w)
         return;
     }
     if (blockIdx.x >= ntiles) return;
+    const bool holes = *w.status & TT_EMB_STATUS_OFFSETS;
 #pragma unroll
     for (int j = 0; j < ITEMS; ++j) {
         const uint32_t i = base + (uint32_t)j * 256 + threadIdx.x;
@@ -204,6 +206,10 @@ __global__ void __launch_bounds__(256) k_seg_starts(WsView w)
     uint32_t mine[ITEMS], s = 0, tot;
 #pragma unroll
     for (int j = 0; j < ITEMS; ++j) { mine[j] = sv[tt_scan_pad(threadIdx.x * ITEMS + j)]; s += mine[j]; }
+    if (holes)
+        for (uint32_t i = base + threadIdx.x; i < n && i < base + TILE; i += 256)
+            if (sv[tt_scan_pad(i - base)] == 0u)
+                for (int e = 0; e < w.D; ++e) w.E[(size_t)i * w.D + e] = 0.f;
     uint32_t ex = tt_block_excl_scan(s, sm, tot);
     if (threadIdx.x == 0) {
         w.scan_tmp[blockIdx.x] = tot;

@@ -43,3 +43,21 @@ def test_repeated_rows(binding, L):  # noqa: F811
     for what, offsets in (("ends", ends), ("falls", falls)):
         check_gradients(binding, emb, wl, offsets.astype(np.int64), what)
         check_gradients(binding, emb, wl, good, "good")
+
+
+SHAPES = [((2, 2, 4), (1, 8, 8, 1)), ((4, 4, 4), (1, 8, 16, 1)), ((4, 8, 4), (1, 8, 8, 1)), ((3, 3, 5), (1, 6, 4, 1)), ((2, 3, 4), (1, 4, 4, 1))]
+
+
+@pytest.mark.parametrize("d,r", SHAPES)
+@pytest.mark.parametrize("rows", [0, 9, 5000])
+def test_rows_without_a_bag(binding, d, r, rows):  # noqa: F811
+    # every other row of 2 x rows in bags, three times each; lookups of all rows in none
+    spec = TableSpec(N=10_400, n=(21, 22, 23), d=d, r=r, alpha=1.0, core_dist="normal", core_scale=0.3)
+    B = 50
+    rng = np.random.default_rng(rows)
+    wl = workloads.custom([spec], B, 1, seed=4, with_grad=True)
+    kept = rng.permutation(np.repeat(2 * np.arange(rows) + 1, 3))
+    wl.indices = np.concatenate([kept, rng.permutation(10_400)]).astype(np.int64)
+    offsets = np.concatenate([[0], np.sort(rng.integers(0, len(kept) + 1, B - 1)), [len(kept)]]).astype(np.int64)
+    emb = binding.from_workload(wl, enable_backward=True)
+    check_gradients(binding, emb, wl, offsets, "kept")
