@@ -382,12 +382,14 @@ struct DePairs {
     uint32_t s, v;                 // row of the last position looked at; start of row s + 1 + lane
     uint32_t bag;
     float factor;
+    bool holes;                    // there may be rows without pairs
 
     __device__ __forceinline__ uint32_t start(uint32_t slot) const { return slot < U ? tt_seg_start(w, slot, U) : total; }
     __device__ __forceinline__ DePairs(const WsView& w_, int64_t chunk) : w(w_)
     {
         U = w.counters[CTR_LEVEL0 + w.K];
         total = w.cnt[U];
+        holes = *w.status & TT_EMB_STATUS_OFFSETS;
         const int64_t a64 = chunk << w.de_chunk_log;
         a = a64 < total ? (uint32_t)a64 : total;
         b = min(a + (1u << w.de_chunk_log), total);
@@ -443,15 +445,14 @@ struct DePairs {
             } else prev = s;
         }
     }
-    // bit j: position p + j starts another row than the one before it (j < n); rows without pairs (lookups that malformed offsets leave out) among
-    // them: false, `rows` then finds the rows, otherwise every start is one row further and s is the row of the last position
+    // bit j: position p + j starts another row than the one before it (j < n); where rows without pairs may be among them (lookups that
+    // malformed offsets leave out): false, `rows` then finds the rows, otherwise every start is one row further and s is the row of the last
+    // position
     __device__ __forceinline__ bool starts(uint32_t p, int n, unsigned& bits)
     {
-        const bool in = v - p < (uint32_t)n;
-        bits = __reduce_or_sync(0xffffffffu, in ? 1u << (v - p) : 0u);
-        const int k = __popc(bits);
-        if (k != __popc(__ballot_sync(0xffffffffu, in))) return false;
-        s += k;
+        bits = __reduce_or_sync(0xffffffffu, v - p < (uint32_t)n ? 1u << (v - p) : 0u);
+        if (holes) return false;
+        s += __popc(bits);
         return true;
     }
     // row of position p + lane (lane < n), all lanes: n positions from p on

@@ -61,3 +61,20 @@ def test_rows_without_a_bag(binding, d, r, rows):  # noqa: F811
     offsets = np.concatenate([[0], np.sort(rng.integers(0, len(kept) + 1, B - 1)), [len(kept)]]).astype(np.int64)
     emb = binding.from_workload(wl, enable_backward=True)
     check_gradients(binding, emb, wl, offsets, "kept")
+
+
+@pytest.mark.parametrize("d,r", SHAPES)
+def test_one_row_without_a_bag_in_every_batch(binding, d, r):  # noqa: F811
+    # rows looked up once, chunks of several batches of 32 sorted positions, a row without a bag behind another position of each batch
+    spec = TableSpec(N=175_000, n=(56, 56, 56), d=d, r=r, alpha=1.0, core_dist="normal", core_scale=0.3)
+    B = 2000
+    rng = np.random.default_rng(5)
+    wl = workloads.custom([spec], B, 1, seed=5, with_grad=True)
+    batches = 5200
+    without = np.array([33 * b + b // 2 % 32 + 1 for b in range(batches)])
+    kept = rng.permutation(np.setdiff1d(np.arange(33 * batches), without))
+    assert len(kept) == 32 * batches and without[-1] < 175_000
+    wl.indices = np.concatenate([kept, without]).astype(np.int64)
+    offsets = np.concatenate([[0], np.sort(rng.integers(0, len(kept) + 1, B - 1)), [len(kept)]]).astype(np.int64)
+    emb = binding.from_workload(wl, enable_backward=True)
+    check_gradients(binding, emb, wl, offsets, "kept")
