@@ -178,7 +178,8 @@ __host__ __device__ __forceinline__ bool tt_weighted(const WsView& w) { return w
 
 enum { CTR_LEVEL0 = 0 /* +k */, CTR_TLEVEL0 = 8 /* +k */, CTR_COST_TOTAL = 16, CTR_SCAN_TICKET = 32 /* tiles of the running scan that have reported */,
        CTR_POOL_NEXT = 34 /* next share of the lookups to be pooled (shares are handed out in order) */,
-       CTR_DIRECT = 40 /* k_direct: CTAs that have reported, their status bits; 1 where the last forward made no grouping, its batch, lookups, idx32 */ };
+       CTR_DIRECT = 40 /* k_direct: CTAs that have reported, their status bits; 1 where the last forward made no grouping, its batch, lookups,
+                          idx32; next bag, long bags (direct.cu): twelve words */ };
 
 struct tt_emb {
     int T, K, D;
