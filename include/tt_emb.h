@@ -245,10 +245,10 @@ int tt_emb_unpack_core(tt_emb_t h, int32_t table, int32_t core, const float* can
  * Device events: time of stage `stage` of the most recent call, in milliseconds, measured with CUDA
  * events recorded on the call's stream when timing is enabled.  SYNCHRONISES on the stage's end event.
  * Stages: 0 grouping, 1 schedule (empty where the prefix levels are small and one kernel makes them and the schedule:
- * then stage 0 is both), 2 contraction, 3 pooling (a small call that makes no grouping is stage 2 alone), 4 backward sort, 5 backward dE,
- * 6 backward contraction, 7 backward middle cores + reductions, 8 sgd; 9..20 the forward sweep kernel of shape
- * variant -1 (generic), 0..10; 21..32 the backward sweep kernel of the same variants (TT_EMB_ERR_STATE for a
- * variant no table uses).
+ * then stage 0 is both), 2 contraction, 3 pooling (a small call that makes no grouping is stage 2, the others are
+ * empty), 4 backward sort, 5 backward dE, 6 backward contraction, 7 backward middle cores + reductions, 8 sgd;
+ * 9..20 the forward sweep kernel of shape variant -1 (generic), 0..10; 21..32 the backward sweep kernel of the
+ * same variants (TT_EMB_ERR_STATE for a variant no table uses).
  * on = 0: no events; 1: events, normal execution; 2: events, and kernels of different shape variants, which
  * normally run side by side on forked streams, run one after the other, so that a per-kernel duration is that
  * kernel's alone (the step is slower in this mode; it is for per-kernel figures, not for throughput).

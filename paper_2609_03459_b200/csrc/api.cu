@@ -623,6 +623,9 @@ static int forward_any(tt_emb* h, const void* indices, bool idx32, const int64_t
     TT_CUDA(tt_launch_direct(h, out, &direct, s));
     if (direct) {
         if ((r = stage_end(h, 2, s))) return r;
+        for (int stage : {0, 1, 3}) TT_STAGE(h, stage, s, cudaSuccess);   // empty ones, and the sweeps
+        for (int i = 0; i <= TT_NUM_VARIANTS; ++i)
+            if (h->vcount[i]) TT_STAGE(h, 9 + i, s, cudaSuccess);
         h->have_forward = true;
         return TT_EMB_OK;
     }

@@ -164,3 +164,16 @@ def test_cores_of_more_than_2_to_the_32_floats(binding, big):  # noqa: F811
     ref = torch.stack([torch.einsum("pa,aqb,bs->pqs", cores[0][0, i].double(), cores[1][:, j].double(), cores[2][:, m, :, 0].double()).reshape(-1)
                        for i, j, m in digits])
     assert_close(out.cpu().numpy(), ref.cpu().numpy(), "out")
+
+
+def test_stage_times(binding):  # noqa: F811
+    # every stage of a forward has a time, as on the grouped path
+    wl = build((4, 4, 4), (1, 8, 8, 1), 64, 2, 1, seed=13)
+    times = []
+    for backward in (False, True):
+        emb = binding.from_workload(wl, enable_backward=backward)
+        emb.enable_timing()
+        emb.forward(dev(wl.indices), dev(wl.offsets), 64)
+        times.append(emb.stage_ms())
+        assert all(t >= 0 for t in times[-1].values())
+    assert set(times[0]) == set(times[1]) >= {"grouping", "schedule", "contraction", "pooling", "k_sweep_fwd<2>"}
