@@ -439,14 +439,12 @@ static cudaError_t make_side_streams(tt_emb* h, int n)
 
 // ------------------------------------------------------------------------------------------------ bind
 
-extern "C" int tt_emb_bind(tt_emb_t h, float* const* core_ptrs, void* workspace, size_t workspace_bytes,
-                           tt_emb_stream_t stream)
+int tt_bind(tt_emb* h, float* const* core_ptrs, void* workspace, size_t workspace_bytes, cudaStream_t s, bool make_streams)
 {
     if (!h || !core_ptrs) return TT_EMB_ERR_ARG;
     if (!workspace || workspace_bytes < h->ws_bytes || (reinterpret_cast<uintptr_t>(workspace) & 255)) return TT_EMB_ERR_WORKSPACE;
     int sms = 0;
     if (!tt_device_ok(&sms)) return TT_EMB_ERR_ARCH;
-    cudaStream_t s = (cudaStream_t)stream;
     h->cluster_ok = tt_group_cluster_ok();
     const int T = h->T, K = h->K;
     for (int t = 0; t < T; ++t)
@@ -515,10 +513,15 @@ extern "C" int tt_emb_bind(tt_emb_t h, float* const* core_ptrs, void* workspace,
         TT_CUDA(cudaMemcpyAsync(base + h->off_guard_list, list, sizeof(list), cudaMemcpyHostToDevice, s));
     }
     // every backward of four cores forks (tt_launch_bwd_contraction): its first call took 120 us longer with the stream made there
-    if (K == 4 && h->enable_backward) TT_CUDA(make_side_streams(h, 1));
+    if (make_streams && K == 4 && h->enable_backward) TT_CUDA(make_side_streams(h, 1));
     h->bound = true;
     h->have_forward = false;
     return TT_EMB_OK;
+}
+
+extern "C" int tt_emb_bind(tt_emb_t h, float* const* core_ptrs, void* workspace, size_t workspace_bytes, tt_emb_stream_t stream)
+{
+    return tt_bind(h, core_ptrs, workspace, workspace_bytes, (cudaStream_t)stream, true);
 }
 
 // ------------------------------------------------------------------------------------------------ timing helpers

@@ -241,6 +241,9 @@ void tt_set_last_cuda_error(cudaError_t e);
 // compute capability 10.x device current? (api.cu)
 int tt_device_ok(int* sm_count);
 
+// tt_emb_bind; make_streams: with the streams that every backward takes (api.cu)
+int tt_bind(tt_emb* h, float* const* core_ptrs, void* workspace, size_t workspace_bytes, cudaStream_t s, bool make_streams);
+
 // fork/join helpers (api.cu): side streams wait for everything enqueued on `s` so far / `s` waits for the side streams
 cudaError_t tt_fork(tt_emb* h, cudaStream_t s, int n);
 cudaError_t tt_join(tt_emb* h, cudaStream_t s, int n);

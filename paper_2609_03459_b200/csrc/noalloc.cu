@@ -62,7 +62,7 @@ extern "C" int tt_emb_forward_static(tt_emb_t h, float* const* core_ptrs, const 
         for (int k = 0; k < h->K; ++k)
             if (h->tab[t].core[k] != core_ptrs[t * h->K + k]) { same = false; break; }
     if (!same) {
-        rc = tt_emb_bind(h, core_ptrs, ws, (size_t)TT_EMB_STATIC_WORKSPACE_BYTES, stream);
+        rc = tt_bind(h, core_ptrs, ws, (size_t)TT_EMB_STATIC_WORKSPACE_BYTES, (cudaStream_t)stream, false);   // no streams for a backward
         if (rc != TT_EMB_OK) return rc;
     }
     return tt_emb_forward(h, indices, offsets, batch, num_lookups, out, stream);

@@ -50,3 +50,11 @@ def test_four_core_step(binding, shapes, lookups):  # noqa: F811
             emb.forward(ids, off, wl.B)
             emb.backward(grad)
         check(emb, f"serial={serial}")
+    # bound to the library's own workspace, which makes no streams, and then the backward, which needs one
+    emb = binding.TTEmbeddingBag([s.N for s in specs], [s.n for s in specs], [s.d for s in specs], [s.r for s in specs], wl.B, wl.L, enable_backward=True)
+    if emb.workspace_bytes <= binding.lib.tt_emb_static_workspace_limit():
+        bound = binding.from_workload(wl, enable_backward=True)
+        emb.cores, emb.grads = bound.cores, bound.grads
+        emb.forward_static(ids, off, wl.B)
+        emb.backward(grad)
+        check(emb, "static")
