@@ -2077,7 +2077,10 @@ cudaError_t tt_launch_bwd_contraction(tt_emb* h, cudaStream_t s)
     }
     cudaError_t e;
     // four cores: the digit-major list of level 2 is made beside the sweeps, as far as the scan's space is free (the segment starts are done
-    // with); the middle level waits for it.  Five short kernels on the way of the call otherwise: 65 k lookups, rank 64, call 380 to 367 us
+    // with); the middle level waits for it.  Five short kernels on the way of the call otherwise: 65 k lookups, rank 64, call 380 to 367 us.
+    // With several shape variants the first one's sweep follows the list on its stream.  The sweeps on the other streams only, backward, us,
+    // behind it / not: one table of rank 64 and one of any shape, 33 k lookups 230 / 246, a third of any shape 269 / 283; two of rank 64 and
+    // one of any shape, 12 k 176 / 166.
     if (h->K == 4 && !h->serial) {
         if ((e = tt_fork(h, s, 1)) != cudaSuccess) return e;
         if ((e = tt_launch_tlist(h, 2, h->side[0])) != cudaSuccess) return e;
