@@ -446,6 +446,7 @@ int tt_bind(tt_emb* h, float* const* core_ptrs, void* workspace, size_t workspac
     int sms = 0;
     if (!tt_device_ok(&sms)) return TT_EMB_ERR_ARCH;
     h->cluster_ok = tt_group_cluster_ok();
+    h->direct_ctas[0] = h->direct_ctas[1] = 0;      // the device may be another one: its attributes are set by the next call
     const int T = h->T, K = h->K;
     for (int t = 0; t < T; ++t)
         for (int k = 0; k < K; ++k) {

@@ -215,7 +215,7 @@ struct tt_emb {
     void* ws_base;
     bool warp_groups;     // every table is swept by warps that take groups one batch at a time (not by whole CTAs)
     int cluster_ok;       // the device takes the cluster of group_cluster.cu
-    int direct_ctas[2];   // resident CTAs per SM of k_direct without / with weights, 0: not asked yet
+    int direct_ctas[2];   // resident CTAs per SM of k_direct without / with weights, 0: not asked since the bind
     int pool_grid;        // CTAs of the pooling kernel (tt_plan_pooling)
     float* carry;         // workspace region of v.carry for chunks of TT_DE_CHUNK lookups
     size_t scan_tmp_elems;

@@ -881,7 +881,7 @@ cudaError_t tt_launch_direct(tt_emb* h, float* out, bool* launched, cudaStream_t
     auto kern = plan.kind == 3 ? (wt ? k_direct<3, true> : k_direct<3, false>) : plan.kind == 0 ? (wt ? k_direct<0, true> : k_direct<0, false>)
               : plan.kind == 1 ? (wt ? k_direct<1, true> : k_direct<1, false>) : (wt ? k_direct<2, true> : k_direct<2, false>);
     cudaError_t e;
-    int& per_sm = h->direct_ctas[wt];     // kernel and shared memory are those of the handle's tables: asked once
+    int& per_sm = h->direct_ctas[wt];     // kernel and shared memory are those of the handle's tables: asked once per bind
     if (per_sm == 0) {
         if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, DIRECT_MOST_SMEM + 32 * DIRECT_WARPS * (int)sizeof(float))) != cudaSuccess) return e;
         if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, DIRECT_THREADS, smem)) != cudaSuccess) return e;
