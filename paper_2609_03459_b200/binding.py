@@ -133,7 +133,10 @@ def make_config(num_rows: Sequence[int], row_factors: Sequence[Sequence[int]], d
 def _stream_ptr(stream=None) -> int:
     import torch
     if stream is None:   # without a Stream object, which took 3.6 of the 8.7 us that a small forward keeps the host
-        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+        raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)     # (not part of torch's interface)
+        if raw is not None:
+            return raw(torch.cuda.current_device())
+        stream = torch.cuda.current_stream()
     return int(stream.cuda_stream)
 
 
@@ -258,7 +261,7 @@ class TTEmbeddingBag:
         """CUDA graph of one forward on fixed buffers (same batch and number of lookups at every replay; the CONTENTS
         of `indices` / `offsets` may change between replays: grouping, schedule and all counts are computed on the
         device).  For launch-latency-bound small batches: replaying the graph saves the launch cost of its
-        kernels (3 to 18, and the level-2 products of four cores, by batch and table sizes).  Returns a torch.cuda.CUDAGraph; call .replay()."""
+        kernels (1 to 18, and the level-2 products of four cores, by batch and table sizes).  Returns a torch.cuda.CUDAGraph; call .replay()."""
         torch = self.torch
         self.forward(indices, offsets, batch, out=out)      # first call outside the capture: creates streams, sets attributes
         torch.cuda.synchronize()

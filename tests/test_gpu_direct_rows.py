@@ -166,6 +166,15 @@ def test_cores_of_more_than_2_to_the_32_floats(binding, big):  # noqa: F811
     assert_close(out.cpu().numpy(), ref.cpu().numpy(), "out")
 
 
+def test_current_stream_without_the_raw_handle(binding, monkeypatch):  # noqa: F811
+    # a torch that no longer has the call behind the shorter way
+    side = torch.cuda.Stream()
+    monkeypatch.delattr(torch._C, "_cuda_getCurrentRawStream")
+    for stream in (torch.cuda.default_stream(), side):
+        with torch.cuda.stream(stream):
+            assert binding._stream_ptr() == stream.cuda_stream
+
+
 def test_stage_times(binding):  # noqa: F811
     # every stage of a forward has a time, as on the grouped path
     wl = build((4, 4, 4), (1, 8, 8, 1), 64, 2, 1, seed=13)
