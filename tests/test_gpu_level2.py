@@ -25,7 +25,7 @@ def rows_by_definition(cores, n, ids):
 
 def handle(binding, n, d, r, lookups):  # noqa: F811
     import torch
-    emb = binding.TTEmbeddingBag([int(np.prod(n))], [n], [d], [r], lookups, lookups)
+    emb = binding.TTEmbeddingBag([int(np.prod(n))], [n], [d], [r], lookups, lookups, enable_backward=True)   # (grouped, however few lookups)
     shapes = [(r[k], n[k], d[k], r[k + 1]) for k in range(4)]
     g = torch.Generator(device="cuda").manual_seed(1)
     emb.set_cores([[torch.empty(s, device="cuda").normal_(generator=g) for s in shapes]])

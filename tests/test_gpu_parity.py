@@ -276,7 +276,7 @@ def test_short_bags_with_rows_outside_the_table(binding):
     t_of = np.searchsorted(wl.offsets[:: wl.B][1:], bad, side="right")
     idx[bad] = np.array([wl.tables[t].N for t in t_of]) + rng.integers(0, 5, size=bad.size)
     wl_bad = workloads.Workload(wl.name, wl.tables, wl.B, idx, wl.offsets, wl.cores, wl.grad_out)
-    emb, out = run_forward(binding, wl_bad)
+    emb, out = run_forward(binding, wl_bad, enable_backward=True)      # (the pooling of grouped rows)
     assert emb.status() & binding.STATUS_INDEX
     assert_close(out, oracle.forward_workload(wl_bad), "short bags with bad ids out")   # the oracle skips them as well
 
@@ -409,7 +409,7 @@ def test_forward_replayed_from_a_cuda_graph(binding):
     wl2 = workloads.custom(tables, B, 7, seed=32, name=name)      # same shapes and lookup count, other rows
     assert wl.L == wl2.L
     wl2.cores = wl.cores
-    emb = binding.from_workload(wl)
+    emb = binding.from_workload(wl, enable_backward=True)      # (a single kernel otherwise)
     d_idx, d_off = dev(wl.indices), dev(wl.offsets)
     out = torch.empty((wl.B, wl.T * wl.D), dtype=torch.float32, device="cuda")
     g = emb.capture_forward(d_idx, d_off, wl.B, out)
@@ -535,13 +535,14 @@ def test_bad_offsets_are_flagged_and_out_is_still_fully_written(binding, d):
     off = wl.offsets.copy()
     for b in (5, 77, 300, 301, 650):
         off[b], off[b + 1] = off[b + 1], off[b] - 1
-    emb = binding.from_workload(wl)
-    out = torch_full((wl.B, wl.D), float("nan"))
-    emb.forward(dev(wl.indices), dev(off), wl.B, out=out)
-    assert emb.status() & binding.STATUS_OFFSETS
     s = wl.tables[0]
     ref = oracle.forward(s.n, s.d, s.r, s.N, wl.cores[0], wl.indices, off)
-    assert_close(out.cpu().numpy(), ref, "out with malformed offsets")
+    for grouped in (False, True):
+        emb = binding.from_workload(wl, enable_backward=grouped)
+        out = torch_full((wl.B, wl.D), float("nan"))
+        emb.forward(dev(wl.indices), dev(off), wl.B, out=out)
+        assert emb.status() & binding.STATUS_OFFSETS
+        assert_close(out.cpu().numpy(), ref, "out with malformed offsets")
 
 
 def torch_full(shape, value):
@@ -612,7 +613,7 @@ def test_invariants_index_order_and_bag_additivity(binding):
     # results do not depend on the order of indices inside a bag; a bag holding two bags' lookups is their sum
     spec = TableSpec(20_000, (28, 28, 28), (4, 4, 4), (1, 8, 8, 1), 1.1, "normal", 0.1)
     wl = workloads.custom([spec], 64, 16, seed=9)
-    emb, out = run_forward(binding, wl)
+    emb, out = run_forward(binding, wl, enable_backward=True)
     rng = np.random.default_rng(1)
     perm = wl.indices.reshape(64, 16).copy()
     for b in range(64):

@@ -28,7 +28,7 @@ def test_grouping(binding, n, N, L):  # noqa: F811
     wl.indices = np.concatenate([rng.integers(0, N, L // 2), rng.choice(sparse, L // 4), np.full(L // 4, N - 1)]).astype(np.int64)
     M = len(wl.indices)
     wl.offsets = np.concatenate([[0], np.sort(rng.integers(0, M + 1, T * B - 1)), [M]]).astype(np.int64)
-    emb = binding.from_workload(wl)
+    emb = binding.from_workload(wl, enable_backward=True)      # (without it few lookups are not grouped)
     for _ in range(2):
         out = emb.forward(dev(wl.indices), dev(wl.offsets), B)
         assert emb.status() == 0
@@ -48,7 +48,7 @@ def test_row_scan_tiles(binding, T, N, L):  # noqa: F811
     wl.indices = np.where(rng.random(L) < 0.6, rng.integers(0, min(N, 33_000), L), rng.integers(0, N, L)).astype(np.int64)
     wl.indices[:2] = 0, N - 1
     wl.offsets = np.concatenate([[0], np.sort(rng.integers(0, L + 1, T * B - 1)), [L]]).astype(np.int64)
-    emb = binding.from_workload(wl)
+    emb = binding.from_workload(wl, enable_backward=True)      # (without it few lookups are not grouped)
     out = emb.forward(dev(wl.indices), dev(wl.offsets), B)
     assert emb.status() == 0
     check_grouping(emb, wl)

@@ -34,7 +34,8 @@ def _dev(a):
     return torch.from_numpy(np.ascontiguousarray(a)).cuda()
 
 
-def test_static_workspace_forward_matches_regular_forward_twice(binding):
+@pytest.mark.parametrize("backward", [False, True])      # lookup by lookup; grouped
+def test_static_workspace_forward_matches_regular_forward_twice(binding, backward):
     import torch
     tables = [TableSpec(30_000, (32, 32, 32), (4, 4, 4), (1, 32, 32, 1), 1.1, "normal", 0.05),
               TableSpec(9_000, (21, 21, 21), (4, 4, 4), (1, 16, 32, 1), 0.9, "normal", 0.05),
@@ -42,13 +43,13 @@ def test_static_workspace_forward_matches_regular_forward_twice(binding):
     wl_a = workloads.custom(tables, 200, (0, 25), seed=11)
     wl_b = workloads.custom(tables, 200, (0, 25), seed=12)
     wl_b.cores = wl_a.cores
-    emb = binding.from_workload(wl_a)                      # regular path: caller-provided workspace
+    emb = binding.from_workload(wl_a, enable_backward=backward)                      # regular path: caller-provided workspace
     assert emb.workspace_bytes <= binding.lib.tt_emb_static_workspace_limit()
     ref_a = emb.forward(_dev(wl_a.indices), _dev(wl_a.offsets), wl_a.B).cpu().numpy()
-    emb_b = binding.from_workload(wl_b)
+    emb_b = binding.from_workload(wl_b, enable_backward=backward)
     ref_b = emb_b.forward(_dev(wl_b.indices), _dev(wl_b.offsets), wl_b.B).cpu().numpy()
 
-    emb_s = binding.from_workload(wl_a if wl_a.L >= wl_b.L else wl_b)   # capacity for the larger batch
+    emb_s = binding.from_workload(wl_a if wl_a.L >= wl_b.L else wl_b, enable_backward=backward)   # capacity for the larger batch
     out1 = emb_s.forward_static(_dev(wl_a.indices), _dev(wl_a.offsets), wl_a.B).cpu().numpy()
     out2 = emb_s.forward_static(_dev(wl_b.indices), _dev(wl_b.offsets), wl_b.B).cpu().numpy()   # second call, other batch
     out3 = emb_s.forward_static(_dev(wl_a.indices), _dev(wl_a.offsets), wl_a.B).cpu().numpy()   # and the first again
