@@ -168,7 +168,8 @@ __global__ void __launch_bounds__(256) k_nodedup_levels(WsView w)
 // Mode 3 against 1, units of equal counts: 12 k words, 25 k lookups 199 / 168, 0.9 M 804 / 763, 14 k words, 0.8 M 683 / 624; 4 k to 8 k words,
 // 0.1 M to 0.6 M 0.96 to 0.99 of the call; 3.5 k words, 4 M 708.5 / 698.5; but 1.5 k words, 0.5 M 240.6 / 237.5 and 0.7 M 216.2 / 217.7, 1.3 k words, 0.3 M 388 / 391,
 // 7 k words, 31 k 229 / 233, 0.2 k words, 12 k 98 / 102, 0.3 M 276 / 279.  Equal costs: 8 k words, four cores, 0.5 M 326 / 331.
-// (8 k to 16 k words with 1 M to 2 M lookups stay with mode 1 only because its line at 2 M is what callers' launch counts have been held to.)
+// 9 k to 15 k words, 1.1 M to 2 M lookups, 28 calls of seven shapes, rank 8 to 32, popular rows first and spread: 0.93 to 0.98 of the forward
+// (155 / 143, 207 / 196, 431 / 403, 376 / 362), 0.97 to 0.99 of the training call (370 / 360, 1129 / 1101, 3620 / 3595).
 #define TT_CLUSTER_SCAN_WORDS (3u << 15)
 #define TT_CLUSTER_ANY_WORDS (1u << 13)
 #define TT_CLUSTER_LEVEL_WORDS (1u << 14)
@@ -192,8 +193,7 @@ static int tt_use_cluster(const tt_emb* h)
     for (int k = 1; k < w.K; ++k)
         if (w.total_words_l[k] > words) words = w.total_words_l[k];
     const bool few_words = words <= (w.L <= TT_CLUSTER_LEVEL_LOOKUPS ? TT_CLUSTER_LEVEL_WORDS : TT_CLUSTER_ANY_WORDS);
-    const bool spread = h->warp_groups && w.L >= (words >= 12288 ? 1 << 14 : words >= 3072 ? 1 << 15 : INT64_MAX) &&
-                        (words <= TT_CLUSTER_ANY_WORDS || w.L <= TT_CLUSTER_LEVEL_LOOKUPS / 2);
+    const bool spread = h->warp_groups && w.L >= (words >= 12288 ? 1 << 14 : words >= 3072 ? 1 << 15 : INT64_MAX);
     // (L <= capU: the digit-major list has room for all the prefixes that the row ids mark)
     if ((!few_words || spread) && words <= TT_CLUSTER_SCAN_WORDS && w.K >= 3 && w.L <= h->capU && tt_prefix_bits(h)) return 3;
     if (!few_words) return 0;

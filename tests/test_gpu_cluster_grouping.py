@@ -92,10 +92,12 @@ def test_schedule_by_cost_in_the_cluster(binding):  # noqa: F811
     assert_close(out.cpu().numpy(), oracle.forward_workload(wl), "out")
 
 
-@pytest.mark.parametrize("T,B,L,way", [(1, 1 << 18, 1000, 2), (1, (1 << 18) + 1, 1000, 1), (20, 64, 1 << 21, 1), (20, 64, (1 << 21) + 1, 0)])
-def test_many_offsets_and_many_lookups(binding, T, B, L, way):  # noqa: F811
+# tables swept by CTAs (ranks 8 and 12): from the prefix levels on up to 2 M lookups; tables swept by warps: the scans only (six launches)
+@pytest.mark.parametrize("T,B,L,rank,way", [(1, 1 << 18, 1000, 8, 2), (1, (1 << 18) + 1, 1000, 8, 1), (20, 64, 1 << 21, 12, 1), (20, 64, (1 << 21) + 1, 12, 0),
+                                            (20, 64, 1 << 21, 8, 0)])
+def test_many_offsets_and_many_lookups(binding, T, B, L, rank, way):  # noqa: F811
     N, n = (300_000, (67, 67, 67)) if T > 1 else (100_000, (47, 47, 47))      # 10 k words per level; 512
-    spec = TableSpec(N=N, n=n, d=(4, 4, 4), r=(1, 8, 8, 1), alpha=1.0, core_dist="normal", core_scale=0.3)
+    spec = TableSpec(N=N, n=n, d=(4, 4, 4), r=(1, 8, rank, 1), alpha=1.0, core_dist="normal", core_scale=0.3)
     wl = workloads.custom([spec] * T, B, 1, seed=2)
     rng = np.random.default_rng(L)
     wl.indices = rng.integers(0, N, L).astype(np.int64)
@@ -103,5 +105,5 @@ def test_many_offsets_and_many_lookups(binding, T, B, L, way):  # noqa: F811
     emb = binding.from_workload(wl)
     took, out = mode(binding, emb, dev(wl.indices), dev(wl.offsets), B)
     assert took == way and emb.status() == 0
-    if T == 1:
-        assert_close(out.cpu().numpy(), oracle.forward_workload(wl, memo=True), "out")
+    assert_close(out.cpu().numpy(), oracle.forward_workload(wl, memo=True), "out")
+    check_grouping(emb, wl)
