@@ -33,3 +33,28 @@ def test_rows_across_chunk_borders(binding, d, L, hot):  # noqa: F811
         for k in range(3):
             assert_close(grads[0][k], ref[0][k], f"dG[{k}]")
     assert emb.check_guards() is None and emb.status() == 0
+
+
+@pytest.mark.parametrize("d", [(2, 2, 4), (2, 4, 4), (4, 4, 4), (4, 8, 4), (3, 3, 5)])
+def test_pieces_around_half_a_chunk_and_blocks_of_32(binding, d):  # noqa: F811
+    # chunks of 32 positions (128 and more for rows of 128 floats): rows whose last piece is half a chunk, one more and one less; one piece, a
+    # block of 32 pieces, one more, 33 blocks; between rows that shift their first position
+    lens = [32 * k + off for k in (1, 2, 31, 32, 33) for off in (-17, -16, -15, -1, 0, 1, 15, 16, 17)] + [32 * 1024 + 5, 32 * 33 * 4, 128 * 32 - 64, 128 * 33 + 65]
+    rng = np.random.default_rng(d[1])
+    lens = np.concatenate([[x, s] for x, s in zip(rng.permutation(lens), rng.integers(1, 32, len(lens)))])
+    L = int(lens.sum())
+    assert len(lens) <= 120 and L < 1 << 17
+    wl = workloads.custom([TableSpec(N=120, n=(4, 5, 6), d=d, r=(1, 3, 2, 1), alpha=1.0, core_dist="normal", core_scale=0.3)], 16, 1, seed=L, with_grad=True)
+    wl.indices = rng.permutation(np.repeat(np.arange(len(lens)), lens)).astype(np.int64)
+    wl.offsets = np.concatenate([[0], np.sort(rng.integers(0, L + 1, 15)), [L]]).astype(np.int64)
+    weights = rng.random(L).astype(np.float32)
+    emb = binding.from_workload(wl, enable_backward=True, enable_weighted=True)
+    for wt in (None, weights):
+        emb.set_pooling("sum", None if wt is None else dev(wt))
+        for _ in range(3):      # (the warps arrive in another order)
+            emb.forward(dev(wl.indices), dev(wl.offsets), wl.B)
+            emb.backward(dev(wl.grad_out))
+            grads, ref = emb.get_grads(), oracle.backward_workload(wl, weights=wt)
+            for k in range(3):
+                assert_close(grads[0][k], ref[0][k], f"dG[{k}]")
+    assert emb.check_guards() is None and emb.status() == 0
