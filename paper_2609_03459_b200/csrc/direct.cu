@@ -790,6 +790,11 @@ static size_t direct_copy_bytes(const tt_emb* h) { return ((size_t)h->T * h->v.B
 //             ns; D = 128 4.8; four cores, rank 64 25), a bag 0.28 ns; and a warp makes its lookups one after the other (one table, 64 bags of 55
 //             lookups, eight warps each, rank 16 / 32 / 64: 17 / 48 / 445 us), a bag of 1.6 times the average length among them.
 //   grouped   36 to 84 us with 1 k lookups, by shape, and 0.28 ns for each of the others.
+//   shared    with at most 2.5 rows in the tables for a lookup: the grouped call once more, and `here` with it, fitted to calls near the
+//             line (1369 calls of 13 shapes, 1 to 40 tables of 300 to 40 M rows each, exponents 0.6 to 1.6).  Rank 8, us, here / grouped: eight tables
+//             of 3 k rows, 0.16 M lookups, 4x4x4 72 / 58, 2x4x4 68 / 56; four of 3 k, 66 k bags of one 69 / 53; sixteen, 0.13 M lookups 82 / 60.  Of
+//             these calls 76 took more than 1.02 of the grouped time (up to 1.4) without this term, 25 do with it (11 others would be faster here,
+//             1.02 to 1.23): how often the rows repeat only the ids say.
 // Near the line both take the same (4x4x4, rank 16: 107 k lookups 87 / 90; rank 8: 203 k 100 / 92; 2x2x4, rank 32: 107 k 102 / 105).
 // Warps of a bag: its lookups by eight, or by two where the bags are few.  With 1 / 2 / 4 / 8 warps, rank 16: bags of 1 lookup, 16 k
 // of them 26 / 42 / 78 / 152; of 1 to 20, 768 of them 24 / 17 / 18 / 17, 4096 51 / 43 / 45 / 59; of 1 to 100, 64 of them 92 / 48 / 26 / 17, 4096
@@ -842,6 +847,13 @@ static bool direct_plan(const tt_emb* h, DirectPlan& plan)
     const double chain = bag <= 1 ? 0 : 1.6 * bag / W * (0.6 + products / 5000);
     const double grouped = 38 + 0.28e-3 * (double)w.L + (products < 45000 ? products / 1500 : 30);
     if (lookups > grouped || chain > grouped) return false;
+    // The line above was drawn for rows spread over large tables.  With few rows for the lookups the grouped call is shorter.
+    if (rows <= 5 * w.L / 2) {
+        const double row = products > bytes / 1.5 ? products : bytes / 1.5;
+        const double shared = 52 + 0.08e-3 * (double)w.L + 0.05e-3 * (double)(w.L < rows ? w.L : rows) + 0.4 * h->T + (products < 45000 ? products / 1500 : 30);
+        const double here = 5 + (double)w.L * (0.26e-3 + (row > 1700 ? row : 1700) / 8.5e6 + (fast ? 0 : 0.5e-3)) + (double)nb * 0.4e-3;
+        if (here > shared) return false;
+    }
     // Long bags, and their pieces: a warp's share of an average bag and a quarter more at least, and long enough to be worth its claim and
     // its sum.  Twice as many in each of the bag's warps are left whole.  Pieces of 0.15 / 0.3 / 0.6 of the grouped time: rank 8, 57 k lookups in one bag 75 / 67 /
     // 84; 3x3x5, 10 k in one 70 / 94 / 146; rank 16, 20 k in one 72 / 72 / 86; power law, 46 k, rank 8 66 / 78 / 78.

@@ -166,6 +166,18 @@ def test_cores_of_more_than_2_to_the_32_floats(binding, big):  # noqa: F811
     assert_close(out.cpu().numpy(), ref.cpu().numpy(), "out")
 
 
+@pytest.mark.parametrize("T,rows,B,lens,direct", [(8, 3000, 400, (1, 100), False), (8, 3_000_000, 400, (1, 100), True), (16, 3000, 4096, (1, 3), False),
+                                                  (4, 3000, 16_384, 1, False), (4, 3000, 4096, 1, True),
+                                                  (4, 60_000, 16_384, 1, True)])
+def test_few_rows_are_shared(binding, T, rows, B, lens, direct):  # noqa: F811
+    n = (round(rows ** (1 / 3)) + 1,) * 3
+    wl = workloads.custom([TableSpec(N=rows, n=n, d=(2, 4, 4), r=(1, 8, 8, 1), alpha=0.8, core_dist="normal", core_scale=0.4)] * T, B, lens, seed=T)
+    emb = binding.from_workload(wl)
+    count, out = launches(binding, emb, dev(wl.indices), dev(wl.offsets), B)
+    assert (count == 1) == direct and emb.status() == 0
+    assert_close(out.cpu().numpy(), oracle.forward_workload(wl, memo=True), "out")
+
+
 def test_current_stream_without_the_raw_handle(binding, monkeypatch):  # noqa: F811
     # a torch that no longer has the call behind the shorter way
     side = torch.cuda.Stream()
