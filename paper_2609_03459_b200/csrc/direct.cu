@@ -790,7 +790,7 @@ static size_t direct_copy_bytes(const tt_emb* h) { return ((size_t)h->T * h->v.B
 //             ns; D = 128 4.8; four cores, rank 64 25), a bag 0.28 ns; and a warp makes its lookups one after the other (one table, 64 bags of 55
 //             lookups, eight warps each, rank 16 / 32 / 64: 17 / 48 / 445 us), a bag of 1.6 times the average length among them.
 //   grouped   36 to 84 us with 1 k lookups, by shape, and 0.28 ns for each of the others.
-//   shared    with at most 2.5 rows in the tables for a lookup: the grouped call once more, and `here` with it, fitted to calls near the
+//   shared    shapes with a kernel of their own, with at most 2.5 rows in the tables for a lookup: the grouped call once more, and `here` with it, fitted to calls near the
 //             line (1369 calls of 13 shapes, 1 to 40 tables of 300 to 40 M rows each, exponents 0.6 to 1.6).  Rank 8, us, here / grouped: eight tables
 //             of 3 k rows, 0.16 M lookups, 4x4x4 72 / 58, 2x4x4 68 / 56; four of 3 k, 66 k bags of one 69 / 53; sixteen, 0.13 M lookups 82 / 60.  Of
 //             these calls 76 took more than 1.02 of the grouped time (up to 1.4) without this term, 25 do with it (11 others would be faster here,
@@ -848,10 +848,10 @@ static bool direct_plan(const tt_emb* h, DirectPlan& plan)
     const double grouped = 38 + 0.28e-3 * (double)w.L + (products < 45000 ? products / 1500 : 30);
     if (lookups > grouped || chain > grouped) return false;
     // The line above was drawn for rows spread over large tables.  With few rows for the lookups the grouped call is shorter.
-    if (rows <= 5 * w.L / 2) {
+    if (fast && rows <= 5 * w.L / 2) {
         const double row = products > bytes / 1.5 ? products : bytes / 1.5;
         const double shared = 52 + 0.08e-3 * (double)w.L + 0.05e-3 * (double)(w.L < rows ? w.L : rows) + 0.4 * h->T + (products < 45000 ? products / 1500 : 30);
-        const double here = 5 + (double)w.L * (0.26e-3 + (row > 1700 ? row : 1700) / 8.5e6 + (fast ? 0 : 0.5e-3)) + (double)nb * 0.4e-3;
+        const double here = 5 + (double)w.L * (0.26e-3 + (row > 1700 ? row : 1700) / 8.5e6) + (double)nb * 0.4e-3;
         if (here > shared) return false;
     }
     // Long bags, and their pieces: a warp's share of an average bag and a quarter more at least, and long enough to be worth its claim and

@@ -166,12 +166,16 @@ def test_cores_of_more_than_2_to_the_32_floats(binding, big):  # noqa: F811
     assert_close(out.cpu().numpy(), ref.cpu().numpy(), "out")
 
 
-@pytest.mark.parametrize("T,rows,B,lens,direct", [(8, 3000, 400, (1, 100), False), (8, 3_000_000, 400, (1, 100), True), (16, 3000, 4096, (1, 3), False),
-                                                  (4, 3000, 16_384, 1, False), (4, 3000, 4096, 1, True),
-                                                  (4, 60_000, 16_384, 1, True)])
-def test_few_rows_are_shared(binding, T, rows, B, lens, direct):  # noqa: F811
+R8, ANY = ((2, 4, 4), (1, 8, 8, 1)), ((3, 3, 5), (1, 6, 4, 1))
+
+
+@pytest.mark.parametrize("shape,T,rows,B,lens,direct", [
+    (R8, 8, 3000, 400, (1, 100), False), (R8, 8, 3_000_000, 400, (1, 100), True), (R8, 16, 3000, 4096, (1, 3), False), (R8, 4, 3000, 16_384, 1, False),
+    (R8, 4, 3000, 4096, 1, True), (R8, 4, 60_000, 16_384, 1, True), (ANY, 1, 60_000, 20_000, (0, 5), True)])
+def test_few_rows_are_shared(binding, shape, T, rows, B, lens, direct):  # noqa: F811
     n = (round(rows ** (1 / 3)) + 1,) * 3
-    wl = workloads.custom([TableSpec(N=rows, n=n, d=(2, 4, 4), r=(1, 8, 8, 1), alpha=0.8, core_dist="normal", core_scale=0.4)] * T, B, lens, seed=T)
+    spec = TableSpec(N=rows, n=n, d=shape[0], r=shape[1], alpha=0.8, core_dist="normal", core_scale=0.4)
+    wl = workloads.custom([spec] * T, B, lens, seed=T)
     emb = binding.from_workload(wl)
     count, out = launches(binding, emb, dev(wl.indices), dev(wl.offsets), B)
     assert (count == 1) == direct and emb.status() == 0
