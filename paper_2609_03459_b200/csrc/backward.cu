@@ -1883,7 +1883,7 @@ __global__ void __launch_bounds__(WIDE_THREADS, 2) k_sweep_bwd_wide(WsView w, in
     extern __shared__ __align__(16) float sm[];
     __shared__ WideBatch batches[2];
     float *Bs = sm, *As = Bs + 64 * WIDE_BP, *Cs = As + 8 * WIDE_GROUPS * WIDE_AP;
-    const int t = w.vlist[vbase + blockIdx.y], K = w.K, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int t = w.vlist[vbase + (FEW ? blockIdx.x : blockIdx.y)], K = w.K, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const TableDesc& td = w.tdesc[t];
     uint32_t step;
     const uint2 rng = tt_sweep_unit<FEW>(w, t, WIDE_GROUPS, step);
@@ -1973,7 +1973,7 @@ __global__ void __launch_bounds__(128, V == 5 ? 6 : V == 1 || V == 8 ? 4 : V == 
 {
     tt_pdl_enter();
     extern __shared__ __align__(16) float sm[];
-    const int t = w.vlist[vbase + blockIdx.y];
+    const int t = w.vlist[vbase + (FEW ? blockIdx.x : blockIdx.y)];
     const TableDesc& td = w.tdesc[t];
     const int stripe = (blockIdx.x + blockIdx.y) % TT_STRIPES;
     float* gk = w.gpart + (size_t)stripe * w.gpart_stride + td.gpart_off;
@@ -2052,11 +2052,11 @@ static cudaError_t launch_sweep_bwd(tt_emb* h, int max_pl, int max_c, cudaStream
     } else if constexpr (V == 4) {
         auto kern = few ? k_sweep_bwd_wide<true> : k_sweep_bwd_wide<false>;
         if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)WIDE_SMEM)) != cudaSuccess) return e;
-        if ((e = tt_launch_pdl(kern, dim3(few ? h->sweep_ctas : h->units_per_table, n), dim3(WIDE_THREADS), WIDE_SMEM, s, h->v, h->vbase[V + 1])) != cudaSuccess) return e;
+        if ((e = tt_launch_pdl(kern, few ? dim3(n, h->sweep_ctas) : dim3(h->units_per_table, n), dim3(WIDE_THREADS), WIDE_SMEM, s, h->v, h->vbase[V + 1])) != cudaSuccess) return e;
     } else {
         auto kern = few ? k_sweep_bwd<V, true> : k_sweep_bwd<V, false>;
         if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
-        if ((e = tt_launch_pdl(kern, dim3(few ? h->sweep_ctas : h->units_per_table, n), dim3(128), smem, s, h->v, max_pl, max_c, h->vbase[V + 1])) != cudaSuccess) return e;
+        if ((e = tt_launch_pdl(kern, few ? dim3(n, h->sweep_ctas) : dim3(h->units_per_table, n), dim3(128), smem, s, h->v, max_pl, max_c, h->vbase[V + 1])) != cudaSuccess) return e;
     }
     tt_note_launch();
     if ((e = tt_stage_end(h, 9 + TT_NUM_VARIANTS + 1 + V + 1, s)) != cudaSuccess) return e;

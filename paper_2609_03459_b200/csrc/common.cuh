@@ -54,9 +54,11 @@
 // schedule's units and so cut: D = 128, rank 32, 1.0 k groups 180 / 96 and 23 / 19; D = 32, rank 32, 0.8 k 52 / 59 and 19 / 23; rank 16,
 // 1.2 k 28 / 43 and 17 / 23; four cores, 0.5 k 56 / 70 and 29 / 37.  Limits of 4 / 8 / 12: 150 drawn calls 0.965 / 0.961 / 0.959 of
 // their time (geometric mean), but above 8 cheap and dear groups in equal parts cost some 3 %.  Six CTAs per SM: as four.
-// The kernels that can do this take 1 % longer where there are more groups after all (a step in shared memory, spills), so they are
-// launched where at most TT_FEW_MAYBE times as many are possible by the lookups and the tables (8 times: 4 tables, D = 128, rank 32, 30 k
-// possible, 0.14 M lookups, training call 616 without, 638 with them; no drawn call with that many possible had few).
+// The kernels that can do this have more CTAs than there are units, so theirs go table by table first: the CTAs without work are the last.
+// (Unit by unit first, as the others', a table's idle CTAs held up the next one's: 4 tables, D = 128, rank 32, 9 k groups, forward sweep 123
+// us, 98 now, 88 without the extra CTAs; D = 16 and 64, rank 32, 5 k groups 36 and 43 / 29 and 35 / 29 and 35.)  They are launched where at most
+// TT_FEW_MAYBE times as many groups are possible by the lookups and the tables: 8 times, 4 tables, D = 128, rank 32, 30 k possible, 0.14 M lookups,
+// training call 616 without, 638 with them; no drawn call with that many possible had few.
 #define TT_FEW_UNITS 4
 #define TT_FEW_GROUPS 4
 #define TT_FEW_LIMIT 8
@@ -452,7 +454,7 @@ __device__ __forceinline__ uint2 tt_sweep_unit(const WsView& w, int t, uint32_t 
 {
     step = ng;
     if (!FEW) return w.unit_rng[t * w.units_per_table + blockIdx.x];
-    const uint32_t q = blockIdx.x, Q = w.units_per_table, total = w.tb[w.K - 1][w.T], a = w.tb[w.K - 1][t], n = w.tb[w.K - 1][t + 1] - a;
+    const uint32_t q = blockIdx.y, Q = w.units_per_table, total = w.tb[w.K - 1][w.T], a = w.tb[w.K - 1][t], n = w.tb[w.K - 1][t + 1] - a;
     const uint2 unit = w.unit_rng[t * Q + min(q, Q - 1)];
     const bool few = total < w.few_units * TT_FEW_LIMIT, none = q >= Q;
     const uint32_t per = max(max((uint32_t)TT_FEW_GROUPS, __float2uint_ru((float)total * w.few_share)), __float2uint_ru((float)n * w.cta_share) + 1);
