@@ -172,7 +172,7 @@ __global__ void __launch_bounds__(256) k_nodedup_levels(WsView w)
 // (155 / 143, 207 / 196, 431 / 403, 376 / 362), 0.97 to 0.99 of the training call (370 / 360, 1129 / 1101, 3620 / 3595).
 // All that by words of whole scan tiles; with few words in them (TT_CLUSTER_SPREAD_WORDS, the possible prefixes alone) mode 1 is the shorter: rank 32, mode
 // 1 / 3, forward, us: 0.25 k words, 0.16 M lookups 91.3 / 93.3; 0.5 k, 0.16 M 96.4 / 97.4, 97.8 / 96.7, 0.5 M 130 / 127.5; 0.8 k, 70 k 94.6 / 93.1, 0.16 M 107.5 / 105.2; 1.3 k,
-// 0.16 M 130 / 125.
+// 0.16 M 130 / 125.  (Not past 12 k words of whole tiles, where mode 2 would have the fewer lookups: 32 tables of 2 k rows, 25 k, training 127 / 111.)
 #define TT_CLUSTER_SCAN_WORDS (3u << 15)
 #define TT_CLUSTER_SPREAD_WORDS 512u
 #define TT_CLUSTER_ANY_WORDS (1u << 13)
@@ -197,8 +197,8 @@ static int tt_use_cluster(const tt_emb* h)
     for (int k = 1; k < w.K; ++k)
         if (w.total_words_l[k] > words) words = w.total_words_l[k];
     const bool few_words = words <= (w.L <= TT_CLUSTER_LEVEL_LOOKUPS ? TT_CLUSTER_LEVEL_WORDS : TT_CLUSTER_ANY_WORDS);
-    const bool spread = h->warp_groups && w.L >= (words >= 12288 ? 1 << 14 : words >= 3072 ? 1 << 15 : INT64_MAX) && w.K >= 3 &&
-                        w.ttotal_words[w.K - 1] >= TT_CLUSTER_SPREAD_WORDS;
+    const bool spread = h->warp_groups && w.K >= 3 &&
+                        (words >= 12288 ? w.L >= 1 << 14 : words >= 3072 && w.L >= 1 << 15 && w.ttotal_words[w.K - 1] >= TT_CLUSTER_SPREAD_WORDS);
     // (L <= capU: the digit-major list has room for all the prefixes that the row ids mark)
     if ((!few_words || spread) && words <= TT_CLUSTER_SCAN_WORDS && w.K >= 3 && w.L <= h->capU && tt_prefix_bits(h)) return 3;
     if (!few_words) return 0;
